@@ -97,11 +97,11 @@ typedef enum rimo_n_weight {
  *                     plan and interpolated by cubic Lagrange polynomials in w_r when tiles
  *                     are built or generated (n >= 16; 8192 keeps the interpolation error
  *                     near 1e-8 relative at the 4096^2 / 50M workload).
- *   uv_order          order of the visibilities within a uv-tile, which sets the groups of
- *                     GTG_CHUNK (20) visibilities the grid step de-grids and grids at once
- *                     (a scheduling choice of this design, no counterpart in the paper):
+ *   uv_order          order of the visibilities within a uv-tile, which sets those that the
+ *                     grid step's warps de-grid and grid at about the same time (a
+ *                     scheduling choice of this design, no counterpart in the paper):
  *                     0 = time-interleaved (the tile's list in time order read as 20 rows,
- *                     column by column: a group's visibilities come from far-apart instants
+ *                     column by column: neighbours in the order come from far-apart instants
  *                     and rarely update the same grid cells; default), 1 = time order,
  *                     2 = shuffled by a counter-based SplitMix64 hash of the visibility
  *                     index.  Results agree within rounding (the grid step sums exactly
@@ -431,13 +431,13 @@ rimo_status rimo_plan_status(rimo_plan_t plan, void* stream);
 /*
  * Failure-detection test of the device-side bounded waits (no counterpart in the paper;
  * the paper's workers fail on the host).  With stall = 1, the grid-step launches of this
- * plan's following applies run with their consumer warps never releasing a ring slot of
- * taps to the producer warp (a flag that nothing sets), and the producer's waits on the
- * other warps limited to `polls` (1 .. 32768) suspended polls of at most 100 us.  A block
- * whose producer has to reuse a slot then gives up: it records RIMO_ERR_TIMEOUT in the
- * plan's status, waits (with the normal bound) for its own bulk copies in flight, and
- * returns, and its consumer warps stop waiting for chunks that will not come.  Results of
- * applies made with stall = 1 are invalid; rimo_plan_status reports the timeout.
+ * plan's following applies fill each slot of their tap rings once and never again, and
+ * their waits for taps are limited to `polls` (1 .. 32768) suspended polls of at most
+ * 100 us.  A warp whose next visibility would need a slot a second time then gives up: it
+ * records RIMO_ERR_TIMEOUT in the plan's status, its block ends at the next unit boundary,
+ * and every warp waits (with the normal bound) for its own copies in flight before it
+ * returns.  Results of applies made with stall = 1 are invalid; rimo_plan_status reports the
+ * timeout.
  * stall = 0 (polls ignored) restores normal operation.  Host-only call.
  * Errors: INVALID_ARG.
  */

@@ -6,20 +6,26 @@
 // holding their first grid cell, and their taps are stored tile after tile, so the
 // taps of consecutive visibilities of a tile are one contiguous byte range.
 //
-// Kernel.  Persistent thread blocks (one per SM) take work units (a uv-tile, or a slice
-// of a heavy one) from a heaviest-first schedule: for plans of dense units (8 chunks of
-// visibilities or more on average, X patches prefetched) the next one through an atomic
-// counter (a block that started late or drew light units takes more; 26.31 -> 25.10 ms per
-// 4096^2/50M apply against a fixed snake order), else in the snake order.  For a unit,
-// the block stages the box of grid cells its visibilities' footprints reach (within the
-// (TS + H)^2 patch, H = largest tile side - 1) in shared memory while a producer warp
-// streams the taps of GTG_CHUNK visibilities at a time with bulk asynchronous copies
-// (cp.async.bulk, completion on an mbarrier) through a shared-memory ring of up to
-// GTG_NBUF chunks.
-//   de-grid : one warp per visibility reads its S x S taps from shared memory (lanes = two
-//             rows of 16 columns), gathers the patch and reduces y_k with warp shuffles;
-//   grid    : the same warp adds conj(taps) y_k into the block's shared accumulator patch
-//             (shared-memory atomic adds: visibilities of different warps may overlap).
+// Kernel.  Persistent thread blocks take work units (a uv-tile, or a slice of a heavy one)
+// from a heaviest-first list through an atomic counter.  For a unit, the block stages the
+// box of grid cells its visibilities' footprints reach (within the (TS + H)^2 patch, H =
+// largest tile side - 1) in shared memory, and its warps take the unit's visibilities round
+// robin, each from a ring of its own:
+//   de-grid : the warp reads the visibility's S x S taps from its ring slot (half a warp per
+//             tile row), gathers the patch and reduces y_k with warp shuffles;
+//   grid    : it adds conj(taps) y_k into the block's shared accumulator patch (shared-memory
+//             integer reductions: visibilities of different warps may overlap);
+//   refill  : it starts the bulk copy (cp.async.bulk, completion on an mbarrier of the slot)
+//             of the visibility after the next one, across the unit's end if need be.
+// Blocks only synchronise at unit boundaries, and two or three blocks per SM hide each other's.
+// What bounds it: with full units (512^2 / 2M visibilities / 4 bins, 488 per unit) the
+// instruction stream (335 per visibility, 72 % of the issue slots) and the shared-memory
+// pipe (82 wavefronts per visibility, 73 % busy); with small units (1024^2 / 2M / 16 bins, 38
+// per unit) their boundaries.  Against one block of 20 visibility warps fed by a producer
+// warp through a common ring of 20-visibility chunks (386 instructions and 90 wavefronts per
+// visibility, a unit's descriptors and the rows of its X box fetched one after the other):
+// 512^2 case 1.06 -> 0.89 ms, 1024^2 de-grid 2.46 -> 0.82 ms and grid 1.86 -> 1.17 ms,
+// 4096^2 / 24M / 32 bins 15.4 -> 10.3 ms per apply.
 // The finished accumulator box is written once to the unit's slot of the patch buffer
 // (slices of a split tile are then added into its first slot); the fold of the inverse
 // transform sums the overlapping halos of neighbouring patches tile by tile, so the gridded
@@ -30,9 +36,6 @@
 #include "internal.h"
 
 namespace rimo {
-
-// e / S for e < 400, S <= 19 by multiply-shift with ceil(2^16 / S)
-__device__ __forceinline__ int div_small(int e, int magic) { return (e * magic) >> 16; }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* ptr) {
     return (uint32_t)__cvta_generic_to_shared(ptr);
@@ -68,16 +71,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
-// The consumers' bounded wait, which also gives up once the block has abandoned the launch
-// (the producer stops issuing chunks after a failed wait of its own).
-__device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort) {
-    for (uint32_t it = 0; it < WAIT_POLLS; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (*abort) return false;
-    }
-    return false;
-}
-
 // Bulk asynchronous copy global -> shared (16-byte aligned, size a multiple of 16).
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile(
@@ -87,71 +80,68 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
         : "memory");
 }
 
-constexpr int GTG_CONSUMERS = GTG_CHUNK;                 // consumer warps
-constexpr int GTG_THREADS = (GTG_CONSUMERS + 1) * 32;   // + one producer warp
-constexpr int GTG_NBUF = 4;   // maximum depth of the tap ring (the plan may use fewer)
-constexpr int GTG_NX = 3;     // maximum number of X patch buffers (prefetch NX - 1 units ahead)
-constexpr int GTG_HDR = 256;  // shared-memory header: the ring's and the X buffers' mbarriers
-constexpr int GTG_CV = GTG_CHUNK;  // visibilities per chunk (one per consumer warp)
+// Asynchronous 16-byte copy global -> shared of this thread (cp.async group).
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// The per-bin side of a grid-step launch: one (plan, w-bin) job.
-struct GtgJob {
-    const TileDesc* units;  // the bin's work units, in patch-slot order
-    const ChunkDesc* chunks;
-    const VisMeta* meta;
-    const float2* const* gblk;
-    const float2* X;        // forward grid [gx][gy]
-    float2* patch;          // accumulator patch per unit slot
-    const uint32_t* fx;     // fixed-point bounds (tap bounds; maxterm of a Phi^dagger apply)
-    const uint8_t* need;    // [tile] of this bin: some footprint reaches the tile
-    int* status;            // the plan's device status word
-    int PW;                 // the plan's patch side (TS + largest tile side - 1)
-};
+constexpr int GTG_MAX_WARPS = 24;  // warps per block (all of them take visibilities)
+constexpr int GTG_SLOTS = 2;       // tap-ring slots of a warp
+constexpr int GTG_RECS = 4;        // ring of unit records
+constexpr int GTG_HDR = GTG_MAX_WARPS * GTG_SLOTS * 8 + GTG_RECS * 64;  // mbarriers, unit records
+constexpr int GTG_TAIL = 256;      // the last slot's tile may be read past its end (lanes beyond its columns)
 
 struct GtgArgs {
-    GtgJob one;             // a one-bin launch: the bin
-    const int* sched;       //   its unit slots, heaviest first
-    const GtgJob* jobs;     // a stage-batched launch: every (plan, bin) of the batch
-    const int2* queue;      //   (job, unit slot) of every unit of every job, heaviest first
-    int nunits;             // units of the launch (schedule or queue length)
-    int* counter;           // dynamic schedule: the next unit to take (zero at launch), or null
+    const UnitRec* recs;    // the launch's units, heaviest first
+    int nunits;
+    int* counter;           // units taken beyond the blocks' first GTG_AHEAD (zero at launch)
+    const float2* X;        // forward grid [gx][gy] and patches of a one-bin launch (null when
+    float2* patch;          //   the records hold the addresses of several jobs)
     const float2* y_in;
     float2* y_out;
-    int gx, gy, TS, PW;
-    int chunk_bytes;
-    int nbuf;               // ring depth in use, 2..GTG_NBUF
-    int ntv, shift;
-    int prefetch;           // the producer bulk-copies the X patches of the next units
-    int xbufs;              // X patch buffers with prefetch (2 or 3: 1 or 2 units ahead)
-    // failure-detection test (rimo_plan_set_wait_test): the consumers withhold their release
-    // of ring slots, and the producer's waits on the consumers give up after peer_polls
+    int gx, gy, TS, PW, pitch;
+    int slot_bytes;         // taps of the largest tile
+    int xbufs;              // X patch buffers: 2 (the next unit's is copied during this one) or 1
+    // failure-detection test (rimo_plan_set_wait_test): ring slots are filled once and never
+    // again, and the waits for taps give up after `polls`
     int stall;
-    uint32_t peer_polls;    // poll limit of the producer's waits on other warps (empty, xfree)
+    uint32_t polls;
 };
+constexpr int GTG_AHEAD = 2;  // units a block takes by its index; the later ones one round ahead
 
-// The job and the patch slot of the launch's unit idx.
-template <bool TABLE>
-__device__ __forceinline__ const GtgJob* unit_job(const GtgArgs& A, int idx, int& slot) {
-    if constexpr (TABLE) {
-        const int2 q = A.queue[idx];
-        slot = q.y;
-        return A.jobs + q.x;
-    } else {
-        slot = A.sched[idx];
-        return &A.one;
-    }
+// Row pitch of the accumulator planes for patches of side PW and tiles of side max_S: the rows
+// one instruction adds to (32 / CW rows of CW lanes, see vis_tile) fall in different banks.
+__host__ __device__ constexpr int pitch_of(int PW, int max_S = 15) {
+    return max_S <= 8 ? PW + (40 - PW % 16) % 16      // 8 modulo 16: four rows of 8 lanes
+         : max_S <= 16 ? PW + (48 - PW % 32) % 32     // 16 modulo 32: two rows of 16
+                       : PW;
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+// Two FP32 numbers in one 64-bit register pair (packed arithmetic: the same roundings as two
+// scalar instructions in one issue slot).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
 }
-
-__device__ __forceinline__ void consumers_sync() {
-    asm volatile("bar.sync 1, %0;" ::"n"(GTG_CONSUMERS * 32) : "memory");
+__device__ __forceinline__ float2 upk(f32x2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
 }
-
-// unit processed by block c in round r: snake order over the heaviest-first schedule
-__device__ __forceinline__ int unit_of(int r, int c, int G) { return r * G + ((r & 1) ? (G - 1 - c) : c); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 
 // rint by the 1.5 x 2^23 shift: for |d| < 2^22, d + FX_MAGIC has unit spacing, so its bits
 // minus those of FX_MAGIC are rint(d) (round to nearest even)
@@ -172,398 +162,420 @@ __device__ __forceinline__ void fx_scale(float maxterm, int64_t n, float& s1, fl
 }
 
 // One visibility by one warp, tile side S known at compile time.
-// Lane = (cell column, component): lane 2c + k handles column c of a tap row and the real
-// (k = 0) or imaginary (k = 1) part, so one instruction covers one row of up to 16 cells
-// (two rows of up to 8 cells when S <= 8): the shared-memory loads of a row are 16
-// consecutive complex cells and each grid-step reduction 32 consecutive words, both free
-// of bank conflicts.  With a = (t.x, t.y)[k], b = (t.y, t.x)[k]:
-//   de-grid:  Re(t x) = sum a x.x - sum b x.y  (k = 0),  Im(t x) = sum a x.x + sum b x.y  (k = 1);
-//   grid:     component k of conj(t) y = a (+-y.x) + b y.y  (sign + for k = 0, - for k = 1),
-//             times the unit's scale s1, added to the fixed-point patch words hi / lo with
-//             32-bit integer reductions.
-// Both parity classes of lanes reduce with four butterfly steps; one more exchange gives
-// every lane y.  Taps stay in registers between the two steps when S <= 16.
+// Lane = cell: CW lanes hold the columns of a tile row (half a warp for the common sides 9 to
+// 15), so one instruction covers 32 / CW rows.  A tap and a patch cell are one 64-bit shared
+// load each (consecutive lanes, consecutive cells), and the four accumulator planes (real and
+// imaginary parts of the words hi and lo) have a row pitch that spreads the rows of one
+// instruction over all 32 banks, so a reduction of 30 of 32 lanes is one wavefront.
+//   de-grid:  y = sum t x : the pair (Re t Re x, Im t Im x) by one packed multiply-add, the
+//             imaginary part by two scalar ones;
+//   grid:     conj(t) y s1 (s1 the unit's scale), split into the two integer words with packed
+//             arithmetic on the pair (real, imaginary).
+// Lanes past the last column or row hold no tap: they are cleared from y's sum and do not
+// add to the patch.  Taps stay in registers between the two steps.  Against one lane per
+// (column, component) with scalar arithmetic: 21 instructions and 8 shared-memory wavefronts
+// per two tile rows instead of 30 and 10.
 template <int S, int MODE, int PWC>  // PWC: the patch side when known at compile time, else 0
-__device__ __forceinline__ void vis_tile(const float2* __restrict__ T, const float2* __restrict__ Xs,
-                                         int* Ahi, int* Alo, float s1, int pbase, int PWr, int lane, uint32_t orig,
-                                         const float2* __restrict__ y_in, float2* __restrict__ y_out) {
-    const int PW = PWC > 0 ? PWC : PWr;  // compile-time row strides fold into the address offsets
+__device__ __forceinline__ void vis_tile(const float2* __restrict__ T, const float2* __restrict__ Xs, int* acc,
+                                         float s1, int du, int dv, int PWr, int pitchr, int planer, int lane,
+                                         uint32_t orig, float2 y, float2* __restrict__ y_out) {
+    // compile-time strides fold into the address offsets
+    const int PW = PWC > 0 ? PWC : PWr, pitch = PWC > 0 ? pitch_of(PWC) : pitchr;
+    const int plane = PWC > 0 ? PWC * pitch_of(PWC) : planer;
     constexpr bool GATHER = MODE != 1, SCATTER = MODE != 0;
-    constexpr int RPI = S <= 8 ? 2 : 1;         // tap rows per instruction
-    constexpr int CW = 16 / RPI;                // cells per row and instruction
-    constexpr int NCG = (S + CW - 1) / CW;      // column groups
-    constexpr int NI = (S + RPI - 1) / RPI;     // row steps
-    constexpr bool KEEP = NI * NCG <= 16;       // keep (a, b) in registers for the grid step
-    const int k = lane & 1;
-    const int c = (lane % (2 * CW)) >> 1;
-    const int roff = lane / (2 * CW);
-    // lane k reads its tap as (component k, component 1 - k): no select on the pair
-    const float* Tl = reinterpret_cast<const float*>(T + roff * S + c) + k;
-    const int tsw = 1 - 2 * k;  // offset of the other component
-    const int xl = pbase + roff * PW + c;
-    float2 ab[KEEP ? NI : 1][KEEP ? NCG : 1];
-    float acc1 = 0.f, acc2 = 0.f;
+    constexpr int CW = S <= 8 ? 8 : (S <= 16 ? 16 : 32);  // lanes per tile row
+    constexpr int RPI = 32 / CW;                          // rows per instruction
+    constexpr int NI = (S + RPI - 1) / RPI;               // row steps
+    const int c = lane % CW, ro = lane / CW;
+    const bool row_ok = (NI - 1) * RPI + ro < S;          // the last step's row exists
+    const f32x2* Tl = reinterpret_cast<const f32x2*>(T) + ro * S + c;
+    const f32x2* Xl = reinterpret_cast<const f32x2*>(Xs) + (du + ro) * PW + dv + c;
+    f32x2 t[NI];
+    f32x2 p = 0ull;
+    float q1 = 0.f, q2 = 0.f;
 #pragma unroll
-    for (int i = 0; i < NI; ++i)
-#pragma unroll
-        for (int j = 0; j < NCG; ++j) {
-            const bool ok = (i * RPI + roff < S) && (c + j * CW < S);
-            const float* tp = Tl + 2 * (i * RPI * S + j * CW);
-            const float2 e = ok ? make_float2(tp[0], tp[tsw]) : make_float2(0.f, 0.f);
-            if (KEEP) ab[KEEP ? i : 0][KEEP ? j : 0] = e;
-            if (GATHER && ok) {
-                const float2 x = Xs[xl + i * RPI * PW + j * CW];
-                acc1 = fmaf(e.x, x.x, acc1);
-                acc2 = fmaf(e.y, x.y, acc2);
-            }
+    for (int i = 0; i < NI; ++i) {
+        const bool ok = (i + 1) * RPI <= S || row_ok;
+        t[i] = ok ? Tl[i * RPI * S] : 0ull;
+        if (GATHER) {
+            const f32x2 x = ok ? Xl[i * RPI * PW] : 0ull;
+            p = fma2(t[i], x, p);
+            const float2 ts = upk(t[i]), xs = upk(x);
+            q1 = fmaf(ts.x, xs.y, q1);
+            q2 = fmaf(ts.y, xs.x, q2);
         }
-    float2 y;
+    }
     if (GATHER) {
-        float v = k ? acc1 + acc2 : acc1 - acc2;
-        v += __shfl_xor_sync(0xffffffffu, v, 16);
+        const float2 ps = upk(p);
+        const float re = c < S ? ps.x - ps.y : 0.f, im = c < S ? q1 + q2 : 0.f;
+        // the low half of the warp reduces the real part, the high half the imaginary one
+        const bool hi = lane & 16;
+        float v = hi ? im : re;
+        v += __shfl_xor_sync(0xffffffffu, hi ? re : im, 16);
         v += __shfl_xor_sync(0xffffffffu, v, 8);
         v += __shfl_xor_sync(0xffffffffu, v, 4);
         v += __shfl_xor_sync(0xffffffffu, v, 2);
-        const float o = __shfl_xor_sync(0xffffffffu, v, 1);
-        y = k ? make_float2(o, v) : make_float2(v, o);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        const float o = __shfl_xor_sync(0xffffffffu, v, 16);
+        y = hi ? make_float2(o, v) : make_float2(v, o);
         if (MODE == 0 && lane == 0) y_out[orig] = y;
-    } else {
-        y = y_in[orig];
     }
     if (SCATTER) {
-        const float ysx = (k ? -y.x : y.x) * s1, yys = y.y * s1;
+        const float yr = y.x * s1, yi = y.y * s1, nyr = -yr;
+        int* al = acc + (du + ro) * pitch + dv + c;
+        const f32x2 M = pk(FX_MAGIC, FX_MAGIC), NM = pk(-FX_MAGIC, -FX_MAGIC), NEG = pk(-1.f, -1.f),
+                    LO = pk(65536.f, 65536.f);
+        if (c < S) {
 #pragma unroll
-        for (int i = 0; i < NI; ++i)
-#pragma unroll
-            for (int j = 0; j < NCG; ++j) {
-                const bool ok = (i * RPI + roff < S) && (c + j * CW < S);
-                if (ok) {
-                    float2 e;
-                    if (KEEP) {
-                        e = ab[KEEP ? i : 0][KEEP ? j : 0];
-                    } else {
-                        const float* tp = Tl + 2 * (i * RPI * S + j * CW);
-                        e = make_float2(tp[0], tp[tsw]);
-                    }
+            for (int i = 0; i < NI; ++i) {
+                if ((i + 1) * RPI <= S || row_ok) {
+                    const float2 ts = upk(t[i]);
+                    const f32x2 d = pk(fmaf(ts.x, yr, ts.y * yi), fmaf(ts.x, yi, ts.y * nyr));
                     // scaled contribution, |d| <= 2^21, split into rint(d) and 2^16 x residual
-                    const float d = fmaf(e.x, ysx, e.y * yys);
-                    const float tq = __fadd_rn(d, FX_MAGIC);
-                    const int q1 = __float_as_int(tq) - FX_MAGIC_BITS;
-                    const float rf = __fsub_rn(d, __fsub_rn(tq, FX_MAGIC));
-                    const int q2 = __float_as_int(__fmaf_rn(rf, 65536.f, FX_MAGIC)) - FX_MAGIC_BITS;
-                    const int ci = 2 * (xl + i * RPI * PW + j * CW) + k;
-                    atomicAdd(Ahi + ci, q1);
-                    atomicAdd(Alo + ci, q2);
+                    const f32x2 h = add2(d, M);
+                    const f32x2 rf = fma2(add2(h, NM), NEG, d);
+                    const float2 hs = upk(h), ls = upk(fma2(rf, LO, M));
+                    int* a = al + i * RPI * pitch;
+                    atomicAdd(a, __float_as_int(hs.x) - FX_MAGIC_BITS);
+                    atomicAdd(a + plane, __float_as_int(hs.y) - FX_MAGIC_BITS);
+                    atomicAdd(a + 2 * plane, __float_as_int(ls.x) - FX_MAGIC_BITS);
+                    atomicAdd(a + 3 * plane, __float_as_int(ls.y) - FX_MAGIC_BITS);
                 }
             }
+        }
     }
 }
 
 template <int MODE, int PWC>
-__device__ __forceinline__ void vis_dispatch(int S, const float2* T, const float2* Xs, int* Ahi, int* Alo, float s1,
-                                             int pbase, int PW, int lane, uint32_t orig, const float2* y_in,
-                                             float2* y_out) {
+__device__ __forceinline__ void vis_dispatch(int S, const float2* T, const float2* Xs, int* acc, float s1, int du,
+                                             int dv, int PW, int pitch, int plane, int lane, uint32_t orig,
+                                             float2 y, float2* y_out) {
+    if (S == 15) {  // the largest support of the common plans, and most of their visibilities
+        vis_tile<15, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out);
+        return;
+    }
     switch (S) {
-        case 3: vis_tile<3, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
-        case 5: vis_tile<5, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
-        case 7: vis_tile<7, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
-        case 9: vis_tile<9, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
-        case 11: vis_tile<11, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
-        case 13: vis_tile<13, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
-        case 15: vis_tile<15, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
-        case 17: vis_tile<17, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
-        default: vis_tile<19, MODE, PWC>(T, Xs, Ahi, Alo, s1, pbase, PW, lane, orig, y_in, y_out); break;
+        case 3: vis_tile<3, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out); break;
+        case 5: vis_tile<5, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out); break;
+        case 7: vis_tile<7, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out); break;
+        case 9: vis_tile<9, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out); break;
+        case 11: vis_tile<11, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out); break;
+        case 13: vis_tile<13, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out); break;
+        default:  // larger tiles have larger patches than the compile-time ones
+            if constexpr (PWC == 0) {
+                if (S == 17) vis_tile<17, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out);
+                else vis_tile<19, MODE, PWC>(T, Xs, acc, s1, du, dv, PW, pitch, plane, lane, orig, y, y_out);
+            }
     }
 }
 
-// Warp-specialised pipeline per block:
-//   producer warp : for each chunk (GTG_CHUNK consecutive visibilities of a unit) streams their
-//                   16-byte metadata and their taps (one contiguous range, from a chunk
-//                   descriptor) into ring slot b with cp.async.bulk, once the consumers
-//                   released the slot;
-//   consumer warps: wait full[b]; each takes one visibility of the chunk, de-grids it
-//                   and grids conj(taps) y_k into the block's shared accumulator patch
-//                   (shared-memory reductions, one tap row per instruction:
-//                   visibilities of different warps may overlap); then arrive on empty[b].
-// Only unit boundaries (patch load / store) synchronise all consumers.
+// The unit's box in pairs of cells (16 bytes): rows [a0, a0 + na), the columns widened to
+// whole pairs, w pairs per row (PW, TS, gy are even: a pair stays within one uv-tile).
+struct UnitBox {
+    int a0, c0, w, n;
+    uint32_t mg;  // e / w = e mg >> 20: e < 2^12 pairs, w <= 41
+    __device__ __forceinline__ UnitBox(const UnitRec* rec) {
+        const uint32_t box = rec->box;
+        a0 = (int)(box & 255u);
+        c0 = box_c0(box);
+        w = box_pairs(box);
+        n = ((int)((box >> 8) & 255u) - a0) * w;
+        mg = rec->mg;
+    }
+    // pair e: patch row a, column c
+    __device__ __forceinline__ void at(int e, int& a, int& c) const {
+        const int r = (int)(((uint32_t)e * mg) >> 20);
+        a = a0 + r;
+        c = c0 + 2 * (e - r * w);
+    }
+};
+
+// Starts the copies of a unit's X box into its patch buffer (rows and columns wrap).
+template <int PWC>
+__device__ __forceinline__ void stage_x(const GtgArgs& A, const UnitRec* rec, float2* dst) {
+    const uint32_t g = rec->geom;
+    const int PW = PWC > 0 ? PWC : (int)(g >> 16);
+    const int u0 = (int)(g & 255u) * A.TS, v0 = (int)((g >> 8) & 255u) * A.TS;
+    const float2* X = reinterpret_cast<const float2*>(reinterpret_cast<const char*>(A.X) + rec->X);
+    const UnitBox B(rec);
+    for (int e = threadIdx.x; e < B.n; e += blockDim.x) {
+        int a, c;
+        B.at(e, a, c);
+        int gu = u0 + a, gv = v0 + c;
+        if (gu >= A.gx) gu -= A.gx;
+        if (gv >= A.gy) gv -= A.gy;
+        cp_async16(dst + a * PW + c, X + (size_t)gu * A.gy + gv);
+    }
+}
+
+// The visibilities of one warp in the order it takes them, unit after unit, in batches of up
+// to 32 held one per lane, and the metadata of the batch after the current one.
+struct VisCursor {
+    int round, base, n;    // the unit's round, the batch's first visibility, the warp's share
+    int b, nb;             // next of the batch, its size
+    const float2* src;     // the lane's visibility: taps, their bytes, VisMeta::pos and orig
+    uint32_t bytes, pos, orig;
+    bool ready;            // nxt is loaded
+    int4 nxt;
+};
+
+// visibilities of a warp: ceil((nvis - warp) / nw), mgw = ceil(2^20 / nw) (nvis <= 2^15)
+__device__ __forceinline__ int unit_share(int nvis, int warp, int nw, uint32_t mgw) {
+    return (int)(((uint64_t)(uint32_t)max(nvis - warp + nw - 1, 0) * mgw) >> 20);
+}
+__device__ __forceinline__ int4 load_meta(const UnitRec* rec, int k, int warp, int nw) {
+    const int i = warp + k * nw;
+    return i < rec->nvis ? __ldg(reinterpret_cast<const int4*>(rec->meta + i)) : make_int4(0, 0, 0, 0);
+}
+
 // MODE 0: de-grid (y_out), 1: grid (y_in), 2: fused de-grid + grid; PWC: the patch side
 // when known at compile time (the common plans), else 0
-// TABLE: the units of many (plan, bin) jobs from one queue (a stage-batched wideband apply).
-template <int MODE, int PWC, bool TABLE>
-__global__ void __launch_bounds__(GTG_THREADS, 1) gtg_kernel(const __grid_constant__ GtgArgs A) {
+// The units may be those of many (plan, bin) jobs: a record holds its job's addresses.
+//
+// Per round (unit) r of a block:
+//   open  : the X box copied during round r - 1 has landed; its max |X| sets the scale;
+//   barrier A; the copy of round r + 1's X box starts (other buffer);
+//   visibilities, each warp on its own;
+//   barrier B; close: the accumulator box goes to the unit's patch slot and back to zero.
+// Unit numbers are taken from the counter one round ahead (of the next round's prefetches), so
+// that no round waits for its descriptors and the last units still spread over the blocks.
+template <int MODE, int PWC>
+__global__ void __launch_bounds__(GTG_MAX_WARPS * 32, 1) gtg_kernel(const __grid_constant__ GtgArgs A) {
     constexpr bool GATHER = MODE != 1, SCATTER = MODE != 0;
     extern __shared__ __align__(128) unsigned char smraw[];
-    uint64_t* full = reinterpret_cast<uint64_t*>(smraw);
-    uint64_t* empty = full + GTG_NBUF;
-    uint64_t* xfull = empty + GTG_NBUF;  // [GTG_NX] X patch buffer landed
-    uint64_t* xfree = xfull + GTG_NX;    // [GTG_NX] consumers are done with the buffer
-    VisMeta* mring = reinterpret_cast<VisMeta*>(smraw + GTG_HDR);      // GTG_NBUF x GTG_CV entries
-    float2* taps = reinterpret_cast<float2*>(smraw + GTG_HDR + GTG_NBUF * GTG_CV * sizeof(VisMeta));
-    // shared memory laid out for the launch's largest patch (a staged batch's jobs may have
+    uint64_t* full = reinterpret_cast<uint64_t*>(smraw);  // [warp][slot] taps landed
+    UnitRec* recs = reinterpret_cast<UnitRec*>(smraw + GTG_MAX_WARPS * GTG_SLOTS * 8);
+    // shared memory laid out for the launch's largest patch (the jobs of a table may have
     // different patch sides; every unit uses its own job's)
     const int PWmax = PWC > 0 ? PWC : A.PW, npmax = PWmax * PWmax;
-    const int chunk_f2 = A.chunk_bytes / 8;
-    const uint32_t NB = (uint32_t)A.nbuf;
-    const bool pre = GATHER && A.prefetch;
-    const int NX = pre ? A.xbufs : 1;  // X patch buffers
-    // dynamic schedule (with prefetch): blocks take units from a counter in heaviest-first
-    // order; otherwise the static snake order
-    const bool dyn = pre && A.counter != nullptr;
-    float2* Xbuf0 = taps + (size_t)NB * chunk_f2;
-    int* Ahi = reinterpret_cast<int*>(Xbuf0 + (GATHER ? (size_t)NX * npmax : 0));  // [cell][re, im] words
-    int* Alo = Ahi + (SCATTER ? 2 * npmax : 0);
-    __shared__ volatile int s_abort;
-    __shared__ volatile int s_fail;           // dynamic schedule: a consumer's wait gave up
-    __shared__ volatile int s_unit[GTG_NX];   // dynamic schedule: the unit of round q (q % NX)
-    __shared__ float s_xmax[GTG_CONSUMERS];
+    const int pitch = PWC > 0 ? pitch_of(PWC) : A.pitch, plane = PWmax * pitch;
+    const int NX = A.xbufs;
+    float2* Xbuf0 = reinterpret_cast<float2*>(smraw + GTG_HDR);
+    int* acc = reinterpret_cast<int*>(Xbuf0 + (GATHER ? NX * npmax : 0));  // planes [hi re, hi im, lo re, lo im]
+    unsigned char* ring = reinterpret_cast<unsigned char*>(acc + (SCATTER ? 4 * plane : 0));
+    __shared__ int s_idx[GTG_RECS];    // unit of round q (q % GTG_RECS)
+    __shared__ uint32_t s_xm[2];       // max |X| of the unit's box (float bits), by round parity
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int G = gridDim.x, cb = blockIdx.x;
-    if (tid == 0) {
-        for (int b = 0; b < GTG_NBUF; ++b) {
-            mbar_init(&full[b], 1);
-            mbar_init(&empty[b], GTG_CONSUMERS);
-        }
-        for (int b = 0; b < GTG_NX; ++b) {
-            mbar_init(&xfull[b], 1);
-            mbar_init(&xfree[b], GTG_CONSUMERS);
-        }
-        s_abort = 0;
-        s_fail = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int G = gridDim.x;
+    const uint32_t mgw = ((1u << 20) + nw - 1) / nw;
+    uint64_t* const wfull = full + warp * GTG_SLOTS;
+    unsigned char* const wring = ring + (size_t)warp * GTG_SLOTS * A.slot_bytes;
+    if (lane == 0)
+        for (int b = 0; b < GTG_SLOTS; ++b) mbar_init(&wfull[b], 1);
+    if (tid < GTG_AHEAD) s_idx[tid] = blockIdx.x + tid * G;
+    if (tid < 2) s_xm[tid] = 0u;
+    if (tid < 4 * GTG_AHEAD) {  // their records (16 bytes per thread)
+        const int q = tid >> 2, idx = blockIdx.x + q * G;
+        if (idx < A.nunits)
+            reinterpret_cast<int4*>(recs + q)[tid & 3] =
+                __ldg(reinterpret_cast<const int4*>(A.recs + idx) + (tid & 3));
     }
+    if (SCATTER)
+        for (int e = tid; e < 4 * plane; e += blockDim.x) acc[e] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
 
-    if (warp == GTG_CONSUMERS) {
-        // ------------------------------------------------------------ producer
-        if (lane != 0) return;
-        uint32_t g = 0;
-        int xq = 0;         // the next round whose X patch is to be copied
-        bool ended = false;  // dynamic schedule: the end of the work was published
-        int* const status0 = TABLE ? A.jobs[0].status : A.one.status;
-        for (int r = 0;; ++r) {
-            int idx = 0;
-            if (!dyn) {
-                idx = unit_of(r, cb, G);
-                if (idx >= A.nunits) break;
-            }
-            // X patches of rounds r .. r + NX - 2 (buffer q % NX, once the consumers released
-            // it after round q - NX); rows wrap along u, a row past the last column splits in
-            // two.  Dynamic schedule: round q's unit is the next of the launch's heaviest-first
-            // order (one atomic per unit), published in s_unit[q % NX] with the copy's barrier
-            // (-1 after the last unit: a plain arrival)
-            while (pre && !ended && xq <= r + NX - 2) {
-                int iq = 0;
-                if (!dyn) {
-                    iq = unit_of(xq, cb, G);
-                    if (iq >= A.nunits) break;
-                }
-                const int j = xq % NX;
-                if (xq >= NX && !s_abort &&
-                    !mbar_wait_bounded(&xfree[j], ((xq / NX) - 1) & 1, A.peer_polls)) {
-                    s_abort = 1;
-                    atomicExch(status0, 1);
-                }
-                if (s_abort) break;
-                if (dyn) {
-                    const int gi = atomicAdd(A.counter, 1);
-                    iq = gi < A.nunits ? gi : -1;
-                    s_unit[j] = iq;
-                    if (iq < 0) {
-                        mbar_arrive(&xfull[j]);
-                        ended = true;
-                        ++xq;
-                        break;
-                    }
-                }
-                int sq;
-                const GtgJob* Jq = unit_job<TABLE>(A, iq, sq);
-                const TileDesc tq = Jq->units[sq];
-                const int PW = PWC > 0 ? PWC : (TABLE ? Jq->PW : A.PW);
-                float2* dst = Xbuf0 + (size_t)j * npmax;
-                const int u0 = tq.tu * A.TS, v0 = tq.tv * A.TS;
-                const int n1 = (v0 + PW <= A.gy) ? PW : A.gy - v0;  // cells before the wrap
-                // the rows of the unit's box, its columns widened to whole 16-byte pairs
-                // (PW, TS, gy and n1 are even)
-                const int a0 = (int)(tq.box & 255u), a1 = (int)((tq.box >> 8) & 255u);
-                const int c0 = (int)((tq.box >> 16) & 254u), c1 = min(PW, (int)(((tq.box >> 24) + 1u) & 254u));
-                const int w1 = max(0, min(c1, n1) - c0), cs = max(c0, n1), w2 = max(0, c1 - cs);
-                mbar_arrive_expect_tx(&xfull[j], (uint32_t)((a1 - a0) * (w1 + w2) * (int)sizeof(float2)));
-                for (int a = a0; a < a1; ++a) {
-                    int gu = u0 + a;
-                    if (gu >= A.gx) gu -= A.gx;
-                    const float2* row = Jq->X + (size_t)gu * A.gy;
-                    if (w1 > 0) bulk_g2s(dst + a * PW + c0, row + v0 + c0, (uint32_t)(w1 * sizeof(float2)), &xfull[j]);
-                    if (w2 > 0) bulk_g2s(dst + a * PW + cs, row + (cs - n1), (uint32_t)(w2 * sizeof(float2)), &xfull[j]);
-                }
-                ++xq;
-            }
-            if (s_abort) {
-                // let the copies already in flight land before the block may exit
-                for (uint32_t q = (g > NB ? g - NB : 0); q < g; ++q)
-                    (void)mbar_wait_bounded(&full[q % NB], (q / NB) & 1);
-                for (int q = (xq > NX ? xq - NX : 0); q < xq; ++q)
-                    (void)mbar_wait_bounded(&xfull[q % NX], (q / NX) & 1);
-                return;
-            }
-            if (dyn) {
-                idx = s_unit[r % NX];  // written by this thread in the loop above
-                if (idx < 0) break;
-            }
-            int slot;
-            const GtgJob* J = unit_job<TABLE>(A, idx, slot);
-            const TileDesc td = J->units[slot];
-            const int nchunks = (int)((td.ve - td.vb + GTG_CV - 1) / GTG_CV);
-            for (int c = 0; c < nchunks; ++c, ++g) {
-                const ChunkDesc cd = J->chunks[td.cb + c];
-                const int64_t v0 = td.vb + (int64_t)c * GTG_CV;
-                const uint32_t nv = (uint32_t)((td.ve - v0) < GTG_CV ? (td.ve - v0) : GTG_CV);
-                const uint32_t b = g % NB, use = g / NB;
-                if (use > 0 && !s_abort && !mbar_wait_bounded(&empty[b], (use - 1) & 1, A.peer_polls)) {
-                    s_abort = 1;
-                    atomicExch(J->status, 1);
-                }
-                if (s_abort) {
-                    // let the copies already in flight land before the block may exit
-                    for (uint32_t q = (g > NB ? g - NB : 0); q < g; ++q)
-                        (void)mbar_wait_bounded(&full[q % NB], (q / NB) & 1);
-                    for (int q = (xq > NX ? xq - NX : 0); q < xq; ++q)
-                        (void)mbar_wait_bounded(&xfull[q % NX], (q / NX) & 1);
-                    return;
-                }
-                mbar_arrive_expect_tx(&full[b], cd.bytes + nv * (uint32_t)sizeof(VisMeta));
-                bulk_g2s(mring + b * GTG_CV, J->meta + v0, nv * (uint32_t)sizeof(VisMeta), &full[b]);
-                bulk_g2s(taps + (size_t)b * chunk_f2, J->gblk[cd.block] + cd.off, cd.bytes, &full[b]);
-            }
-        }
-        return;
-    }
+    if (GATHER) stage_x<PWC>(A, recs, Xbuf0);  // round 0 (every block has a first unit)
+    cp_async_commit();
 
-    // ---------------------------------------------------------------- consumers
-    uint32_t g = 0;
-    for (int r = 0;; ++r) {
-        int idx;
-        if (dyn) {
-            // the round's unit as the producer published it; a failed wait (abort) records
-            // s_fail, and every consumer warp decides to stop from s_fail and the unit after
-            // the barrier below, all alike
-            const bool ok = !s_abort && mbar_wait_or_abort(&xfull[r % NX], (r / NX) & 1, &s_abort);
-            if (!ok) s_fail = 1;
-            idx = ok ? s_unit[r % NX] : -1;
-        } else {
-            idx = unit_of(r, cb, G);
-            if (idx >= A.nunits) break;
+    // ---- this warp's visibilities
+    VisCursor C;
+    auto unpack = [&](const float2* taps, const int4& m) {  // a lane's visibility of the new batch
+        const uint32_t S = ((uint32_t)m.w >> 16) & 255u, n = S * S;
+        C.src = taps + (int64_t)(((uint64_t)(uint32_t)m.y << 32) | (uint32_t)m.x);
+        C.bytes = (n + (n & 1u)) * (uint32_t)sizeof(float2);
+        C.pos = (uint32_t)m.w;
+        C.orig = (uint32_t)m.z;
+    };
+    // loads the batch after the current one, if its unit's record is there in round r
+    auto look_ahead = [&](int r) {
+        if (C.base + 32 < C.n) {
+            C.nxt = load_meta(recs + C.round % GTG_RECS, C.base + 32 + lane, warp, nw);
+            C.ready = true;
+        } else if (C.round <= r && s_idx[(C.round + 1) % GTG_RECS] < A.nunits) {
+            C.nxt = load_meta(recs + (C.round + 1) % GTG_RECS, lane, warp, nw);
+            C.ready = true;
         }
-        const bool have = idx >= 0;
-        int slot = 0;
-        const GtgJob* J = have ? unit_job<TABLE>(A, idx, slot) : (TABLE ? A.jobs : &A.one);
-        TileDesc td;
-        if (have) {
-            td = J->units[slot];
-        } else {  // no unit: nothing to stage or process
-            td.tu = td.tv = 0;
-            td.vb = td.ve = td.cb = 0;
-            td.box = 0u;
-        }
-        const int nchunks = (int)((td.ve - td.vb + GTG_CV - 1) / GTG_CV);
-        const int PW = PWC > 0 ? PWC : (TABLE ? J->PW : A.PW), npatch = PW * PW;
-        const int u0 = td.tu * A.TS, v0 = td.tv * A.TS;
-        // the unit's box: the only cells its footprints read and write
-        const int ba0 = (int)(td.box & 255u), ba1 = (int)((td.box >> 8) & 255u);
-        const int bb0 = (int)((td.box >> 16) & 255u), bb1 = (int)(td.box >> 24);
-        float xm = 0.f;
-        float2* Xs = Xbuf0 + (pre ? (size_t)(r % NX) * npmax : 0);
-        if (!dyn && pre && !s_abort && !mbar_wait_or_abort(&xfull[r % NX], (r / NX) & 1, &s_abort)) {
-            s_abort = 1;
-            atomicExch(J->status, 1);
-        }
-        for (int a = ba0 + warp; a < ba1; a += GTG_CONSUMERS) {
-            int gu = u0 + a;
-            if (gu >= A.gx) gu -= A.gx;
-            for (int b = bb0 + lane; b < bb1; b += 32) {
-                if (GATHER) {
-                    float2 x;
-                    if (pre) {
-                        x = Xs[a * PW + b];  // landed by the producer (cells outside the bin's
-                                             // footprints hold finite values of other bins)
-                    } else {
-                        int gv = v0 + b;
-                        if (gv >= A.gy) gv -= A.gy;
-                        // cells of tiles no footprint reaches hold no grid values of this bin
-                        x = J->need[(gu >> A.shift) * A.ntv + (gv >> A.shift)] ? J->X[(size_t)gu * A.gy + gv]
-                                                                              : make_float2(0.f, 0.f);
-                        Xs[a * PW + b] = x;
-                    }
-                    const float m = fabsf(x.x) + fabsf(x.y);
-                    if (m <= 3.4028234e38f) xm = fmaxf(xm, m);  // non-finite input is flagged elsewhere
-                }
-                if (SCATTER) {
-                    reinterpret_cast<int2*>(Ahi)[a * PW + b] = make_int2(0, 0);
-                    reinterpret_cast<int2*>(Alo)[a * PW + b] = make_int2(0, 0);
-                }
+    };
+    // the next batch, of the unit of round r + 1 at most; false: none
+    auto advance = [&](int r) {
+        if (A.stall) return false;
+        do {
+            if (C.base + 32 < C.n) {
+                C.base += 32;
+            } else {
+                if (C.round > r || s_idx[(C.round + 1) % GTG_RECS] >= A.nunits) return false;
+                ++C.round;
+                C.base = 0;
+                C.n = unit_share(recs[C.round % GTG_RECS].nvis, warp, nw, mgw);
             }
+            const UnitRec* rec = recs + C.round % GTG_RECS;
+            unpack(rec->taps, C.ready ? C.nxt : load_meta(rec, C.base + lane, warp, nw));
+            C.b = 0;
+            C.nb = min(32, C.n - C.base);
+            C.ready = false;
+            look_ahead(r);
+        } while (C.nb <= 0);
+        return true;
+    };
+    C.round = C.base = C.b = 0;
+    C.n = unit_share(recs[0].nvis, warp, nw, mgw);
+    C.nb = min(32, C.n);
+    unpack(recs[0].taps, load_meta(recs, lane, warp, nw));
+    C.ready = false;
+    look_ahead(0);
+    int inflight = 0, islot = 0, tslot = 0;  // copies under way or landed; next slots to fill and to take
+    uint32_t tphase = 0;
+    uint32_t posA = 0, posB = 0, origA = 0, origB = 0;  // of the visibilities in slots 0 and 1
+    float2 yA = make_float2(0.f, 0.f), yB = yA;
+    // starts the copy of the next visibility's taps (and the load of its y when gridding)
+    auto refill = [&](int r) {
+        if (C.b >= C.nb && !advance(r)) return;
+        if (lane == C.b) {
+            mbar_arrive_expect_tx(&wfull[islot], C.bytes);
+            bulk_g2s(wring + islot * A.slot_bytes, C.src, C.bytes, &wfull[islot]);
         }
-        if (MODE == 2) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) xm = fmaxf(xm, __shfl_xor_sync(0xffffffffu, xm, o));
-            if (lane == 0) s_xmax[warp] = xm;
+        const uint32_t pos = __shfl_sync(0xffffffffu, C.pos, C.b);
+        const uint32_t orig = MODE != 2 ? __shfl_sync(0xffffffffu, C.orig, C.b) : 0u;
+        if (islot) {
+            posB = pos;
+            origB = orig;
+            if (MODE == 1) yB = __ldg(&A.y_in[orig]);
+        } else {
+            posA = pos;
+            origA = orig;
+            if (MODE == 1) yA = __ldg(&A.y_in[orig]);
         }
-        consumers_sync();
-        if (dyn && (s_fail || !have)) break;
+        ++C.b;
+        ++inflight;
+        islot ^= 1;
+    };
+    if (A.stall && C.nb > GTG_SLOTS) C.nb = GTG_SLOTS;
+    refill(0);
+    refill(0);
+
+    const uint32_t* fxp = nullptr;  // the bounds read last (one plan: read once)
+    float fx0 = 0.f, fx1 = 0.f;
+    bool bad = false;
+    for (int r = 0;; ++r) {
+        const UnitRec* rec = recs + r % GTG_RECS;
+        const bool have = s_idx[r % GTG_RECS] < A.nunits;
+        const int PW = PWC > 0 ? PWC : (have ? (int)(rec->geom >> 16) : A.PW);
+        float2* Xs = Xbuf0 + (NX == 2 && (r & 1) ? npmax : 0);
+        cp_async_wait_all();
+        if (MODE == 2 && have) {
+            // max |X| of the pairs this thread copied
+            float xm = 0.f;
+            const UnitBox B(rec);
+            for (int e = tid; e < B.n; e += blockDim.x) {
+                int a, c;
+                B.at(e, a, c);
+                const float4 x = *reinterpret_cast<const float4*>(Xs + a * PW + c);
+                const float m0 = fabsf(x.x) + fabsf(x.y), m1 = fabsf(x.z) + fabsf(x.w);
+                if (m0 <= 3.4028234e38f) xm = fmaxf(xm, m0);  // non-finite input is flagged elsewhere
+                if (m1 <= 3.4028234e38f) xm = fmaxf(xm, m1);
+            }
+            const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(xm));
+            if (lane == 0) atomicMax(&s_xm[r & 1], wm);
+        }
+        // barrier A: the box, the cleared accumulators and the unit ring are visible; every
+        // warp learns of a failed wait
+        if (__syncthreads_or(bad) || !have) break;
+        int next_idx = 0;
+        if (tid == (nw - 1) * 32) next_idx = atomicAdd(A.counter, 1) + GTG_AHEAD * G;
+        const bool more = s_idx[(r + 1) % GTG_RECS] < A.nunits;
+        if (GATHER && NX == 2 && more)
+            stage_x<PWC>(A, recs + (r + 1) % GTG_RECS, Xbuf0 + (r & 1 ? 0 : npmax));
+        if (!C.ready && more) look_ahead(r);
+        if (warp == nw - 1) {  // the unit of round r + 2 and its record (this warp has the smallest share)
+            next_idx = __shfl_sync(0xffffffffu, next_idx, 0);
+            const int q = (r + 2) % GTG_RECS;
+            if (lane == 0) s_idx[q] = next_idx;
+            if (lane < 4 && next_idx < A.nunits)
+                cp_async16(reinterpret_cast<int4*>(recs + q) + lane,
+                           reinterpret_cast<const int4*>(A.recs + next_idx) + lane);
+        }
+        cp_async_commit();
+
+        const int nvis = rec->nvis;
         float s1 = 1.f, inv_s1 = 1.f;
         if (MODE == 2) {
             // per-unit bound: a de-gridded y of this unit has |y.x| + |y.y| <= 2 T1 max|X|_1
-            // over the patch, a contribution component at most tmax times that (margin 2)
-            float xmax = 0.f;
-#pragma unroll
-            for (int w = 0; w < GTG_CONSUMERS; ++w) xmax = fmaxf(xmax, s_xmax[w]);
-            const float mt = 4.f * __uint_as_float(__ldg(J->fx + FX_TMAX)) * __uint_as_float(__ldg(J->fx + FX_T1)) * xmax;
-            fx_scale(mt, td.ve - td.vb, s1, inv_s1);
+            // over the box, a contribution component at most tmax times that (margin 2)
+            const float xmax = __uint_as_float(s_xm[r & 1]);
+            if (rec->fx != fxp) {
+                fxp = rec->fx;
+                fx0 = __uint_as_float(__ldg(fxp + FX_TMAX));
+                fx1 = __uint_as_float(__ldg(fxp + FX_T1));
+            }
+            const float mt = 4.f * fx0 * fx1 * xmax;
+            fx_scale(mt, nvis, s1, inv_s1);
+            if (tid == 0) s_xm[(r + 1) & 1] = 0u;  // last read in round r - 1, next used in round r + 1
         } else if (SCATTER) {
             // twice tmax max|y|_1 (rounding margin); both words final before this launch
-            const float mt = 2.f * __uint_as_float(__ldcg(J->fx + FX_TMAX)) * __uint_as_float(__ldcg(J->fx + FX_YB));
-            if (!(mt <= 3.4028234e38f)) atomicExch(J->status, 3);
-            fx_scale(mt, td.ve - td.vb, s1, inv_s1);
-        }
-        for (int c = 0; c < nchunks; ++c, ++g) {
-            const uint32_t b = g % NB, par = (g / NB) & 1;
-            if (!s_abort && !mbar_wait_or_abort(&full[b], par, &s_abort)) {
-                s_abort = 1;
-                atomicExch(J->status, 1);
+            if (rec->fx != fxp) {
+                fxp = rec->fx;
+                fx0 = __uint_as_float(__ldg(fxp + FX_TMAX));
+                fx1 = __uint_as_float(__ldg(fxp + FX_YB));
             }
-            const int64_t cv0 = td.vb + (int64_t)c * GTG_CV;
-            const int ncv = (int)((td.ve - cv0) < GTG_CV ? (td.ve - cv0) : GTG_CV);
-            if (!s_abort && warp < ncv) {
-                const VisMeta mt = mring[b * GTG_CV + warp];
-                const int du = mt.pos & 255, dv = (mt.pos >> 8) & 255, S = (mt.pos >> 16) & 255;
-                const int loc = (int)(mt.off - mring[b * GTG_CV].off);
-                vis_dispatch<MODE, PWC>(S, taps + (size_t)b * chunk_f2 + loc, Xs, Ahi, Alo, s1, du * PW + dv, PW, lane,
-                                   mt.orig, A.y_in, A.y_out);
+            const float mt = 2.f * fx0 * fx1;
+            if (!(mt <= 3.4028234e38f)) atomicExch(rec->status, 3);
+            fx_scale(mt, nvis, s1, inv_s1);
+        }
+        // (nothing is in flight after a unit that left this warp no visibility)
+        if (inflight == 0) {
+            refill(r);
+            refill(r);
+        }
+        const int mine = unit_share(nvis, warp, nw, mgw);
+        for (int k = 0; k < mine; ++k) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&wfull[tslot], tphase, A.polls))) {
+                bad = true;
+                if (lane == 0) atomicExch(rec->status, 1);
+                break;
             }
-            __syncwarp();
-            if (lane == 0 && !A.stall) mbar_arrive(&empty[b]);
+            const uint32_t pos = tslot ? posB : posA, orig = tslot ? origB : origA;
+            const float2 y = MODE == 1 ? (tslot ? yB : yA) : make_float2(0.f, 0.f);
+            const int du = pos & 255, dv = (pos >> 8) & 255, S = (pos >> 16) & 255;
+            vis_dispatch<MODE, PWC>(S, reinterpret_cast<const float2*>(wring + tslot * A.slot_bytes), Xs, acc, s1, du,
+                                    dv, PW, pitch, plane, lane, orig, y, A.y_out);
+            __syncwarp();  // every lane has read the slot
+            --inflight;
+            tphase ^= (uint32_t)tslot;
+            tslot ^= 1;
+            refill(r);
         }
-        if (pre) {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&xfree[r % NX]);
+        if (SCATTER || NX == 1) __syncthreads();  // barrier B
+        if (GATHER && NX == 1 && more) {
+            stage_x<PWC>(A, recs + (r + 1) % GTG_RECS, Xbuf0);
+            cp_async_commit();
         }
-        consumers_sync();
-        if (SCATTER && !s_abort) {
+        if (SCATTER) {
             // the box of the patch (the fold and the merge read no cell outside it)
-            float2* dst = J->patch + (size_t)slot * npatch;
+            float2* dst = reinterpret_cast<float2*>(reinterpret_cast<char*>(A.patch) + rec->patch);
             const float inv_lo = inv_s1 * (1.f / 65536.f);
-            const int bw = bb1 - bb0, nb = (ba1 - ba0) * bw;
-            // e / bw = umulhi(e, ceil(2^32 / bw)) while e bw < 2^32 (e < PW^2, bw <= PW)
-            const uint32_t mg = 0xffffffffu / (uint32_t)max(bw, 2) + 1u;
-            for (int e = tid; e < nb; e += GTG_CONSUMERS * 32) {
-                const int da = bw > 1 ? (int)__umulhi((uint32_t)e, mg) : e;
-                const int c = (ba0 + da) * PW + bb0 + (e - da * bw);
-                const int2 h = reinterpret_cast<const int2*>(Ahi)[c], l = reinterpret_cast<const int2*>(Alo)[c];
-                dst[c] = make_float2(fmaf((float)l.x, inv_lo, (float)h.x * inv_s1),
-                                     fmaf((float)l.y, inv_lo, (float)h.y * inv_s1));
+            const UnitBox B(rec);
+            for (int e = tid; e < B.n; e += blockDim.x) {
+                int a, c;
+                B.at(e, a, c);
+                int2* q = reinterpret_cast<int2*>(acc + a * pitch + c);
+                const int2 hr = q[0], hi = q[plane / 2], lr = q[plane], li = q[3 * plane / 2];
+                q[0] = q[plane / 2] = q[plane] = q[3 * plane / 2] = make_int2(0, 0);
+                *reinterpret_cast<float4*>(dst + a * PW + c) =
+                    make_float4(fmaf((float)lr.x, inv_lo, (float)hr.x * inv_s1),
+                                fmaf((float)li.x, inv_lo, (float)hi.x * inv_s1),
+                                fmaf((float)lr.y, inv_lo, (float)hr.y * inv_s1),
+                                fmaf((float)li.y, inv_lo, (float)hi.y * inv_s1));
             }
         }
-        consumers_sync();
+    }
+    // copies in flight land before the block may exit
+    cp_async_wait_all();
+    for (; inflight > 0; --inflight) {
+        (void)mbar_wait_bounded(&wfull[tslot], tphase);
+        tphase ^= (uint32_t)tslot;
+        tslot ^= 1;
     }
 }
 
@@ -601,69 +613,51 @@ __global__ void __launch_bounds__(256) merge_patches_kernel(const __grid_constan
     }
 }
 
-static size_t gtg_smem_dims(int PW, int chunk_bytes, int mode, int nbuf, bool prefetch, int xbufs = 2) {
-    const size_t npatch = (size_t)PW * PW * sizeof(float2);
-    // X patches (float2; xbufs of them when prefetched) when de-gridding, hi + lo words
-    // (2 x int2) when gridding
-    const int nx = mode != 1 ? (prefetch ? xbufs : 1) : 0;
-    return GTG_HDR + GTG_NBUF * GTG_CV * sizeof(VisMeta) + (size_t)nbuf * chunk_bytes +
-           (size_t)(nx + (mode != 0 ? 2 : 0)) * npatch;
+static size_t gtg_smem(int PW, int pitch, int slot_bytes, int mode, int warps, int xbufs) {
+    return GTG_HDR + (mode != 1 ? (size_t)xbufs * PW * PW * sizeof(float2) : 0) +
+           (mode != 0 ? (size_t)4 * PW * pitch * sizeof(int) : 0) + (size_t)warps * GTG_SLOTS * slot_bytes + GTG_TAIL;
 }
 
-size_t gtg_smem(const rimo_plan* p, int mode, int nbuf, bool prefetch) {
-    return gtg_smem_dims(p->PW, p->chunk_bytes, mode, nbuf, prefetch);
-}
-
-// Launch shape of the grid step for a patch side and tap-ring chunk (prefetch, X buffers,
-// ring depth, shared memory); `mode` as in launch_gtg.  Units of a few chunks (mean below
-// 8 chunks of visibilities) leave too little time between two X patch copies for one copy
-// ahead to land: they get a third X buffer, two units ahead, at the price of a ring slot.
-static void gtg_shape(const rimo_plan* p, int PW, int chunk_bytes, int mode, double vis_per_unit, GtgArgs& A,
-                      size_t& sm) {
-    const size_t limit = 227 * 1024 - 2048;  // minus the kernel's static shared memory
-    A.xbufs = vis_per_unit < 8.0 * GTG_CV ? GTG_NX : 2;
-    // prefetch the X patches when the buffers still leave a 3-deep tap ring (4-deep with two)
-    const int ring = A.xbufs == 2 ? GTG_NBUF : GTG_NBUF - 1;
-    A.prefetch = mode != 1 && gtg_smem_dims(PW, chunk_bytes, mode, ring, true, A.xbufs) <= limit;
-    if (mode != 1 && !A.prefetch && A.xbufs > 2) {
-        A.xbufs = 2;
-        A.prefetch = gtg_smem_dims(PW, chunk_bytes, mode, GTG_NBUF, true, 2) <= limit;
-    }
-    A.nbuf = GTG_NBUF;
-    while (A.nbuf > 2 && gtg_smem_dims(PW, chunk_bytes, mode, A.nbuf, A.prefetch, A.xbufs) > limit) --A.nbuf;
-    sm = gtg_smem_dims(PW, chunk_bytes, mode, A.nbuf, A.prefetch, A.xbufs);
-    if (sm > limit) fail(RIMO_ERR_UNSUPPORTED, "tile patch and tap ring exceed shared memory");
+// Launch shape of the grid step for patches of side PW and tiles of side max_S; `mode` as in
+// launch_gtg.  24 warps per SM, as three, two or one block, the most blocks that fit: a
+// block's unit boundaries then hide behind the other blocks' visibilities (15 x 15 tiles on
+// 32-wide uv-tiles: three blocks when only de-gridding or gridding, two when fused).  A
+// single block gives up its second X buffer when that leaves fewer than 16 warps a ring.
+struct GtgShape {
+    int warps, blocks_per_sm;
+    size_t smem;
+};
+static GtgShape gtg_shape(const rimo_plan* p, int PW, int max_S, int mode, GtgArgs& A) {
+    const int n = max_S * max_S;
     A.gx = p->gx;
     A.gy = p->gy;
     A.TS = p->TS;
     A.PW = PW;
-    A.chunk_bytes = chunk_bytes;
-    A.ntv = p->gy / p->TS;
-    A.shift = p->TS == 64 ? 6 : 5;
+    A.pitch = pitch_of(PW, max_S);
+    A.slot_bytes = (n + (n & 1)) * (int)sizeof(float2);
     A.stall = p->test_stall;
-    A.peer_polls = p->test_stall ? p->test_polls : WAIT_POLLS;
-}
-
-static GtgJob gtg_job(const rimo_plan* p, int bin, const float2* X, float2* patch) {
-    GtgJob J;
-    J.units = p->d_tiles + p->bins[bin].t0;
-    J.chunks = p->d_chunks;
-    J.meta = p->d_meta;
-    J.gblk = p->d_gblock_ptrs;
-    J.X = X;
-    J.patch = patch;
-    J.fx = p->d_fx;
-    J.need = p->d_need + (size_t)bin * (size_t)(p->gx / p->TS) * (p->gy / p->TS);
-    J.status = p->d_status;
-    J.PW = p->PW;
-    return J;
+    A.polls = p->test_stall ? p->test_polls : WAIT_POLLS;
+    GtgShape g{};
+    A.xbufs = 2;
+    for (g.blocks_per_sm = 3; g.blocks_per_sm >= 2; --g.blocks_per_sm) {
+        g.warps = GTG_MAX_WARPS / g.blocks_per_sm;
+        g.smem = gtg_smem(PW, A.pitch, A.slot_bytes, mode, g.warps, 2);
+        // 228 KB per SM, 1 KB of each block's share reserved, 512 bytes for static shared memory
+        if (g.smem + 1024 + 512 <= (size_t)(228 * 1024) / g.blocks_per_sm) return g;
+    }
+    for (A.xbufs = 2; A.xbufs >= 1; --A.xbufs)
+        for (g.warps = GTG_MAX_WARPS; g.warps >= (A.xbufs == 2 ? 16 : 1); --g.warps) {
+            g.smem = gtg_smem(PW, A.pitch, A.slot_bytes, mode, g.warps, A.xbufs);
+            if (g.smem <= 226 * 1024) return g;
+        }
+    fail(RIMO_ERR_UNSUPPORTED, "tile patch and tap ring exceed shared memory");
 }
 
 // the kernel instance: patch sides of the uv-tiles 32 and 64 with 15 x 15 tiles are
 // compile-time constants
-template <int MODE, bool TABLE>
+template <int MODE>
 static void (*gtg_kernel_for(int PW))(GtgArgs) {
-    return PW == 46 ? gtg_kernel<MODE, 46, TABLE> : PW == 78 ? gtg_kernel<MODE, 78, TABLE> : gtg_kernel<MODE, 0, TABLE>;
+    return PW == 46 ? gtg_kernel<MODE, 46> : PW == 78 ? gtg_kernel<MODE, 78> : gtg_kernel<MODE, 0>;
 }
 
 template <int MODE>
@@ -673,19 +667,17 @@ static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_o
     if (nu <= 0) return;
     GtgArgs A;
     std::memset(&A, 0, sizeof(A));
-    A.one = gtg_job(p, bin, p->d_X, p->d_patch);
-    A.sched = p->d_sched + br.t0;
+    A.recs = p->d_recs + br.t0;
     A.nunits = nu;
-    // dense units take the dynamic schedule (zeroed counter at the start of every apply)
-    A.counter = (double)(br.ve - br.vb) / nu >= 8.0 * GTG_CV ? p->d_counter + bin : nullptr;
+    A.counter = p->d_counter + bin;  // zeroed at the start of every apply
+    A.X = p->d_X;
+    A.patch = p->d_patch;
     A.y_in = y_in;
     A.y_out = y_out;
-    size_t sm = 0;
-    gtg_shape(p, p->PW, p->chunk_bytes, MODE, (double)(br.ve - br.vb) / nu, A, sm);
-    void (*kern)(GtgArgs) = gtg_kernel_for<MODE, false>(p->PW);
-    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    const int grid = std::min(nu, p->n_sm);
-    kern<<<grid, GTG_THREADS, sm, s>>>(A);
+    const GtgShape g = gtg_shape(p, p->PW, p->max_S, MODE, A);
+    void (*kern)(GtgArgs) = gtg_kernel_for<MODE>(p->PW);
+    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+    kern<<<std::min(nu, p->n_sm * g.blocks_per_sm), g.warps * 32, g.smem, s>>>(A);
     if (MODE != 0 && br.m1 > br.m0) {
         MergeJob mj;
         mj.patch = p->d_patch;
@@ -697,20 +689,18 @@ static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_o
 
 // ---------------------------------------------------------------------------
 // The grid step of a stage-batched apply: one persistent launch over the units of every
-// (plan, bin) job, taken heaviest first from one queue, then one merge launch.
+// (plan, bin) job, taken heaviest first from one list, then one merge launch.
 struct WideGtg {
     GtgArgs A;
-    size_t sm = 0;
+    GtgShape shape{};
     int grid = 0, merge_blocks = 0, njobs = 0, PW = 0;
-    GtgJob* jobs = nullptr;
-    int2* queue = nullptr;
+    UnitRec* recs = nullptr;
     MergeJob* mjobs = nullptr;
     int* mfirst = nullptr;
-    int* counter = nullptr;  // the dynamic schedule's next unit (zeroed before every launch)
+    int* counter = nullptr;  // the units taken (zeroed before every launch)
     int64_t units = 0;
     ~WideGtg() {
-        cudaFree(jobs);
-        cudaFree(queue);
+        cudaFree(recs);
         cudaFree(mjobs);
         cudaFree(mfirst);
         cudaFree(counter);
@@ -722,39 +712,30 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, cudaStream_t s) {
     auto* w = new WideGtg();
     try {
         const rimo_plan* p0 = jobs[0].p;
-        int pw_max = 0, cb_max = 0;
+        int pw_max = 0, s_max = 0;
         bool one_pw = true;
         for (const WideJob& j : jobs) {
             pw_max = std::max(pw_max, j.p->PW);
-            cb_max = std::max(cb_max, j.p->chunk_bytes);
+            s_max = std::max(s_max, j.p->max_S);
             one_pw = one_pw && j.p->PW == p0->PW;
         }
-        int64_t nvis = 0, nun = 0;
-        for (const WideJob& j : jobs) {
-            nvis += j.p->bins[j.bin].ve - j.p->bins[j.bin].vb;
-            nun += j.p->bins[j.bin].t1 - j.p->bins[j.bin].t0;
-        }
         std::memset(&w->A, 0, sizeof(w->A));
-        gtg_shape(p0, pw_max, cb_max, 2, (double)nvis / std::max<int64_t>(1, nun), w->A, w->sm);
+        w->shape = gtg_shape(p0, pw_max, s_max, 2, w->A);
         // one patch side: its compile-time kernel; several: the kernel reading each job's
         w->PW = one_pw ? p0->PW : 0;
-        std::vector<GtgJob> gj;
         std::vector<MergeJob> mj;
         std::vector<int> mf{0};
-        struct Q {
-            int64_t n;
-            int job, slot;
-        };
-        std::vector<Q> q;
+        std::vector<UnitRec> recs;
         for (size_t j = 0; j < jobs.size(); ++j) {
             const rimo_plan* p = jobs[j].p;
             if (p->TS != p0->TS || p->gx != p0->gx || p->gy != p0->gy)
                 fail(RIMO_ERR_UNSUPPORTED, "jobs of one grid-step launch need one grid and uv-tile size");
             const auto& br = p->bins[jobs[j].bin];
-            gj.push_back(gtg_job(p, jobs[j].bin, jobs[j].X, jobs[j].patch));
-            for (int u = 0; u < br.t1 - br.t0; ++u) {
-                const TileDesc& td = p->tiles_host[(size_t)br.t0 + u];
-                q.push_back(Q{td.ve - td.vb, (int)j, u});
+            for (int u = br.t0; u < br.t1; ++u) {
+                UnitRec q = p->recs_host[(size_t)u];
+                q.X = (int64_t)(uintptr_t)jobs[j].X;
+                q.patch += (int64_t)(uintptr_t)jobs[j].patch;
+                recs.push_back(q);
             }
             MergeJob m;
             m.patch = jobs[j].patch;
@@ -763,30 +744,26 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, cudaStream_t s) {
             mj.push_back(m);
             mf.push_back(mf.back() + (br.m1 - br.m0));
         }
-        // heaviest first over the whole batch (ties: job, then slot), dealt in snake order
-        std::stable_sort(q.begin(), q.end(), [](const Q& a, const Q& b) { return a.n > b.n; });
-        std::vector<int2> qq(q.size());
-        for (size_t i = 0; i < q.size(); ++i) qq[i] = make_int2(q[i].job, q[i].slot);
-        w->units = (int64_t)q.size();
+        // heaviest first over the whole batch (ties: job, then the bin's order)
+        std::stable_sort(recs.begin(), recs.end(), [](const UnitRec& a, const UnitRec& b) { return a.nvis > b.nvis; });
+        w->units = (int64_t)recs.size();
         w->njobs = (int)jobs.size();
         w->merge_blocks = mf.back();
-        RIMO_CUDA(cudaMalloc(&w->jobs, gj.size() * sizeof(GtgJob)));
-        RIMO_CUDA(cudaMalloc(&w->queue, std::max<size_t>(1, qq.size()) * sizeof(int2)));
+        // (a unit index plus the blocks' look-ahead stays an int)
+        if (w->units > 0x7fffffffLL - 8 * 4096) fail(RIMO_ERR_UNSUPPORTED, "too many work units for one launch");
+        RIMO_CUDA(cudaMalloc(&w->recs, std::max<size_t>(1, recs.size()) * sizeof(UnitRec)));
         RIMO_CUDA(cudaMalloc(&w->mjobs, mj.size() * sizeof(MergeJob)));
         RIMO_CUDA(cudaMalloc(&w->mfirst, mf.size() * sizeof(int)));
         RIMO_CUDA(cudaMalloc(&w->counter, sizeof(int)));
-        RIMO_CUDA(cudaMemcpyAsync(w->jobs, gj.data(), gj.size() * sizeof(GtgJob), cudaMemcpyHostToDevice, s));
-        if (!qq.empty())
-            RIMO_CUDA(cudaMemcpyAsync(w->queue, qq.data(), qq.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+        if (!recs.empty())
+            RIMO_CUDA(cudaMemcpyAsync(w->recs, recs.data(), recs.size() * sizeof(UnitRec), cudaMemcpyHostToDevice, s));
         RIMO_CUDA(cudaMemcpyAsync(w->mjobs, mj.data(), mj.size() * sizeof(MergeJob), cudaMemcpyHostToDevice, s));
         RIMO_CUDA(cudaMemcpyAsync(w->mfirst, mf.data(), mf.size() * sizeof(int), cudaMemcpyHostToDevice, s));
         RIMO_CUDA(cudaStreamSynchronize(s));
-        w->A.jobs = w->jobs;
-        w->A.queue = w->queue;
-        w->A.nunits = (int)q.size();
-        w->A.counter = (double)nvis / std::max<int64_t>(1, nun) >= 8.0 * GTG_CV ? w->counter : nullptr;
-        if ((int64_t)w->A.nunits != w->units) fail(RIMO_ERR_UNSUPPORTED, "too many work units for one launch");
-        w->grid = (int)std::min<int64_t>(w->units, p0->n_sm);
+        w->A.recs = w->recs;
+        w->A.nunits = (int)w->units;
+        w->A.counter = w->counter;
+        w->grid = (int)std::min<int64_t>(w->units, (int64_t)p0->n_sm * w->shape.blocks_per_sm);
     } catch (...) {
         delete w;
         throw;
@@ -800,10 +777,10 @@ int64_t wide_gtg_units(const WideGtg* w) { return w->units; }
 
 void wide_gtg(const WideGtg* w, cudaStream_t s) {
     if (w->units == 0) return;
-    void (*kern)(GtgArgs) = gtg_kernel_for<2, true>(w->PW);
-    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->sm));
-    if (w->A.counter) RIMO_CUDA(cudaMemsetAsync(w->counter, 0, sizeof(int), s));
-    kern<<<w->grid, GTG_THREADS, w->sm, s>>>(w->A);
+    void (*kern)(GtgArgs) = gtg_kernel_for<2>(w->PW);
+    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->shape.smem));
+    RIMO_CUDA(cudaMemsetAsync(w->counter, 0, sizeof(int), s));
+    kern<<<w->grid, w->shape.warps * 32, w->shape.smem, s>>>(w->A);
     if (w->merge_blocks > 0) {
         MergeJob none;
         none.patch = nullptr;

@@ -10,7 +10,8 @@
 #include "rimo.h"
 
 namespace rimo {
-// visibilities per tap-ring chunk of the grid step, one per consumer warp
+// rows of the time interleave of a uv-tile's visibilities (uv_order 0): that many visibilities
+// in a row come from far-apart instants
 constexpr int GTG_CHUNK = 20;
 
 // ---------------------------------------------------------------------------
@@ -62,7 +63,6 @@ constexpr uint32_t SHARD_SKIP = 255;
 struct TileDesc {
     int32_t tu, tv;
     int64_t vb, ve;
-    int64_t cb;   // index of the unit's first chunk descriptor
     // the unit's box within its patch: the cells [a0, a1) x [b0, b1) its footprints reach
     // (a0 | a1 << 8 | b0 << 16 | b1 << 24); the whole patch for the units of a split tile
     uint32_t box;
@@ -72,14 +72,25 @@ __host__ __device__ inline uint32_t box_pack(int a0, int a1, int b0, int b1) {
     return (uint32_t)a0 | ((uint32_t)a1 << 8) | ((uint32_t)b0 << 16) | ((uint32_t)b1 << 24);
 }
 
-// One chunk of at most GTG_CHUNK consecutive visibilities of a unit: their taps are the byte
-// range [8 off, 8 off + bytes) of Fourier block `block`.
-struct ChunkDesc {
-    int64_t off;
-    uint32_t bytes;
-    uint32_t block;
+// A work unit as the grid step reads it (64 bytes, one record per unit in launch order).  The
+// forward grid and the patches of a plan's own records count from the launch's base pointers;
+// in a launch over several jobs the records hold the jobs' addresses (base pointers null).
+struct alignas(16) UnitRec {
+    uint32_t geom;         // uv-tile (tu | tv << 8) and patch side << 16
+    uint32_t box;          // TileDesc::box
+    uint32_t mg;           // ceil(2^20 / w), w the box's pairs of columns: divides a pair's number by w
+    int32_t nvis;
+    const VisMeta* meta;   // the unit's first visibility
+    const float2* taps;    // the Fourier block VisMeta::off counts from
+    int64_t X;             // bytes from the base to the forward grid ...
+    int64_t patch;         // ... and to the unit's patch
+    const uint32_t* fx;    // the plan's fixed-point bounds
+    int* status;           // the plan's device status word
 };
-static_assert(sizeof(ChunkDesc) == 16, "ChunkDesc must stay 16 bytes");
+// the box's columns widened to whole pairs of cells: first column, pairs
+__host__ __device__ inline int box_c0(uint32_t box) { return (int)((box >> 16) & 254u); }
+__host__ __device__ inline int box_pairs(uint32_t box) { return ((int)(box >> 24) + 1 - box_c0(box)) >> 1; }
+static_assert(sizeof(UnitRec) == 64, "UnitRec must stay 64 bytes");
 
 struct BinRange {
     int64_t vb = 0, ve = 0;       // visibilities of the bin in sorted order
@@ -122,15 +133,13 @@ struct rimo_plan {
     std::vector<int32_t> inv_perm;               // caller index -> sorted position
     std::vector<rimo::BinRange> bins;
     std::vector<rimo::TileDesc> tiles_host;      // work units (uv-tiles or parts), grouped by bin
-    std::vector<int32_t> sched_host;             // per bin: unit indices, heaviest first
+    std::vector<rimo::UnitRec> recs_host;        // the same units per bin, heaviest first
     std::vector<int2> merge_host;                // per bin: (first slot, units) of split tiles
     std::vector<int64_t> block_bytes;
 
     // device
     rimo::VisMeta* d_meta = nullptr;
-    rimo::TileDesc* d_tiles = nullptr;
-    int32_t* d_sched = nullptr;
-    rimo::ChunkDesc* d_chunks = nullptr;
+    rimo::UnitRec* d_recs = nullptr;
     int2* d_merge = nullptr;
     std::vector<float2*> d_gblocks;
     float2** d_gblock_ptrs = nullptr;
@@ -146,7 +155,7 @@ struct rimo_plan {
     int32_t* d_counter = nullptr;  // per-bin dynamic tile schedulers (reset at each apply)
     int32_t* d_status = nullptr;   // device-side error flag (bounded waits)
     uint32_t* d_fx = nullptr;      // fixed-point grid-step bounds (layout: rimo::FX_*)
-    int max_tiles_bin = 0, chunk_vis = rimo::GTG_CHUNK, chunk_bytes = 0, nbuf = 4, n_sm = 0;
+    int max_tiles_bin = 0, n_sm = 0;
     int device = 0;                // CUDA device the plan lives on
     int test_stall = 0;            // failure-detection test of the grid step's bounded waits
     uint32_t test_polls = 0;       // (rimo_plan_set_wait_test)
@@ -292,6 +301,9 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, cudaStream_t s);
 void wide_gtg_destroy(WideGtg* w);
 int64_t wide_gtg_units(const WideGtg* w);
 void wide_gtg(const WideGtg* w, cudaStream_t s);  // G_p^H G_p of every job: one persistent launch
+
+// Whether a plan of max_units work units per w-bin fits the allocation-free apply's scratch.
+bool noalloc_fits(const rimo_plan* p, int max_units);
 
 // The three applies on stream s (defined in apply.cu).
 void apply_phi(rimo_plan* p, const float2* x, float2* y, cudaStream_t s);

@@ -2,6 +2,7 @@
 // transformed rows, the forward / folded grid, the tile patches and the tile schedulers)
 // is carved from one statically allocated device array of this file instead of the
 // plan's own scratch buffers.  The computation is the plan's regular apply, unchanged.
+#include <algorithm>
 #include <mutex>
 
 #include "internal.h"
@@ -40,6 +41,17 @@ static unsigned char* noalloc_scratch() {
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// bytes of the array a plan takes: its parts' sizes, each on a 256-byte boundary
+struct NoallocParts {
+    size_t counters, ab, grid, patches;
+    NoallocParts(const rimo_plan* p, int max_units)
+        : counters(align256((size_t)p->P * sizeof(int32_t))),
+          ab(align256((size_t)2 * p->nx * p->ny * sizeof(float2))),
+          grid(align256((size_t)p->gx * p->gy * sizeof(float2))),
+          patches(align256((size_t)std::max(1, max_units) * p->PW * p->PW * sizeof(float2))) {}
+    size_t total() const { return counters + ab + grid + patches; }
+};
+bool noalloc_fits(const rimo_plan* p, int max_units) { return NoallocParts(p, max_units).total() <= NOALLOC_BYTES; }
 
 }  // namespace rimo
 
@@ -54,11 +66,8 @@ extern "C" rimo_status rimo_apply_phi_adj_phi_noalloc(rimo_plan_t p, const rimo_
         if ((const void*)x == (const void*)out) fail(RIMO_ERR_INVALID_ARG, "x and out must be distinct");
         if (p->mode != RIMO_MODE_STORED_G || p->h_built)
             fail(RIMO_ERR_UNSUPPORTED, "the allocation-free apply covers stored-G plans only");
-        const size_t counters = align256((size_t)p->P * sizeof(int32_t));
-        const size_t ab = align256((size_t)2 * p->nx * p->ny * sizeof(float2));
-        const size_t grid = align256((size_t)p->gx * p->gy * sizeof(float2));
-        const size_t patches = align256((size_t)std::max(1, p->max_tiles_bin) * p->PW * p->PW * sizeof(float2));
-        const size_t need = counters + ab + grid + patches;
+        const NoallocParts parts(p, p->max_tiles_bin);
+        const size_t counters = parts.counters, ab = parts.ab, grid = parts.grid, need = parts.total();
         if (need > NOALLOC_BYTES)
             fail(RIMO_ERR_UNSUPPORTED, "plan needs " + std::to_string(need) + " bytes of scratch, above the " +
                                            std::to_string(NOALLOC_BYTES) + "-byte static scratch");

@@ -394,9 +394,8 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
             // Interleave the tile's visibilities (arrival order within a tile is time, so
             // neighbours are the same few baselines a fraction of a cell apart): viewed
             // as GTG_CHUNK rows of nc, the new order reads the list column by column, so
-            // that the GTG_CHUNK consecutive visibilities of one ring chunk, de-gridded and
-            // gridded at the same time by as many warps, come from far-apart instants and
-            // rarely update the same grid cells.
+            // that consecutive visibilities, de-gridded and gridded at the same time by as
+            // many warps, come from far-apart instants and rarely update the same grid cells.
             // (uv_order 0; 1 keeps the time order; 2 orders the tile's visibilities by a
             // SplitMix64 hash of their index)
             if (q.uv_order == 0) {
@@ -499,8 +498,13 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
     // work units: active uv-tiles, split into units of at most `cap` visibilities so that
     // no unit outweighs a fraction of one SM's share of the bin; slots group the units of
     // a tile contiguously (merge groups), the schedule orders units heaviest first
+    // (a block commits to a unit one ahead, so the last units' blocks end within about two
+    // units of one another: an eighth of an SM's share keeps that tail small; half a share,
+    // with two blocks per SM, left the SMs of 512^2/2M/4 bins idle for 28 % of the launch).
+    // A plan that fits the allocation-free apply's scratch with half shares takes the finest
+    // split that still does.
     p->tiles_host.clear();
-    p->sched_host.clear();
+    p->recs_host.clear();
     p->merge_host.clear();
     int n_active = 0;
     std::vector<int32_t> slot((size_t)P * ntile, -1);
@@ -510,10 +514,25 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
         RIMO_CUDA(cudaGetDevice(&dev));
         RIMO_CUDA(cudaDeviceGetAttribute(&nsm_host, cudaDevAttrMultiProcessorCount, dev));
     }
-    for (int b = 0; b < P; ++b) {
+    auto unit_cap = [&](int b, int64_t parts) {
         const int64_t bin_vis = bstart[b + 1] - bstart[b];
-        const int64_t cap = std::min<int64_t>(
-            FX_MAX_UNIT, std::max<int64_t>(256, (bin_vis + 2 * nsm_host - 1) / (2 * (int64_t)nsm_host)));
+        return std::min<int64_t>(FX_MAX_UNIT, std::max<int64_t>(256, (bin_vis + parts - 1) / parts));
+    };
+    auto max_units = [&](int64_t parts) {
+        int64_t most = 0;
+        for (int b = 0; b < P; ++b) {
+            const int64_t cap = unit_cap(b, parts);
+            int64_t k = 0;
+            for (const auto& x : tl[b]) k += (x.ve - x.vb + cap - 1) / cap;
+            most = std::max(most, k);
+        }
+        return (int)most;
+    };
+    int64_t parts = 8 * (int64_t)nsm_host;
+    if (noalloc_fits(p, max_units(2 * (int64_t)nsm_host)))
+        while (!noalloc_fits(p, max_units(parts))) parts -= nsm_host;
+    for (int b = 0; b < P; ++b) {
+        const int64_t cap = unit_cap(b, parts);
         p->bins[b].t0 = (int32_t)p->tiles_host.size();
         p->bins[b].m0 = (int32_t)p->merge_host.size();
         for (const auto& x : tl[b]) {
@@ -522,7 +541,7 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
             const int64_t k = (n + cap - 1) / cap;
             for (int64_t q = 0; q < k; ++q) {
                 const int64_t a = x.vb + n * q / k, e = x.vb + n * (q + 1) / k;
-                TileDesc u{x.tu, x.tv, a, e, 0, 0u, 0u};
+                TileDesc u{x.tu, x.tv, a, e, 0u, 0u};
                 if (k > 1) {
                     u.box = box_pack(0, p->PW, 0, p->PW);  // the merge adds the slices' whole patches
                 } else {
@@ -552,7 +571,17 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
             const auto& B = p->tiles_host[p->bins[b].t0 + j];
             return (A.ve - A.vb) > (B.ve - B.vb);
         });
-        p->sched_host.insert(p->sched_host.end(), ord.begin(), ord.end());
+        for (int32_t i : ord) {  // (the device addresses follow once they are known)
+            const TileDesc& u = p->tiles_host[(size_t)p->bins[b].t0 + i];
+            UnitRec r{};
+            r.geom = (uint32_t)u.tu | ((uint32_t)u.tv << 8) | ((uint32_t)p->PW << 16);
+            r.box = u.box;
+            r.nvis = (int32_t)(u.ve - u.vb);
+            const int w = box_pairs(u.box);
+            r.mg = (uint32_t)(((1 << 20) + w - 1) / w);
+            r.patch = (int64_t)i * p->PW * p->PW * (int64_t)sizeof(float2);
+            p->recs_host.push_back(r);
+        }
         n_active += (int)tl[b].size();
         p->max_tiles_bin = std::max(p->max_tiles_bin, nu);
     }
@@ -574,24 +603,6 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
         launch_kwtab(p, s);
     }
     p->d_meta = upload(p, meta, s);
-    // chunk descriptors: GTG_CHUNK consecutive visibilities of a unit share one tap range
-    {
-        std::vector<ChunkDesc> ch;
-        for (auto& u : p->tiles_host) {
-            u.cb = (int64_t)ch.size();
-            for (int64_t v0 = u.vb; v0 < u.ve; v0 += GTG_CHUNK) {
-                const int64_t v1 = std::min<int64_t>(u.ve, v0 + GTG_CHUNK);
-                const VisMeta& m0 = meta[v0];
-                const VisMeta& m1 = meta[v1 - 1];
-                const int64_t S1 = (m1.pos >> 16) & 255;
-                const int64_t end = m1.off + S1 * S1 + ((S1 * S1) & 1);
-                ch.push_back(ChunkDesc{m0.off, (uint32_t)((end - m0.off) * 8), m0.pos >> 24});
-            }
-        }
-        p->d_chunks = upload(p, ch, s);
-    }
-    p->d_tiles = upload(p, p->tiles_host, s);
-    p->d_sched = upload(p, p->sched_host, s);
     p->d_merge = upload(p, p->merge_host, s);
     p->d_wr = upload(p, wr_s, s);
     p->d_phiu = upload(p, pu_s, s);
@@ -681,10 +692,18 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
         RIMO_CUDA(cudaGetDevice(&dev));
         RIMO_CUDA(cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, dev));
         p->device = dev;
-        const int s2 = p->max_S * p->max_S;
-        p->chunk_vis = GTG_CHUNK;
-        p->chunk_bytes = p->chunk_vis * (s2 + (s2 & 1)) * (int)sizeof(float2);
     }
+    const int64_t patch_bytes = (int64_t)p->PW * p->PW * (int64_t)sizeof(float2);
+    for (int b = 0; b < P; ++b)
+        for (int i = p->bins[b].t0; i < p->bins[b].t1; ++i) {
+            UnitRec& r = p->recs_host[(size_t)i];
+            const TileDesc& u = p->tiles_host[(size_t)(p->bins[b].t0 + r.patch / patch_bytes)];
+            r.meta = p->d_meta + u.vb;
+            r.taps = ptrs[meta[(size_t)u.vb].pos >> 24];
+            r.fx = p->d_fx;
+            r.status = p->d_status;
+        }
+    p->d_recs = upload(p, p->recs_host, s);
     p->d_AB = (float2*)dev_alloc(p, (size_t)2 * p->nx * p->ny * sizeof(float2));
     p->d_delta = (float2*)dev_alloc(p, (size_t)p->nx * p->ny * sizeof(float2));
     RIMO_CUDA(cudaMemsetAsync(p->d_delta, 0, (size_t)p->nx * p->ny * sizeof(float2), s));

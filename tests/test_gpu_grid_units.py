@@ -1,0 +1,40 @@
+"""The grid step at the edges of its work units (GPU): units of fewer visibilities than a block
+has warps, of one more, and around the 32 visibilities per warp that it holds metadata for;
+every tile side; both uv-tile sizes; units split over several slices; against the FP64 oracle."""
+import math
+
+import numpy as np
+import pytest
+
+from parity_util import TOL, both, rel, to_dev, to_host
+
+pytestmark = pytest.mark.gpu
+
+# (visibilities, kb_support, max_wsupport, uv-tile, spread in grid cells)
+CASES = [
+    (1, 7, 9, 32, 4), (7, 7, 9, 32, 4), (8, 7, 9, 32, 4), (9, 7, 9, 32, 4), (13, 7, 9, 32, 4), (25, 7, 9, 32, 4),
+    (256, 7, 9, 32, 6), (257, 7, 9, 32, 6), (385, 7, 9, 32, 6), (769, 7, 9, 32, 6),
+    (300, 3, 1, 32, 40), (300, 5, 3, 32, 40), (300, 9, 1, 32, 40), (300, 11, 5, 32, 40),
+    (300, 11, 7, 32, 40), (300, 11, 9, 32, 40), (300, 11, 9, 64, 60), (300, 7, 9, 64, 60), (1200, 7, 9, 64, 6),
+]
+
+
+@pytest.mark.parametrize("m, kb, cap, tile, spread", CASES)
+def test_units_of_every_size_and_tile_side(m, kb, cap, tile, spread):
+    n, fov = 64, math.radians(2.0)
+    rng = np.random.default_rng(m * 31 + kb * 7 + cap)
+    uvw = np.empty((m, 3))
+    # a patch of `spread` cells that straddles the wrap of the grid in v
+    uvw[:, 0] = (10.0 + spread * rng.random(m)) / (2.0 * fov)
+    uvw[:, 1] = (spread * (rng.random(m) - 0.5)) / (2.0 * fov)
+    uvw[:, 2] = 2000.0 * (rng.random(m) - 0.5)
+    plan, op = both(uvw, n, n, fov, fov, n_wbins=1, kb_support=kb, max_wsupport=cap, tile_size=tile)
+    x = (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))).astype(np.complex64)
+    y = (rng.standard_normal(m) + 1j * rng.standard_normal(m)).astype(np.complex64)
+    assert rel(to_host(plan.phi(to_dev(x))), op.phi(x)) < TOL
+    assert rel(to_host(plan.phi_adj(to_dev(y))), op.phi_adj(y)) < TOL
+    first = to_host(plan.phi_adj_phi(to_dev(x)))
+    assert rel(first, op.phi_adj_phi(x)) < TOL
+    assert np.array_equal(to_host(plan.phi_adj_phi(to_dev(x))), first)  # fixed-point sums: bit for bit
+    plan.status()
+    plan.close()
