@@ -76,7 +76,7 @@ void destroy_batch(rimo_batch* b) {
 }
 
 // Whether the plans can run as one staged pipeline: stored G (no H, no generated tiles),
-// square images of one size and one uv-tile size (patch sides and tap chunks may differ).
+// square images of one size and one uv-tile size (patch sides may differ).
 bool stage_eligible(const std::vector<rimo_plan*>& plans) {
     const rimo_plan* a = plans[0];
     for (const rimo_plan* p : plans) {
@@ -116,7 +116,7 @@ void stage(rimo_batch* b, cudaStream_t s) {
         b->jobs[j].X = reinterpret_cast<float2*>(base + off[j][1]);
         b->jobs[j].patch = reinterpret_cast<float2*>(base + off[j][2]);
     }
-    b->wgtg = wide_gtg_create(b->jobs, s);
+    b->wgtg = wide_gtg_create(b->jobs, nullptr, s);
 }
 
 // Records the staged pipeline for (x, out): per channel the image bound (flags non-finite
@@ -128,9 +128,11 @@ void record_staged(rimo_batch* b, const float2* x, float2* out, int real_only, c
         else RIMO_CUDA(cudaMemsetAsync(out + c * img, 0, img * sizeof(float2), s));
     }
     if (b->jobs.empty()) return;
-    wide_fwd(b->wfft, s);
-    wide_gtg(b->wgtg, s);
-    wide_inv(b->wfft, real_only, s);
+    wide_fwd_rows(b->wfft, nullptr, s);
+    wide_fwd_cols(b->wfft, s);
+    wide_gtg(b->wgtg, 2, nullptr, nullptr, s);
+    wide_inv_cols(b->wfft, s);
+    wide_inv_rows(b->wfft, nullptr, 0, real_only, s);
 }
 
 // Records all channels' applies into a graph on the batch's own root stream (staged: one

@@ -547,6 +547,9 @@ __device__ __forceinline__ int sel_row0(const RowSel& sel, int b, int rows_per_b
 // shape (a wideband batch, every channel's every bin in one launch per pass): job j owns
 // the launch's blocks [first[j], first[j + 1]), and a block finds its job by bisection and
 // then runs as in a one-job launch, with its block index within the job.
+// The image pointer of a rows job counts from the launch's `img` bytes: 0 with the image's
+// address in the job, or the image's address with null jobs (a plan's tables, whose images
+// come with the call).
 struct RowsJob {          // a rows pass: image rows -> transposed half transforms, or back
     const float2* in;
     float2* out;
@@ -586,13 +589,13 @@ __device__ __forceinline__ const J& block_job(const J& one, const JobTable<J>& t
 // is column i of At (At[k][i], k < 2N).
 template <int N, int RB, int C, bool TABLE>
 __global__ void __launch_bounds__(RB * N / 8, (1024 / (RB * N / 8)) > 0 ? (1024 / (RB * N / 8)) : 1)
-    fwd_rows_kernel(const __grid_constant__ RowsJob one, const JobTable<RowsJob> tab, int ny,
+    fwd_rows_kernel(const __grid_constant__ RowsJob one, const JobTable<RowsJob> tab, int64_t img, int ny,
                     const float2* __restrict__ tws) {
     constexpr int L = 2 * N, T = L / 16, SR = L + L / 16;
     extern __shared__ float2 smem[];
     int bk;
     const RowsJob& J = block_job<TABLE>(one, tab, bk);
-    const float2* __restrict__ x = J.in;
+    const float2* __restrict__ x = reinterpret_cast<const float2*>(reinterpret_cast<const char*>(J.in) + img);
     const ZArgs z = J.z;
     const RowSel& sel = J.sel;
     const int g = threadIdx.x / T, t = threadIdx.x % T;
@@ -886,7 +889,7 @@ __global__ void __launch_bounds__(RB * N / 8, (1024 / (RB * N / 8)) > 0 ? (1024 
 template <int N, int RG, bool TABLE>
 __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 / (RG * N / 8)) : 1)
     inv_rows_kernel(const __grid_constant__ RowsJob one, const JobTable<RowsJob> tab, const int* __restrict__ group,
-                    int ny, int accumulate, int real_only, const float2* __restrict__ tws) {
+                    int64_t img, int ny, int accumulate, int real_only, const float2* __restrict__ tws) {
     constexpr int L = 2 * N, T = L / 16, SR = L + L / 16;
     extern __shared__ float2 smem[];
     const int g = threadIdx.x / T, t = threadIdx.x % T;
@@ -905,7 +908,8 @@ __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 
         const RowSel& sel = J.sel;
         const ZArgs z = J.z;
         const float2* __restrict__ in = J.in + (size_t)i * L;
-        float2* __restrict__ orow = J.out + (size_t)i * N;
+        float2* __restrict__ orow =
+            reinterpret_cast<float2*>(reinterpret_cast<char*>(J.out) + img) + (size_t)i * N;
         const int acc = accumulate || jj > j0;
         float2 v[16];
         // columns u of tile rows the inverse column pass skipped are zero (not stored)
@@ -1095,8 +1099,8 @@ static int tile_shift(int TS) { return TS == 64 ? 6 : 5; }
 
 // One launch of each pass, for one job (TABLE = false: `one`) or a job table.
 template <int N, bool TABLE>
-static void run_fwd_rows(const RowsJob& one, const JobTable<RowsJob>& tab, int grid, int ny, const float2* tws,
-                         cudaStream_t s) {
+static void run_fwd_rows(const RowsJob& one, const JobTable<RowsJob>& tab, int64_t img, int grid, int ny,
+                         const float2* tws, cudaStream_t s) {
     constexpr int RB = rows_per_block<N>();
     constexpr int C = cluster_of<RB>();
     const size_t sm = (size_t)RB * (2 * N + N / 8) * sizeof(float2);
@@ -1104,10 +1108,10 @@ static void run_fwd_rows(const RowsJob& one, const JobTable<RowsJob>& tab, int g
     if constexpr (C > 1) {
         if (grid % C != 0) fail(RIMO_ERR_UNSUPPORTED, "image rows do not fill the transposed-store clusters");
         set_smem(fwd_rows_kernel<N, RB, C, TABLE>, sm);
-        launch_clustered(fwd_rows_kernel<N, RB, C, TABLE>, grid, RB * N / 8, sm, C, s, one, tab, ny, tws);
+        launch_clustered(fwd_rows_kernel<N, RB, C, TABLE>, grid, RB * N / 8, sm, C, s, one, tab, img, ny, tws);
     } else {
         set_smem(fwd_rows_kernel<N, RB, 1, TABLE>, sm);
-        fwd_rows_kernel<N, RB, 1, TABLE><<<grid, RB * N / 8, sm, s>>>(one, tab, ny, tws);
+        fwd_rows_kernel<N, RB, 1, TABLE><<<grid, RB * N / 8, sm, s>>>(one, tab, img, ny, tws);
     }
 }
 
@@ -1169,13 +1173,13 @@ static void run_inv_cols(const ColsJob& one, const JobTable<ColsJob>& tab, int g
 }
 
 template <int N, bool TABLE>
-static void run_inv_rows(const RowsJob& one, const JobTable<RowsJob>& tab, const int* group, int grid, int ny, int acc,
-                         int re, const float2* tws, cudaStream_t s) {
+static void run_inv_rows(const RowsJob& one, const JobTable<RowsJob>& tab, const int* group, int64_t img, int grid,
+                         int ny, int acc, int re, const float2* tws, cudaStream_t s) {
     constexpr int RG = rows_per_block<N>();
     const size_t sm = (size_t)RG * (2 * N + N / 8) * sizeof(float2);
     if (grid == 0) return;
     set_smem(inv_rows_kernel<N, RG, TABLE>, sm);
-    inv_rows_kernel<N, RG, TABLE><<<grid, RG * N / 8, sm, s>>>(one, tab, group, ny, acc, re, tws);
+    inv_rows_kernel<N, RG, TABLE><<<grid, RG * N / 8, sm, s>>>(one, tab, group, img, ny, acc, re, tws);
 }
 
 template <class J>
@@ -1189,7 +1193,7 @@ static JobTable<J> no_table() {
 
 template <int N>
 static void fwd_rows(const rimo_plan* p, int bin, const float2* x, float2* At, cudaStream_t s) {
-    run_fwd_rows<N, false>(rows_job(p, bin, x, At, fwd_sel(p, bin)), no_table<RowsJob>(),
+    run_fwd_rows<N, false>(rows_job(p, bin, x, At, fwd_sel(p, bin)), no_table<RowsJob>(), 0,
                            p->ny / rows_per_block<N>(), p->ny, p->tab.tws_x, s);
 }
 
@@ -1213,7 +1217,7 @@ static void inv_cols(const rimo_plan* p, int bin, bool holo, float2* B, cudaStre
 template <int N>
 static void inv_rows(const rimo_plan* p, int bin, const float2* B, float2* out, int acc, int re,
                      cudaStream_t s) {
-    run_inv_rows<N, false>(rows_job(p, bin, B, out, inv_sel(p, bin)), no_table<RowsJob>(), nullptr,
+    run_inv_rows<N, false>(rows_job(p, bin, B, out, inv_sel(p, bin)), no_table<RowsJob>(), nullptr, 0,
                            p->ny / rows_per_block<N>(), p->ny, acc, re, p->tab.tws_x, s);
 }
 
@@ -1231,30 +1235,17 @@ struct WideFft {
     };
     Pass rows_fwd, cols_fwd, fold, cols_inv, rows_inv;
     int* group = nullptr;  // rows_inv: jobs of channel c are [group[c], group[c + 1])
-    std::vector<void*> owned;
-    ~WideFft() {
-        for (void* q : owned) cudaFree(q);
-    }
+    char* tables = nullptr;  // every table, one allocation
+    ~WideFft() { cudaFree(tables); }
 };
 
-template <class J>
-static WideFft::Pass upload_pass(WideFft* w, const std::vector<J>& jobs, const std::vector<int>& first,
-                                 cudaStream_t s) {
-    WideFft::Pass ps;
-    ps.njobs = (int)jobs.size();
-    ps.blocks = first.empty() ? 0 : first.back();
-    if (jobs.empty()) return ps;
-    void* dj = nullptr;
-    void* df = nullptr;
-    RIMO_CUDA(cudaMalloc(&dj, jobs.size() * sizeof(J)));
-    w->owned.push_back(dj);
-    RIMO_CUDA(cudaMalloc(&df, first.size() * sizeof(int)));
-    w->owned.push_back(df);
-    RIMO_CUDA(cudaMemcpyAsync(dj, jobs.data(), jobs.size() * sizeof(J), cudaMemcpyHostToDevice, s));
-    RIMO_CUDA(cudaMemcpyAsync(df, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-    ps.jobs = dj;
-    ps.first = (int*)df;
-    return ps;
+// Appends an array to the host image of the tables (256-byte aligned); its offset.
+template <class T>
+static size_t append(std::vector<char>& blob, const std::vector<T>& v) {
+    const size_t at = (blob.size() + 255) & ~(size_t)255;
+    blob.resize(at + v.size() * sizeof(T));
+    if (!v.empty()) std::memcpy(blob.data() + at, v.data(), v.size() * sizeof(T));
+    return at;
 }
 
 WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<const float2*>& x,
@@ -1271,7 +1262,7 @@ WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<con
         w->tws_y = p0->tab.tws_y;
         w->tws32 = p0->tab.tws32;
         w->ngroups = (int)x.size();
-        const int rb = 4096 / p0->nx;  // rows per block of every pass (nx = ny)
+        const int rb = 4096 / p0->nx, cb = 4096 / p0->ny;  // rows per block of the rows and the cols passes
         std::vector<RowsJob> rf, ri;
         std::vector<ColsJob> cf, ci;
         std::vector<FoldArgs> fo;
@@ -1282,24 +1273,37 @@ WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<con
             rf.push_back(rows_job(p, j.bin, x[j.group], j.AB, fs));
             frf.push_back(frf.back() + p->ny / rb);
             cf.push_back(cols_job(p, j.bin, j.AB, j.X, fs));
-            fcf.push_back(fcf.back() + sel_blocks(p, j.bin, fs, rb));
+            fcf.push_back(fcf.back() + sel_blocks(p, j.bin, fs, cb));
             fo.push_back(fold_args(p, j.bin, j.patch, nullptr, j.X));
             ffo.push_back(ffo.back() + (p->bins[j.bin].n1 - p->bins[j.bin].n0));
             ci.push_back(cols_job(p, j.bin, j.X, j.AB, is));
-            fci.push_back(fci.back() + sel_blocks(p, j.bin, is, rb));
+            fci.push_back(fci.back() + sel_blocks(p, j.bin, is, cb));
             ri.push_back(rows_job(p, j.bin, j.AB, out[j.group], is));
             grp[j.group + 1]++;
         }
         for (int c = 0; c < w->ngroups; ++c) grp[c + 1] += grp[c];
-        w->rows_fwd = upload_pass(w, rf, frf, s);
-        w->cols_fwd = upload_pass(w, cf, fcf, s);
-        w->fold = upload_pass(w, fo, ffo, s);
-        w->cols_inv = upload_pass(w, ci, fci, s);
-        w->rows_inv = upload_pass(w, ri, std::vector<int>{0, w->ngroups * (p0->ny / rb)}, s);
-        RIMO_CUDA(cudaMalloc(&w->group, grp.size() * sizeof(int)));
-        w->owned.push_back(w->group);
-        RIMO_CUDA(cudaMemcpyAsync(w->group, grp.data(), grp.size() * sizeof(int), cudaMemcpyHostToDevice, s));
-        RIMO_CUDA(cudaStreamSynchronize(s));  // the host vectors go out of scope
+        std::vector<char> blob;
+        std::vector<std::pair<WideFft::Pass*, std::pair<size_t, size_t>>> at;
+        auto pass = [&](WideFft::Pass& ps, const auto& jobs, const std::vector<int>& first) {
+            ps.njobs = (int)jobs.size();
+            ps.blocks = first.back();
+            const size_t a = append(blob, jobs);
+            at.push_back({&ps, {a, append(blob, first)}});
+        };
+        pass(w->rows_fwd, rf, frf);
+        pass(w->cols_fwd, cf, fcf);
+        pass(w->fold, fo, ffo);
+        pass(w->cols_inv, ci, fci);
+        pass(w->rows_inv, ri, std::vector<int>{0, w->ngroups * (p0->ny / rb)});
+        const size_t gat = append(blob, grp);
+        RIMO_CUDA(cudaMalloc(&w->tables, blob.size()));
+        RIMO_CUDA(cudaMemcpyAsync(w->tables, blob.data(), blob.size(), cudaMemcpyHostToDevice, s));
+        for (auto& q : at) {
+            q.first->jobs = w->tables + q.second.first;
+            q.first->first = reinterpret_cast<int*>(w->tables + q.second.second);
+        }
+        w->group = reinterpret_cast<int*>(w->tables + gat);
+        RIMO_CUDA(cudaStreamSynchronize(s));  // the host image goes out of scope
     } catch (...) {
         delete w;
         throw;
@@ -1318,34 +1322,43 @@ static JobTable<J> table_of(const WideFft::Pass& ps) {
     return t;
 }
 
-template <int N>
-static void wide_fwd_n(const WideFft* w, cudaStream_t s) {
-    RowsJob r1;
-    ColsJob c1;
-    std::memset(&r1, 0, sizeof(r1));
-    std::memset(&c1, 0, sizeof(c1));
-    run_fwd_rows<N, true>(r1, table_of<RowsJob>(w->rows_fwd), w->rows_fwd.blocks, w->ny, w->tws_x, s);
-    run_fwd_cols<N, true>(c1, table_of<ColsJob>(w->cols_fwd), w->cols_fwd.blocks, w->TS, w->tws_y, s, w->tws32);
+template <class J>
+static J no_job() {
+    J j;
+    std::memset(&j, 0, sizeof(j));
+    return j;
 }
 
 template <int N>
-static void wide_inv_n(const WideFft* w, int real_only, cudaStream_t s) {
-    RowsJob r1;
-    ColsJob c1;
-    FoldArgs f1;
-    std::memset(&r1, 0, sizeof(r1));
-    std::memset(&c1, 0, sizeof(c1));
-    std::memset(&f1, 0, sizeof(f1));
-    run_fold<true>(f1, table_of<FoldArgs>(w->fold), w->fold.blocks, w->TS, s);
-    run_inv_cols<N, true>(c1, table_of<ColsJob>(w->cols_inv), w->cols_inv.blocks, w->gx, w->TS, w->tws_y, s,
+static void wide_rows_fwd(const WideFft* w, int64_t img, cudaStream_t s) {
+    run_fwd_rows<N, true>(no_job<RowsJob>(), table_of<RowsJob>(w->rows_fwd), img, w->rows_fwd.blocks, w->ny, w->tws_x, s);
+}
+template <int N>
+static void wide_cols_fwd(const WideFft* w, cudaStream_t s) {
+    run_fwd_cols<N, true>(no_job<ColsJob>(), table_of<ColsJob>(w->cols_fwd), w->cols_fwd.blocks, w->TS, w->tws_y, s,
                           w->tws32);
-    run_inv_rows<N, true>(r1, table_of<RowsJob>(w->rows_inv), w->group, w->rows_inv.blocks, w->ny, 0, real_only,
-                          w->tws_x, s);
+}
+template <int N>
+static void wide_cols_inv(const WideFft* w, cudaStream_t s) {
+    run_inv_cols<N, true>(no_job<ColsJob>(), table_of<ColsJob>(w->cols_inv), w->cols_inv.blocks, w->gx, w->TS, w->tws_y,
+                          s, w->tws32);
+}
+template <int N>
+static void wide_rows_inv(const WideFft* w, int64_t img, int acc, int real_only, cudaStream_t s) {
+    run_inv_rows<N, true>(no_job<RowsJob>(), table_of<RowsJob>(w->rows_inv), w->group, img, w->rows_inv.blocks, w->ny,
+                          acc, real_only, w->tws_x, s);
 }
 
-void wide_fwd(const WideFft* w, cudaStream_t s) { RIMO_DISPATCH_N(w->nx, wide_fwd_n<NN>(w, s)); }
-void wide_inv(const WideFft* w, int real_only, cudaStream_t s) {
-    RIMO_DISPATCH_N(w->nx, wide_inv_n<NN>(w, real_only, s));
+void wide_fwd_rows(const WideFft* w, const float2* x, cudaStream_t s) {
+    RIMO_DISPATCH_N(w->nx, wide_rows_fwd<NN>(w, (int64_t)(uintptr_t)x, s));
+}
+void wide_fwd_cols(const WideFft* w, cudaStream_t s) { RIMO_DISPATCH_N(w->ny, wide_cols_fwd<NN>(w, s)); }
+void wide_inv_cols(const WideFft* w, cudaStream_t s) {
+    run_fold<true>(no_job<FoldArgs>(), table_of<FoldArgs>(w->fold), w->fold.blocks, w->TS, s);
+    RIMO_DISPATCH_N(w->ny, wide_cols_inv<NN>(w, s));
+}
+void wide_inv_rows(const WideFft* w, float2* out, int acc, int real_only, cudaStream_t s) {
+    RIMO_DISPATCH_N(w->nx, wide_rows_inv<NN>(w, (int64_t)(uintptr_t)out, acc, real_only, s));
 }
 
 void launch_fwd_rows(const rimo_plan* p, int bin, const float2* x, float2* At, cudaStream_t s) {

@@ -661,7 +661,8 @@ static void (*gtg_kernel_for(int PW))(GtgArgs) {
 }
 
 template <int MODE>
-static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_out, cudaStream_t s) {
+static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_out, cudaStream_t s, const float2* X,
+                    float2* patch) {
     const auto& br = p->bins[bin];
     const int nu = br.t1 - br.t0;
     if (nu <= 0) return;
@@ -670,8 +671,8 @@ static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_o
     A.recs = p->d_recs + br.t0;
     A.nunits = nu;
     A.counter = p->d_counter + bin;  // zeroed at the start of every apply
-    A.X = p->d_X;
-    A.patch = p->d_patch;
+    A.X = X ? X : p->d_X;
+    A.patch = patch ? patch : p->d_patch;
     A.y_in = y_in;
     A.y_out = y_out;
     const GtgShape g = gtg_shape(p, p->PW, p->max_S, MODE, A);
@@ -680,7 +681,7 @@ static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_o
     kern<<<std::min(nu, p->n_sm * g.blocks_per_sm), g.warps * 32, g.smem, s>>>(A);
     if (MODE != 0 && br.m1 > br.m0) {
         MergeJob mj;
-        mj.patch = p->d_patch;
+        mj.patch = A.patch;
         mj.groups = p->d_merge + br.m0;
         mj.npatch = p->PW * p->PW;
         merge_patches_kernel<false><<<br.m1 - br.m0, 256, 0, s>>>(mj, nullptr, nullptr, 0);
@@ -691,41 +692,43 @@ static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_o
 // The grid step of a stage-batched apply: one persistent launch over the units of every
 // (plan, bin) job, taken heaviest first from one list, then one merge launch.
 struct WideGtg {
-    GtgArgs A;
-    GtgShape shape{};
-    int grid = 0, merge_blocks = 0, njobs = 0, PW = 0;
+    const rimo_plan* p0 = nullptr;
+    int merge_blocks = 0, njobs = 0;
+    int PW = 0, max_S = 0;   // the jobs' largest patch and tile sides
+    bool one_pw = true;      // one patch side: its compile-time kernel; several: the kernel reading each record's
     UnitRec* recs = nullptr;
     MergeJob* mjobs = nullptr;
     int* mfirst = nullptr;
-    int* counter = nullptr;  // the units taken (zeroed before every launch)
+    int* counter = nullptr;
+    int* own_counter = nullptr;
     int64_t units = 0;
     ~WideGtg() {
         cudaFree(recs);
         cudaFree(mjobs);
         cudaFree(mfirst);
-        cudaFree(counter);
+        cudaFree(own_counter);
     }
 };
 
-WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, cudaStream_t s) {
+WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStream_t s) {
     if (jobs.empty()) fail(RIMO_ERR_INVALID_ARG, "no jobs");
     auto* w = new WideGtg();
     try {
         const rimo_plan* p0 = jobs[0].p;
-        int pw_max = 0, s_max = 0;
-        bool one_pw = true;
+        w->p0 = p0;
         for (const WideJob& j : jobs) {
-            pw_max = std::max(pw_max, j.p->PW);
-            s_max = std::max(s_max, j.p->max_S);
-            one_pw = one_pw && j.p->PW == p0->PW;
+            w->PW = std::max(w->PW, j.p->PW);
+            w->max_S = std::max(w->max_S, j.p->max_S);
+            w->one_pw = w->one_pw && j.p->PW == p0->PW;
         }
-        std::memset(&w->A, 0, sizeof(w->A));
-        w->shape = gtg_shape(p0, pw_max, s_max, 2, w->A);
-        // one patch side: its compile-time kernel; several: the kernel reading each job's
-        w->PW = one_pw ? p0->PW : 0;
         std::vector<MergeJob> mj;
         std::vector<int> mf{0};
         std::vector<UnitRec> recs;
+        size_t nrec = 0;
+        for (const WideJob& j : jobs) nrec += (size_t)(j.p->bins[j.bin].t1 - j.p->bins[j.bin].t0);
+        // (a unit index plus the blocks' look-ahead stays an int)
+        if (nrec > (size_t)0x7fffffff - 8 * 4096) fail(RIMO_ERR_UNSUPPORTED, "too many work units for one launch");
+        recs.reserve(nrec);
         for (size_t j = 0; j < jobs.size(); ++j) {
             const rimo_plan* p = jobs[j].p;
             if (p->TS != p0->TS || p->gx != p0->gx || p->gy != p0->gy)
@@ -744,26 +747,29 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, cudaStream_t s) {
             mj.push_back(m);
             mf.push_back(mf.back() + (br.m1 - br.m0));
         }
-        // heaviest first over the whole batch (ties: job, then the bin's order)
-        std::stable_sort(recs.begin(), recs.end(), [](const UnitRec& a, const UnitRec& b) { return a.nvis > b.nvis; });
+        // heaviest first over all jobs (ties: job, then the bin's order)
+        {
+            std::vector<uint64_t> key(recs.size());
+            for (size_t i = 0; i < recs.size(); ++i)
+                key[i] = ((uint64_t)(0xffffffffu - (uint32_t)recs[i].nvis) << 32) | (uint32_t)i;
+            std::sort(key.begin(), key.end());
+            std::vector<UnitRec> sorted(recs.size());
+            for (size_t i = 0; i < recs.size(); ++i) sorted[i] = recs[(uint32_t)key[i]];
+            recs.swap(sorted);
+        }
         w->units = (int64_t)recs.size();
         w->njobs = (int)jobs.size();
         w->merge_blocks = mf.back();
-        // (a unit index plus the blocks' look-ahead stays an int)
-        if (w->units > 0x7fffffffLL - 8 * 4096) fail(RIMO_ERR_UNSUPPORTED, "too many work units for one launch");
         RIMO_CUDA(cudaMalloc(&w->recs, std::max<size_t>(1, recs.size()) * sizeof(UnitRec)));
         RIMO_CUDA(cudaMalloc(&w->mjobs, mj.size() * sizeof(MergeJob)));
         RIMO_CUDA(cudaMalloc(&w->mfirst, mf.size() * sizeof(int)));
-        RIMO_CUDA(cudaMalloc(&w->counter, sizeof(int)));
+        if (!counter) RIMO_CUDA(cudaMalloc(&w->own_counter, sizeof(int)));
+        w->counter = counter ? counter : w->own_counter;
         if (!recs.empty())
             RIMO_CUDA(cudaMemcpyAsync(w->recs, recs.data(), recs.size() * sizeof(UnitRec), cudaMemcpyHostToDevice, s));
         RIMO_CUDA(cudaMemcpyAsync(w->mjobs, mj.data(), mj.size() * sizeof(MergeJob), cudaMemcpyHostToDevice, s));
         RIMO_CUDA(cudaMemcpyAsync(w->mfirst, mf.data(), mf.size() * sizeof(int), cudaMemcpyHostToDevice, s));
         RIMO_CUDA(cudaStreamSynchronize(s));
-        w->A.recs = w->recs;
-        w->A.nunits = (int)w->units;
-        w->A.counter = w->counter;
-        w->grid = (int)std::min<int64_t>(w->units, (int64_t)p0->n_sm * w->shape.blocks_per_sm);
     } catch (...) {
         delete w;
         throw;
@@ -775,26 +781,35 @@ void wide_gtg_destroy(WideGtg* w) { delete w; }
 
 int64_t wide_gtg_units(const WideGtg* w) { return w->units; }
 
-void wide_gtg(const WideGtg* w, cudaStream_t s) {
-    if (w->units == 0) return;
-    void (*kern)(GtgArgs) = gtg_kernel_for<2>(w->PW);
-    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w->shape.smem));
-    RIMO_CUDA(cudaMemsetAsync(w->counter, 0, sizeof(int), s));
-    kern<<<w->grid, w->shape.warps * 32, w->shape.smem, s>>>(w->A);
-    if (w->merge_blocks > 0) {
-        MergeJob none;
-        none.patch = nullptr;
-        none.groups = nullptr;
-        none.npatch = 0;
-        merge_patches_kernel<true><<<w->merge_blocks, 256, 0, s>>>(none, w->mjobs, w->mfirst, w->njobs);
-    }
+int wide_gtg(const WideGtg* w, int mode, const float2* y_in, float2* y_out, cudaStream_t s) {
+    if (w->units == 0) return 0;
+    GtgArgs A;
+    std::memset(&A, 0, sizeof(A));
+    const GtgShape g = gtg_shape(w->p0, w->PW, w->max_S, mode, A);
+    A.recs = w->recs;
+    A.nunits = (int)w->units;
+    A.counter = w->counter;
+    A.y_in = y_in;
+    A.y_out = y_out;
+    const int pw = w->one_pw ? w->PW : 0;
+    void (*kern)(GtgArgs) = mode == 0 ? gtg_kernel_for<0>(pw) : mode == 1 ? gtg_kernel_for<1>(pw) : gtg_kernel_for<2>(pw);
+    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+    if (w->own_counter) RIMO_CUDA(cudaMemsetAsync(w->counter, 0, sizeof(int), s));
+    kern<<<(int)std::min<int64_t>(w->units, (int64_t)w->p0->n_sm * g.blocks_per_sm), g.warps * 32, g.smem, s>>>(A);
+    if (mode == 0 || w->merge_blocks == 0) return 1;
+    MergeJob none;
+    none.patch = nullptr;
+    none.groups = nullptr;
+    none.npatch = 0;
+    merge_patches_kernel<true><<<w->merge_blocks, 256, 0, s>>>(none, w->mjobs, w->mfirst, w->njobs);
+    return 2;
 }
 
 void launch_gtg(const rimo_plan* p, int bin, int mode, const float2* y_in, float2* y_out,
-                cudaStream_t s) {
-    if (mode == 0) gtg_run<0>(p, bin, y_in, y_out, s);
-    else if (mode == 1) gtg_run<1>(p, bin, y_in, y_out, s);
-    else gtg_run<2>(p, bin, y_in, y_out, s);
+                cudaStream_t s, const float2* X, float2* patch) {
+    if (mode == 0) gtg_run<0>(p, bin, y_in, y_out, s, X, patch);
+    else if (mode == 1) gtg_run<1>(p, bin, y_in, y_out, s, X, patch);
+    else gtg_run<2>(p, bin, y_in, y_out, s, X, patch);
 }
 
 // ---------------------------------------------------------------------------

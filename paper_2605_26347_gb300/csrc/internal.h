@@ -119,6 +119,10 @@ struct DevTables {
 
 }  // namespace rimo
 
+namespace rimo {
+struct PlanStage;
+}
+
 // The plan object behind rimo_plan_t.
 struct rimo_plan {
     rimo_plan_params prm{};
@@ -191,6 +195,8 @@ struct rimo_plan {
     int32_t* d_hslot = nullptr;           // [bin][tile] -> needed-tile index in the bin, or -1
     float2* d_hpatch = nullptr;           // H-apply output patches of one bin [needed tile][PW*PW]
     int32_t* d_hent = nullptr;            // entry table (type << 16 | a << 8 | |b|)
+    rimo::PlanStage* stage = nullptr;     // groups of bins that share launches, or null
+    bool bin_by_bin = false;              // this call keeps to one bin at a time (allocation-free apply)
     float2* d_AB = nullptr;    // half-transformed intermediates (2 nx ny)
     float2* d_delta = nullptr; // delta image for the PSF
     rimo::DevTables tab;
@@ -260,8 +266,9 @@ void launch_inv_rows(const rimo_plan* p, int bin, const float2* B, float2* out, 
                      int real_only, cudaStream_t s);
 // mode 0: degrid (y_out), 1: grid (y_in), 2: fused degrid + grid.  Modes 1 and 2 write the
 // accumulator patch of every active tile of the bin to p->d_patch.
+// X, patch: the bin's forward grid and patches (null: the plan's d_X and d_patch)
 void launch_gtg(const rimo_plan* p, int bin, int mode, const float2* y_in, float2* y_out,
-                cudaStream_t s);
+                cudaStream_t s, const float2* X = nullptr, float2* patch = nullptr);
 void launch_gbuild(const rimo_plan* p, cudaStream_t s);
 // exact tiles of the sorted visibilities [v0, v0 + n) into their block (the on-the-fly mode's
 // scratch), with the tap bounds of the fixed-point grid step
@@ -291,16 +298,40 @@ __device__ __forceinline__ int job_of(const int* first, int njobs, int b) {
     return lo;
 }
 struct WideFft;   // device job tables of the transform passes (fft.cu)
-struct WideGtg;   // device unit queue of the grid step (grid.cu)
+struct WideGtg;   // device unit list of the grid step (grid.cu)
+// x, out: the images of each group (null: every group's images come with the launches)
 WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<const float2*>& x,
                          const std::vector<float2*>& out, cudaStream_t s);
 void wide_fft_destroy(WideFft* w);
-void wide_fwd(const WideFft* w, cudaStream_t s);                 // F Z_p of every job
-void wide_inv(const WideFft* w, int real_only, cudaStream_t s);  // fold, Z_p^H F^H, Sigma_p per channel
-WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, cudaStream_t s);
+// F Z_p of every job: rows and cols pass (x: see wide_fft_create, null with tables that hold it)
+void wide_fwd_rows(const WideFft* w, const float2* x, cudaStream_t s);
+void wide_fwd_cols(const WideFft* w, cudaStream_t s);
+// the fold and F^H, then Z_p^H and Sigma_p per group (acc: added to the image)
+void wide_inv_cols(const WideFft* w, cudaStream_t s);
+void wide_inv_rows(const WideFft* w, float2* out, int acc, int real_only, cudaStream_t s);
+// counter: the launches' unit counter (device, zero before each launch), or null for one of its
+// own, which every launch clears
+WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStream_t s);
 void wide_gtg_destroy(WideGtg* w);
 int64_t wide_gtg_units(const WideGtg* w);
-void wide_gtg(const WideGtg* w, cudaStream_t s);  // G_p^H G_p of every job: one persistent launch
+// the grid step of every job, one persistent launch (mode, y_in, y_out as in launch_gtg), and
+// the merge of split tiles; returns the kernel launches
+int wide_gtg(const WideGtg* w, int mode, const float2* y_in, float2* y_out, cudaStream_t s);
+
+// The bins of one plan in groups that share a launch per pass (see stage_plan in apply.cu).
+struct PlanStage {
+    struct Group {
+        std::vector<WideJob> jobs;
+        WideFft* fft = nullptr;
+        WideGtg* gtg = nullptr;   // stored G; else the bins' grid steps follow their tile generation
+    };
+    std::vector<Group> groups;
+    void* scratch = nullptr;
+    int64_t scratch_bytes = 0;
+    ~PlanStage();
+};
+// Sets p->stage where it pays and its scratch can be had (at the end of plan creation).
+void stage_plan(rimo_plan* p, cudaStream_t s);
 
 // Whether a plan of max_units work units per w-bin fits the allocation-free apply's scratch.
 bool noalloc_fits(const rimo_plan* p, int max_units);

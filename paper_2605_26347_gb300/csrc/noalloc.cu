@@ -84,6 +84,7 @@ extern "C" rimo_status rimo_apply_phi_adj_phi_noalloc(rimo_plan_t p, const rimo_
         float2* own_ab = p->d_AB;
         float2* own_x = p->d_X;
         float2* own_patch = p->d_patch;
+        p->bin_by_bin = true;
         p->d_counter = reinterpret_cast<int32_t*>(base);
         p->d_AB = reinterpret_cast<float2*>(base + counters);
         p->d_X = reinterpret_cast<float2*>(base + counters + ab);
@@ -92,12 +93,14 @@ extern "C" rimo_status rimo_apply_phi_adj_phi_noalloc(rimo_plan_t p, const rimo_
             apply_phi_adj_phi(p, (const float2*)x, (float2*)out, real_part_only, s);
             RIMO_CUDA(cudaGetLastError());
         } catch (...) {
+            p->bin_by_bin = false;
             p->d_counter = own_counter;
             p->d_AB = own_ab;
             p->d_X = own_x;
             p->d_patch = own_patch;
             throw;
         }
+        p->bin_by_bin = false;
         p->d_counter = own_counter;
         p->d_AB = own_ab;
         p->d_X = own_x;

@@ -505,6 +505,12 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
     // split that still does.
     p->tiles_host.clear();
     p->recs_host.clear();
+    {
+        size_t n = 0;
+        for (const auto& v : tl) n += v.size();
+        p->recs_host.reserve(n);
+        p->tiles_host.reserve(n);
+    }
     p->merge_host.clear();
     int n_active = 0;
     std::vector<int32_t> slot((size_t)P * ntile, -1);
@@ -721,6 +727,8 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
     for (const TileDesc& u : p->tiles_host)
         p->info.box_cells += (int64_t)(((u.box >> 8) & 255u) - (u.box & 255u)) * (int64_t)((u.box >> 24) - ((u.box >> 16) & 255u));
 
+    stage_plan(p, s);
+
     // ---- stage 3: precompute G on the device (the surrogate generates it at apply time)
     if (!generated) {
         prof_begin(p, ST_GBUILD, s);
@@ -800,6 +808,7 @@ rimo_status rimo_plan_create(const double* uvw, int64_t M, const rimo_plan_param
 
 rimo_status rimo_plan_destroy(rimo_plan_t p) {
     if (!p) return RIMO_OK;
+    delete p->stage;
     for (void* ptr : p->owned) cudaFree(ptr);
     for (auto& m : p->prof_pending) {
         cudaEventDestroy(m.a);
