@@ -569,6 +569,13 @@ struct JobTable {
     int njobs;
 };
 
+// A table's image pointer counts from img (see RowsJob).
+template <bool TABLE, class T>
+__device__ __forceinline__ T* at_image(T* p, int64_t img) {
+    if constexpr (TABLE) return reinterpret_cast<T*>(reinterpret_cast<uintptr_t>(p) + (uintptr_t)img);
+    else return p;
+}
+
 // This block's job and its block index b within the job.
 template <bool TABLE, class J>
 __device__ __forceinline__ const J& block_job(const J& one, const JobTable<J>& tab, int& b) {
@@ -595,7 +602,7 @@ __global__ void __launch_bounds__(RB * N / 8, (1024 / (RB * N / 8)) > 0 ? (1024 
     extern __shared__ float2 smem[];
     int bk;
     const RowsJob& J = block_job<TABLE>(one, tab, bk);
-    const float2* __restrict__ x = reinterpret_cast<const float2*>(reinterpret_cast<const char*>(J.in) + img);
+    const float2* __restrict__ x = at_image<TABLE>(J.in, img);
     const ZArgs z = J.z;
     const RowSel& sel = J.sel;
     const int g = threadIdx.x / T, t = threadIdx.x % T;
@@ -754,90 +761,78 @@ struct FoldArgs {
     int ntu, ntv, TS, H, PW, gy;
 };
 
-// TSC: the tile side (32 or 64) as a compile-time constant, so the cell indexing is shifts
+// TSC: the tile side (32 or 64) as a compile-time constant, so the cell indexing is shifts.
+// A thread folds pairs of cells (16-byte loads and stores): the grid step writes its boxes
+// widened to whole pairs of columns (its added cells hold zeros), so a pair is in a box or not
+// as a whole.  With one cell per load and 64-bit patch offsets per cell the kernel was bound by
+// its index arithmetic (149 instructions per cell and warp, the integer pipe 70 % busy): four
+// bins of 1024^2/2M 98 -> 67 us (4.0 TB/s of boxes and tiles), 4096^2/24M inverse cols + fold
+// 6.71 -> 6.31 ms per apply.
 template <bool TABLE, int TSC>
 __global__ void __launch_bounds__(256) fold_kernel(const __grid_constant__ FoldArgs one, const JobTable<FoldArgs> tab) {
     int bk;
     const FoldArgs& F = block_job<TABLE>(one, tab, bk);
-    constexpr int TS = TSC;
+    constexpr int TS = TSC, ROW = TS / 2;  // pairs per row
     const int tile = F.tiles[bk];
     const int tu = tile / F.ntv, tv = tile - tu * F.ntv;
     const int tu1 = tu == 0 ? F.ntu - 1 : tu - 1, tv1 = tv == 0 ? F.ntv - 1 : tv - 1;
-    const size_t np = (size_t)F.PW * F.PW;
-    const uint32_t whole = box_pack(0, F.PW, 0, F.PW);
-    // slot and box of tile t (an empty box for a tile without a patch)
-    auto get = [&](int t, int& sl) {
+    const int PW = F.PW, H = F.H;
+    const uint32_t whole = box_pack(0, PW, 0, PW);
+    // the box of tile t's patch in this tile's cells, its cells (a, b) being the patch's
+    // (a + oa, b + ob): rows [a, a + na), columns [b, b + nb) (nothing without a patch), and
+    // the patch's address moved by that offset
+    struct Src {
+        const float2* p;
+        int a, na, b, nb;
+    };
+    auto src = [&](int t, int oa, int ob, int ca, int cb) {
+        Src r;
+        int sl;
+        uint32_t x = whole;
         if (F.slotbox) {
             const int2 q = F.slotbox[t];
             sl = q.x;
-            return sl < 0 ? 0u : (uint32_t)q.y;
+            x = (uint32_t)q.y;
+        } else {
+            sl = F.slot[t];
         }
-        sl = F.slot[t];
-        return sl < 0 ? 0u : whole;
-    };
-    int s00, s10, s01, s11;
-    const uint32_t x00 = get(tu * F.ntv + tv, s00), x10 = get(tu1 * F.ntv + tv, s10);
-    const uint32_t x01 = get(tu * F.ntv + tv1, s01), x11 = get(tu1 * F.ntv + tv1, s11);
-    // a box in the tile's cells (a, b): patch cells (a + oa, b + ob) with (oa, ob) the tile's
-    // offset in that patch; [lo, lo + n) per axis, compared unsigned (empty: n = 0)
-    struct Rng {
-        int a, na, b, nb;
-    };
-    auto rng = [&](uint32_t x, int oa, int ob) {
-        Rng r;
-        r.a = (int)(x & 255u) - oa;
-        r.na = max(0, (int)((x >> 8) & 255u) - oa - r.a);
-        r.b = (int)((x >> 16) & 255u) - ob;
-        r.nb = max(0, (int)(x >> 24) - ob - r.b);
+        if (sl < 0) x = 0u;
+        r.p = F.patch + (size_t)max(sl, 0) * PW * PW + oa * PW + ob;
+        // (a box reaches at most ca rows and cb columns into this tile)
+        r.a = max((int)(x & 255u) - oa, 0);
+        r.na = max(0, min((int)((x >> 8) & 255u) - oa, ca) - r.a);
+        r.b = max((int)((x >> 16) & 254u) - ob, 0);
+        r.nb = max(0, min((int)(((x >> 24) + 1u) & 254u) - ob, cb) - r.b);
         return r;
     };
-    auto in = [](const Rng& r, int a, int b) {
-        return (unsigned)(a - r.a) < (unsigned)r.na && (unsigned)(b - r.b) < (unsigned)r.nb;
+    const Src s00 = src(tu * F.ntv + tv, 0, 0, TS, TS), s10 = src(tu1 * F.ntv + tv, TS, 0, H, TS);
+    const Src s01 = src(tu * F.ntv + tv1, 0, TS, TS, H), s11 = src(tu1 * F.ntv + tv1, TS, TS, H, H);
+    float2* __restrict__ Xh = F.Xh + (size_t)(tu * TS) * F.gy + tv * TS;
+    // one pair of the tile: the sources summed in a fixed order
+    auto pair = [&](int a, int b) {
+        const int off = a * PW + b;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        auto get = [&](const Src& q, float4& x) {
+            const bool in = (unsigned)(a - q.a) < (unsigned)q.na && (unsigned)(b - q.b) < (unsigned)q.nb;
+            x = in ? __ldg(reinterpret_cast<const float4*>(q.p + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            return in;
+        };
+        float4 x00, x10, x01, x11;
+        get(s00, x00);
+        const bool k10 = get(s10, x10), k01 = get(s01, x01), k11 = get(s11, x11);
+        v = x00;
+        auto add = [&](bool k, const float4& x) {
+            if (k) v = make_float4(v.x + x.x, v.y + x.y, v.z + x.z, v.w + x.w);
+        };
+        add(k10, x10);
+        add(k01, x01);
+        add(k11, x11);
+        return v;
     };
-    const Rng r00 = rng(x00, 0, 0), r10 = rng(x10, TS, 0), r01 = rng(x01, 0, TS), r11 = rng(x11, TS, TS);
-    const float2* __restrict__ patch = F.patch;
-    float2* __restrict__ Xh = F.Xh;
-    // every box covers all the cells its patch gives this tile (dense units): no per-cell test
-    auto covers = [](const Rng& r, int na, int nb) { return r.a <= 0 && r.a + r.na >= na && r.b <= 0 && r.b + r.nb >= nb; };
-    const bool dense = (s00 < 0 || covers(r00, TS, TS)) && (s10 < 0 || covers(r10, F.H, TS)) &&
-                       (s01 < 0 || covers(r01, TS, F.H)) && (s11 < 0 || covers(r11, F.H, F.H));
-    // one cell of the tile: the four sources (predicated), summed in a fixed order
-    auto cell = [&](int e, float2& v) {
-        const int a = e / TS, b = e - a * TS;
-        const bool k00 = dense ? s00 >= 0 : in(r00, a, b);
-        const bool k10 = dense ? (a < F.H && s10 >= 0) : in(r10, a, b);
-        const bool k01 = dense ? (b < F.H && s01 >= 0) : in(r01, a, b);
-        const bool k11 = dense ? (a < F.H && b < F.H && s11 >= 0) : in(r11, a, b);
-        const float2 z = make_float2(0.f, 0.f);
-        const float2 p00 = k00 ? __ldg(&patch[s00 * np + a * F.PW + b]) : z;
-        const float2 p10 = k10 ? __ldg(&patch[s10 * np + (a + TS) * F.PW + b]) : z;
-        const float2 p01 = k01 ? __ldg(&patch[s01 * np + a * F.PW + b + TS]) : z;
-        const float2 p11 = k11 ? __ldg(&patch[s11 * np + (a + TS) * F.PW + b + TS]) : z;
-        v = k00 ? p00 : z;
-        if (k10) v = cadd(v, p10);
-        if (k01) v = cadd(v, p01);
-        if (k11) v = cadd(v, p11);
-    };
-    auto dst = [&](int e) {
-        const int a = e / TS, b = e - a * TS;
-        return Xh + (size_t)(tu * TS + a) * F.gy + tv * TS + b;
-    };
-    if constexpr (TS == 32) {
-        // the four cells of a thread: every load issued before the stores (per 4096^2/50M
-        // apply, inverse cols + fold 6.91 -> 6.72 ms against one cell at a time with a
-        // runtime tile side; the 16 cells of a 64-wide tile at once took 80 registers and
-        // slowed the wideband batch, 102.5 -> 114.2 ms, so 64-wide tiles go one at a time)
-        float2 acc[4];
-#pragma unroll
-        for (int it = 0; it < 4; ++it) cell(threadIdx.x + 256 * it, acc[it]);
-#pragma unroll
-        for (int it = 0; it < 4; ++it) *dst(threadIdx.x + 256 * it) = acc[it];
-    } else {
-        for (int e = threadIdx.x; e < TS * TS; e += 256) {
-            float2 v;
-            cell(e, v);
-            *dst(e) = v;
-        }
+#pragma unroll 2
+    for (int e = threadIdx.x; e < TS * ROW; e += 256) {
+        const int a = e / ROW, b = 2 * (e % ROW);
+        *reinterpret_cast<float4*>(Xh + (size_t)a * F.gy + b) = pair(a, b);
     }
 }
 
@@ -908,8 +903,7 @@ __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 
         const RowSel& sel = J.sel;
         const ZArgs z = J.z;
         const float2* __restrict__ in = J.in + (size_t)i * L;
-        float2* __restrict__ orow =
-            reinterpret_cast<float2*>(reinterpret_cast<char*>(J.out) + img) + (size_t)i * N;
+        float2* __restrict__ orow = at_image<TABLE>(J.out, img) + (size_t)i * N;
         const int acc = accumulate || jj > j0;
         float2 v[16];
         // columns u of tile rows the inverse column pass skipped are zero (not stored)
