@@ -121,8 +121,11 @@ PlanStage::~PlanStage() {
     for (Group& g : groups) {
         if (g.fft) wide_fft_destroy(g.fft);
         if (g.gtg) wide_gtg_destroy(g.gtg);
+        if (g.hfft) wide_fft_destroy(g.hfft);
+        if (g.h) wide_h_destroy(g.h);
     }
     cudaFree(scratch);
+    cudaFree(hpatch);
 }
 
 void stage_plan(rimo_plan* p, cudaStream_t s) {
@@ -166,21 +169,29 @@ void stage_plan(rimo_plan* p, cudaStream_t s) {
     p->info.scratch_bytes += st->scratch_bytes;
 }
 
-static bool staged(const rimo_plan* p) { return p->stage && !p->bin_by_bin && !p->h_built; }
+// `holo`: Phi^dagger Phi through H
+static bool staged(const rimo_plan* p, bool holo) {
+    return p->stage && !p->bin_by_bin && (!holo || p->stage->hpatch);
+}
 
-// One group: F Z_p x (mode 0 and 2), the grid step, and the image (mode 1 and 2; `first`: written,
-// else added to).
-static void apply_group(rimo_plan* p, const PlanStage::Group& g, int mode, const float2* x, const float2* y_in,
-                        float2* y_out, float2* out, bool first, int real_only, cudaStream_t s) {
+// One group: F Z_p x (mode 0 and 2), the grid step (`holo`: H), and the image (mode 1 and 2;
+// `first`: written, else added to).
+static void apply_group(rimo_plan* p, const PlanStage::Group& g, int mode, bool holo, const float2* x,
+                        const float2* y_in, float2* y_out, float2* out, bool first, int real_only, cudaStream_t s) {
+    const WideFft* fft = holo ? g.hfft : g.fft;
     if (mode != 1) {
         prof_begin(p, ST_FWD_ROWS, s);
-        wide_fwd_rows(g.fft, x, s);
+        wide_fwd_rows(fft, x, s);
         prof_end(p, 1, s);
         prof_begin(p, ST_FWD_COLS, s);
-        wide_fwd_cols(g.fft, s);
+        wide_fwd_cols(fft, s);
         prof_end(p, 1, s);
     }
-    if (g.gtg) {
+    if (holo) {
+        prof_begin(p, ST_HAPPLY, s);
+        wide_happly(g.h, s);
+        prof_end(p, 1, s);
+    } else if (g.gtg) {
         prof_begin(p, ST_GTG, s);
         const int nl = wide_gtg(g.gtg, mode, y_in, y_out, s);
         prof_end(p, nl, s);
@@ -189,10 +200,10 @@ static void apply_group(rimo_plan* p, const PlanStage::Group& g, int mode, const
     }
     if (mode == 0) return;
     prof_begin(p, ST_INV_COLS, s);
-    wide_inv_cols(g.fft, s);
+    wide_inv_cols(fft, s);
     prof_end(p, 2, s);
     prof_begin(p, ST_INV_ROWS, s);
-    wide_inv_rows(g.fft, out, first ? 0 : 1, real_only, s);
+    wide_inv_rows(fft, out, first ? 0 : 1, real_only, s);
     prof_end(p, 1, s);
 }
 
@@ -205,8 +216,8 @@ static void begin_apply(rimo_plan* p, cudaStream_t s) {
 
 void apply_phi(rimo_plan* p, const float2* x, float2* y, cudaStream_t s) {
     begin_apply(p, s);
-    if (staged(p)) {
-        for (const auto& g : p->stage->groups) apply_group(p, g, 0, x, nullptr, y, nullptr, false, 0, s);
+    if (staged(p, false)) {
+        for (const auto& g : p->stage->groups) apply_group(p, g, 0, false, x, nullptr, y, nullptr, false, 0, s);
         return;
     }
     for (int b = 0; b < p->P; ++b) {
@@ -222,9 +233,9 @@ void apply_phi_adj(rimo_plan* p, const float2* y, float2* x, cudaStream_t s) {
     prof_begin(p, ST_BOUND, s);
     launch_y_bound(p, y, s);
     prof_end(p, p->M > 0 ? 1 : 0, s);
-    if (staged(p)) {
+    if (staged(p, false)) {
         for (const auto& g : p->stage->groups) {
-            apply_group(p, g, 1, nullptr, y, nullptr, x, first, 0, s);
+            apply_group(p, g, 1, false, nullptr, y, nullptr, x, first, 0, s);
             first = false;
         }
         if (first) zero_image(p, (rimo_cfloat*)x, s);
@@ -250,9 +261,9 @@ void apply_phi_adj_phi_bins(rimo_plan* p, const float2* x, float2* out, int real
     prof_begin(p, ST_BOUND, s);
     launch_image_bound(p, x, s);
     prof_end(p, 1, s);
-    if (staged(p) && !mask) {
+    if (!mask && staged(p, p->h_built)) {
         for (const auto& g : p->stage->groups) {
-            apply_group(p, g, 2, x, nullptr, nullptr, out, first, real_only, s);
+            apply_group(p, g, 2, p->h_built, x, nullptr, nullptr, out, first, real_only, s);
             first = false;
         }
         if (first) zero_image(p, (rimo_cfloat*)out, s);

@@ -1243,7 +1243,7 @@ static size_t append(std::vector<char>& blob, const std::vector<T>& v) {
 }
 
 WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<const float2*>& x,
-                         const std::vector<float2*>& out, cudaStream_t s) {
+                         const std::vector<float2*>& out, cudaStream_t s, bool holographic) {
     if (jobs.empty()) fail(RIMO_ERR_INVALID_ARG, "no jobs");
     auto* w = new WideFft();
     try {
@@ -1268,7 +1268,7 @@ WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<con
             frf.push_back(frf.back() + p->ny / rb);
             cf.push_back(cols_job(p, j.bin, j.AB, j.X, fs));
             fcf.push_back(fcf.back() + sel_blocks(p, j.bin, fs, cb));
-            fo.push_back(fold_args(p, j.bin, j.patch, nullptr, j.X));
+            fo.push_back(fold_args(p, j.bin, j.patch, holographic ? p->d_hslot : nullptr, j.X));
             ffo.push_back(ffo.back() + (p->bins[j.bin].n1 - p->bins[j.bin].n0));
             ci.push_back(cols_job(p, j.bin, j.X, j.AB, is));
             fci.push_back(fci.back() + sel_blocks(p, j.bin, is, cb));

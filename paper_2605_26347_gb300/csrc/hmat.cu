@@ -21,13 +21,14 @@
 // owner keeping its entries in shared memory (no atomics); the candidate visibilities
 // (anchor within D before the block) come from an anchor index sorted by (g0, h0) that the
 // host prepares.  Apply: one CTA per needed tile, one warp per owner; the gathered sum
-// of the type-A row and the scattered conjugate terms are accumulated in the two-word
-// fixed-point patch of the gridding step.
+// of the type-A row, its scattered conjugate terms and the type-B block's row and column sums
+// are accumulated in the two-word fixed-point patch of the gridding step.
 #include <algorithm>
 #include <cstring>
 #include <numeric>
 #include <vector>
 
+#include "fixed.cuh"
 #include "internal.h"
 #include "planner.h"
 
@@ -40,9 +41,7 @@ namespace {
 constexpr int HB_OWN = 4;                 // owner block edge of the build
 constexpr int HB_WARPS = HB_OWN * HB_OWN;  // one warp per owner
 constexpr int HB_CHUNK = 16;              // candidate visibilities staged at a time
-constexpr int HA_WARPS = 16;              // apply: consumer warps per CTA
-constexpr float HX_MAGIC = 12582912.0f;   // 1.5 x 2^23 (rint by the shift)
-constexpr int HX_MAGIC_BITS = 0x4B400000;
+constexpr int HA_WARPS = 8;               // apply: warps per CTA, two CTAs per SM
 
 // entry e of an owner row -> (type, a, b), packed type << 16 | a << 8 | b
 std::vector<int32_t> entry_table(int D) {
@@ -303,142 +302,300 @@ struct HApplyArgs {
     const uint16_t* idx;      // compressed: the entry numbers
     const int64_t* roff;      // compressed: [owner + 1] first entry of each owner row (null: dense)
     const uint32_t* tmax;     // [needed tile] max |h|_1 of the tile's rows
-    const int32_t* ent;
     float2* patch;            // [needed tile][PW * PW]
-    int gx, gy, ntv, TS, D, PW, ne, shift;
+    int gx, gy, ntv, TS, PW, pitch, shift;
 };
 
-__device__ __forceinline__ void fx_add(int* hi, int* lo, int ci, float d) {
-    const float tq = __fadd_rn(d, HX_MAGIC);
-    const int q1 = __float_as_int(tq) - HX_MAGIC_BITS;
-    const float rf = __fsub_rn(d, __fsub_rn(tq, HX_MAGIC));
-    const int q2 = __float_as_int(__fmaf_rn(rf, 65536.f, HX_MAGIC)) - HX_MAGIC_BITS;
-    atomicAdd(hi + ci, q1);
-    atomicAdd(lo + ci, q2);
+// sum over the W lanes of a group (W a power of two, lanes of one group consecutive) of W values
+// per lane: lane l of the group gets the sum of value l (W - 1 exchanges instead of W log W)
+template <int W>
+__device__ __forceinline__ float lane_sums(float (&v)[W], int lane) {
+#pragma unroll
+    for (int w = W / 2; w >= 1; w >>= 1) {
+        const bool up = lane & w;
+#pragma unroll
+        for (int j = 0; j < w; ++j) {
+            const float send = up ? v[j] : v[j + w];
+            v[j] = (up ? v[j + w] : v[j]) + __shfl_xor_sync(0xffffffffu, send, w);
+        }
+    }
+    return v[0];
 }
 
-__global__ void __launch_bounds__(HA_WARPS * 32, 1) happly_kernel(HApplyArgs A) {
+// One owner's dense row in registers, spread over a warp as in the grid step's vis_tile: CW
+// lanes hold the columns of a row, 32 / CW rows per step.
+template <int S>
+struct HRow {
+    static constexpr int CW = S <= 8 ? 8 : (S <= 16 ? 16 : 32), RPI = 32 / CW, D = S - 1;
+    static constexpr int NA = (S + RPI - 1) / RPI, NB = (D + RPI - 1) / RPI;
+    f32x2 a[NA], b[NB];  // type A: h[a][b], a, b in [0, D]; type B: a, b in [1, D]
+    template <class Ld>  // ld(e): entry e
+    __device__ __forceinline__ void load(int lane, Ld ld) {
+        const int c = lane % CW, ro = lane / CW;
+#pragma unroll
+        for (int i = 0; i < NA; ++i) a[i] = c < S && i * RPI + ro < S ? ld((i * RPI + ro) * S + c) : 0ull;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) b[i] = c < D && i * RPI + ro < D ? ld(S * S + (i * RPI + ro) * D + c) : 0ull;
+    }
+};
+
+// The products of one owner's row (cell (lu, lv) of the patch) with the input patch Z, added to
+// the accumulator planes.
+//   type A (the owner with the cells c2 below and right of it): the row's sum h z[c2] is the
+//     owner's, conj(h) z[owner] goes to each c2;
+//   type B (the cells c1 right of the owner with the cells c2 below it): with lanes along b and
+//     steps along a the sums over a stay in registers (h z[c2] of c1) and those over b are one
+//     exchange tree for all of them (conj(h) z[c1] of c2), so only the (2 D) sums are added to
+//     the patch, not every product.
+template <int S>
+__device__ __forceinline__ void h_owner(const HRow<S>& h, const float2* Z, int* acc, int PW, int pitch, int plane,
+                                        int lu, int lv, float s1, int lane) {
+    constexpr int CW = HRow<S>::CW, RPI = HRow<S>::RPI, NA = HRow<S>::NA, NB = HRow<S>::NB, D = S - 1;
+    const int c = lane % CW, ro = lane / CW;
+    const float2 zo = Z[lu * PW + lv];
+    {
+        const bool row_ok = (NA - 1) * RPI + ro < S;
+        const f32x2* Zl = reinterpret_cast<const f32x2*>(Z) + (lu + ro) * PW + lv + c;
+        f32x2 p = 0ull;
+        float q1 = 0.f, q2 = 0.f;
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            const f32x2 z = (i + 1) * RPI <= S || row_ok ? Zl[i * RPI * PW] : 0ull;
+            p = fma2(h.a[i], z, p);
+            const float2 hs = upk(h.a[i]), zs = upk(z);
+            q1 = fmaf(hs.x, zs.y, q1);
+            q2 = fmaf(hs.y, zs.x, q2);
+        }
+        const float2 ps = upk(p);
+        const float re = c < S ? ps.x - ps.y : 0.f, im = c < S ? q1 + q2 : 0.f;
+        const bool hi = lane & 16;
+        float v = hi ? im : re;
+        v += __shfl_xor_sync(0xffffffffu, hi ? re : im, 16);
+        v += __shfl_xor_sync(0xffffffffu, v, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        const float o = __shfl_xor_sync(0xffffffffu, v, 16);  // lane 0: the sum is (v, o)
+        const float zr = zo.x * s1, zi = zo.y * s1, nzr = -zr;
+        int* al = acc + (lu + ro) * pitch + lv + c;
+        if (c < S) {
+#pragma unroll
+            for (int i = 0; i < NA; ++i) {
+                if ((i + 1) * RPI <= S || row_ok) {
+                    const float2 hs = upk(h.a[i]);
+                    f32x2 d = pk(fmaf(hs.x, zr, hs.y * zi), fmaf(hs.x, zi, hs.y * nzr));
+                    if (i == 0 && lane == 0) d = pk(v * s1, o * s1);  // the owner's own cell: the row's sum
+                    fx_add2(al + i * RPI * pitch, plane, d);
+                }
+            }
+        }
+    }
+    {
+        const float2 zero = make_float2(0.f, 0.f);
+        const float2 z1 = c < D ? Z[lu * PW + lv + c + 1] : zero;  // z[c1]
+        float rx = 0.f, ry = 0.f;
+        constexpr int NC = (2 * NB + CW - 1) / CW;
+        float w[NC][CW];
+#pragma unroll
+        for (int i = 0; i < NC * CW; ++i) w[i / CW][i % CW] = 0.f;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int a = i * RPI + ro;
+            const float2 z2 = (i + 1) * RPI <= D || a < D ? Z[(lu + a + 1) * PW + lv] : zero;  // z[c2]
+            const float2 hs = upk(h.b[i]);
+            rx = fmaf(hs.x, z2.x, fmaf(-hs.y, z2.y, rx));
+            ry = fmaf(hs.x, z2.y, fmaf(hs.y, z2.x, ry));
+            w[2 * i / CW][2 * i % CW] = fmaf(hs.x, z1.x, hs.y * z1.y);
+            w[(2 * i + 1) / CW][(2 * i + 1) % CW] = fmaf(hs.x, z1.y, -hs.y * z1.x);
+        }
+#pragma unroll
+        for (int o = CW; o < 32; o <<= 1) {
+            rx += __shfl_xor_sync(0xffffffffu, rx, o);
+            ry += __shfl_xor_sync(0xffffffffu, ry, o);
+        }
+        if (ro == 0 && c < D) fx_add2(acc + lu * pitch + lv + c + 1, plane, pk(rx * s1, ry * s1));
+#pragma unroll
+        for (int q = 0; q < NC; ++q) {
+            const float t = lane_sums<CW>(w[q], lane) * s1;
+            const int e = q * CW + c, a = (e >> 1) * RPI + ro;
+            if (e < 2 * NB && a < D) {
+                const float tq = __fadd_rn(t, FX_MAGIC);
+                const float rf = __fsub_rn(t, __fsub_rn(tq, FX_MAGIC));
+                int* p = acc + (lu + a + 1) * pitch + lv + (e & 1) * plane;
+                atomicAdd(p, __float_as_int(tq) - FX_MAGIC_BITS);
+                atomicAdd(p + 2 * plane, __float_as_int(__fmaf_rn(rf, 65536.f, FX_MAGIC)) - FX_MAGIC_BITS);
+            }
+        }
+    }
+}
+
+// One block per needed tile, one warp per owner (covered cells round robin).  A warp loads the
+// row of its next owner (dense rows: into registers, coalesced) while it multiplies the
+// current one, which keeps about 54 KB per SM in flight; a compressed row is first spread into
+// a dense one in the warp's shared buffer.
+// Bound by HBM at best (8 bytes per entry); before, with one entry per lane and every product
+// added to the patch (8 shared reductions per type-B entry, no load ahead of the reductions),
+// 256^2/1M/4 bins (1M rows, 3.4 GB) took 3.00 ms; now 0.75 ms, 4.7 TB/s, in one launch over the
+// bins (the rows' 120-byte segments fetch 1.6 times their bytes from L2).
+template <int S>
+__global__ void __launch_bounds__(HA_WARPS * 32, 2)
+    happly_kernel(const __grid_constant__ HApplyArgs one, const HApplyArgs* __restrict__ jobs,
+                  const int* __restrict__ first, int njobs) {
+    constexpr int D = S - 1, NE = S * S + D * D;
     extern __shared__ __align__(16) unsigned char hsm[];
-    const int PW = A.PW, np = PW * PW, ne = A.ne;
-    float2* Z = reinterpret_cast<float2*>(hsm);          // input patch
-    int* Ohi = reinterpret_cast<int*>(Z + np);            // [cell][re, im]
-    int* Olo = Ohi + 2 * np;
-    int* sent = Olo + 2 * np;
     __shared__ uint32_t tbits[128];
-    __shared__ float s_scale[2];
-    __shared__ float s_zmax[HA_WARPS];
-    const int t_idx = blockIdx.x;
+    __shared__ int wsum[129];          // covered cells before each bitmap word
+    __shared__ uint16_t cells[4096];   // the covered cells in row-major order
+    __shared__ uint32_t s_zmax;
+    int t_idx = (int)blockIdx.x;
+    const HApplyArgs* pa = &one;
+    if (jobs) {
+        const int j = job_of(first, njobs, t_idx);
+        t_idx -= __ldg(first + j);
+        pa = jobs + j;
+    }
+    const HApplyArgs& A = *pa;
+    const int PW = A.PW, np = PW * PW, TS = A.TS, pitch = A.pitch, plane = PW * pitch;
+    float2* Z = reinterpret_cast<float2*>(hsm);               // input patch
+    int* acc = reinterpret_cast<int*>(Z + np);                // planes [hi re, hi im, lo re, lo im]
+    f32x2* rows = reinterpret_cast<f32x2*>(acc + 4 * plane);  // compressed rows spread out, one per warp
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tile = A.need[t_idx];
     const int tu = tile / A.ntv, tv = tile - tu * A.ntv;
-    const int u0 = tu * A.TS, v0 = tv * A.TS;
-    const int words = A.TS * A.TS / 32;
-    const int ntu = A.gx / A.TS;
-    for (int e = threadIdx.x; e < words; e += blockDim.x) tbits[e] = A.bits[(size_t)t_idx * words + e];
-    for (int e = threadIdx.x; e < ne; e += blockDim.x) sent[e] = A.ent[e];
+    const int u0 = tu * TS, v0 = tv * TS;
+    const int words = TS * TS / 32;
+    for (int e = tid; e < words; e += blockDim.x) tbits[e] = A.bits[(size_t)t_idx * words + e];
+    for (int e = tid; e < 4 * plane; e += blockDim.x) acc[e] = 0;
+    if (tid == 0) s_zmax = 0u;
+    __syncthreads();
+    if (warp == 0) {  // running count over the bitmap words
+        int base = 0;
+        for (int q = 0; q < words; q += 32) {
+            int n = __popc(tbits[q + lane]);
+            const int own = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int m = __shfl_up_sync(0xffffffffu, n, o);
+                if (lane >= o) n += m;
+            }
+            wsum[q + lane] = base + n - own;
+            base += __shfl_sync(0xffffffffu, n, 31);
+        }
+    }
     float zm = 0.f;
-    for (int e = threadIdx.x; e < np; e += blockDim.x) {
+    for (int e = tid; e < np; e += blockDim.x) {
         const int a = e / PW, b = e - a * PW;
         const int gu = wrap(u0 + a, A.gx), gv = wrap(v0 + b, A.gy);
         const int tt = (gu >> A.shift) * A.ntv + (gv >> A.shift);
         const float2 z = A.need_mask[tt] ? A.X[(size_t)gu * A.gy + gv] : make_float2(0.f, 0.f);
         Z[e] = z;
         zm = fmaxf(zm, fabsf(z.x) + fabsf(z.y));
-        Ohi[2 * e] = Ohi[2 * e + 1] = 0;
-        Olo[2 * e] = Olo[2 * e + 1] = 0;
     }
-    (void)ntu;
-    for (int o = 16; o > 0; o >>= 1) zm = fmaxf(zm, __shfl_xor_sync(0xffffffffu, zm, o));
-    if ((threadIdx.x & 31) == 0) s_zmax[threadIdx.x >> 5] = zm;
+    zm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(zm)));
+    if (lane == 0) atomicMax(&s_zmax, __float_as_uint(zm));
     __syncthreads();
-    if (threadIdx.x == 0) {
-        // bound on one accumulated term of this tile: the gathered type-A sum, (D+1)^2
-        // entries of |h|_1 <= the tile's max times |z|_1 <= the patch's max (margin 2);
-        // at most 2 ne terms per cell.  Per-tile bounds keep the fixed-point resolution
-        // relative to the tile's own values where H spans orders of magnitude.
-        float zmax = 0.f;
-        for (int w = 0; w < HA_WARPS; ++w) zmax = fmaxf(zmax, s_zmax[w]);
-        const float hmax = __uint_as_float(__ldg(A.tmax + t_idx));
-        const float mt = 2.f * (float)((A.D + 1) * (A.D + 1)) * hmax * zmax;
-        float s1 = 1.f, inv = 1.f;
-        if (mt > 0.f) {
-            const float lim = fminf(2097152.f, 1073741824.f / (float)(2 * ne));
-            int ex = (int)((__float_as_uint(lim / mt) >> 23) & 255u) - 127;
-            ex = ex < -120 ? -120 : (ex > 120 ? 120 : ex);
-            s1 = __uint_as_float((uint32_t)(ex + 127) << 23);
-            inv = __uint_as_float((uint32_t)(127 - ex) << 23);
-        }
-        s_scale[0] = s1;
-        s_scale[1] = inv;
+    for (int e = tid; e < TS * TS; e += blockDim.x) {
+        const uint32_t w = tbits[e >> 5], m = 1u << (e & 31);
+        if (w & m) cells[wsum[e >> 5] + __popc(w & (m - 1u))] = (uint16_t)e;
     }
     __syncthreads();
-    const float s1 = s_scale[0];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // bound on one accumulated term of this tile: the gathered type-A sum, (D+1)^2
+    // entries of |h|_1 <= the tile's max times |z|_1 <= the patch's max (margin 2);
+    // at most 2 ne terms per cell.  Per-tile bounds keep the fixed-point resolution
+    // relative to the tile's own values where H spans orders of magnitude.
+    float s1 = 1.f, inv = 1.f;
+    const float mt = 2.f * (float)(S * S) * __uint_as_float(__ldg(A.tmax + t_idx)) * __uint_as_float(s_zmax);
+    if (mt > 0.f) {
+        const float lim = fminf(2097152.f, 1073741824.f / (float)(2 * NE));
+        int ex = (int)((__float_as_uint(lim / mt) >> 23) & 255u) - 127;
+        ex = ex < -120 ? -120 : (ex > 120 ? 120 : ex);
+        s1 = __uint_as_float((uint32_t)(ex + 127) << 23);
+        inv = __uint_as_float((uint32_t)(127 - ex) << 23);
+    }
     const int64_t base = A.hoff[t_idx];
     const int nown = (int)(A.hoff[t_idx + 1] - base);
-    // owners of this warp: covered cells w, w + HA_WARPS, ... in row-major rank order
-    int cell = -1, rank = -1;
-    for (int k = warp; k < nown; k += HA_WARPS) {
-        // advance (cell, rank) to the k-th covered cell
-        while (rank < k) {
-            ++cell;
-            if ((tbits[cell >> 5] >> (cell & 31)) & 1u) ++rank;
+    auto multiply = [&](const HRow<S>& h, int k) {
+        const int cell = cells[k], lu = cell >> A.shift, lv = cell & (TS - 1);
+        h_owner<S>(h, Z, acc, PW, pitch, plane, lu, lv, s1, lane);
+    };
+    if (A.roff == nullptr) {
+        const f32x2* val = reinterpret_cast<const f32x2*>(A.val) + base * NE;
+        auto fetch = [&](HRow<S>& h, int k) {
+            const f32x2* row = val + (int64_t)k * NE;
+            h.load(lane, [&](int e) { return (f32x2)__ldg(row + e); });
+        };
+        HRow<S> h0, h1;
+        int k = warp;
+        if (k < nown) fetch(h0, k);
+        for (; k < nown; k += 2 * HA_WARPS) {
+            if (k + HA_WARPS < nown) fetch(h1, k + HA_WARPS);
+            multiply(h0, k);
+            if (k + HA_WARPS >= nown) break;
+            if (k + 2 * HA_WARPS < nown) fetch(h0, k + 2 * HA_WARPS);
+            multiply(h1, k + HA_WARPS);
         }
-        const int lu = cell / A.TS, lv = cell - lu * A.TS;
-        const bool dense = A.roff == nullptr;
-        const int64_t q0 = dense ? (base + k) * ne : __ldg(&A.roff[base + k]);
-        const int64_t q1 = dense ? q0 + ne : __ldg(&A.roff[base + k + 1]);
-        const float2 zo = Z[lu * PW + lv];
-        float gx = 0.f, gy = 0.f;
-        for (int64_t q = q0 + lane; q < q1; q += 32) {
-            const float2 h = __ldg(&A.val[q]);
-            const int e = dense ? (int)(q - q0) : __ldg(&A.idx[q]);
-            const int en = sent[e];
-            const int a = (en >> 8) & 255, b = en & 255;
-            if ((en >> 16) == 0) {
-                const int c2 = (lu + a) * PW + lv + b;
-                const float2 z2 = Z[c2];
-                gx = fmaf(h.x, z2.x, fmaf(-h.y, z2.y, gx));  // h z2
-                gy = fmaf(h.x, z2.y, fmaf(h.y, z2.x, gy));
-                if (a | b) {  // conj(h) z_owner into c2
-                    fx_add(Ohi, Olo, 2 * c2, s1 * fmaf(h.x, zo.x, h.y * zo.y));
-                    fx_add(Ohi, Olo, 2 * c2 + 1, s1 * fmaf(h.x, zo.y, -h.y * zo.x));
+    } else {
+        f32x2* row = rows + warp * NE;
+        const f32x2* val = reinterpret_cast<const f32x2*>(A.val);
+        for (int k = warp; k < nown; k += HA_WARPS) {
+            const int64_t q0 = __ldg(&A.roff[base + k]), q1 = __ldg(&A.roff[base + k + 1]);
+            for (int e = lane; e < NE; e += 32) row[e] = 0ull;
+            __syncwarp();
+            for (int64_t q = q0 + lane; q < q1; q += 32 * 7) {
+                f32x2 h[7];
+                int e[7];
+#pragma unroll
+                for (int i = 0; i < 7; ++i) {
+                    const bool on = q + 32 * i < q1;
+                    h[i] = on ? (f32x2)__ldg(val + q + 32 * i) : 0ull;
+                    e[i] = on ? (int)__ldg(A.idx + q + 32 * i) : -1;
                 }
-            } else {
-                const int c1 = lu * PW + lv + b, c2 = (lu + a) * PW + lv;
-                const float2 z1 = Z[c1], z2 = Z[c2];
-                fx_add(Ohi, Olo, 2 * c1, s1 * fmaf(h.x, z2.x, -h.y * z2.y));      // h z2 into c1
-                fx_add(Ohi, Olo, 2 * c1 + 1, s1 * fmaf(h.x, z2.y, h.y * z2.x));
-                fx_add(Ohi, Olo, 2 * c2, s1 * fmaf(h.x, z1.x, h.y * z1.y));       // conj(h) z1 into c2
-                fx_add(Ohi, Olo, 2 * c2 + 1, s1 * fmaf(h.x, z1.y, -h.y * z1.x));
+#pragma unroll
+                for (int i = 0; i < 7; ++i)
+                    if (e[i] >= 0) row[e[i]] = h[i];
             }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            gx += __shfl_xor_sync(0xffffffffu, gx, o);
-            gy += __shfl_xor_sync(0xffffffffu, gy, o);
-        }
-        if (lane == 0) {
-            const int co = lu * PW + lv;
-            fx_add(Ohi, Olo, 2 * co, s1 * gx);
-            fx_add(Ohi, Olo, 2 * co + 1, s1 * gy);
+            __syncwarp();
+            HRow<S> h;
+            h.load(lane, [&](int e) { return row[e]; });
+            multiply(h, k);
+            __syncwarp();  // every lane has read the row
         }
     }
     __syncthreads();
-    const float inv = s_scale[1], inv_lo = inv * (1.f / 65536.f);
+    const float inv_lo = inv * (1.f / 65536.f);
     float2* dst = A.patch + (size_t)t_idx * np;
-    for (int e = threadIdx.x; e < np; e += blockDim.x)
-        dst[e] = make_float2(fmaf((float)Olo[2 * e], inv_lo, (float)Ohi[2 * e] * inv),
-                             fmaf((float)Olo[2 * e + 1], inv_lo, (float)Ohi[2 * e + 1] * inv));
+    for (int e = tid; e < np; e += blockDim.x) {
+        const int a = e / PW, q = a * pitch + (e - a * PW);
+        dst[e] = make_float2(fmaf((float)acc[q + 2 * plane], inv_lo, (float)acc[q] * inv),
+                             fmaf((float)acc[q + 3 * plane], inv_lo, (float)acc[q + plane] * inv));
+    }
+}
+
+static void (*happly_for(int S))(HApplyArgs, const HApplyArgs*, const int*, int) {
+    switch (S) {
+        case 3: return happly_kernel<3>;
+        case 5: return happly_kernel<5>;
+        case 7: return happly_kernel<7>;
+        case 9: return happly_kernel<9>;
+        case 11: return happly_kernel<11>;
+        case 13: return happly_kernel<13>;
+        case 15: return happly_kernel<15>;
+        case 17: return happly_kernel<17>;
+        default: return happly_kernel<19>;
+    }
+}
+
+// (the row buffers only where some bin's rows are compressed)
+size_t happly_smem(int PW, int S, bool compressed) {
+    const size_t ne = (size_t)S * S + (size_t)(S - 1) * (S - 1);
+    return (size_t)PW * PW * sizeof(float2) + (size_t)4 * PW * pitch_of(PW, S) * sizeof(int) +
+           (compressed ? HA_WARPS * ne * sizeof(float2) : 0);
 }
 
 size_t hbuild_smem(int ne, int S_max, int D) {
     return (size_t)HB_WARPS * ne * sizeof(float2) + (size_t)HB_CHUNK * S_max * S_max * sizeof(float2) +
            HB_CHUNK * sizeof(int4) + (size_t)(ne + 2) * sizeof(int) +
            (size_t)2 * (HB_OWN + D) * (2 * sizeof(int64_t) + sizeof(int)) + 64;
-}
-
-size_t happly_smem(int PW, int ne) {
-    const size_t np = (size_t)PW * PW;
-    return np * sizeof(float2) + 4 * np * sizeof(int) + (size_t)ne * sizeof(int);
 }
 
 struct DevBuf {
@@ -494,14 +651,12 @@ __global__ void __launch_bounds__(256) hcompact_kernel(const float2* __restrict_
 
 }  // namespace
 
-void launch_happly(const rimo_plan* p, int bin, cudaStream_t s) {
+static HApplyArgs happly_args(const rimo_plan* p, int bin, const float2* X, float2* patch) {
     const auto& br = p->bins[bin];
-    const int nneed = br.n1 - br.n0;
-    if (nneed <= 0) return;
-    const int ntu = p->gx / p->TS, ntv = p->gy / p->TS;
-    const size_t ntile = (size_t)ntu * ntv;
+    const size_t ntile = (size_t)(p->gx / p->TS) * (p->gy / p->TS);
     HApplyArgs A;
-    A.X = p->d_X;
+    std::memset(&A, 0, sizeof(A));
+    A.X = X;
     A.need_mask = p->d_need + (size_t)bin * ntile;
     A.need = p->d_need_list + br.n0;
     A.bits = p->d_hbits[bin];
@@ -510,19 +665,95 @@ void launch_happly(const rimo_plan* p, int bin, cudaStream_t s) {
     A.idx = p->h_dense[bin] ? nullptr : p->d_hidx[bin];
     A.roff = p->h_dense[bin] ? nullptr : p->d_hroff[bin];
     A.tmax = p->d_htmax[bin];
-    A.ent = p->d_hent;
-    A.patch = p->d_hpatch;
+    A.patch = patch;
     A.gx = p->gx;
     A.gy = p->gy;
-    A.ntv = ntv;
+    A.ntv = p->gy / p->TS;
     A.TS = p->TS;
-    A.D = p->H;
     A.PW = p->PW;
-    A.ne = p->h_ne;
+    A.pitch = pitch_of(p->PW, p->max_S);
     A.shift = p->TS == 64 ? 6 : 5;
-    const size_t sm = happly_smem(p->PW, p->h_ne);
-    RIMO_CUDA(cudaFuncSetAttribute(happly_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    happly_kernel<<<nneed, HA_WARPS * 32, sm, s>>>(A);
+    return A;
+}
+
+static void happly_launch(const rimo_plan* p, const HApplyArgs& one, const HApplyArgs* jobs, const int* first, int njobs,
+                          int blocks, bool compressed, cudaStream_t s) {
+    if (blocks <= 0) return;
+    auto kern = happly_for(p->max_S);
+    const size_t sm = happly_smem(p->PW, p->max_S, compressed);
+    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    kern<<<blocks, HA_WARPS * 32, sm, s>>>(one, jobs, first, njobs);
+}
+
+void launch_happly(const rimo_plan* p, int bin, cudaStream_t s) {
+    happly_launch(p, happly_args(p, bin, p->d_X, p->d_hpatch), nullptr, nullptr, 0, p->bins[bin].n1 - p->bins[bin].n0,
+                  !p->h_dense[bin], s);
+}
+
+// The holographic applies of a group of bins as one launch over a table of jobs.
+struct WideH {
+    const rimo_plan* p = nullptr;
+    HApplyArgs* jobs = nullptr;
+    int* first = nullptr;
+    int njobs = 0, blocks = 0;
+    bool compressed = false;
+    ~WideH() {
+        cudaFree(jobs);
+        cudaFree(first);
+    }
+};
+
+static WideH* wide_h_create(const rimo_plan* p, const std::vector<WideJob>& jobs, cudaStream_t s) {
+    auto* w = new WideH();
+    try {
+        w->p = p;
+        std::vector<HApplyArgs> a;
+        std::vector<int> f{0};
+        for (const WideJob& j : jobs) {
+            a.push_back(happly_args(p, j.bin, j.X, j.patch));
+            f.push_back(f.back() + (p->bins[j.bin].n1 - p->bins[j.bin].n0));
+            w->compressed = w->compressed || !p->h_dense[j.bin];
+        }
+        w->njobs = (int)a.size();
+        w->blocks = f.back();
+        RIMO_CUDA(cudaMalloc(&w->jobs, a.size() * sizeof(HApplyArgs)));
+        RIMO_CUDA(cudaMalloc(&w->first, f.size() * sizeof(int)));
+        RIMO_CUDA(cudaMemcpyAsync(w->jobs, a.data(), a.size() * sizeof(HApplyArgs), cudaMemcpyHostToDevice, s));
+        RIMO_CUDA(cudaMemcpyAsync(w->first, f.data(), f.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+        RIMO_CUDA(cudaStreamSynchronize(s));
+    } catch (...) {
+        delete w;
+        throw;
+    }
+    return w;
+}
+void wide_h_destroy(WideH* w) { delete w; }
+void wide_happly(const WideH* w, cudaStream_t s) {
+    HApplyArgs none;
+    std::memset(&none, 0, sizeof(none));
+    happly_launch(w->p, none, w->jobs, w->first, w->njobs, w->blocks, w->compressed, s);
+}
+
+// Once H is built, the plan's groups of bins apply it too (patches of their own; without room
+// for them, one bin at a time).
+static void stage_holographic(rimo_plan* p, int max_need, cudaStream_t s) {
+    if (!p->stage) return;
+    size_t most = 0;
+    for (const auto& g : p->stage->groups) most = std::max(most, g.jobs.size());
+    const size_t each = (size_t)max_need * p->PW * p->PW;
+    if (most * each * sizeof(float2) > ((size_t)512 << 20)) return;
+    if (cudaMalloc(&p->stage->hpatch, most * each * sizeof(float2)) != cudaSuccess) {
+        cudaGetLastError();
+        p->stage->hpatch = nullptr;
+        return;
+    }
+    for (auto& g : p->stage->groups) {
+        std::vector<WideJob> jobs = g.jobs;
+        for (size_t k = 0; k < jobs.size(); ++k) jobs[k].patch = static_cast<float2*>(p->stage->hpatch) + k * each;
+        g.hfft = wide_fft_create(jobs, {nullptr}, {nullptr}, s, true);
+        g.h = wide_h_create(p, jobs, s);
+    }
+    p->info.scratch_bytes += (int64_t)(most * each * sizeof(float2));
 }
 
 // Builds H for every bin; see the file comment.  Synchronises s.
@@ -748,6 +979,7 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
     p->info.h_nnz = 2 * (nnz - (int64_t)diag) + (int64_t)diag;
     p->h_ne = ne;
     p->info.h_bytes = h_bytes + (int64_t)patch_bytes;
+    stage_holographic(p, max_need, s);
     p->h_built = true;
 }
 

@@ -299,9 +299,13 @@ __device__ __forceinline__ int job_of(const int* first, int njobs, int b) {
 }
 struct WideFft;   // device job tables of the transform passes (fft.cu)
 struct WideGtg;   // device unit list of the grid step (grid.cu)
+struct WideH;     // device job table of the holographic apply (hmat.cu)
+void wide_h_destroy(WideH* w);
+void wide_happly(const WideH* w, cudaStream_t s);
 // x, out: the images of each group (null: every group's images come with the launches)
+// holographic: the jobs' patches are those of the holographic apply
 WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<const float2*>& x,
-                         const std::vector<float2*>& out, cudaStream_t s);
+                         const std::vector<float2*>& out, cudaStream_t s, bool holographic = false);
 void wide_fft_destroy(WideFft* w);
 // F Z_p of every job: rows and cols pass (x: see wide_fft_create, null with tables that hold it)
 void wide_fwd_rows(const WideFft* w, const float2* x, cudaStream_t s);
@@ -324,9 +328,12 @@ struct PlanStage {
         std::vector<WideJob> jobs;
         WideFft* fft = nullptr;
         WideGtg* gtg = nullptr;   // stored G; else the bins' grid steps follow their tile generation
+        WideFft* hfft = nullptr;  // once H is built: the passes with its patches ...
+        WideH* h = nullptr;       // ... and its apply
     };
     std::vector<Group> groups;
     void* scratch = nullptr;
+    void* hpatch = nullptr;       // the groups' holographic patches
     int64_t scratch_bytes = 0;
     ~PlanStage();
 };

@@ -68,3 +68,35 @@ def test_bins_in_groups_equal_one_bin_at_a_time(nx, ny, m, bins, kw):
     assert rel(to_host(c), to_host(a)) < 2e-6  # each within 1e-6 of 64 bits
     plan.status()
     plan.close()
+
+
+@pytest.mark.parametrize("m, kb, cap, tile, dense", [
+    (300, 7, 9, 32, False), (300, 7, 9, 64, False), (60000, 7, 9, 32, True), (60000, 7, 9, 64, True),
+    (300, 3, 1, 32, False), (60000, 3, 1, 32, True), (60000, 5, 1, 32, True), (60000, 5, 3, 32, True),
+    (60000, 9, 1, 32, True), (60000, 11, 1, 32, True), (60000, 11, 3, 32, True), (60000, 11, 7, 32, True),
+    (60000, 11, 9, 32, True), (400, 11, 9, 64, False), (1, 7, 9, 32, False),
+])
+def test_holographic_apply_of_every_tile_side(m, kb, cap, tile, dense):
+    """H against G^dagger G of the same plan, rows kept dense (a visibility or more per cell) and
+    compressed, for every tile side; with bins in groups and one at a time."""
+    import torch
+
+    import paper_2605_26347_gb300 as pkg
+    n, fov = 64, math.radians(2.0)
+    rng = np.random.default_rng(m + kb + cap)
+    uvw = (rng.random((m, 3)) - 0.5) * np.array([2 * n / (2 * fov), 2 * n / (2 * fov), 3000.0])
+    bins = 1 if m < 2 else 2
+    plan = pkg.Plan(uvw, pkg.default_params(n, n, fov, fov, n_wbins=bins, kb_support=kb, max_wsupport=cap,
+                                            tile_size=tile))
+    x = to_dev((rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))))
+    g = to_host(plan.phi_adj_phi(x))
+    plan.build_holographic()
+    i = plan.info()
+    if dense:
+        assert i["h_nonzero"] > 0.8 * i["h_entries"]
+    a = plan.phi_adj_phi(x)
+    assert rel(to_host(a), g) < TOL  # both within a few 1e-7 of the operator
+    b = plan.phi_adj_phi_bins(x, np.ones(bins, np.uint8))
+    assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
+    plan.status()
+    plan.close()
