@@ -14,6 +14,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <random>
@@ -83,12 +84,16 @@ __device__ __forceinline__ bool mbar_wait_(uint64_t* bar, uint32_t parity) {
 
 // --------------------------------------------------------------------------------------
 // C[m][n] (+)= sum_k A[m][k] B[n][k]: A (M x K) and B (N x K) bf16 row-major with K
-// contiguous, C fp32.  Block: 128 threads, tile 128 (m) x up to 256 (n), K staged in
-// chunks of 64 into shared memory in the canonical K-major layout; one thread issues
-// the tcgen05.mma (K = 16 each), the accumulator lives in tensor memory.
-constexpr int GEMM_NT = 256;
+// contiguous, C fp32.  Block: 128 threads, tile 128 (m) x nt (n), K staged in chunks of 64
+// into shared memory in the canonical K-major layout by 16-byte asynchronous copies, two
+// chunks deep; one thread issues the tcgen05.mma (K = 16 each), the accumulator lives in
+// tensor memory.  These products are a few hundred MFLOP: they are bound by the latency of a
+// block's chunks (loads, barrier, MMA, wait), so the copies of a chunk are all in flight at
+// once and the tiles are small enough for 64 blocks or more (B = 4096, serialised: dY W3 67 -> 13 us,
+// dY^T H2 91 -> 10 us, dZ2^T H1 93 -> 7 us, H1 W2^T 22 -> 7 us; loss and gradients with their copy to
+// the host 460 -> 155 us).
 constexpr int GEMM_KC = 64;
-constexpr size_t GEMM_SMEM = 100 * 1024;  // also caps residency at two blocks per SM
+constexpr int GEMM_MAX_NT = 128;
 
 struct GemmArgs {
     const bf16* A;
@@ -96,78 +101,97 @@ struct GemmArgs {
     float* C;
     int lda, ldb, ldc;
     int M, N, K;
+    int nt;      // columns of a tile: 64 or 128 (tensor-memory columns)
+    int m_store; // rows of C stored
     int kspan;   // K range of one split (grid.z)
     int atomic;  // add into C (split-K) instead of storing
     int* status;
 };
 
+__device__ __forceinline__ void cp_async16_(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
 __global__ void __launch_bounds__(128) gemm_tc_kernel(GemmArgs g) {
     extern __shared__ __align__(1024) unsigned char sm[];
-    unsigned char* sA = sm;                          // 128 x 64 bf16 = 16 KB
-    unsigned char* sB = sm + 16384;                  // 256 x 64 bf16 = 32 KB
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bar[2];
     __shared__ uint32_t tslot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int n0 = blockIdx.x * GEMM_NT, m0 = blockIdx.y * 128;
-    const int nt = min(GEMM_NT, g.N - n0);
+    const int n0 = blockIdx.x * g.nt, m0 = blockIdx.y * 128;
+    const int nt = min(g.nt, g.N - n0);
     const int k_begin = blockIdx.z * g.kspan, k_end = min(g.K, k_begin + g.kspan);
-    if (warp == 0) tc::tmem_alloc(&tslot, GEMM_NT);
+    const uint32_t sA = tc::smem_addr(sm), stage = 128 * GEMM_KC * 2 + g.nt * GEMM_KC * 2;
+    if (warp == 0) tc::tmem_alloc(&tslot, g.nt);
     if (tid == 0) {
-        mbar_init_(&bar, 1);
+        mbar_init_(&bar[0], 1);
+        mbar_init_(&bar[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    const int nch = (k_end - k_begin + GEMM_KC - 1) / GEMM_KC;
+    // starts the copies of chunk c into its stage (c & 1): 128 rows of A, nt rows of B
+    auto load = [&](int c) {
+        const int k0 = k_begin + c * GEMM_KC, nv = min(GEMM_KC, k_end - k0) / 8;  // 16-byte vectors per row
+        const uint32_t a = sA + (c & 1) * stage, b = a + 128 * GEMM_KC * 2;
+        const int r0 = tid >> 3, v = tid & 7;
+        if (v < nv) {
+#pragma unroll
+            for (int r = r0; r < 128; r += 16)
+                cp_async16_(a + tc::kmajor_offset(r, v * 8, 128), g.A + (size_t)(m0 + r) * g.lda + k0 + v * 8);
+            for (int r = r0; r < nt; r += 16)
+                cp_async16_(b + tc::kmajor_offset(r, v * 8, nt), g.B + (size_t)(n0 + r) * g.ldb + k0 + v * 8);
+        }
+    };
+    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+    if (nch > 0) load(0);
+    commit();
+    if (nch > 1) load(1);
+    commit();
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = tslot;
     const uint32_t idesc = tc::idesc_bf16_f32(128, nt);
-    uint32_t phase = 0;
     bool ok = true;
-    for (int k0 = k_begin; k0 < k_end; k0 += GEMM_KC) {
-        const int kc = min(GEMM_KC, k_end - k0);   // multiple of 16
-        const int nv = kc / 8;                      // 16-byte vectors per row
-        for (int e = tid; e < 128 * nv; e += 128) {
-            const int r = e / nv, v = e - r * nv;
-            const uint4 val = *reinterpret_cast<const uint4*>(g.A + (size_t)(m0 + r) * g.lda + k0 + v * 8);
-            *reinterpret_cast<uint4*>(sA + tc::kmajor_offset(r, v * 8, 128)) = val;
-        }
-        for (int e = tid; e < nt * nv; e += 128) {
-            const int r = e / nv, v = e - r * nv;
-            const uint4 val = *reinterpret_cast<const uint4*>(g.B + (size_t)(n0 + r) * g.ldb + k0 + v * 8);
-            *reinterpret_cast<uint4*>(sB + tc::kmajor_offset(r, v * 8, nt)) = val;
-        }
+    for (int c = 0; c < nch; ++c) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");  // chunk c (the later group may be under way)
         tc::fence_proxy_async();
         tc::fence_before_sync();
         __syncthreads();
         tc::fence_after_sync();
         if (tid == 0) {
-            for (int s = 0; s < kc / 16; ++s) {
-                const uint64_t ad = tc::smem_desc(tc::smem_addr(sA) + s * 128 * 32, 128, 256);
-                const uint64_t bd = tc::smem_desc(tc::smem_addr(sB) + s * nt * 32, 128, 256);
-                tc::mma_bf16(tmem, ad, bd, idesc, (k0 > k_begin || s > 0) ? 1u : 0u);
-            }
-            tc::mma_commit(&bar);
+            const uint32_t a = sA + (c & 1) * stage, b = a + 128 * GEMM_KC * 2;
+            const int ns = min(GEMM_KC, k_end - k_begin - c * GEMM_KC) / 16;
+            for (int s = 0; s < ns; ++s)
+                tc::mma_bf16(tmem, tc::smem_desc(a + s * 128 * 32, 128, 256), tc::smem_desc(b + s * nt * 32, 128, 256),
+                             idesc, (c > 0 || s > 0) ? 1u : 0u);
+            tc::mma_commit(&bar[c & 1]);
         }
-        ok = mbar_wait_(&bar, phase);
-        phase ^= 1;
-        if (__syncthreads_or(!ok)) break;
+        if (c + 2 < nch || c + 1 == nch) {  // the stage is read: refill it, or the product is complete
+            ok = mbar_wait_(&bar[c & 1], (c >> 1) & 1);
+            if (__syncthreads_or(!ok)) {
+                ok = false;
+                break;
+            }
+            if (c + 2 < nch) load(c + 2);
+        }
+        commit();
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     if (!ok) {
         if (tid == 0) atomicExch(g.status, 2);
-    } else if (k_end > k_begin) {
+    } else if (nch > 0) {
         tc::fence_after_sync();
         const int row = m0 + 32 * warp + lane;
         for (int c = 0; c < nt; c += 16) {
             float v[16];
             tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + c, v);
-            float* dst = g.C + (size_t)row * g.ldc + n0 + c;
-            if (g.atomic) {
+            if (row >= g.m_store) continue;
+            float4* dst = reinterpret_cast<float4*>(g.C + (size_t)row * g.ldc + n0 + c);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) atomicAdd(dst + i, v[i]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 16; i += 4)
-                    *reinterpret_cast<float4*>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+            for (int i = 0; i < 4; ++i) {
+                const float4 x = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                if (g.atomic) atomicAdd(dst + i, x);
+                else dst[i] = x;
             }
         }
     }
@@ -175,17 +199,21 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(GemmArgs g) {
     __syncthreads();
     tc::fence_after_sync();
     if (warp == 0) {
-        tc::tmem_dealloc(tmem, GEMM_NT);
+        tc::tmem_dealloc(tmem, g.nt);
         tc::tmem_relinquish();
     }
 }
 
-static void gemm(const bf16* A, int lda, const bf16* B, int ldb, float* C, int ldc, int M, int N, int K,
-                 int splits, bool atomic, int* status, cudaStream_t s) {
-    static bool attr = false;
-    if (!attr) {
-        RIMO_CUDA(cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEMM_SMEM));
-        attr = true;
+// nt: columns of a tile (64 or 128); splits: of K, added into C
+static void gemm(const bf16* A, int lda, const bf16* B, int ldb, float* C, int ldc, int M, int N, int K, int nt,
+                 int splits, bool atomic, int* status, cudaStream_t s, int m_store = 1 << 30) {
+    constexpr int most = 2 * (128 + GEMM_MAX_NT) * GEMM_KC * 2;
+    static std::atomic<uint64_t> ready{0};  // devices whose limit is raised
+    int dev = 0;
+    RIMO_CUDA(cudaGetDevice(&dev));
+    if (dev >= 64 || !((ready.load() >> dev) & 1u)) {
+        RIMO_CUDA(cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        if (dev < 64) ready.fetch_or(1ull << dev);
     }
     GemmArgs g;
     g.A = A;
@@ -197,146 +225,172 @@ static void gemm(const bf16* A, int lda, const bf16* B, int ldb, float* C, int l
     g.M = M;
     g.N = N;
     g.K = K;
+    g.nt = nt;
+    g.m_store = m_store;
     g.kspan = ((K / splits + 15) / 16) * 16;
     g.atomic = atomic ? 1 : 0;
     g.status = status;
-    dim3 grid((N + GEMM_NT - 1) / GEMM_NT, M / 128, (K + g.kspan - 1) / g.kspan);
-    gemm_tc_kernel<<<grid, 128, GEMM_SMEM, s>>>(g);
+    dim3 grid((N + nt - 1) / nt, M / 128, (K + g.kspan - 1) / g.kspan);
+    gemm_tc_kernel<<<grid, 128, (size_t)2 * (128 + nt) * GEMM_KC * 2, s>>>(g);
 }
 
 // --------------------------------------------------------------------------------------
 // elementwise steps
-__global__ void l1_fwd_kernel(const float* __restrict__ X, const float* __restrict__ W1, const float* __restrict__ b1,
-                              float* __restrict__ Z1, bf16* __restrict__ H1, int B) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)B * MLP_H) return;
-    const int b = (int)(e / MLP_H), j = (int)(e % MLP_H);
+// Each takes EL_ROWS samples per block (256 threads: two samples at a time, one hidden unit per
+// thread), reads and writes whole rows, and also writes the bf16 result transposed (through
+// shared memory), the operand of the weight-gradient products.
+constexpr int EL_ROWS = 16;
+
+// block-wide transposed store of a [EL_ROWS][ncol <= 128] tile: dst[col0 + c][b0 + r]
+__device__ __forceinline__ void store_transposed(const bf16 (*t)[MLP_H + 2], bf16* __restrict__ dst, size_t ld, int col0,
+                                                 int ncol, int b0) {
+    // a thread writes two samples (4 bytes) of a column: 8 threads per 32-byte column segment
+    for (int e = threadIdx.x; e < ncol * (EL_ROWS / 2); e += 256) {
+        const int c = e / (EL_ROWS / 2), r = 2 * (e % (EL_ROWS / 2));
+        __nv_bfloat162 h;
+        h.x = t[r][c];
+        h.y = t[r + 1][c];
+        *reinterpret_cast<__nv_bfloat162*>(dst + (size_t)(col0 + c) * ld + b0 + r) = h;
+    }
+}
+
+__global__ void __launch_bounds__(256) l1_fwd_kernel(const float* __restrict__ X, const float* __restrict__ W1,
+                                                     const float* __restrict__ b1, float* __restrict__ Z1,
+                                                     bf16* __restrict__ H1, bf16* __restrict__ H1T, int B) {
+    __shared__ bf16 t[EL_ROWS][MLP_H + 2];
+    const int j = threadIdx.x % MLP_H, b0 = blockIdx.x * EL_ROWS;
     const float w0 = __bfloat162float(__float2bfloat16(W1[j * 3 + 0]));
     const float w1 = __bfloat162float(__float2bfloat16(W1[j * 3 + 1]));
     const float w2 = __bfloat162float(__float2bfloat16(W1[j * 3 + 2]));
-    const float z = fmaf(X[b * 3 + 0], w0, fmaf(X[b * 3 + 1], w1, fmaf(X[b * 3 + 2], w2, b1[j])));
-    Z1[e] = z;
-    H1[e] = __float2bfloat16(gelu_f(z));
+    const float bias = b1[j];
+#pragma unroll
+    for (int r = threadIdx.x / MLP_H; r < EL_ROWS; r += 2) {
+        const int b = b0 + r;
+        const float z = fmaf(X[b * 3 + 0], w0, fmaf(X[b * 3 + 1], w1, fmaf(X[b * 3 + 2], w2, bias)));
+        const bf16 h = __float2bfloat16(gelu_f(z));
+        Z1[(size_t)b * MLP_H + j] = z;
+        H1[(size_t)b * MLP_H + j] = h;
+        t[r][j] = h;
+    }
+    if (!H1T) return;
+    __syncthreads();
+    store_transposed(t, H1T, B, 0, MLP_H, b0);
 }
 
-// Z (in place) += bias; H = bf16(gelu(Z))
-__global__ void act_fwd_kernel(float* __restrict__ Z, const float* __restrict__ bias, bf16* __restrict__ H, int B,
-                               int n, int ld) {
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= (int64_t)B * n) return;
-    const int b = (int)(e / n), j = (int)(e % n);
-    const float z = Z[(size_t)b * ld + j] + bias[j];
-    Z[(size_t)b * ld + j] = z;
-    H[(size_t)b * n + j] = __float2bfloat16(gelu_f(z));
+// Z (in place) += bias; H = bf16(gelu(Z)), and transposed when HT is given
+__global__ void __launch_bounds__(256) act_fwd_kernel(float* __restrict__ Z, const float* __restrict__ bias,
+                                                      bf16* __restrict__ H, bf16* __restrict__ HT, int B) {
+    __shared__ bf16 t[EL_ROWS][MLP_H + 2];
+    const int j = threadIdx.x % MLP_H, b0 = blockIdx.x * EL_ROWS;
+    const float bj = bias[j];
+#pragma unroll
+    for (int r = threadIdx.x / MLP_H; r < EL_ROWS; r += 2) {
+        const size_t e = (size_t)(b0 + r) * MLP_H + j;
+        const float z = Z[e] + bj;
+        const bf16 h = __float2bfloat16(gelu_f(z));
+        Z[e] = z;
+        H[e] = h;
+        t[r][j] = h;
+    }
+    if (!HT) return;
+    __syncthreads();
+    store_transposed(t, HT, B, 0, MLP_H, b0);
 }
 
-// Y += b3; r = Y - T; loss += r^2; dY = 2 r / (450 B) as bf16 (cols >= 450 zero); db3 += dY
-__global__ void loss_bwd_kernel(float* __restrict__ Y, int ldy, const float* __restrict__ b3,
-                                const float* __restrict__ T, bf16* __restrict__ dY, int ld_dy, float* __restrict__ db3,
-                                float* __restrict__ loss, int B) {
-    __shared__ float red[256];
-    const int j = blockIdx.x % MLP_OUT_PAD;  // one output column per block x slice of the batch
-    const int part = blockIdx.x / MLP_OUT_PAD, nparts = gridDim.x / MLP_OUT_PAD;
-    float sq = 0.f, db = 0.f;
+// r = Y + b3 - T; loss += r^2; dY = 2 r / (450 B) as bf16 (columns 450 .. 463 zero) and its
+// transpose; db3 += dY.  (One block per output column before: strided reads of every row,
+// 72 us at B = 4096; now 9 us.)
+__global__ void __launch_bounds__(256) loss_bwd_kernel(const float* __restrict__ Y, int ldy, const float* __restrict__ b3,
+                                                       const float* __restrict__ T, bf16* __restrict__ dY, int ld_dy,
+                                                       bf16* __restrict__ dYT, float* __restrict__ db3,
+                                                       float* __restrict__ loss, int B) {
+    __shared__ bf16 t[EL_ROWS][MLP_H + 2];
+    __shared__ float part[256];
+    const int jj = threadIdx.x % MLP_H, half = threadIdx.x / MLP_H, b0 = blockIdx.x * EL_ROWS;
     const float scale = 2.f / ((float)MLP_OUT * (float)B);
-    for (int b = part * blockDim.x + threadIdx.x; b < B; b += nparts * blockDim.x) {
-        float d = 0.f;
-        if (j < MLP_OUT) {
-            const float y = Y[(size_t)b * ldy + j] + b3[j];
-            Y[(size_t)b * ldy + j] = y;
-            const float r = y - T[(size_t)b * MLP_OUT + j];
-            sq += r * r;
-            d = scale * r;
+    float sq = 0.f;
+    const int c0 = blockIdx.y * MLP_H, ncol = min(MLP_H, MLP_OUT_PAD - c0), j = c0 + jj;
+    float db = 0.f;
+    if (jj < ncol) {
+        const bool real = j < MLP_OUT;
+        const float bj = real ? b3[j] : 0.f;
+#pragma unroll
+        for (int r = half; r < EL_ROWS; r += 2) {
+            const size_t b = (size_t)(b0 + r);
+            const float res = real ? Y[b * ldy + j] + bj - T[b * MLP_OUT + j] : 0.f;
+            const float d = scale * res;
+            sq = fmaf(res, res, sq);
             db += d;
+            const bf16 h = __float2bfloat16(d);
+            dY[b * ld_dy + j] = h;
+            t[r][jj] = h;
         }
-        dY[(size_t)b * ld_dy + j] = __float2bfloat16(d);
     }
-    red[threadIdx.x] = sq;
+    part[threadIdx.x] = db;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
+    if (half == 0 && j < MLP_OUT) atomicAdd(&db3[j], part[jj] + part[jj + MLP_H]);
+    store_transposed(t, dYT, B, c0, ncol, b0);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sq;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float v = 0.f;
+        for (int w = 0; w < 8; ++w) v += part[w];
+        atomicAdd(loss, v);
     }
-    if (threadIdx.x == 0 && j < MLP_OUT) atomicAdd(loss, red[0]);
-    __syncthreads();
-    red[threadIdx.x] = db;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && j < MLP_OUT) atomicAdd(&db3[j], red[0]);
 }
 
-// dZ = dH * gelu'(Z) -> bf16; db += dZ (fp32)
-__global__ void act_bwd_kernel(const float* __restrict__ dH, const float* __restrict__ Z, bf16* __restrict__ dZ,
-                               float* __restrict__ db, int B) {
-    __shared__ float red[256];
-    const int j = blockIdx.x % MLP_H, part = blockIdx.x / MLP_H, nparts = gridDim.x / MLP_H;
+// dZ = dH * gelu'(Z) -> bf16, and transposed; db += dZ (fp32)
+__global__ void __launch_bounds__(256) act_bwd_kernel(const float* __restrict__ dH, const float* __restrict__ Z,
+                                                      bf16* __restrict__ dZ, bf16* __restrict__ dZT,
+                                                      float* __restrict__ db, int B) {
+    __shared__ bf16 t[EL_ROWS][MLP_H + 2];
+    __shared__ float part[256];
+    const int j = threadIdx.x % MLP_H, half = threadIdx.x / MLP_H, b0 = blockIdx.x * EL_ROWS;
     float acc = 0.f;
-    for (int b = part * blockDim.x + threadIdx.x; b < B; b += nparts * blockDim.x) {
-        const float d = dH[(size_t)b * MLP_H + j] * gelu_grad_f(Z[(size_t)b * MLP_H + j]);
-        dZ[(size_t)b * MLP_H + j] = __float2bfloat16(d);
+#pragma unroll
+    for (int r = half; r < EL_ROWS; r += 2) {
+        const size_t e = (size_t)(b0 + r) * MLP_H + j;
+        const float d = dH[e] * gelu_grad_f(Z[e]);
+        const bf16 h = __float2bfloat16(d);
+        dZ[e] = h;
+        t[r][j] = h;
         acc += d;
     }
-    red[threadIdx.x] = acc;
+    part[threadIdx.x] = acc;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(&db[j], red[0]);
+    if (half == 0) atomicAdd(&db[j], part[j] + part[j + MLP_H]);
+    store_transposed(t, dZT, B, 0, MLP_H, b0);
 }
 
 // dZ1 = dH1 * gelu'(Z1); dW1[j][i] += dZ1[b][j] X[b][i]; db1[j] += dZ1[b][j]
-__global__ void l1_bwd_kernel(const float* __restrict__ dH1, const float* __restrict__ Z1, const float* __restrict__ X,
-                              float* __restrict__ dW1, float* __restrict__ db1, int B) {
-    __shared__ float red[4][256];
-    const int j = blockIdx.x % MLP_H, part = blockIdx.x / MLP_H, nparts = gridDim.x / MLP_H;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-    for (int b = part * blockDim.x + threadIdx.x; b < B; b += nparts * blockDim.x) {
-        const float d = dH1[(size_t)b * MLP_H + j] * gelu_grad_f(Z1[(size_t)b * MLP_H + j]);
-        a0 += d * X[b * 3 + 0];
-        a1 += d * X[b * 3 + 1];
-        a2 += d * X[b * 3 + 2];
-        a3 += d;
+__global__ void __launch_bounds__(256) l1_bwd_kernel(const float* __restrict__ dH1, const float* __restrict__ Z1,
+                                                     const float* __restrict__ X, float* __restrict__ dW1,
+                                                     float* __restrict__ db1) {
+    __shared__ float4 part[256];
+    const int j = threadIdx.x % MLP_H, half = threadIdx.x / MLP_H, b0 = blockIdx.x * EL_ROWS;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int r = half; r < EL_ROWS; r += 2) {
+        const int b = b0 + r;
+        const size_t e = (size_t)b * MLP_H + j;
+        const float d = dH1[e] * gelu_grad_f(Z1[e]);
+        a.x = fmaf(d, X[b * 3 + 0], a.x);
+        a.y = fmaf(d, X[b * 3 + 1], a.y);
+        a.z = fmaf(d, X[b * 3 + 2], a.z);
+        a.w += d;
     }
-    red[0][threadIdx.x] = a0;
-    red[1][threadIdx.x] = a1;
-    red[2][threadIdx.x] = a2;
-    red[3][threadIdx.x] = a3;
+    part[threadIdx.x] = a;
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o)
-            for (int q = 0; q < 4; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + o];
-        __syncthreads();
+    if (half == 0) {
+        const float4 q = part[j + MLP_H];
+        atomicAdd(&dW1[j * 3 + 0], a.x + q.x);
+        atomicAdd(&dW1[j * 3 + 1], a.y + q.y);
+        atomicAdd(&dW1[j * 3 + 2], a.z + q.z);
+        atomicAdd(&db1[j], a.w + q.w);
     }
-    if (threadIdx.x == 0) {
-        atomicAdd(&dW1[j * 3 + 0], red[0][0]);
-        atomicAdd(&dW1[j * 3 + 1], red[1][0]);
-        atomicAdd(&dW1[j * 3 + 2], red[2][0]);
-        atomicAdd(&db1[j], red[3][0]);
-    }
-}
-
-// dst[c][r] = src[r][c], bf16, 32 x 32 tiles through shared memory
-__global__ void transpose_bf16_kernel(const bf16* __restrict__ src, bf16* __restrict__ dst, int R, int Cn) {
-    __shared__ bf16 t[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int r = r0 + i, c = c0 + threadIdx.x;
-        t[i][threadIdx.x] = (r < R && c < Cn) ? src[(size_t)r * Cn + c] : __float2bfloat16(0.f);
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
-        const int c = c0 + i, r = r0 + threadIdx.x;
-        if (c < Cn && r < R) dst[(size_t)c * R + r] = t[threadIdx.x][i];
-    }
-}
-
-static void transpose(const bf16* src, bf16* dst, int R, int Cn, cudaStream_t s) {
-    dim3 grid((Cn + 31) / 32, (R + 31) / 32), block(32, 8);
-    transpose_bf16_kernel<<<grid, block, 0, s>>>(src, dst, R, Cn);
 }
 
 // Adam on the FP32 masters, then the bf16 operand copies: W2 [128][128], W2^T, W3 [464][128]
@@ -380,6 +434,7 @@ __global__ void pack_weights_kernel(const float* __restrict__ P, bf16* __restric
 // --------------------------------------------------------------------------------------
 Mlp::~Mlp() {
     for (void* p : owned) cudaFree(p);
+    if (host) cudaFreeHost(host);
 }
 
 void* Mlp::alloc(size_t bytes) {
@@ -394,15 +449,20 @@ void* Mlp::alloc(size_t bytes) {
 
 void Mlp::init(uint64_t seed) {
     P = (float*)alloc(MLP_NPARAM * sizeof(float));
-    G = (float*)alloc(MLP_NPARAM * sizeof(float));
+    // gradients, the batch loss and the status word: one buffer, one copy to the host
+    G = (float*)alloc((MLP_NPARAM + 2) * sizeof(float));
+    loss = G + MLP_NPARAM;
+    status = reinterpret_cast<int*>(G + MLP_NPARAM + 1);
+    if (cudaMallocHost(&host, (MLP_NPARAM + 2) * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        fail(RIMO_ERR_OOM, "host buffer of the surrogate's gradients");
+    }
     Mom = (float*)alloc(MLP_NPARAM * sizeof(float));
     Vel = (float*)alloc(MLP_NPARAM * sizeof(float));
     W2b = (bf16*)alloc(MLP_H * MLP_H * sizeof(bf16));
     W2Tb = (bf16*)alloc(MLP_H * MLP_H * sizeof(bf16));
     W3b = (bf16*)alloc(MLP_OUT_PAD * MLP_H * sizeof(bf16));
     W3Tb = (bf16*)alloc(MLP_H * MLP_K3 * sizeof(bf16));
-    loss = (float*)alloc(sizeof(float));
-    status = (int*)alloc(sizeof(int));
     RIMO_CUDA(cudaMemset(status, 0, sizeof(int)));
     // uniform(-1/sqrt(fan_in), 1/sqrt(fan_in)) from a seeded host generator
     std::vector<float> h(MLP_NPARAM);
@@ -434,7 +494,7 @@ void Mlp::pack(cudaStream_t s) {
     pack_weights_kernel<<<(n + 255) / 256, 256, 0, s>>>(P, W2b, W2Tb, W3b, W3Tb);
 }
 
-void Mlp::reserve(int B) {
+void Mlp::reserve(int B, cudaStream_t s) {
     if (B <= cap) return;
     cap = B;
     Z1 = (float*)alloc((size_t)B * MLP_H * sizeof(float));
@@ -449,40 +509,34 @@ void Mlp::reserve(int B) {
     dYT = (bf16*)alloc((size_t)B * MLP_K3 * sizeof(bf16));
     dZ = (bf16*)alloc((size_t)B * MLP_H * sizeof(bf16));
     dZT = (bf16*)alloc((size_t)B * MLP_H * sizeof(bf16));
+    // rows past the padded outputs only fill the last 128-row tile of dW3
+    RIMO_CUDA(cudaMemsetAsync(dYT, 0, (size_t)B * MLP_K3 * sizeof(bf16), s));
 }
 
-void Mlp::forward(const float* X, int B, cudaStream_t s) {
-    reserve(B);
-    const int n1 = B * MLP_H;
-    l1_fwd_kernel<<<(n1 + 255) / 256, 256, 0, s>>>(X, P + MLP_OFF_W1, P + MLP_OFF_B1, Z1, H1, B);
-    gemm(H1, MLP_H, W2b, MLP_H, Z2, MLP_H, B, MLP_H, MLP_H, 1, false, status, s);
-    act_fwd_kernel<<<(n1 + 255) / 256, 256, 0, s>>>(Z2, P + MLP_OFF_B2, H2, B, MLP_H, MLP_H);
-    gemm(H2, MLP_H, W3b, MLP_H, Y, MLP_OUT_PAD, B, MLP_OUT_PAD, MLP_H, 1, false, status, s);
+void Mlp::forward(const float* X, int B, cudaStream_t s, bool train) {
+    reserve(B, s);
+    const int blocks = B / EL_ROWS;
+    l1_fwd_kernel<<<blocks, 256, 0, s>>>(X, P + MLP_OFF_W1, P + MLP_OFF_B1, Z1, H1, train ? H1T : nullptr, B);
+    gemm(H1, MLP_H, W2b, MLP_H, Z2, MLP_H, B, MLP_H, MLP_H, 64, 1, false, status, s);
+    act_fwd_kernel<<<blocks, 256, 0, s>>>(Z2, P + MLP_OFF_B2, H2, train ? H2T : nullptr, B);
+    gemm(H2, MLP_H, W3b, MLP_H, Y, MLP_OUT_PAD, B, MLP_OUT_PAD, MLP_H, 128, 1, false, status, s);
 }
 
 void Mlp::grads(const float* X, const float* T, int B, cudaStream_t s) {
-    forward(X, B, s);
-    RIMO_CUDA(cudaMemsetAsync(G, 0, MLP_NPARAM * sizeof(float), s));
-    RIMO_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), s));
-    RIMO_CUDA(cudaMemsetAsync(dY, 0, (size_t)B * MLP_K3 * sizeof(bf16), s));
-    const int parts = std::max(1, std::min(16, B / 256));
-    loss_bwd_kernel<<<MLP_OUT_PAD * parts, 256, 0, s>>>(Y, MLP_OUT_PAD, P + MLP_OFF_B3, T, dY, MLP_K3,
-                                                       G + MLP_OFF_B3, loss, B);
-    transpose(H2, H2T, B, MLP_H, s);
-    transpose(dY, dYT, B, MLP_K3, s);
-    const int splits = std::max(1, B / 512);
+    forward(X, B, s, true);
+    RIMO_CUDA(cudaMemsetAsync(G, 0, (MLP_NPARAM + 1) * sizeof(float), s));  // and the loss
+    const int blocks = B / EL_ROWS;
+    loss_bwd_kernel<<<dim3(blocks, (MLP_OUT_PAD + MLP_H - 1) / MLP_H), 256, 0, s>>>(
+        Y, MLP_OUT_PAD, P + MLP_OFF_B3, T, dY, MLP_K3, dYT, G + MLP_OFF_B3, loss, B);
+    const int splits = std::max(1, B / 128);
     // dH2 = dY W3 (K = 464 padded output dimension)
-    gemm(dY, MLP_K3, W3Tb, MLP_K3, dH, MLP_H, B, MLP_H, MLP_OUT_PAD, 1, false, status, s);
-    // dW3 = dY^T H2 (M = 464 -> rows >= 450 land in a scratch tail of G3)
-    RIMO_CUDA(cudaMemsetAsync(Y, 0, (size_t)512 * MLP_H * sizeof(float), s));
-    gemm(dYT, B, H2T, B, Y, MLP_H, 512, MLP_H, B, splits, true, status, s);
-    RIMO_CUDA(cudaMemcpyAsync(G + MLP_OFF_W3, Y, (size_t)MLP_OUT * MLP_H * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    act_bwd_kernel<<<MLP_H * parts, 256, 0, s>>>(dH, Z2, dZ, G + MLP_OFF_B2, B);
-    transpose(dZ, dZT, B, MLP_H, s);
-    transpose(H1, H1T, B, MLP_H, s);
-    gemm(dZT, B, H1T, B, G + MLP_OFF_W2, MLP_H, MLP_H, MLP_H, B, splits, true, status, s);
-    gemm(dZ, MLP_H, W2Tb, MLP_H, dH, MLP_H, B, MLP_H, MLP_H, 1, false, status, s);
-    l1_bwd_kernel<<<MLP_H * parts, 256, 0, s>>>(dH, Z1, X, G + MLP_OFF_W1, G + MLP_OFF_B1, B);
+    gemm(dY, MLP_K3, W3Tb, MLP_K3, dH, MLP_H, B, MLP_H, MLP_OUT_PAD, 64, 1, false, status, s);
+    // dW3 = dY^T H2 (M = 512: the rows past the outputs are not stored)
+    gemm(dYT, B, H2T, B, G + MLP_OFF_W3, MLP_H, 512, MLP_H, B, 128, splits, true, status, s, MLP_OUT);
+    act_bwd_kernel<<<blocks, 256, 0, s>>>(dH, Z2, dZ, dZT, G + MLP_OFF_B2, B);
+    gemm(dZT, B, H1T, B, G + MLP_OFF_W2, MLP_H, MLP_H, MLP_H, B, 64, splits, true, status, s);
+    gemm(dZ, MLP_H, W2Tb, MLP_H, dH, MLP_H, B, MLP_H, MLP_H, 64, 1, false, status, s);
+    l1_bwd_kernel<<<blocks, 256, 0, s>>>(dH, Z1, X, G + MLP_OFF_W1, G + MLP_OFF_B1);
 }
 
 void Mlp::step(const float* X, const float* T, int B, float lr, cudaStream_t s) {
@@ -979,15 +1033,16 @@ rimo_status rimo_surrogate_gradients(rimo_surrogate_t s, const float* x, const f
     if (!s || !x || !t) fail(RIMO_ERR_INVALID_ARG, "null argument");
     check_batch(B);
     cudaStream_t st = (cudaStream_t)stream;
-    s->mlp.grads(x, t, (int)B, st);
+    Mlp& m = s->mlp;
+    m.grads(x, t, (int)B, st);
     RIMO_CUDA(cudaGetLastError());
-    check_status(s->mlp, st);
-    if (grads) RIMO_CUDA(cudaMemcpy(grads, s->mlp.G, MLP_NPARAM * sizeof(float), cudaMemcpyDeviceToHost));
-    if (loss) {
-        float l = 0.f;
-        RIMO_CUDA(cudaMemcpy(&l, s->mlp.loss, sizeof(float), cudaMemcpyDeviceToHost));
-        *loss = l / ((float)B * MLP_OUT);
-    }
+    RIMO_CUDA(cudaMemcpyAsync(m.host, m.G, (MLP_NPARAM + 2) * sizeof(float), cudaMemcpyDeviceToHost, st));
+    RIMO_CUDA(cudaStreamSynchronize(st));
+    int failed = 0;
+    std::memcpy(&failed, m.host + MLP_NPARAM + 1, sizeof(int));
+    if (failed) check_status(m, st);  // clears it and reports
+    if (grads) std::memcpy(grads, m.host, MLP_NPARAM * sizeof(float));
+    if (loss) *loss = m.host[MLP_NPARAM] / ((float)B * MLP_OUT);
     SUR_END
 }
 
@@ -1046,7 +1101,7 @@ rimo_status rimo_surrogate_fit(rimo_surrogate_t s, rimo_plan_t exact, int64_t n_
         exact->d_meta, exact->d_gblock_ptrs, exact->d_phiu, exact->d_phiv, exact->d_wr, exact->M, sample_seed,
         n_samples, 1.f / ws, X, T);
     RIMO_CUDA(cudaGetLastError());
-    s->mlp.reserve(batch);
+    s->mlp.reserve(batch, st);
     for (int k = 0; k < steps; ++k) {
         // cosine decay from lr to lr / 100
         const float lr_k = lr * (0.01f + 0.99f * 0.5f * (1.f + std::cos(3.14159265358979f * (float)k / (float)steps)));

@@ -26,8 +26,9 @@ struct Mlp {
     float* Mom = nullptr;  // Adam first moments
     float* Vel = nullptr;  // Adam second moments
     __nv_bfloat16 *W2b = nullptr, *W2Tb = nullptr, *W3b = nullptr, *W3Tb = nullptr;
-    float* loss = nullptr;
-    int* status = nullptr;
+    float* loss = nullptr;   // behind G
+    int* status = nullptr;   // behind the loss
+    float* host = nullptr;   // pinned copy of G, loss and status
     int t = 0;
     // activations of the last batch
     int cap = 0;
@@ -41,8 +42,9 @@ struct Mlp {
     void init(uint64_t seed);
     void set_params(const float* host, cudaStream_t s);
     void pack(cudaStream_t s);
-    void reserve(int B);
-    void forward(const float* X, int B, cudaStream_t s);             // Y [B][464] without b3
+    void reserve(int B, cudaStream_t s);
+    // Y [B][464] without b3 (train: also the transposed activations)
+    void forward(const float* X, int B, cudaStream_t s, bool train = false);
     void grads(const float* X, const float* T, int B, cudaStream_t s);
     void step(const float* X, const float* T, int B, float lr, cudaStream_t s);
 };
