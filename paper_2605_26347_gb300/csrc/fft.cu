@@ -161,7 +161,11 @@ __device__ __forceinline__ void dft_r(float2* v) {
     else dft16<INV>(v);
 }
 
+// Exchange buffers are padded: element i at i + i / 16.  A stage's addresses are one base per
+// thread and compile-time offsets (a multiple of 16 moves by padded16): the index arithmetic,
+// spelled out per element, was 15 to 20 % of the passes' instructions (see the stages below).
 __device__ __forceinline__ int pidx(int i) { return i + (i >> 4); }
+__host__ __device__ constexpr int padded16(int i) { return i + i / 16; }
 
 // One Stockham stage of radix R after NS points have been combined (NS * R <= N).
 // Thread t owns butterflies j = t + q T (q < 16/R, T = N/16); butterfly j reads
@@ -174,10 +178,12 @@ __device__ __forceinline__ void fft_stage(float2 (&v)[16], float2* sm, int t, co
     constexpr int T = N / 16;
     constexpr int Q = 16 / R;
     if (!FIRST) {
+        const float2* rd = sm + pidx(t);
 #pragma unroll
         for (int q = 0; q < Q; ++q)
 #pragma unroll
-            for (int r = 0; r < R; ++r) v[q * R + r] = sm[pidx(t + q * T + r * (N / R))];
+            // element t + q T + r N / R: T and N / R are multiples of 16, or T = 8 and q < 2
+            for (int r = 0; r < R; ++r) v[q * R + r] = rd[padded16(q * T) + padded16(r * (N / R))];
         __syncthreads();
     }
 #pragma unroll
@@ -211,14 +217,12 @@ __device__ __forceinline__ void fft_stage(float2 (&v)[16], float2* sm, int t, co
         if constexpr (HZ && R == 16) dft16_hz<INV>(&v[q * R]);
         else dft_r<R, INV>(&v[q * R]);
     }
-    if (!LAST) {
+    if constexpr (!LAST) {
+        // butterfly j = t (R = 16, Q = 1): element (j / NS) 16 NS + j mod NS + r NS
+        static_assert(R == 16, "only a last stage has a smaller radix");
+        float2* wr = sm + padded16((t / NS) * NS * 16) + (NS == 1 ? 0 : pidx(t & (NS - 1)));
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const int j = t + q * T;
-            const int base = (j / NS) * NS * R + (j & (NS - 1));
-#pragma unroll
-            for (int r = 0; r < R; ++r) sm[pidx(base + r * NS)] = v[q * R + r];
-        }
+        for (int r = 0; r < R; ++r) wr[NS == 1 ? r : padded16(r * NS)] = v[r];
         __syncthreads();
     }
 }
@@ -274,16 +278,21 @@ __device__ __forceinline__ void dft32(float2* v) {
 // out_k32(t, s).  All 256 threads of the row must call it.
 template <bool INV, bool HZ>
 __device__ __forceinline__ void fft8192_32(float2 (&v)[32], float2* sm, int t, const float2* __restrict__ tw) {
+    // every address is one base per thread and a compile-time offset (multiples of 32 move by
+    // 33 / 32): 9 % of the pass was index arithmetic without that
     dft32<INV, HZ>(v);  // stage 1: butterfly j = t, outputs at 32 t + r
+    float2* w1 = sm + 33 * t;
 #pragma unroll
-    for (int r = 0; r < 32; ++r) sm[pidx32(32 * t + r)] = v[r];
+    for (int r = 0; r < 32; ++r) w1[r] = v[r];
     __syncthreads();
     // stage 2: NS = 32, R = 16, butterflies j = t + 256 q, reads j + 512 r
+    const float2* rd = sm + pidx32(t);
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll
-        for (int r = 0; r < 16; ++r) v[16 * q + r] = sm[pidx32(t + 256 * q + 512 * r)];
+        for (int r = 0; r < 16; ++r) v[16 * q + r] = rd[264 * q + 528 * r];
     __syncthreads();
+    float2* w2 = sm + (t >> 5) * 528 + (t & 31);  // outputs at (j / 32) 512 + j mod 32 + 32 r
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
         const int j = t + 256 * q, jm = j & 31;
@@ -300,16 +309,15 @@ __device__ __forceinline__ void fft8192_32(float2 (&v)[32], float2* sm, int t, c
 #pragma unroll
         for (int r = 1; r < 16; ++r) v[16 * q + r] = INV ? cmulc(v[16 * q + r], w[r]) : cmul(v[16 * q + r], w[r]);
         dft16<INV>(&v[16 * q]);
-        const int base = (j >> 5) * 512 + jm;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) sm[pidx32(base + 32 * r)] = v[16 * q + r];
+        for (int r = 0; r < 16; ++r) w2[8 * 528 * q + 33 * r] = v[16 * q + r];
     }
     __syncthreads();
     // stage 3: NS = 512, R = 16, butterflies j = t + 256 q (< 512), reads j + 512 r
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll
-        for (int r = 0; r < 16; ++r) v[16 * q + r] = sm[pidx32(t + 256 * q + 512 * r)];
+        for (int r = 0; r < 16; ++r) v[16 * q + r] = rd[264 * q + 528 * r];
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -506,20 +514,27 @@ __device__ __forceinline__ void transposed_store(float2* smem, Src src, Dst dst,
         }
         __syncthreads();
     } else {
-        cluster_sync_all();
-        constexpr int NP = C * RB / 2, KPC = NK / C;
-        static_assert(THREADS % NP == 0, "a thread keeps one row pair");
+        constexpr int NP = C * RB / 2, KPC = NK / C, STEP = THREADS / NP, IT = KPC / STEP;
+        static_assert(THREADS % NP == 0 && STEP % 16 == 0 && KPC % STEP == 0, "a thread keeps one row pair");
         const int rank = (int)(blockIdx.x % C);
         const int rbase = r0_block - rank * RB;  // first row of the cluster
         const int q = threadIdx.x % NP;                   // rows 2q, 2q + 1 of the cluster
-        const uint32_t b0 = dsmem_map(smem + ((2 * q) % RB) * SR, (2 * q) / RB);
-        const uint32_t b1 = dsmem_map(smem + ((2 * q + 1) % RB) * SR, (2 * q + 1) / RB);
-        for (int e = threadIdx.x; e < KPC * NP; e += THREADS) {
-            const int kk = rank * KPC + e / NP;
-            if (!keep(kk)) continue;
-            const uint32_t off = (uint32_t)pidx(src(kk)) * 8u;
-            const float2 a = dsmem_ld2(b0 + off), b = dsmem_ld2(b1 + off);
-            *reinterpret_cast<float4*>(&out[(size_t)dst(kk) * ld + rbase + 2 * q]) = make_float4(a.x, a.y, b.x, b.y);
+        // src and dst are shifts within a rank's range, so a thread's values are STEP apart
+        const int kk0 = rank * KPC + threadIdx.x / NP;
+        uint32_t on = 0;
+#pragma unroll
+        for (int it = 0; it < IT; ++it) on |= (keep(kk0 + it * STEP) ? 1u : 0u) << it;
+        const uint32_t off = (uint32_t)pidx(src(kk0)) * 8u;
+        const uint32_t b0 = dsmem_map(smem + ((2 * q) % RB) * SR, (2 * q) / RB) + off;
+        const uint32_t b1 = dsmem_map(smem + ((2 * q + 1) % RB) * SR, (2 * q + 1) / RB) + off;
+        float2* o = out + (size_t)dst(kk0) * ld + rbase + 2 * q;
+        cluster_sync_all();
+#pragma unroll
+        for (int it = 0; it < IT; ++it) {
+            if ((on >> it) & 1u) {
+                const float2 a = dsmem_ld2(b0 + padded16(it * STEP) * 8), b = dsmem_ld2(b1 + padded16(it * STEP) * 8);
+                *reinterpret_cast<float4*>(o + (size_t)(it * STEP) * ld) = make_float4(a.x, a.y, b.x, b.y);
+            }
         }
         cluster_sync_relaxed();  // partners are done reading before the block may exit
     }
@@ -624,7 +639,7 @@ __global__ void __launch_bounds__(RB * N / 8, (1024 / (RB * N / 8)) > 0 ? (1024 
     }
     fft_n<L, false, true>(v, sm, t, tws);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) sm[pidx(t + T * m)] = v[out_slot<L>(m)];
+    for (int m = 0; m < 16; ++m) sm[pidx(t) + padded16(T * m)] = v[out_slot<L>(m)];
     // rows k of At the forward column pass does not transform are not stored
     transposed_store<RB, C, SR, L, RB * N / 8>(
         smem, [](int kk) { return kk; }, [](int kk) { return kk; },
@@ -740,7 +755,7 @@ __global__ void __launch_bounds__(256, 2)
     }
     fft8192_32<true, false>(v, smem, t, tw);
 #pragma unroll
-    for (int q = 0; q < 32; ++q) smem[pidx(out_k32(t, q))] = v[q];
+    for (int q = 0; q < 32; ++q) smem[pidx(t) + padded16(out_k32(0, q))] = v[q];
     transposed_store<1, 4, SR, N, 256>(
         smem, [](int kk) { return kk < N / 2 ? kk : kk + N; },
         [](int kk) { return kk < N / 2 ? kk + N / 2 : kk - N / 2; }, [](int) { return true; }, J.out, (size_t)gx, r0);
@@ -868,7 +883,7 @@ __global__ void __launch_bounds__(RB * N / 8, (1024 / (RB * N / 8)) > 0 ? (1024 
     }
     fft_n<L, true>(v, sm, t, tws);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) sm[pidx(t + T * m)] = v[out_slot<L>(m)];
+    for (int m = 0; m < 16; ++m) sm[pidx(t) + padded16(T * m)] = v[out_slot<L>(m)];
     // kept output kk < N: k = kk (kk < N/2) or kk + N; image row i = (k < N/2 ? k : k - L) + N/2
     transposed_store<RB, C, SR, N, RB * N / 8>(
         smem, [](int kk) { return kk < N / 2 ? kk : kk + N; },
