@@ -114,12 +114,13 @@ constexpr int GTG_AHEAD = 2;  // units a block takes by its index; the later one
 
 // Scale of one work unit of n visibilities: the largest power of two s with
 // s maxterm <= min(2^21, 2^30 / n) (see the fixed-point layout in internal.h).
-__device__ __forceinline__ void fx_scale(float maxterm, int64_t n, float& s1, float& inv) {
+__device__ __forceinline__ void fx_scale(float maxterm, int n, float& s1, float& inv) {
     s1 = 1.f;
     inv = 1.f;
     if (!(maxterm > 0.f)) return;  // all contributions vanish (or the input was flagged)
-    const float lim = fminf(2097152.f, 1073741824.f / (float)(n > 1 ? n : 1));
-    int ex = (int)((__float_as_uint(lim / maxterm) >> 23) & 255u) - 127;
+    // (approximate quotients: a power of two, the margins of maxterm cover an ulp)
+    const float lim = fminf(2097152.f, __fdividef(1073741824.f, (float)(n > 1 ? n : 1)));
+    int ex = (int)((__float_as_uint(__fdividef(lim, maxterm)) >> 23) & 255u) - 127;
     ex = ex < -120 ? -120 : (ex > 120 ? 120 : ex);
     s1 = __uint_as_float((uint32_t)(ex + 127) << 23);
     inv = __uint_as_float((uint32_t)(127 - ex) << 23);
@@ -244,15 +245,16 @@ struct UnitBox {
     }
 };
 
-// Starts the copies of a unit's X box into its patch buffer (rows and columns wrap).
+// Starts the copies of a unit's X box into its patch buffer (rows and columns wrap), as thread t
+// of nt.
 template <int PWC>
-__device__ __forceinline__ void stage_x(const GtgArgs& A, const UnitRec* rec, float2* dst) {
+__device__ __forceinline__ void stage_x(const GtgArgs& A, const UnitRec* rec, float2* dst, int t, int nt) {
     const uint32_t g = rec->geom;
     const int PW = PWC > 0 ? PWC : (int)(g >> 16);
     const int u0 = (int)(g & 255u) * A.TS, v0 = (int)((g >> 8) & 255u) * A.TS;
     const float2* X = reinterpret_cast<const float2*>(reinterpret_cast<const char*>(A.X) + rec->X);
     const UnitBox B(rec);
-    for (int e = threadIdx.x; e < B.n; e += blockDim.x) {
+    for (int e = t; e < B.n; e += nt) {
         int a, c;
         B.at(e, a, c);
         int gu = u0 + a, gv = v0 + c;
@@ -330,7 +332,10 @@ __global__ void __launch_bounds__(GTG_MAX_WARPS * 32, 1) gtg_kernel(const __grid
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
 
-    if (GATHER) stage_x<PWC>(A, recs, Xbuf0);  // round 0 (every block has a first unit)
+    // the last third of the warps (the smallest shares of a small unit) copies the X boxes and
+    // finds their maxima
+    const int st0 = (nw - (nw + 2) / 3) * 32, stn = (int)blockDim.x - st0;
+    if (GATHER && tid >= st0) stage_x<PWC>(A, recs, Xbuf0, tid - st0, stn);  // round 0 (every block has a first unit)
     cp_async_commit();
 
     // ---- this warp's visibilities
@@ -348,29 +353,32 @@ __global__ void __launch_bounds__(GTG_MAX_WARPS * 32, 1) gtg_kernel(const __grid
             C.nxt = load_meta(recs + C.round % GTG_RECS, C.base + 32 + lane, warp, nw);
             C.ready = true;
         } else if (C.round <= r && s_idx[(C.round + 1) % GTG_RECS] < A.nunits) {
-            C.nxt = load_meta(recs + (C.round + 1) % GTG_RECS, lane, warp, nw);
-            C.ready = true;
+            const UnitRec* rec = recs + (C.round + 1) % GTG_RECS;
+            if (warp < rec->nvis) {
+                C.nxt = load_meta(rec, lane, warp, nw);
+                C.ready = true;
+            }
         }
     };
     // the next batch, of the unit of round r + 1 at most; false: none
     auto advance = [&](int r) {
         if (A.stall) return false;
-        do {
-            if (C.base + 32 < C.n) {
-                C.base += 32;
-            } else {
+        if (C.base + 32 < C.n) {
+            C.base += 32;
+        } else {
+            do {
                 if (C.round > r || s_idx[(C.round + 1) % GTG_RECS] >= A.nunits) return false;
                 ++C.round;
-                C.base = 0;
-                C.n = unit_share(recs[C.round % GTG_RECS].nvis, warp, nw, mgw);
-            }
-            const UnitRec* rec = recs + C.round % GTG_RECS;
-            unpack(rec->taps, C.ready ? C.nxt : load_meta(rec, C.base + lane, warp, nw));
-            C.b = 0;
-            C.nb = min(32, C.n - C.base);
-            C.ready = false;
-            look_ahead(r);
-        } while (C.nb <= 0);
+                C.base = C.n = C.b = C.nb = 0;  // (a unit of fewer visibilities has none for this warp)
+            } while (warp >= recs[C.round % GTG_RECS].nvis);
+            C.n = unit_share(recs[C.round % GTG_RECS].nvis, warp, nw, mgw);
+        }
+        const UnitRec* rec = recs + C.round % GTG_RECS;
+        unpack(rec->taps, C.ready ? C.nxt : load_meta(rec, C.base + lane, warp, nw));
+        C.b = 0;
+        C.nb = min(32, C.n - C.base);
+        C.ready = false;
+        look_ahead(r);
         return true;
     };
     C.round = C.base = C.b = 0;
@@ -418,11 +426,11 @@ __global__ void __launch_bounds__(GTG_MAX_WARPS * 32, 1) gtg_kernel(const __grid
         const int PW = PWC > 0 ? PWC : (have ? (int)(rec->geom >> 16) : A.PW);
         float2* Xs = Xbuf0 + (NX == 2 && (r & 1) ? npmax : 0);
         cp_async_wait_all();
-        if (MODE == 2 && have) {
+        if (MODE == 2 && have && tid >= st0) {
             // max |X| of the pairs this thread copied
             float xm = 0.f;
             const UnitBox B(rec);
-            for (int e = tid; e < B.n; e += blockDim.x) {
+            for (int e = tid - st0; e < B.n; e += stn) {
                 int a, c;
                 B.at(e, a, c);
                 const float4 x = *reinterpret_cast<const float4*>(Xs + a * PW + c);
@@ -439,8 +447,8 @@ __global__ void __launch_bounds__(GTG_MAX_WARPS * 32, 1) gtg_kernel(const __grid
         int next_idx = 0;
         if (tid == (nw - 1) * 32) next_idx = atomicAdd(A.counter, 1) + GTG_AHEAD * G;
         const bool more = s_idx[(r + 1) % GTG_RECS] < A.nunits;
-        if (GATHER && NX == 2 && more)
-            stage_x<PWC>(A, recs + (r + 1) % GTG_RECS, Xbuf0 + (r & 1 ? 0 : npmax));
+        if (GATHER && NX == 2 && more && tid >= st0)
+            stage_x<PWC>(A, recs + (r + 1) % GTG_RECS, Xbuf0 + (r & 1 ? 0 : npmax), tid - st0, stn);
         if (!C.ready && more) look_ahead(r);
         if (warp == nw - 1) {  // the unit of round r + 2 and its record (this warp has the smallest share)
             next_idx = __shfl_sync(0xffffffffu, next_idx, 0);
@@ -501,8 +509,8 @@ __global__ void __launch_bounds__(GTG_MAX_WARPS * 32, 1) gtg_kernel(const __grid
             refill(r);
         }
         if (SCATTER || NX == 1) __syncthreads();  // barrier B
-        if (GATHER && NX == 1 && more) {
-            stage_x<PWC>(A, recs + (r + 1) % GTG_RECS, Xbuf0);
+        if (GATHER && NX == 1 && more && tid >= st0) {
+            stage_x<PWC>(A, recs + (r + 1) % GTG_RECS, Xbuf0, tid - st0, stn);
             cp_async_commit();
         }
         if (SCATTER) {
