@@ -86,19 +86,23 @@ static void inv(rimo_plan* p, int b, float2* out, bool first, int real_only, cud
     prof_end(p, 1, s);
 }
 
-static void gtg(rimo_plan* p, int b, int mode, const float2* y_in, float2* y_out, cudaStream_t s,
-                const float2* X = nullptr, float2* patch = nullptr) {
+// Plans without stored G: the tiles of bins [b0, b1] into the tap scratch.
+static void generate(rimo_plan* p, int b0, int b1, cudaStream_t s) {
+    const int64_t v0 = p->bins[b0].vb, n = p->bins[b1].ve - v0;
     if (p->mode == RIMO_MODE_SURROGATE) {
         prof_begin(p, ST_MLP, s);
-        const int nl = surrogate_generate(p, b, s);  // this bin's tiles into the tap scratch
-        prof_end(p, nl, s);
+        prof_end(p, surrogate_generate(p, v0, n, s), s);
     } else if (p->mode == RIMO_MODE_ONTHEFLY || p->mode == RIMO_MODE_HOLOGRAPHIC) {
         prof_begin(p, ST_GBUILD, s);
-        launch_gbuild_range(p, p->bins[b].vb, p->bins[b].ve - p->bins[b].vb, s);  // exact tiles
+        launch_gbuild_range(p, v0, n, s);  // exact tiles
         prof_end(p, 1, s);
     }
+}
+
+static void gtg(rimo_plan* p, int b, int mode, const float2* y_in, float2* y_out, cudaStream_t s) {
+    generate(p, b, b, s);
     prof_begin(p, ST_GTG, s);
-    launch_gtg(p, b, mode, y_in, y_out, s, X, patch);
+    launch_gtg(p, b, mode, y_in, y_out, s);
     const bool merge = mode != 0 && p->bins[b].m1 > p->bins[b].m0;
     prof_end(p, gtg_launches(p, b, mode) + (merge ? 1 : 0), s);
 }
@@ -111,16 +115,20 @@ static void gtg(rimo_plan* p, int b, int mode, const float2* y_in, float2* y_out
 // and patches of their own (the kernels and the order of every sum are those of one bin at a
 // time, so the results are the same bit for bit).  The scratch of a group is at most
 // STAGE_BYTES; from 2048^2 on that is less than two bins, whose passes fill the GPU anyway.
+// Plans that generate their tiles do so for as many bins of a group as fit STAGE_TAPS (at
+// 1024^2/1M/16 bins, generation and grid step of four bins at a time: tabulated kernels 0.82 ->
+// 0.56 and 0.96 -> 0.87 ms per apply, the network 1.03 -> 0.80 ms).
 // Measured, us per call: Phi^dagger Phi and an update at 256^2/20k/4 bins 200 -> 100, Phi at
 // 512x256/100k/3 bins 108 -> 60, Phi and Phi^dagger at 1024^2/2M/16 bins 1269 -> 1062 and
 // 2010 -> 1854.
 constexpr int STAGE_BLOCKS = 1216;                       // four waves of two blocks per SM
 constexpr int64_t STAGE_BYTES = (int64_t)512 << 20;
+constexpr int64_t STAGE_TAPS = (int64_t)1 << 30;
 
 PlanStage::~PlanStage() {
     for (Group& g : groups) {
         if (g.fft) wide_fft_destroy(g.fft);
-        if (g.gtg) wide_gtg_destroy(g.gtg);
+        for (Run& r : g.runs) wide_gtg_destroy(r.gtg);
         if (g.hfft) wide_fft_destroy(g.hfft);
         if (g.h) wide_h_destroy(g.h);
     }
@@ -128,43 +136,77 @@ PlanStage::~PlanStage() {
     cudaFree(hpatch);
 }
 
+static int64_t al256(int64_t x) { return (x + 255) & ~(int64_t)255; }
+// scratch of one bin: half transforms, grid, patches
+struct BinScratch {
+    int64_t ab, gx, pt;
+    explicit BinScratch(const rimo_plan* p)
+        : ab(al256((int64_t)2 * p->nx * p->ny * 8)), gx(al256((int64_t)p->gx * p->gy * 8)),
+          pt(al256((int64_t)std::max(1, p->max_tiles_bin) * p->PW * p->PW * 8)) {}
+    int64_t total() const { return ab + gx + pt; }
+};
+
+void stage_bins(rimo_plan* p, bool share_taps) {
+    int nb = 0;
+    for (int b = 0; b < p->P; ++b) nb += p->bins[b].t1 > p->bins[b].t0;
+    const int per_bin = std::max(1, p->nx * p->ny / 4096);
+    const int64_t most = std::min<int64_t>({(int64_t)nb, (STAGE_BLOCKS + per_bin - 1) / per_bin,
+                                            STAGE_BYTES / BinScratch(p).total()});
+    // groups of nearly equal size
+    const int64_t ng = most < 2 ? nb : (nb + most - 1) / most;
+    p->stage_each = ng > 0 ? (int)((nb + ng - 1) / ng) : 1;
+    // generated tiles: runs of a group's bins that share the tap scratch
+    p->tap_run.assign((size_t)nb, 1);
+    if (p->mode == RIMO_MODE_STORED_G) {
+        for (int i = 0; i < nb; ++i) p->tap_run[i] = i % p->stage_each == 0;
+    } else if (share_taps) {
+        int64_t sum = 0;
+        for (int i = 0; i < nb; ++i) {
+            p->tap_run[i] = i % p->stage_each == 0 || sum + p->block_bytes[i] > STAGE_TAPS;
+            sum = (p->tap_run[i] ? 0 : sum) + p->block_bytes[i];
+        }
+    }
+}
+
 void stage_plan(rimo_plan* p, cudaStream_t s) {
-    auto al = [](int64_t x) { return (x + 255) & ~(int64_t)255; };
+    if (p->stage_each < 2) return;
     std::vector<int> bins;
     for (int b = 0; b < p->P; ++b)
         if (p->bins[b].t1 > p->bins[b].t0) bins.push_back(b);
-    const int per_bin = std::max(1, p->nx * p->ny / 4096);
-    const int64_t ab = al((int64_t)2 * p->nx * p->ny * 8), gx = al((int64_t)p->gx * p->gy * 8);
-    const int64_t pt = al((int64_t)std::max(1, p->max_tiles_bin) * p->PW * p->PW * 8);
-    const int64_t most = std::min<int64_t>({(int64_t)bins.size(), (STAGE_BLOCKS + per_bin - 1) / per_bin,
-                                            STAGE_BYTES / (ab + gx + pt)});
-    if (most < 2) return;
-    // groups of nearly equal size
-    const int ng = (int)(((int64_t)bins.size() + most - 1) / most);
-    const int64_t each = ((int64_t)bins.size() + ng - 1) / ng;
+    const BinScratch sc(p);
+    const int64_t each = p->stage_each;
     auto* st = new PlanStage();
     p->stage = st;  // freed with the plan
-    if (cudaMalloc(&st->scratch, (size_t)(each * (ab + gx + pt))) != cudaSuccess) {
+    if (cudaMalloc(&st->scratch, (size_t)(each * sc.total())) != cudaSuccess) {
         cudaGetLastError();  // no room: one bin at a time
         st->scratch = nullptr;
         p->stage = nullptr;
         delete st;
         return;
     }
-    st->scratch_bytes = each * (ab + gx + pt);
+    st->scratch_bytes = each * sc.total();
     char* base = static_cast<char*>(st->scratch);
+    int runs = 0;
     for (size_t i = 0; i < bins.size(); i += (size_t)each) {
         PlanStage::Group g;
         for (size_t k = i; k < std::min(bins.size(), i + (size_t)each); ++k) {
-            char* q = base + (int64_t)(k - i) * (ab + gx + pt);
-            g.jobs.push_back(WideJob{p, bins[k], 0, reinterpret_cast<float2*>(q), reinterpret_cast<float2*>(q + ab),
-                                     reinterpret_cast<float2*>(q + ab + gx)});
+            char* q = base + (int64_t)(k - i) * sc.total();
+            g.jobs.push_back(WideJob{p, bins[k], 0, reinterpret_cast<float2*>(q), reinterpret_cast<float2*>(q + sc.ab),
+                                     reinterpret_cast<float2*>(q + sc.ab + sc.gx)});
         }
         st->groups.push_back(g);
         PlanStage::Group& h = st->groups.back();
         h.fft = wide_fft_create(h.jobs, {nullptr}, {nullptr}, s);
-        // (the counters are cleared at the start of every apply; there are at most P groups)
-        if (p->mode == RIMO_MODE_STORED_G) h.gtg = wide_gtg_create(h.jobs, p->d_counter + st->groups.size() - 1, s);
+        for (size_t k = 0; k < h.jobs.size(); ++k) {
+            if (!p->tap_run[i + k]) continue;
+            size_t e = k + 1;
+            while (e < h.jobs.size() && !p->tap_run[i + e]) ++e;
+            PlanStage::Run r{h.jobs[k].bin, h.jobs[e - 1].bin, nullptr};
+            // (the counters are cleared at the start of every apply; there are at most P runs)
+            r.gtg = wide_gtg_create(std::vector<WideJob>(h.jobs.begin() + (long)k, h.jobs.begin() + (long)e),
+                                    p->d_counter + runs++, s);
+            h.runs.push_back(r);
+        }
     }
     p->info.scratch_bytes += st->scratch_bytes;
 }
@@ -191,12 +233,14 @@ static void apply_group(rimo_plan* p, const PlanStage::Group& g, int mode, bool 
         prof_begin(p, ST_HAPPLY, s);
         wide_happly(g.h, s);
         prof_end(p, 1, s);
-    } else if (g.gtg) {
-        prof_begin(p, ST_GTG, s);
-        const int nl = wide_gtg(g.gtg, mode, y_in, y_out, s);
-        prof_end(p, nl, s);
     } else {
-        for (const WideJob& j : g.jobs) gtg(p, j.bin, mode, y_in, y_out, s, j.X, j.patch);
+        for (const PlanStage::Run& r : g.runs) {
+            // (its bins are neighbours but for empty ones: one range of visibilities)
+            generate(p, r.bin0, r.bin1, s);
+            prof_begin(p, ST_GTG, s);
+            const int nl = wide_gtg(r.gtg, mode, y_in, y_out, s);
+            prof_end(p, nl, s);
+        }
     }
     if (mode == 0) return;
     prof_begin(p, ST_INV_COLS, s);

@@ -623,8 +623,7 @@ static void (*gtg_kernel_for(int PW))(GtgArgs) {
 }
 
 template <int MODE>
-static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_out, cudaStream_t s, const float2* X,
-                    float2* patch) {
+static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_out, cudaStream_t s) {
     const auto& br = p->bins[bin];
     const int nu = br.t1 - br.t0;
     if (nu <= 0) return;
@@ -633,8 +632,8 @@ static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_o
     A.recs = p->d_recs + br.t0;
     A.nunits = nu;
     A.counter = p->d_counter + bin;  // zeroed at the start of every apply
-    A.X = X ? X : p->d_X;
-    A.patch = patch ? patch : p->d_patch;
+    A.X = p->d_X;
+    A.patch = p->d_patch;
     A.y_in = y_in;
     A.y_out = y_out;
     const GtgShape g = gtg_shape(p, p->PW, p->max_S, MODE, A);
@@ -768,10 +767,10 @@ int wide_gtg(const WideGtg* w, int mode, const float2* y_in, float2* y_out, cuda
 }
 
 void launch_gtg(const rimo_plan* p, int bin, int mode, const float2* y_in, float2* y_out,
-                cudaStream_t s, const float2* X, float2* patch) {
-    if (mode == 0) gtg_run<0>(p, bin, y_in, y_out, s, X, patch);
-    else if (mode == 1) gtg_run<1>(p, bin, y_in, y_out, s, X, patch);
-    else gtg_run<2>(p, bin, y_in, y_out, s, X, patch);
+                cudaStream_t s) {
+    if (mode == 0) gtg_run<0>(p, bin, y_in, y_out, s);
+    else if (mode == 1) gtg_run<1>(p, bin, y_in, y_out, s);
+    else gtg_run<2>(p, bin, y_in, y_out, s);
 }
 
 // ---------------------------------------------------------------------------

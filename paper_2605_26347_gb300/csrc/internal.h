@@ -174,8 +174,11 @@ struct rimo_plan {
     // kernel surrogate (mode RIMO_MODE_SURROGATE) or exact on-the-fly tiles (mode
     // RIMO_MODE_ONTHEFLY): tiles generated per bin at apply time
     struct rimo_surrogate* sur = nullptr;  // attached by rimo_plan_set_surrogate (not owned)
-    float2* d_sur_taps = nullptr;          // one bin's taps, laid out like its G block
+    float2* d_sur_taps = nullptr;          // the taps of one run of bins
     int64_t sur_taps_bytes = 0;
+    std::vector<float2*> gblock_host;      // address of every block (host copy of d_gblock_ptrs)
+    int stage_each = 1;                    // bins per group (see stage_plan)
+    std::vector<uint8_t> tap_run;          // per non-empty bin: 1 = starts a run (see stage_bins)
 
     // holographic matrices (Section 3.3), once rimo_build_holographic has run.  Each pair of
     // cells (c1, c2) of H_p = G_p^dagger G_p with |c2 - c1| <= H per axis is stored once, at
@@ -266,9 +269,8 @@ void launch_inv_rows(const rimo_plan* p, int bin, const float2* B, float2* out, 
                      int real_only, cudaStream_t s);
 // mode 0: degrid (y_out), 1: grid (y_in), 2: fused degrid + grid.  Modes 1 and 2 write the
 // accumulator patch of every active tile of the bin to p->d_patch.
-// X, patch: the bin's forward grid and patches (null: the plan's d_X and d_patch)
 void launch_gtg(const rimo_plan* p, int bin, int mode, const float2* y_in, float2* y_out,
-                cudaStream_t s, const float2* X = nullptr, float2* patch = nullptr);
+                cudaStream_t s);
 void launch_gbuild(const rimo_plan* p, cudaStream_t s);
 // exact tiles of the sorted visibilities [v0, v0 + n) into their block (the on-the-fly mode's
 // scratch), with the tap bounds of the fixed-point grid step
@@ -324,10 +326,15 @@ int wide_gtg(const WideGtg* w, int mode, const float2* y_in, float2* y_out, cuda
 
 // The bins of one plan in groups that share a launch per pass (see stage_plan in apply.cu).
 struct PlanStage {
+    // bins whose tiles are there together: one grid-step launch
+    struct Run {
+        int bin0, bin1;
+        WideGtg* gtg;
+    };
     struct Group {
         std::vector<WideJob> jobs;
         WideFft* fft = nullptr;
-        WideGtg* gtg = nullptr;   // stored G; else the bins' grid steps follow their tile generation
+        std::vector<Run> runs;
         WideFft* hfft = nullptr;  // once H is built: the passes with its patches ...
         WideH* h = nullptr;       // ... and its apply
     };
@@ -337,6 +344,9 @@ struct PlanStage {
     int64_t scratch_bytes = 0;
     ~PlanStage();
 };
+// Bins of a group (1: no groups) and the runs of bins that share the tap scratch, from the
+// plan's sizes and blocks, into p->stage_each and p->tap_run.
+void stage_bins(rimo_plan* p, bool share_taps);
 // Sets p->stage where it pays and its scratch can be had (at the end of plan creation).
 void stage_plan(rimo_plan* p, cudaStream_t s);
 
@@ -356,9 +366,9 @@ void launch_image_bound(const rimo_plan* p, const float2* x, cudaStream_t s);
 // Z_p of bin `bin` at every pixel into out (ny x nx)
 void launch_zlayer(const rimo_plan* p, int bin, float2* out, cudaStream_t s);
 void launch_y_bound(const rimo_plan* p, const float2* y, cudaStream_t s);
-// Kernel surrogate: fill d_sur_taps with the MLP's tiles of bin `bin` (and the tap bounds
+// Kernel surrogate: the MLP's tiles of the sorted visibilities [v0, v0 + n) into their blocks (and the tap bounds
 // of the fixed-point grid step); reset_surrogate_bounds clears those bounds for an apply.
-int surrogate_generate(rimo_plan* p, int bin, cudaStream_t s);  // returns kernel launches
+int surrogate_generate(rimo_plan* p, int64_t v0, int64_t n, cudaStream_t s);  // returns kernel launches
 void reset_surrogate_bounds(rimo_plan* p, cudaStream_t s);
 // Holographic apply of bin `bin` (forward grid in d_X -> output patches in d_hpatch).
 void launch_happly(const rimo_plan* p, int bin, cudaStream_t s);

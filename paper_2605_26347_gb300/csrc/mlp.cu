@@ -639,7 +639,7 @@ __global__ void pack_w3g_kernel(const float* __restrict__ P, bf16* __restrict__ 
 
 struct GenArgs {
     const VisMeta* meta;
-    float2* taps;
+    float2* const* gblk;
     const float* phiu;
     const float* phiv;
     const float* wr;
@@ -669,7 +669,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 1) sur_gen_kernel(GenArgs A) {
     float* sb2 = sb1 + 128;
     float* sb3 = sb2 + 128;
     float* sx = sb3 + GEN_N3;
-    int64_t* soff = reinterpret_cast<int64_t*>(sx + 384);
+    float2** sdst = reinterpret_cast<float2**>(sx + 384);  // each row's tile
     __shared__ float swt[128];  // data weight of each row
     __shared__ float s_tsum[GEN_WG][128];  // per warp group: partial tap sums of each row
     __shared__ __align__(8) uint64_t bar;
@@ -712,7 +712,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 1) sur_gen_kernel(GenArgs A) {
     const int ntile = (A.n + 127) / 128;
     // the next tile's inputs are loaded (raw) while this tile computes
     float in_u = 0.f, in_v = 0.f, in_w = 0.f, in_wt = 1.f;
-    int64_t in_off = 0;
+    float2* in_dst = nullptr;
     auto load_inputs = [&](int t) {
         if (tid < 128 && t < ntile) {
             const int j = t * 128 + tid < A.n ? t * 128 + tid : A.n - 1;
@@ -720,7 +720,8 @@ __global__ void __launch_bounds__(GEN_THREADS, 1) sur_gen_kernel(GenArgs A) {
             in_u = __ldg(A.phiu + k);
             in_v = __ldg(A.phiv + k);
             in_w = __ldg(A.wr + k);
-            in_off = A.meta[k].off;
+            const VisMeta mt = A.meta[k];
+            in_dst = A.gblk[mt.pos >> 24] + mt.off;
             in_wt = A.wt ? __ldg(A.wt + k) : 1.f;
         }
     };
@@ -731,7 +732,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 1) sur_gen_kernel(GenArgs A) {
             sx[3 * tid + 0] = 2.f * in_u - 1.f;
             sx[3 * tid + 1] = 2.f * in_v - 1.f;
             sx[3 * tid + 2] = in_w * A.inv_w;
-            soff[tid] = in_off;
+            sdst[tid] = in_dst;
             swt[tid] = in_wt;
         }
         load_inputs(tile + gridDim.x);
@@ -853,7 +854,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 1) sur_gen_kernel(GenArgs A) {
                     const int row = 4 * it + (lane >> 3), pc = lane & 7;
                     const int rg = 32 * (warp & 3) + row;
                     if (pc < npc && base + rg < A.n)
-                        *reinterpret_cast<float4*>(A.taps + soff[rg] + q0 + 2 * pc) = stage[row * 8 + (pc ^ (row & 7))];
+                        *reinterpret_cast<float4*>(sdst[rg] + q0 + 2 * pc) = stage[row * 8 + (pc ^ (row & 7))];
                 }
                 __syncwarp();
             }
@@ -896,18 +897,17 @@ void reset_surrogate_bounds(rimo_plan* p, cudaStream_t s) {
         pack_w3g_kernel<<<(GEN_N3 * MLP_H + 255) / 256, 256, 0, s>>>(p->sur->mlp.P, p->sur->W3g);
 }
 
-int surrogate_generate(rimo_plan* p, int bin, cudaStream_t s) {
+int surrogate_generate(rimo_plan* p, int64_t v0, int64_t n, cudaStream_t s) {
     rimo_surrogate* sur = p->sur;
     const float ws = sur->w_scale > 0.f ? sur->w_scale : (p->info.wr_max > 0 ? (float)p->info.wr_max : 1.f);
-    const int64_t vb = p->bins[bin].vb, n = p->bins[bin].ve - vb;
     if (n <= 0) return 0;
     GenArgs A;
     A.meta = p->d_meta;
-    A.taps = p->d_sur_taps;
+    A.gblk = p->d_gblock_ptrs;
     A.phiu = p->d_phiu;
     A.phiv = p->d_phiv;
     A.wr = p->d_wr;
-    A.v0 = vb;
+    A.v0 = v0;
     A.n = (int)n;
     A.inv_w = 1.f / ws;
     A.P = sur->mlp.P;

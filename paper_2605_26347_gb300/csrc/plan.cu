@@ -614,15 +614,36 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
     p->d_phiu = upload(p, pu_s, s);
     p->d_phiv = upload(p, pv_s, s);
     int64_t gbytes = 0;
+    stage_bins(p, true);
     std::vector<float2*> ptrs;
     if (generated) {
-        // no stored G: every bin's (single) block points at one scratch that is refilled
-        // for each bin of each apply
-        int64_t mx = 16;
-        for (int64_t bb : p->block_bytes) mx = std::max(mx, bb);
-        p->d_sur_taps = (float2*)dev_alloc(p, (size_t)mx);
+        // no stored G: every bin's (single) block points into one scratch that is refilled for
+        // each run of bins of each apply
+        std::vector<int64_t> at;
+        auto place = [&]() {  // the blocks' offsets; the largest run's bytes
+            int64_t mx = 16, off = 0;
+            at.clear();
+            for (size_t i = 0; i < p->block_bytes.size(); ++i) {
+                if (p->tap_run[i]) off = 0;
+                at.push_back(off);
+                off += p->block_bytes[i];
+                mx = std::max(mx, off);
+            }
+            return mx;
+        };
+        int64_t mx = place();
+        void* taps = nullptr;
+        if (p->stage_each > 1 && cudaMalloc(&taps, (size_t)mx) != cudaSuccess) {
+            cudaGetLastError();  // no room for several bins: one at a time
+            taps = nullptr;
+            stage_bins(p, false);
+            mx = place();
+        }
+        if (taps) p->owned.push_back(taps);
+        else taps = dev_alloc(p, (size_t)mx);
+        p->d_sur_taps = (float2*)taps;
         p->sur_taps_bytes = mx;
-        for (size_t i = 0; i < p->block_bytes.size(); ++i) ptrs.push_back(p->d_sur_taps);
+        for (int64_t o : at) ptrs.push_back(p->d_sur_taps + o / (int64_t)sizeof(float2));
     } else {
         for (int64_t bb : p->block_bytes) {
             p->d_gblocks.push_back((float2*)dev_alloc(p, (size_t)std::max<int64_t>(bb, 16)));
@@ -630,6 +651,7 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
         }
         ptrs = p->d_gblocks;
     }
+    p->gblock_host = ptrs;
     p->d_gblock_ptrs = upload(p, ptrs, s);
     const size_t grid_elems = (size_t)gx * gy;
     p->d_X = (float2*)dev_alloc(p, grid_elems * sizeof(float2));
@@ -871,7 +893,8 @@ rimo_status rimo_plan_get_tiles(rimo_plan_t p, const int64_t* idx, int64_t n, in
             int b = p->bins_user[idx[q]];
             if (generated && b != have_bin) {  // tiles of generated plans: this bin, as an apply makes them
                 RIMO_CUDA(cudaStreamSynchronize(s));  // earlier copies out of the scratch are done
-                if (p->mode == RIMO_MODE_SURROGATE) surrogate_generate(p, b, s);
+                if (p->mode == RIMO_MODE_SURROGATE)
+                    surrogate_generate(p, p->bins[b].vb, p->bins[b].ve - p->bins[b].vb, s);
                 else launch_gbuild_range(p, p->bins[b].vb, p->bins[b].ve - p->bins[b].vb, s);
                 have_bin = b;
             }
@@ -884,8 +907,7 @@ rimo_status rimo_plan_get_tiles(rimo_plan_t p, const int64_t* idx, int64_t n, in
             g0[q] = tu * p->TS + du;
             h0[q] = tv * p->TS + dv;
             S[q] = Sq;
-            // generated plans: every block is the one tap scratch
-            const float2* src = generated ? p->d_sur_taps : p->d_gblocks.at((size_t)blk);
+            const float2* src = p->gblock_host.at((size_t)blk);  // (generated plans: in the tap scratch)
             RIMO_CUDA(cudaMemcpyAsync(taps + q * 361, src + m.off,
                                       (size_t)Sq * Sq * sizeof(float2), cudaMemcpyDeviceToHost, s));
         }

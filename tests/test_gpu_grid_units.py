@@ -47,7 +47,9 @@ def test_units_of_every_size_and_tile_side(m, kb, cap, tile, spread):
 ])
 def test_bins_in_groups_equal_one_bin_at_a_time(nx, ny, m, bins, kw):
     """Plans of small images run their bins in groups; a call that selects every bin by a mask
-    takes them one at a time: the same sums in the same order, bit for bit."""
+    takes them one at a time: the same sums in the same order, bit for bit with stored G.  With
+    tiles generated per group the fixed-point scale comes from the group's tap bound, which may
+    be a power of two above a bin's: 2^-46 of the bound, far below an FP32 rounding."""
     import synth
     import torch
 
@@ -61,7 +63,10 @@ def test_bins_in_groups_equal_one_bin_at_a_time(nx, ny, m, bins, kw):
     for real in (False, True):
         a = plan.phi_adj_phi(x, real_part_only=real)
         b = plan.phi_adj_phi_bins(x, np.ones(bins, np.uint8), real_part_only=real)
-        assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
+        if kw.get("mode") == 4:
+            assert rel(to_host(a), to_host(b)) < 1e-7
+        else:
+            assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
     # Phi^dagger Phi x = Phi^dagger (Phi x), the two halves in groups as well
     c = plan.phi_adj(plan.phi(x))
     a = plan.phi_adj_phi(x)
