@@ -28,6 +28,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "phase.cuh"
 
 namespace rimo {
 
@@ -379,17 +380,15 @@ __device__ __forceinline__ int out_slot(int m) {
 
 // e^{-2 pi i w dn} from the double-float phase w * dn, reduced modulo 1 before sincos.
 // The product and reduction keep ~48 significant bits (error-free FMA product), which is
-// the FP64-accurate w-phase argument; only the final sincospi is single precision.
+// the FP64-accurate w-phase argument; only the final sine and cosine are single precision.
 __device__ __forceinline__ float2 wphase(float w_hi, float w_lo, float2 d) {
     float p = w_hi * d.x;
     float e = fmaf(w_hi, d.x, -p);
     e = fmaf(w_hi, d.y, e);
     e = fmaf(w_lo, d.x, e);
     float k = rintf(p);
-    float r = (p - k) + e;
-    float s, c;
-    sincospif(2.0f * r, &s, &c);
-    return make_float2(c, -s);
+    const float2 cs = cis_turn((p - k) + e);
+    return make_float2(cs.x, -cs.y);
 }
 
 struct ZArgs {

@@ -6,6 +6,7 @@
 #include <cstring>
 
 #include "internal.h"
+#include "phase.cuh"
 
 namespace rimo {
 
@@ -65,10 +66,10 @@ constexpr int BUILD_WARPS = 8;
 // Chirp sample c(a', b') of the folded grid (a', b' in [0, L/2]) for residual w
 __device__ __forceinline__ float2 chirp_at(const float* s_dn, const float* s_tx, const float* s_ty, int Q,
                                           int a, int b, float w, int literal) {
-    float sn, cs;
-    sincospif(2.f * w * s_dn[a * Q + b], &sn, &cs);
+    const float turns = w * s_dn[a * Q + b];
+    const float2 cs = cis_turn(turns - rintf(turns));
     const float tt = s_tx[a] * s_ty[b];
-    return literal ? make_float2(tt * cs, -tt * sn) : make_float2(1.f + tt * (cs - 1.f), -tt * sn);
+    return literal ? make_float2(tt * cs.x, -tt * cs.y) : make_float2(1.f + tt * (cs.x - 1.f), -tt * cs.y);
 }
 
 // The folded residual w-kernel K(t_x, t_y; w) for t in [0, hq)^2 into Kq[t_x][t_y] (row
