@@ -949,6 +949,60 @@ __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 
     }
 }
 
+// The same pass with the bins of a group side by side: a block of 4096 / N slots takes
+// 4096 / N / BP image rows, BP bins of each at a time (BP = 1 << lb slots), whose products meet in
+// shared memory and are summed there in the order of the bins, so the sums are those of
+// inv_rows_kernel bit for bit.  For launches whose blocks, each with its bins one after the
+// other, would not fill the GPU (N <= 512; four bins of 256^2 22.6 -> 15.0 us, of 512^2 24.8 ->
+// 15.8 us; at 1024^2, with four rows per block, it was slower: 0.164 -> 0.172 ms per apply).
+template <int N, int RG>
+__global__ void __launch_bounds__(RG * N / 8, 2)
+    inv_rows_bins_kernel(const JobTable<RowsJob> tab, const int* __restrict__ group, int64_t img, int ny,
+                         int accumulate, int real_only, int lb, const float2* __restrict__ tws) {
+    constexpr int L = 2 * N, T = L / 16, SR = L + L / 16, THREADS = RG * N / 8;
+    extern __shared__ float2 smem[];
+    const int g = threadIdx.x / T, t = threadIdx.x % T;
+    float2* sm = smem + g * SR;
+    const int BP = 1 << lb, rows = RG >> lb, per = ny / rows;
+    const int c = (int)blockIdx.x / per, row0 = ((int)blockIdx.x - c * per) * rows;
+    const int j0 = __ldg(group + c), j1 = __ldg(group + c + 1);
+    const int i = row0 + (g >> lb), ic = i - ny / 2;
+    float2* __restrict__ out = at_image<true>(tab.jobs[j0].out, img) + (size_t)row0 * N;
+    for (int jc = j0; jc < j1; jc += BP) {
+        const int nb = min(BP, j1 - jc);
+        const bool on = (g & (BP - 1)) < nb;
+        const RowsJob& J = tab.jobs[on ? jc + (g & (BP - 1)) : j0];
+        const RowSel& sel = J.sel;
+        const float2* __restrict__ in = J.in + (size_t)i * L;
+        float2 v[16];
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            const int tr = (t + T * m) >> sel.shift;
+            const bool keep = on && (!sel.on || ((sel.bits[tr >> 5] >> (tr & 31)) & 1u));
+            v[m] = keep ? __ldg(&in[t + T * m]) : make_float2(0.f, 0.f);
+        }
+        fft_n<L, true>(v, sm, t, tws);
+        const ZArgs z = J.z;
+#pragma unroll
+        for (int m = 0; m < 16; ++m) {
+            const int k = t + T * m;
+            if (k >= N / 2 && k < 3 * N / 2) continue;  // outside the crop
+            const int jc2 = k < N / 2 ? k : k - L;
+            sm[jc2 + N / 2] = cmulc(v[out_slot<L>(m)], z_factor(z, i, jc2 + N / 2, ic, jc2));
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < rows * N; e += THREADS) {
+            const float2* p = smem + (size_t)((e / N) << lb) * SR + e % N;
+            float2 val = p[0];
+            if (accumulate || jc > j0) val = cadd(val, out[e]);
+            for (int s = 1; s < nb; ++s) val = cadd(p[s * SR], val);
+            if (real_only) val.y = 0.f;
+            out[e] = val;
+        }
+        __syncthreads();  // the next bins' first stage rewrites the slots
+    }
+}
+
 // ----------------------------------------------------------------------------- Z_p
 // Z_p(i, j) of every pixel, as the row passes apply it (for checking the w-phase).
 __global__ void __launch_bounds__(256) zlayer_kernel(ZArgs z, int nx, int ny, float2* __restrict__ out) {
@@ -1233,6 +1287,7 @@ static void inv_rows(const rimo_plan* p, int bin, const float2* B, float2* out, 
 // The transform passes of a stage-batched apply: one launch per pass over every job.
 struct WideFft {
     int nx = 0, ny = 0, gx = 0, TS = 0, ngroups = 0;
+    int group_max = 0;     // jobs of the largest group
     const float2* tws_x = nullptr;
     const float2* tws_y = nullptr;
     const float2* tws32 = nullptr;
@@ -1289,6 +1344,7 @@ WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<con
             ri.push_back(rows_job(p, j.bin, j.AB, out[j.group], is));
             grp[j.group + 1]++;
         }
+        for (int c = 0; c < w->ngroups; ++c) w->group_max = std::max(w->group_max, grp[c + 1]);
         for (int c = 0; c < w->ngroups; ++c) grp[c + 1] += grp[c];
         std::vector<char> blob;
         std::vector<std::pair<WideFft::Pass*, std::pair<size_t, size_t>>> at;
@@ -1353,6 +1409,19 @@ static void wide_cols_inv(const WideFft* w, cudaStream_t s) {
 }
 template <int N>
 static void wide_rows_inv(const WideFft* w, int64_t img, int acc, int real_only, cudaStream_t s) {
+    // under two waves of 304 blocks, several bins side by side (more, smaller blocks' worth of rows)
+    if constexpr (N <= 512) {
+        constexpr int RG = rows_per_block<N>();
+        int lb = 0;
+        while ((RG >> (lb + 1)) >= 1 && (1 << lb) < w->group_max && (w->rows_inv.blocks << lb) < 608) ++lb;
+        if (lb > 0) {
+            const size_t sm = (size_t)RG * (2 * N + N / 8) * sizeof(float2);
+            set_smem(inv_rows_bins_kernel<N, RG>, sm);
+            inv_rows_bins_kernel<N, RG><<<w->rows_inv.blocks << lb, RG * N / 8, sm, s>>>(
+                table_of<RowsJob>(w->rows_inv), w->group, img, w->ny, acc, real_only, lb, w->tws_x);
+            return;
+        }
+    }
     run_inv_rows<N, true>(no_job<RowsJob>(), table_of<RowsJob>(w->rows_inv), w->group, img, w->rows_inv.blocks, w->ny,
                           acc, real_only, w->tws_x, s);
 }
