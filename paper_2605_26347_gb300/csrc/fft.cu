@@ -767,86 +767,57 @@ __global__ void __launch_bounds__(256, 2)
 // patch reaches are never written and read as zero by the inverse transform.
 struct FoldArgs {
     const float2* patch;   // [slot][PW * PW]
-    const int2* slotbox;   // [tu * ntv + tv] -> (slot or -1, the slot's box: cells outside it
-                           //   are zero and not stored), or null: `slot` with whole patches
-    const int* slot;       // [tu * ntv + tv] -> slot or -1 (this bin)
-    const int* tiles;      // needed tiles of this bin, tu * ntv + tv
+    const FoldRec* recs;   // needed tiles of this bin
     float2* Xh;            // [gx][gy]
-    int ntu, ntv, TS, H, PW, gy;
+    int PW, gy;
 };
 
-// TSC: the tile side (32 or 64) as a compile-time constant, so the cell indexing is shifts.
-// A thread folds pairs of cells (16-byte loads and stores): the grid step writes its boxes
-// widened to whole pairs of columns (its added cells hold zeros), so a pair is in a box or not
-// as a whole.  With one cell per load and 64-bit patch offsets per cell the kernel was bound by
-// its index arithmetic (149 instructions per cell and warp, the integer pipe 70 % busy): four
-// bins of 1024^2/2M 98 -> 67 us (4.0 TB/s of boxes and tiles), 4096^2/24M inverse cols + fold
-// 6.71 -> 6.31 ms per apply.
-template <bool TABLE, int TSC>
+// TS: the tile side (32 or 64) as a compile-time constant, so the cell indexing is shifts.
+// A thread folds pairs of cells of one pair of columns (16-byte loads and stores): the grid step
+// writes its boxes widened to whole pairs of columns (the added cells hold zeros), so a pair is
+// in a box or not as a whole.  The sources' places and ranges come from the tile's record: with
+// slots and boxes looked up and clipped here, one cell per load and 64-bit offsets per cell the
+// kernel was bound by its index arithmetic.  Measured, one cell per load / pairs / pairs and
+// records: four bins of 1024^2/2M 98 / 67 / 55 us (4.9 TB/s of boxes and tiles).
+template <bool TABLE, int TS>
 __global__ void __launch_bounds__(256) fold_kernel(const __grid_constant__ FoldArgs one, const JobTable<FoldArgs> tab) {
     int bk;
     const FoldArgs& F = block_job<TABLE>(one, tab, bk);
-    constexpr int TS = TSC, ROW = TS / 2;  // pairs per row
-    const int tile = F.tiles[bk];
-    const int tu = tile / F.ntv, tv = tile - tu * F.ntv;
-    const int tu1 = tu == 0 ? F.ntu - 1 : tu - 1, tv1 = tv == 0 ? F.ntv - 1 : tv - 1;
-    const int PW = F.PW, H = F.H;
-    const uint32_t whole = box_pack(0, PW, 0, PW);
-    // the box of tile t's patch in this tile's cells, its cells (a, b) being the patch's
-    // (a + oa, b + ob): rows [a, a + na), columns [b, b + nb) (nothing without a patch), and
-    // the patch's address moved by that offset
+    constexpr int ROW = TS / 2, STEP = 256 / ROW;  // pairs per row, rows per pass of the block
+    const int4 off = __ldg(reinterpret_cast<const int4*>(F.recs + bk));
+    const uint4 rng = __ldg(reinterpret_cast<const uint4*>(F.recs + bk) + 1);
+    const int a = threadIdx.x / ROW, b = 2 * (threadIdx.x % ROW), PW = F.PW;
+    // a source's first row and rows in this pair of columns, and the address of its row 0 there
     struct Src {
         const float2* p;
-        int a, na, b, nb;
+        int a0, na;
     };
-    auto src = [&](int t, int oa, int ob, int ca, int cb) {
-        Src r;
-        int sl;
-        uint32_t x = whole;
-        if (F.slotbox) {
-            const int2 q = F.slotbox[t];
-            sl = q.x;
-            x = (uint32_t)q.y;
-        } else {
-            sl = F.slot[t];
-        }
-        if (sl < 0) x = 0u;
-        r.p = F.patch + (size_t)max(sl, 0) * PW * PW + oa * PW + ob;
-        // (a box reaches at most ca rows and cb columns into this tile)
-        r.a = max((int)(x & 255u) - oa, 0);
-        r.na = max(0, min((int)((x >> 8) & 255u) - oa, ca) - r.a);
-        r.b = max((int)((x >> 16) & 254u) - ob, 0);
-        r.nb = max(0, min((int)(((x >> 24) + 1u) & 254u) - ob, cb) - r.b);
-        return r;
+    auto src = [&](int o, uint32_t x) {
+        const int a0 = (int)(x & 127u), a1 = (int)((x >> 7) & 127u), b0 = (int)((x >> 14) & 127u);
+        const int b1 = (int)((x >> 21) & 127u);
+        return Src{F.patch + 2 * (int64_t)o + b, a0, b >= b0 && b < b1 ? a1 - a0 : 0};
     };
-    const Src s00 = src(tu * F.ntv + tv, 0, 0, TS, TS), s10 = src(tu1 * F.ntv + tv, TS, 0, H, TS);
-    const Src s01 = src(tu * F.ntv + tv1, 0, TS, TS, H), s11 = src(tu1 * F.ntv + tv1, TS, TS, H, H);
-    float2* __restrict__ Xh = F.Xh + (size_t)(tu * TS) * F.gy + tv * TS;
-    // one pair of the tile: the sources summed in a fixed order
-    auto pair = [&](int a, int b) {
-        const int off = a * PW + b;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        auto get = [&](const Src& q, float4& x) {
-            const bool in = (unsigned)(a - q.a) < (unsigned)q.na && (unsigned)(b - q.b) < (unsigned)q.nb;
-            x = in ? __ldg(reinterpret_cast<const float4*>(q.p + off)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            return in;
-        };
-        float4 x00, x10, x01, x11;
-        get(s00, x00);
-        const bool k10 = get(s10, x10), k01 = get(s01, x01), k11 = get(s11, x11);
-        v = x00;
+    const Src s00 = src(off.x, rng.x), s10 = src(off.y, rng.y), s01 = src(off.z, rng.z), s11 = src(off.w, rng.w);
+    const int tu = (int)(rng.x >> 28 | (rng.y >> 28) << 4), tv = (int)(rng.z >> 28 | (rng.w >> 28) << 4);
+    float2* __restrict__ Xh = F.Xh + (size_t)(tu * TS + a) * F.gy + tv * TS + b;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+    for (int r = 0; r < TS; r += STEP) {
+        // the sources' pairs, then their sum in a fixed order
+        bool k00 = (unsigned)(a + r - s00.a0) < (unsigned)s00.na, k10 = (unsigned)(a + r - s10.a0) < (unsigned)s10.na;
+        bool k01 = (unsigned)(a + r - s01.a0) < (unsigned)s01.na, k11 = (unsigned)(a + r - s11.a0) < (unsigned)s11.na;
+        const int o = (a + r) * PW;
+        float4 v = k00 ? __ldg(reinterpret_cast<const float4*>(s00.p + o)) : zero;
+        const float4 x10 = k10 ? __ldg(reinterpret_cast<const float4*>(s10.p + o)) : zero;
+        const float4 x01 = k01 ? __ldg(reinterpret_cast<const float4*>(s01.p + o)) : zero;
+        const float4 x11 = k11 ? __ldg(reinterpret_cast<const float4*>(s11.p + o)) : zero;
         auto add = [&](bool k, const float4& x) {
             if (k) v = make_float4(v.x + x.x, v.y + x.y, v.z + x.z, v.w + x.w);
         };
         add(k10, x10);
         add(k01, x01);
         add(k11, x11);
-        return v;
-    };
-#pragma unroll 2
-    for (int e = threadIdx.x; e < TS * ROW; e += 256) {
-        const int a = e / ROW, b = 2 * (e % ROW);
-        *reinterpret_cast<float4*>(Xh + (size_t)a * F.gy + b) = pair(a, b);
+        *reinterpret_cast<float4*>(Xh + (size_t)r * F.gy) = v;
     }
 }
 
@@ -1137,22 +1108,13 @@ static ColsJob cols_job(const rimo_plan* p, int bin, const float2* in, float2* o
     J.sel = sel;
     return J;
 }
-// grid-step patches (one per active tile, merged) or holographic-apply patches (one per
-// needed tile): both cover [tile origin, + PW) on each axis
-// the grid step's patches (slots and boxes from the plan) or, with `hslot`, the holographic
-// apply's whole patches
-static FoldArgs fold_args(const rimo_plan* p, int bin, const float2* patch, const int* hslot, float2* Xh) {
-    const int ntu = p->gx / p->TS, ntv = p->gy / p->TS;
+// the grid step's patches (one per active tile, merged, over their boxes) or, with `holo`, the
+// holographic apply's (one per needed tile, whole): both cover [tile origin, + PW) on each axis
+static FoldArgs fold_args(const rimo_plan* p, int bin, const float2* patch, bool holo, float2* Xh) {
     FoldArgs F;
     F.patch = patch;
-    F.slotbox = hslot ? nullptr : p->d_slot + (size_t)bin * ntu * ntv;
-    F.slot = hslot ? hslot + (size_t)bin * ntu * ntv : nullptr;
-    F.tiles = p->d_need_list + p->bins[bin].n0;
+    F.recs = (holo ? p->d_hfold : p->d_fold) + p->bins[bin].n0;
     F.Xh = Xh;
-    F.ntu = ntu;
-    F.ntv = ntv;
-    F.TS = p->TS;
-    F.H = p->H;
     F.PW = p->PW;
     F.gy = p->gy;
     return F;
@@ -1269,7 +1231,7 @@ static void fwd_cols(const rimo_plan* p, int bin, const float2* At, float2* X, c
 template <int N>
 static void inv_cols(const rimo_plan* p, int bin, bool holo, float2* B, cudaStream_t s) {
     const auto& br = p->bins[bin];
-    run_fold<false>(fold_args(p, bin, holo ? p->d_hpatch : p->d_patch, holo ? p->d_hslot : nullptr, p->d_X),
+    run_fold<false>(fold_args(p, bin, holo ? p->d_hpatch : p->d_patch, holo, p->d_X),
                     no_table<FoldArgs>(), br.n1 - br.n0, p->TS, s);
     const RowSel sel = inv_sel(p, bin);
     run_inv_cols<N, false>(cols_job(p, bin, p->d_X, B, sel), no_table<ColsJob>(),
@@ -1337,7 +1299,7 @@ WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<con
             frf.push_back(frf.back() + p->ny / rb);
             cf.push_back(cols_job(p, j.bin, j.AB, j.X, fs));
             fcf.push_back(fcf.back() + sel_blocks(p, j.bin, fs, cb));
-            fo.push_back(fold_args(p, j.bin, j.patch, holographic ? p->d_hslot : nullptr, j.X));
+            fo.push_back(fold_args(p, j.bin, j.patch, holographic, j.X));
             ffo.push_back(ffo.back() + (p->bins[j.bin].n1 - p->bins[j.bin].n0));
             ci.push_back(cols_job(p, j.bin, j.X, j.AB, is));
             fci.push_back(fci.back() + sel_blocks(p, j.bin, is, cb));

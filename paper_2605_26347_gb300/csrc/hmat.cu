@@ -816,7 +816,7 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
     std::vector<int32_t> hslot((size_t)P * ntile, -1);
     for (int b = 0; b < P; ++b)
         for (int k = p->bins[b].n0; k < p->bins[b].n1; ++k) hslot[(size_t)b * ntile + p->need_host[k]] = k - p->bins[b].n0;
-    p->d_hslot = upload_vec(p, hslot, s);
+    p->d_hfold = upload_vec(p, fold_records(p, hslot, true), s);
     p->d_hbits.assign(P, nullptr);
     p->d_hoff.assign(P, nullptr);
     p->d_hval.assign(P, nullptr);

@@ -92,6 +92,17 @@ __host__ __device__ inline int box_c0(uint32_t box) { return (int)((box >> 16) &
 __host__ __device__ inline int box_pairs(uint32_t box) { return ((int)(box >> 24) + 1 - box_c0(box)) >> 1; }
 static_assert(sizeof(UnitRec) == 64, "UnitRec must stay 64 bytes");
 
+// One needed tile as the fold reads it: per source patch - the tile's own, those of the tile
+// before it along u, along v and both - the tile's first cell within the patches, in pairs of
+// cells, and the part of the tile that the patch's box (widened to pairs of columns) covers:
+// rows [a0, a1), columns [b0, b1) as a0 | a1 << 7 | b0 << 14 | b1 << 21, empty without a patch.
+// The top four bits hold the tile's place: tu in those of rng[0] and rng[1], tv in rng[2], rng[3].
+struct alignas(16) FoldRec {
+    int32_t off[4];
+    uint32_t rng[4];
+};
+static_assert(sizeof(FoldRec) == 32, "FoldRec must stay 32 bytes");
+
 struct BinRange {
     int64_t vb = 0, ve = 0;       // visibilities of the bin in sorted order
     int32_t t0 = 0, t1 = 0;       // work units of the bin: tiles_host[t0 .. t1) (patch slots 0 ..)
@@ -152,8 +163,7 @@ struct rimo_plan {
     float* d_phiv = nullptr;
     float2* d_X = nullptr;     // forward grid   (gx rows u, gy cols v)
     float2* d_patch = nullptr; // gridded accumulator patch of every active tile of one bin
-    int2* d_slot = nullptr;    // [bin][tu][tv] -> (index of the tile's patch in d_patch, or -1;
-                               //   the box of that patch, TileDesc::box)
+    rimo::FoldRec* d_fold = nullptr;  // per needed tile (as d_need_list): the patches it sums
     uint8_t* d_need = nullptr; // [bin][tu][tv] != 0: some active patch of the bin reads the tile
     int32_t* d_need_list = nullptr;  // per bin: the needed tiles as tu * ntv + tv
     int32_t* d_counter = nullptr;  // per-bin dynamic tile schedulers (reset at each apply)
@@ -195,7 +205,7 @@ struct rimo_plan {
     std::vector<uint32_t*> d_hbits;       // per bin: [needed tile][TS*TS/32] covered cells
     std::vector<int64_t*> d_hoff;         // per bin: [needed tile + 1] first owner of the tile
     std::vector<std::vector<int64_t>> hoff_host;
-    int32_t* d_hslot = nullptr;           // [bin][tile] -> needed-tile index in the bin, or -1
+    rimo::FoldRec* d_hfold = nullptr;     // per needed tile: the holographic patches it sums
     float2* d_hpatch = nullptr;           // H-apply output patches of one bin [needed tile][PW*PW]
     int32_t* d_hent = nullptr;            // entry table (type << 16 | a << 8 | |b|)
     rimo::PlanStage* stage = nullptr;     // groups of bins that share launches, or null
@@ -258,6 +268,10 @@ constexpr int FX_MAX_UNIT = 32768;  // visibilities per work unit (lo word range
 // Bracket a group of `launches` kernel launches of one stage on stream s (no-op when off).
 void prof_begin(rimo_plan* p, int stage, cudaStream_t s);
 void prof_end(rimo_plan* p, int launches, cudaStream_t s);
+
+// The fold's records of every bin's needed tiles, from the patch slot of each tile ([bin][tile],
+// or -1) and the box of each unit (null: whole patches).
+std::vector<FoldRec> fold_records(const rimo_plan* p, const std::vector<int32_t>& slot, bool whole);
 
 // Kernel launchers (defined in the .cu files).
 void launch_fwd_rows(const rimo_plan* p, int bin, const float2* x, float2* At, cudaStream_t s);
