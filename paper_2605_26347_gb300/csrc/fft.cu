@@ -493,6 +493,10 @@ __device__ __forceinline__ float2 dsmem_ld2(uint32_t addr) {
 // m >= 12 (c = t + T m - L); the other slots are zero.  Inverse: of the L outputs only
 // c mod L with c in [-N/2, N/2) (the crop) are kept.
 
+// The thread slots m of the kept (or non-zero) half: m = 0 .. 3 and 12 .. 15, known at compile
+// time, so that a pruned last stage and the staging skip the others.
+__host__ __device__ constexpr int kept_slot(int q) { return q < 4 ? q : q + 8; }
+
 // Transposed store of a CTA's (C = 1) or a cluster's (C > 1) rows: output row dst(kk) of
 // `out` (leading dimension ld) gets, at columns [r0, r0 + C RB), value src(kk) of each of
 // the C RB rows, for the nk kept values kk with keep(kk) (the others are not written).  With C > 1, after a cluster barrier each CTA
@@ -754,7 +758,8 @@ __global__ void __launch_bounds__(256, 2)
     }
     fft8192_32<true, false>(v, smem, t, tw);
 #pragma unroll
-    for (int q = 0; q < 32; ++q) smem[pidx(t) + padded16(out_k32(0, q))] = v[q];
+    for (int q = 0; q < 32; ++q)  // outputs k < N / 2 and k >= 3 N / 2: q mod 16 < 4 and >= 12
+        if ((q & 15) < 4 || (q & 15) >= 12) smem[pidx(t) + padded16(out_k32(0, q))] = v[q];
     transposed_store<1, 4, SR, N, 256>(
         smem, [](int kk) { return kk < N / 2 ? kk : kk + N; },
         [](int kk) { return kk < N / 2 ? kk + N / 2 : kk - N / 2; }, [](int) { return true; }, J.out, (size_t)gx, r0);
@@ -853,7 +858,8 @@ __global__ void __launch_bounds__(RB * N / 8, (1024 / (RB * N / 8)) > 0 ? (1024 
     }
     fft_n<L, true>(v, sm, t, tws);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) sm[pidx(t) + padded16(T * m)] = v[out_slot<L>(m)];
+    for (int q = 0; q < 8; ++q)
+        sm[pidx(t) + padded16(T * kept_slot(q))] = v[out_slot<L>(kept_slot(q))];
     // kept output kk < N: k = kk (kk < N/2) or kk + N; image row i = (k < N/2 ? k : k - L) + N/2
     transposed_store<RB, C, SR, N, RB * N / 8>(
         smem, [](int kk) { return kk < N / 2 ? kk : kk + N; },
@@ -905,10 +911,8 @@ __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 
         for (int m = 0; m < 16; ++m) v[m] = (keep >> m) & 1u ? __ldg(&in[t + T * m]) : make_float2(0.f, 0.f);
         fft_n<L, true>(v, sm, t, tws);
 #pragma unroll
-        for (int m = 0; m < 16; ++m) {
-            const int k = t + T * m;
-            if (k >= N / 2 && k < 3 * N / 2) continue;  // outside the crop
-            const int jc = k < N / 2 ? k : k - L;
+        for (int q = 0; q < 8; ++q) {
+            const int m = kept_slot(q), jc = t + T * m - (m < 4 ? 0 : L);
             const int j = jc + N / 2;
             float2 val = cmulc(v[out_slot<L>(m)], z_factor(z, i, j, ic, jc));
             if (acc) val = cadd(val, orow[j]);
@@ -955,10 +959,8 @@ __global__ void __launch_bounds__(RG * N / 8, 2)
         fft_n<L, true>(v, sm, t, tws);
         const ZArgs z = J.z;
 #pragma unroll
-        for (int m = 0; m < 16; ++m) {
-            const int k = t + T * m;
-            if (k >= N / 2 && k < 3 * N / 2) continue;  // outside the crop
-            const int jc2 = k < N / 2 ? k : k - L;
+        for (int q = 0; q < 8; ++q) {
+            const int m = kept_slot(q), jc2 = t + T * m - (m < 4 ? 0 : L);
             sm[jc2 + N / 2] = cmulc(v[out_slot<L>(m)], z_factor(z, i, jc2 + N / 2, ic, jc2));
         }
         __syncthreads();
