@@ -32,34 +32,39 @@
 
 namespace rimo {
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// Complex additions of the butterflies: packed (both halves in one issue slot, with the roundings of
+// two scalar additions) or, with PK = false, scalar (see fft_n).
+template <bool PK = true>
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) {
+    return PK ? __fadd2_rn(a, b) : make_float2(a.x + b.x, a.y + b.y);
+}
+template <bool PK = true>
+__device__ __forceinline__ float2 csub(float2 a, float2 b) {
+    return PK ? __ffma2_rn(b, make_float2(-1.f, -1.f), a) : make_float2(a.x - b.x, a.y - b.y);
+}
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {  // a * conj(b)
     return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
 }
-// multiply by -i (forward) or +i (inverse)
-template <bool INV>
-__device__ __forceinline__ float2 mul_mi(float2 a) {
-    return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
-}
 
-template <bool INV>
+template <bool PK>
 __device__ __forceinline__ void dft2(float2& a, float2& b) {
     float2 t = a;
-    a = cadd(t, b);
-    b = csub(t, b);
+    a = cadd<PK>(t, b);
+    b = csub<PK>(t, b);
 }
 
-template <bool INV>
+template <bool INV, bool PK>
 __device__ __forceinline__ void dft4(float2& x0, float2& x1, float2& x2, float2& x3) {
-    float2 a0 = cadd(x0, x2), a1 = csub(x0, x2), a2 = cadd(x1, x3), a3 = mul_mi<INV>(csub(x1, x3));
-    x0 = cadd(a0, a2);
-    x2 = csub(a0, a2);
-    x1 = cadd(a1, a3);
-    x3 = csub(a1, a3);
+    const float2 a0 = cadd<PK>(x0, x2), a1 = csub<PK>(x0, x2), a2 = cadd<PK>(x1, x3), d = csub<PK>(x1, x3);
+    x0 = cadd<PK>(a0, a2);
+    x2 = csub<PK>(a0, a2);
+    // a1 -+ i d: the halves swap, so these additions are scalar
+    const float2 p = make_float2(a1.x + d.y, a1.y - d.x), q = make_float2(a1.x - d.y, a1.y + d.x);
+    x1 = INV ? q : p;
+    x3 = INV ? p : q;
 }
 
 #define RS2 0.70710678118654752440f
@@ -74,20 +79,20 @@ __device__ __forceinline__ float2 w8(int k) {
     return make_float2(c[k], INV ? s[k] : -s[k]);
 }
 
-template <bool INV>
+template <bool INV, bool PK = true>
 __device__ __forceinline__ void dft8(float2* v) {
-    dft4<INV>(v[0], v[2], v[4], v[6]);
-    dft4<INV>(v[1], v[3], v[5], v[7]);
+    dft4<INV, PK>(v[0], v[2], v[4], v[6]);
+    dft4<INV, PK>(v[1], v[3], v[5], v[7]);
     float2 o1 = cmul(v[3], w8<INV>(1)), o2 = cmul(v[5], w8<INV>(2)), o3 = cmul(v[7], w8<INV>(3));
     float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6], o0 = v[1];
-    v[0] = cadd(e0, o0);
-    v[4] = csub(e0, o0);
-    v[1] = cadd(e1, o1);
-    v[5] = csub(e1, o1);
-    v[2] = cadd(e2, o2);
-    v[6] = csub(e2, o2);
-    v[3] = cadd(e3, o3);
-    v[7] = csub(e3, o3);
+    v[0] = cadd<PK>(e0, o0);
+    v[4] = csub<PK>(e0, o0);
+    v[1] = cadd<PK>(e1, o1);
+    v[5] = csub<PK>(e1, o1);
+    v[2] = cadd<PK>(e2, o2);
+    v[6] = csub<PK>(e2, o2);
+    v[3] = cadd<PK>(e3, o3);
+    v[7] = csub<PK>(e3, o3);
 }
 
 template <bool INV>
@@ -98,10 +103,10 @@ __device__ __forceinline__ float2 w16(int k) {  // k in [0, 9]
 }
 
 // 16-point DFT as 4 x 4: inner DFT_4 over n1 (stride 4), twiddle W16^{n2 k1}, outer DFT_4.
-template <bool INV>
+template <bool INV, bool PK = true>
 __device__ __forceinline__ void dft16(float2* v) {
 #pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) dft4<INV>(v[n2], v[n2 + 4], v[n2 + 8], v[n2 + 12]);
+    for (int n2 = 0; n2 < 4; ++n2) dft4<INV, PK>(v[n2], v[n2 + 4], v[n2 + 8], v[n2 + 12]);
     // now v[n2 + 4 k1] = A[n2][k1]
 #pragma unroll
     for (int n2 = 1; n2 < 4; ++n2)
@@ -111,7 +116,7 @@ __device__ __forceinline__ void dft16(float2* v) {
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1) {
         float2 a = v[0 + 4 * k1], b = v[1 + 4 * k1], c = v[2 + 4 * k1], d = v[3 + 4 * k1];
-        dft4<INV>(a, b, c, d);
+        dft4<INV, PK>(a, b, c, d);
         t[k1 + 0] = a;
         t[k1 + 4] = b;
         t[k1 + 8] = c;
@@ -125,16 +130,16 @@ __device__ __forceinline__ void dft16(float2* v) {
 // row holds its samples in the centred half): the first layer of 4-point DFTs reduces to
 // sums and differences of x_n2 and x_n2+12 (written out, since the compiler may not drop an
 // addition of +0, which would turn -0 into +0)
-template <bool INV>
+template <bool INV, bool PK = true>
 __device__ __forceinline__ void dft16_hz(float2* v) {
 #pragma unroll
     for (int n2 = 0; n2 < 4; ++n2) {
         const float2 a = v[n2], d = v[n2 + 12];
-        const float2 md = mul_mi<INV>(make_float2(-d.x, -d.y));
-        v[n2] = cadd(a, d);
-        v[n2 + 8] = csub(a, d);
-        v[n2 + 4] = cadd(a, md);
-        v[n2 + 12] = csub(a, md);
+        v[n2] = cadd<PK>(a, d);
+        v[n2 + 8] = csub<PK>(a, d);
+        const float2 p = make_float2(a.x + d.y, a.y - d.x), q = make_float2(a.x - d.y, a.y + d.x);
+        v[n2 + 4] = INV ? p : q;
+        v[n2 + 12] = INV ? q : p;
     }
 #pragma unroll
     for (int n2 = 1; n2 < 4; ++n2)
@@ -144,7 +149,7 @@ __device__ __forceinline__ void dft16_hz(float2* v) {
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1) {
         float2 a = v[0 + 4 * k1], b = v[1 + 4 * k1], c = v[2 + 4 * k1], d = v[3 + 4 * k1];
-        dft4<INV>(a, b, c, d);
+        dft4<INV, PK>(a, b, c, d);
         t[k1 + 0] = a;
         t[k1 + 4] = b;
         t[k1 + 8] = c;
@@ -154,12 +159,12 @@ __device__ __forceinline__ void dft16_hz(float2* v) {
     for (int k = 0; k < 16; ++k) v[k] = t[k];
 }
 
-template <int R, bool INV>
+template <int R, bool INV, bool PK>
 __device__ __forceinline__ void dft_r(float2* v) {
-    if constexpr (R == 2) dft2<INV>(v[0], v[1]);
-    else if constexpr (R == 4) dft4<INV>(v[0], v[1], v[2], v[3]);
-    else if constexpr (R == 8) dft8<INV>(v);
-    else dft16<INV>(v);
+    if constexpr (R == 2) dft2<PK>(v[0], v[1]);
+    else if constexpr (R == 4) dft4<INV, PK>(v[0], v[1], v[2], v[3]);
+    else if constexpr (R == 8) dft8<INV, PK>(v);
+    else dft16<INV, PK>(v);
 }
 
 // Exchange buffers are padded: element i at i + i / 16.  A stage's addresses are one base per
@@ -174,7 +179,7 @@ __host__ __device__ constexpr int padded16(int i) { return i + i / 16; }
 // W_{NS R}^{r (j mod NS)} come from the stage table tws[r NS + j mod NS], laid out so that
 // consecutive threads read consecutive entries.
 // HZ: a first stage whose inputs m = 4 .. 11 are zero (forward passes)
-template <int N, int R, int NS, bool INV, bool FIRST, bool LAST, bool HZ = false>
+template <int N, int R, int NS, bool INV, bool FIRST, bool LAST, bool HZ = false, bool PK = true>
 __device__ __forceinline__ void fft_stage(float2 (&v)[16], float2* sm, int t, const float2* __restrict__ tws) {
     constexpr int T = N / 16;
     constexpr int Q = 16 / R;
@@ -215,8 +220,8 @@ __device__ __forceinline__ void fft_stage(float2 (&v)[16], float2* sm, int t, co
                 }
             }
         }
-        if constexpr (HZ && R == 16) dft16_hz<INV>(&v[q * R]);
-        else dft_r<R, INV>(&v[q * R]);
+        if constexpr (HZ && R == 16) dft16_hz<INV, PK>(&v[q * R]);
+        else dft_r<R, INV, PK>(&v[q * R]);
     }
     if constexpr (!LAST) {
         // butterfly j = t (R = 16, Q = 1): element (j / NS) 16 NS + j mod NS + r NS
@@ -353,21 +358,25 @@ struct Plan16 {
 // tws: the stage twiddle tables of length N (see stage_twiddles on the host): the second
 // stage's W_{16 R}^{r j} at [0, 16 R), the third stage's W_{256 R}^{r j} at [256, 256 + 256 R),
 // a fourth stage's W_{4096 R}^{r j} at [4352, 4352 + 4096 R).
-template <int N, bool INV, bool HZ = false>
+// PK: packed additions.  Off for the 8192-point row passes and for inv_rows_bins_kernel, which hold
+// every register: the moves and spills that register pairs cost are more than the issue slots they
+// save.  Per 4096^2/24M apply, scalar and packed: forward rows 5.18 and 5.29 ms, inverse rows 4.04
+// and 4.12; 512^2 in one bin, inverse rows 15.9 and 18.5 us.  The other passes gain: forward cols at
+// 4096^2 3.53 -> 3.19 ms, inverse cols 5.65 -> 5.55, 2048^2 inverse rows 0.612 -> 0.561.
+template <int N, bool INV, bool HZ = false, bool PK = N <= 4096>
 __device__ __forceinline__ void fft_n(float2 (&v)[16], float2* sm, int t, const float2* __restrict__ tws) {
     constexpr int RL = Plan16<N>::R_LAST;
+    fft_stage<N, 16, 1, INV, true, false, HZ, PK>(v, sm, t, tws);
     if constexpr (Plan16<N>::STAGES == 2) {
-        fft_stage<N, 16, 1, INV, true, false, HZ>(v, sm, t, tws);
-        fft_stage<N, RL, 16, INV, false, true>(v, sm, t, tws);
-    } else if constexpr (Plan16<N>::STAGES == 3) {
-        fft_stage<N, 16, 1, INV, true, false, HZ>(v, sm, t, tws);
-        fft_stage<N, 16, 16, INV, false, false>(v, sm, t, tws);
-        fft_stage<N, RL, 256, INV, false, true>(v, sm, t, tws + 256);
+        fft_stage<N, RL, 16, INV, false, true, false, PK>(v, sm, t, tws);
     } else {
-        fft_stage<N, 16, 1, INV, true, false, HZ>(v, sm, t, tws);
-        fft_stage<N, 16, 16, INV, false, false>(v, sm, t, tws);
-        fft_stage<N, 16, 256, INV, false, false>(v, sm, t, tws + 256);
-        fft_stage<N, RL, 4096, INV, false, true>(v, sm, t, tws + 256 + 4096);
+        fft_stage<N, 16, 16, INV, false, false, false, PK>(v, sm, t, tws);
+        if constexpr (Plan16<N>::STAGES == 3) {
+            fft_stage<N, RL, 256, INV, false, true, false, PK>(v, sm, t, tws + 256);
+        } else {
+            fft_stage<N, 16, 256, INV, false, false, false, PK>(v, sm, t, tws + 256);
+            fft_stage<N, RL, 4096, INV, false, true, false, PK>(v, sm, t, tws + 256 + 4096);
+        }
     }
 }
 
@@ -915,7 +924,7 @@ __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 
             const int m = kept_slot(q), jc = t + T * m - (m < 4 ? 0 : L);
             const int j = jc + N / 2;
             float2 val = cmulc(v[out_slot<L>(m)], z_factor(z, i, j, ic, jc));
-            if (acc) val = cadd(val, orow[j]);
+            if (acc) val = cadd<false>(val, orow[j]);
             if (real_only) val.y = 0.f;
             orow[j] = val;
         }
@@ -956,7 +965,7 @@ __global__ void __launch_bounds__(RG * N / 8, 2)
             const bool keep = on && (!sel.on || ((sel.bits[tr >> 5] >> (tr & 31)) & 1u));
             v[m] = keep ? __ldg(&in[t + T * m]) : make_float2(0.f, 0.f);
         }
-        fft_n<L, true>(v, sm, t, tws);
+        fft_n<L, true, false, false>(v, sm, t, tws);
         const ZArgs z = J.z;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -967,8 +976,8 @@ __global__ void __launch_bounds__(RG * N / 8, 2)
         for (int e = threadIdx.x; e < rows * N; e += THREADS) {
             const float2* p = smem + (size_t)((e / N) << lb) * SR + e % N;
             float2 val = p[0];
-            if (accumulate || jc > j0) val = cadd(val, out[e]);
-            for (int s = 1; s < nb; ++s) val = cadd(p[s * SR], val);
+            if (accumulate || jc > j0) val = cadd<false>(val, out[e]);
+            for (int s = 1; s < nb; ++s) val = cadd<false>(p[s * SR], val);
             if (real_only) val.y = 0.f;
             out[e] = val;
         }
