@@ -15,8 +15,14 @@
 // thread, 2N/16 threads per row), exchanging through shared memory between stages; at
 // 2N = 8192 the two column passes hold 32 points per thread instead (256 threads per row,
 // radix 32 x 16 x 16: two exchanges and barriers instead of three; measured per 4096^2/50M
-// apply, forward cols 4.28 -> 3.81 ms and inverse cols + fold 7.56 -> 6.90 ms, while the row
-// passes, which also evaluate Z_p per point, were slower so: 5.32 -> 5.55 and 4.30 -> 4.61 ms).  The
+// apply when it was introduced, forward cols 4.28 -> 3.81 ms and inverse cols + fold 7.56 ->
+// 6.90 ms, while the row passes, which also evaluate Z_p per point, were slower so: 5.32 -> 5.55
+// and 4.30 -> 4.61 ms).  What bounds the passes at 4096^2 (32 bins, 24M visibilities, per apply):
+// forward cols 3.19 ms, latency and half the issue slots; fold + inverse cols 5.46 ms, the same and
+// the clusters' barriers; forward rows 5.10 ms, barriers (block and cluster), the exchange and the
+// 32-byte pieces of the transposed store (69 % of the load/store pipe); inverse rows 4.05 ms,
+// memory latency at 4.2 TB/s with two 512-thread rows per SM (with the 8192 points as two halves of
+// 4096, two exchanges instead of three, they took the same 5.18 and 4.09 ms).  The
 // zero padding and the crop are exploited where they cost nothing: forward passes never
 // load the zero half of their input (those points enter the first butterflies as
 // constants), inverse passes store only the kept half of their output, and the
@@ -1035,13 +1041,17 @@ static void launch_clustered(void (*kernel)(KArgs...), int grid, int block, size
     cfg.blockDim = dim3((unsigned)block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    // clusters placed where the SMs are least loaded: forward rows 5.19 -> 5.10 ms and inverse cols +
+    // fold 5.54 -> 5.46 per 4096^2/24M apply (equal at 2048^2; spread over the SMs: as the default)
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)C;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeClusterSchedulingPolicyPreference;
+    at[1].val.clusterSchedulingPolicyPreference = cudaClusterSchedulingPolicyLoadBalancing;
+    cfg.numAttrs = 2;
     RIMO_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
 }
 
