@@ -116,9 +116,9 @@ static void gtg(rimo_plan* p, int b, int mode, const float2* y_in, float2* y_out
 // time, so the results are the same bit for bit).  The scratch of a group is at most
 // STAGE_BYTES; from 2048^2 on that is less than two bins, whose passes fill the GPU anyway.
 // Plans that generate their tiles do so for as many bins of a group as fit STAGE_TAPS (at
-// 1024^2/1M/16 bins, generation and grid step of four bins at a time: tabulated kernels 0.82 ->
-// 0.56 and 0.96 -> 0.87 ms per apply, the network 1.03 -> 0.80 ms).
-// Measured, us per call: Phi^dagger Phi and an update at 256^2/20k/4 bins 200 -> 100, Phi at
+// 1024^2/1M/16 bins, generation and grid step of four bins instead of one at a time: tabulated
+// kernels 0.82 -> 0.56 and 0.96 -> 0.87 ms per apply, the network 1.03 -> 0.80 ms).
+// Measured, us per call, this change alone: Phi^dagger Phi and an update at 256^2/20k/4 bins 200 -> 100, Phi at
 // 512x256/100k/3 bins 108 -> 60, Phi and Phi^dagger at 1024^2/2M/16 bins 1269 -> 1062 and
 // 2010 -> 1854.
 constexpr int STAGE_BLOCKS = 1216;                       // four waves of two blocks per SM
@@ -177,7 +177,10 @@ void stage_plan(rimo_plan* p, cudaStream_t s) {
     const int64_t each = p->stage_each;
     auto* st = new PlanStage();
     p->stage = st;  // freed with the plan
-    if (cudaMalloc(&st->scratch, (size_t)(each * sc.total())) != cudaSuccess) {
+    // only from memory that is plentiful: what a caller allocates next fits as it did without groups
+    size_t room = 0, total = 0;
+    RIMO_CUDA(cudaMemGetInfo(&room, &total));
+    if (room < (size_t)(4 * each * sc.total()) || cudaMalloc(&st->scratch, (size_t)(each * sc.total())) != cudaSuccess) {
         cudaGetLastError();  // no room: one bin at a time
         st->scratch = nullptr;
         p->stage = nullptr;

@@ -672,7 +672,10 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
         };
         int64_t mx = place();
         void* taps = nullptr;
-        if (p->stage_each > 1 && cudaMalloc(&taps, (size_t)mx) != cudaSuccess) {
+        // several bins' tiles only where the rest of the plan surely fits beside them
+        size_t room = 0, total = 0;
+        if (p->stage_each > 1) RIMO_CUDA(cudaMemGetInfo(&room, &total));
+        if (p->stage_each > 1 && (room < 2 * (size_t)mx + ((size_t)4 << 30) || cudaMalloc(&taps, (size_t)mx) != cudaSuccess)) {
             cudaGetLastError();  // no room for several bins: one at a time
             taps = nullptr;
             stage_bins(p, false);
