@@ -625,8 +625,9 @@ rimo_status rimo_image_dot(const rimo_cfloat* a, const rimo_cfloat* b, int64_t n
  * Kernel surrogate as the plan's tile generator.  A plan created with mode
  * RIMO_MODE_SURROGATE (kb_support + max_wsupport - 1 must be 15) places every visibility
  * with the largest support (15 x 15 tiles), keeps one Fourier block per w-bin and stores
- * no G: each apply generates one bin's tiles at a time with the attached network into a
- * scratch the size of the largest bin, then grids them as the stored-G path does.
+ * no G: each apply generates the tiles of a few bins at a time (runs of bins whose taps
+ * come to at most 1 GiB, else one bin) with the attached network into a scratch the size
+ * of the largest run, then grids them as the stored-G path does.
  * rimo_plan_set_surrogate attaches s (not owned; it must outlive its use, and one
  * surrogate must not serve two applies at once) and allocates the generation buffers.
  * Applies and tile read-back of a surrogate plan without a surrogate fail with STATE;

@@ -19,13 +19,14 @@
 //             of the visibility after the next one, across the unit's end if need be.
 // Blocks only synchronise at unit boundaries, and two or three blocks per SM hide each other's.
 // What bounds it: with full units (512^2 / 2M visibilities / 4 bins, 488 per unit) the
-// instruction stream (335 per visibility, 72 % of the issue slots) and the shared-memory
-// pipe (82 wavefronts per visibility, 73 % busy); with small units (1024^2 / 2M / 16 bins, 38
-// per unit) their boundaries.  Against one block of 20 visibility warps fed by a producer
+// shared-memory pipe (86 wavefronts per visibility, 79 % busy; 328 instructions, 73 % of the
+// issue slots, 5 TB/s of taps); with small units (1024^2 / 2M / 16 bins, 38 per unit) their
+// boundaries and the bookkeeping per visibility (gridding: half the issue slots and half the
+// pipe).  Against one block of 20 visibility warps fed by a producer
 // warp through a common ring of 20-visibility chunks (386 instructions and 90 wavefronts per
 // visibility, a unit's descriptors and the rows of its X box fetched one after the other):
-// 512^2 case 1.06 -> 0.89 ms, 1024^2 de-grid 2.46 -> 0.82 ms and grid 1.86 -> 1.17 ms,
-// 4096^2 / 24M / 32 bins 15.4 -> 10.3 ms per apply.
+// 512^2 case 1.06 -> 0.74 ms, 1024^2 de-grid 2.46 -> 0.70 ms and grid 1.86 -> 0.98 ms,
+// 4096^2 / 24M / 32 bins 15.4 -> 9.8 ms per apply.
 // The finished accumulator box is written once to the unit's slot of the patch buffer
 // (slices of a split tile are then added into its first slot); the fold of the inverse
 // transform sums the overlapping halos of neighbouring patches tile by tile, so the gridded

@@ -182,7 +182,7 @@ struct rimo_plan {
     float* d_wt_buf = nullptr;  // their buffer (kept when the weighting is removed)
 
     // kernel surrogate (mode RIMO_MODE_SURROGATE) or exact on-the-fly tiles (mode
-    // RIMO_MODE_ONTHEFLY): tiles generated per bin at apply time
+    // RIMO_MODE_ONTHEFLY): tiles generated per run of bins at apply time
     struct rimo_surrogate* sur = nullptr;  // attached by rimo_plan_set_surrogate (not owned)
     float2* d_sur_taps = nullptr;          // the taps of one run of bins
     int64_t sur_taps_bytes = 0;

@@ -819,7 +819,7 @@ __global__ void __launch_bounds__(GEN_THREADS, 1) sur_gen_kernel(GenArgs A) {
         if (__syncthreads_or(!ok)) break;
         tc::fence_after_sync();
         {   // layer-3 read-out: chunks of 16 taps (warp groups take every GEN_WG-th chunk).  The
-            // chunk's 32 rows pass through a warp-private 4 KB of the A buffer (free once the
+            // chunk's 32 rows pass through a warp-private 4 KB laid over the A buffer (free once the
             // layer-3 MMAs completed) so that the warp writes 128-byte row segments, not
             // scattered 16-byte pieces; pieces are XOR-swizzled by row against bank conflicts.
             const int r = 32 * (warp & 3) + lane;

@@ -10,7 +10,8 @@ namespace rimo {
 // |f| <= 1/8 goes through the Taylor series of sin and cos in x = 2 pi f, |x| <= pi / 4, to x^9
 // and x^10 (first omitted terms 2e-9 and 1e-10; against 64 bits over a turn: at most 8.7e-8,
 // 1.9e-8 rms, where rounding alone is 1.5e-8).  About 25 instructions, none on the special
-// function unit, where sincospif took about 45 with four there: PHASE_FIGURES
+// function unit, where sincospif took about 45 with four there (row
+// passes 2 to 6 % faster: forward rows of 4096^2 / 32 bins 5.33 -> 5.21 ms)
 __device__ __forceinline__ float2 cis_turn(float r) {
     const float t = __fadd_rn(4.f * r, 12582912.f);
     const int q = __float_as_int(t);
