@@ -623,6 +623,17 @@ __device__ __forceinline__ const J& block_job(const J& one, const JobTable<J>& t
     }
 }
 
+// Which of a warp's values lie in needed tiles, as one bit per value m < n: the warp's 32
+// consecutive cells at pos(m) share a tile (sides 32 and 64), so lane m reads that tile's flag
+// and a ballot hands all of them to every lane.  With the flags staged in shared memory behind a
+// barrier and a load per value, 4096^2/24M took 3.20 instead of 2.91 ms of forward cols and 5.46
+// instead of 5.26 of inverse cols + fold, 2048^2/10M 0.668 for 0.606 and 1.33 for 1.25.
+template <class Pos>
+__device__ __forceinline__ uint32_t needed(const uint8_t* __restrict__ need_row, int shift, int n, Pos pos) {
+    const int lane = threadIdx.x & 31;
+    return __ballot_sync(0xffffffffu, lane < n && __ldg(need_row + (pos(lane) >> shift)) != 0);
+}
+
 // ----------------------------------------------------------------------------- forward rows
 // grid: ny / RB blocks of RB * N/8 threads per job; block b transforms image rows
 // [b RB, b RB + RB): Z_p times the row, zero-padded to 2N, DFT along l; row i of the result
@@ -685,9 +696,14 @@ __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 
     const size_t u = (size_t)r0 + g;
     const float2* __restrict__ in = J.in + u * N;
     float2* __restrict__ out = J.out + u * L;
-    for (int e = threadIdx.x; e < RG * ntv; e += blockDim.x) {
-        const size_t uu = (size_t)r0 + e / ntv;
-        s_need[e] = need[(uu >> shift) * ntv + e % ntv];
+    uint32_t on = 0;
+    if constexpr (T >= 32) {
+        on = needed(need + (u >> shift) * ntv, shift, 16, [&](int m) { return (t & ~31) + T * m; });
+    } else {
+        for (int e = threadIdx.x; e < RG * ntv; e += blockDim.x) {
+            const size_t uu = (size_t)r0 + e / ntv;
+            s_need[e] = need[(uu >> shift) * ntv + e % ntv];
+        }
     }
     float2 v[16];
 #pragma unroll
@@ -700,12 +716,12 @@ __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 
             v[m] = __ldg(&in[jc + N / 2]);
         }
     }
-    __syncthreads();
+    if constexpr (T < 32) __syncthreads();
     fft_n<L, false, true>(v, sm, t, tws);
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
         const int k = t + T * m;
-        if (s_need[g * ntv + (k >> shift)]) out[k] = v[out_slot<L>(m)];
+        if (T >= 32 ? (on >> m) & 1u : s_need[g * ntv + (k >> shift)]) out[k] = v[out_slot<L>(m)];
     }
 }
 
@@ -720,13 +736,12 @@ __global__ void __launch_bounds__(256, 2)
     const ColsJob& J = block_job<TABLE>(one, tab, bk);
     const uint8_t* __restrict__ need = J.need;
     const int ntv = L >> shift;
-    uint8_t* s_need = reinterpret_cast<uint8_t*>(smem + L + L / 32);
     const int t = threadIdx.x;
     const int r0 = sel_row0(J.sel, bk, 1);
     const size_t u = (size_t)r0;
     const float2* __restrict__ in = J.in + u * N;
     float2* __restrict__ out = J.out + u * L;
-    for (int e = threadIdx.x; e < ntv; e += blockDim.x) s_need[e] = need[(u >> shift) * ntv + e];
+    const uint32_t on = needed(need + (u >> shift) * ntv, shift, 32, [&](int q) { return out_k32(t & ~31, q); });
     float2 v[32];
 #pragma unroll
     for (int m = 0; m < 32; ++m) {
@@ -738,12 +753,11 @@ __global__ void __launch_bounds__(256, 2)
             v[m] = __ldg(&in[jc + N / 2]);
         }
     }
-    __syncthreads();
     fft8192_32<false, true>(v, smem, t, tw);
 #pragma unroll
     for (int q = 0; q < 32; ++q) {
         const int k = out_k32(t, q);
-        if (s_need[k >> shift]) out[k] = v[q];
+        if ((on >> q) & 1u) out[k] = v[q];
     }
 }
 
@@ -758,18 +772,16 @@ __global__ void __launch_bounds__(256, 2)
     const ColsJob& J = block_job<TABLE>(one, tab, bk);
     const uint8_t* __restrict__ need = J.need;
     const int ntv = L >> shift;
-    uint8_t* s_need = reinterpret_cast<uint8_t*>(smem + SR);
     const int t = threadIdx.x;
     const int r0 = sel_row0(J.sel, bk, 1);
     const int u = r0;
-    for (int e = threadIdx.x; e < ntv; e += blockDim.x) s_need[e] = need[(size_t)(u >> shift) * ntv + e];
-    __syncthreads();
+    const uint32_t on = needed(need + (size_t)(u >> shift) * ntv, shift, 32, [&](int m) { return (t & ~31) + 256 * m; });
     const float2* __restrict__ in = J.in + (size_t)u * L;
     float2 v[32];
 #pragma unroll
     for (int m = 0; m < 32; ++m) {
         const int p = t + 256 * m;
-        v[m] = s_need[p >> shift] ? __ldg(&in[p]) : make_float2(0.f, 0.f);
+        v[m] = (on >> m) & 1u ? __ldg(&in[p]) : make_float2(0.f, 0.f);
     }
     fft8192_32<true, false>(v, smem, t, tw);
 #pragma unroll
@@ -859,17 +871,22 @@ __global__ void __launch_bounds__(RB * N / 8, (1024 / (RB * N / 8)) > 0 ? (1024 
     float2* sm = smem + g * SR;
     const int r0 = sel_row0(J.sel, bk, RB);
     const int u = r0 + g;
-    for (int e = threadIdx.x; e < RB * ntv; e += blockDim.x) {
-        const int uu = r0 + e / ntv;
-        s_need[e] = need[(size_t)(uu >> shift) * ntv + e % ntv];
+    uint32_t on = 0;
+    if constexpr (T >= 32) {
+        on = needed(need + (size_t)(u >> shift) * ntv, shift, 16, [&](int m) { return (t & ~31) + T * m; });
+    } else {
+        for (int e = threadIdx.x; e < RB * ntv; e += blockDim.x) {
+            const int uu = r0 + e / ntv;
+            s_need[e] = need[(size_t)(uu >> shift) * ntv + e % ntv];
+        }
+        __syncthreads();
     }
-    __syncthreads();
     const float2* __restrict__ in = J.in + (size_t)u * L;
     float2 v[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) {
         const int p = t + T * m;
-        v[m] = s_need[g * ntv + (p >> shift)] ? __ldg(&in[p]) : make_float2(0.f, 0.f);
+        v[m] = (T >= 32 ? (on >> m) & 1u : s_need[g * ntv + (p >> shift)]) ? __ldg(&in[p]) : make_float2(0.f, 0.f);
     }
     fft_n<L, true>(v, sm, t, tws);
 #pragma unroll
@@ -1167,14 +1184,14 @@ static void run_fwd_cols(const ColsJob& one, const JobTable<ColsJob>& tab, int g
                          cudaStream_t s, const float2* tw32) {
     if constexpr (N == 4096) {
         if (!tw32) fail(RIMO_ERR_STATE, "8192-point column transforms without their twiddle table");
-        const size_t sm = (size_t)(8192 + 8192 / 32) * sizeof(float2) + 8192 / 32 + 16;
+        const size_t sm = (size_t)(8192 + 8192 / 32) * sizeof(float2);
         if (grid == 0) return;
         set_smem(fwd_cols32_kernel<TABLE>, sm);
         fwd_cols32_kernel<TABLE><<<grid, 256, sm, s>>>(one, tab, tile_shift(TS), tw32);
     } else {
         constexpr int RG = rows_per_block<N>();
         const int ntv = (2 * N) / TS;
-        const size_t sm = (size_t)RG * (2 * N + N / 8) * sizeof(float2) + (size_t)RG * ntv + 16;
+        const size_t sm = (size_t)RG * (2 * N + N / 8) * sizeof(float2) + (N < 256 ? (size_t)RG * ntv : 0);  // N < 256: flags
         if (grid == 0) return;
         set_smem(fwd_cols_kernel<N, RG, TABLE>, sm);
         fwd_cols_kernel<N, RG, TABLE><<<grid, RG * N / 8, sm, s>>>(one, tab, tile_shift(TS), tws);
@@ -1193,7 +1210,7 @@ static void run_inv_cols(const ColsJob& one, const JobTable<ColsJob>& tab, int g
                          const float2* tws, cudaStream_t s, const float2* tw32) {
     if constexpr (N == 4096) {
         if (!tw32) fail(RIMO_ERR_STATE, "8192-point column transforms without their twiddle table");
-        const size_t sm = (size_t)(8192 + 8192 / 16) * sizeof(float2) + 8192 / 32 + 16;
+        const size_t sm = (size_t)(8192 + 8192 / 16) * sizeof(float2);
         if (grid == 0) return;
         if (grid % 4 != 0) fail(RIMO_ERR_UNSUPPORTED, "grid rows do not fill the transposed-store clusters");
         set_smem(inv_cols32_kernel<TABLE>, sm);
@@ -1202,7 +1219,7 @@ static void run_inv_cols(const ColsJob& one, const JobTable<ColsJob>& tab, int g
         constexpr int RB = rows_per_block<N>();
         constexpr int C = cluster_of<RB>();
         const int ntv = (2 * N) / TS;
-        const size_t sm = (size_t)RB * (2 * N + N / 8) * sizeof(float2) + (size_t)RB * ntv + 16;
+        const size_t sm = (size_t)RB * (2 * N + N / 8) * sizeof(float2) + (N < 256 ? (size_t)RB * ntv : 0);  // N < 256: flags
         if (grid == 0) return;
         // C consecutive blocks of a cluster stay in one tile row: TS / RB is a multiple of C
         if constexpr (C > 1) {

@@ -105,3 +105,22 @@ def test_holographic_apply_of_every_tile_side(m, kb, cap, tile, dense):
     assert torch.equal(torch.view_as_real(a), torch.view_as_real(b))
     plan.status()
     plan.close()
+
+
+@pytest.mark.parametrize("n, tile", [(64, 32), (64, 64), (128, 32), (256, 32), (256, 64), (512, 64), (1024, 32),
+                                     (2048, 64)])
+def test_needed_tiles_of_the_column_passes(n, tile):
+    """Few visibilities, scattered over the whole grid and its edges: most tiles are not needed, so
+    the column passes' marks (per warp, or in shared memory below 256) decide what is stored and read."""
+    fov = math.radians(2.0)
+    rng = np.random.default_rng(n + tile)
+    m = 40
+    uvw = np.empty((m, 3))
+    uvw[:, :2] = (rng.random((m, 2)) - 0.5) * (2 * n - 1) / (2.0 * fov)
+    uvw[:2, :2] = [[0.4999 * n / fov, 0.0], [0.0, -0.4999 * n / fov]]
+    uvw[:, 2] = 100.0 * (rng.random(m) - 0.5)
+    plan, op = both(uvw, n, n, fov, fov, n_wbins=2, tile_size=tile)
+    x = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+    assert rel(to_host(plan.phi(to_dev(x))), op.phi(x.astype(np.complex64).astype(np.complex128))) < TOL
+    assert rel(to_host(plan.phi_adj_phi(to_dev(x))), op.phi_adj_phi(x.astype(np.complex64).astype(np.complex128))) < TOL
+    plan.close()
