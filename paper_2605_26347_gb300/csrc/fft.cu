@@ -32,6 +32,7 @@
 
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 #include "internal.h"
 #include "phase.cuh"
@@ -512,6 +513,22 @@ __device__ __forceinline__ float2 dsmem_ld2(uint32_t addr) {
 // time, so that a pruned last stage and the staging skip the others.
 __host__ __device__ constexpr int kept_slot(int q) { return q < 4 ? q : q + 8; }
 
+// Which steps of a transposed store a warp takes part in: its values of one step share a uv-tile
+// (at most 16 in a row, aligned), so lane i asks for step i and a ballot tells every lane.
+struct KeepAll {
+    __device__ bool operator()(int) const { return true; }
+};
+template <int IT, class Keep, class At>
+__device__ __forceinline__ uint32_t kept_steps(Keep keep, At at) {
+    static_assert(IT <= 32, "one lane per step");
+    if constexpr (std::is_same<Keep, KeepAll>::value) {
+        return 0xffffffffu;
+    } else {
+        const int lane = threadIdx.x & 31;
+        return __ballot_sync(0xffffffffu, lane < IT && keep(at(lane)));
+    }
+}
+
 // Transposed store of a CTA's (C = 1) or a cluster's (C > 1) rows: output row dst(kk) of
 // `out` (leading dimension ld) gets, at columns [r0, r0 + C RB), value src(kk) of each of
 // the C RB rows, for the nk kept values kk with keep(kk) (the others are not written).  With C > 1, after a cluster barrier each CTA
@@ -522,10 +539,13 @@ __device__ __forceinline__ void transposed_store(float2* smem, Src src, Dst dst,
                                                  int r0_block) {  // r0_block: this CTA's first row
     if constexpr (C == 1) {
         __syncthreads();
-        constexpr int NP = RB / 2;
-        for (int e = threadIdx.x; e < NK * NP; e += THREADS) {
-            const int kk = e / NP, q = e % NP;
-            if (!keep(kk)) continue;
+        constexpr int NP = RB / 2, IT = NK * NP / THREADS;
+        static_assert(NK * NP % THREADS == 0 && NP >= 2, "a warp holds at most 16 values");
+        const uint32_t on = kept_steps<IT>(keep, [](int i) { return (int)((threadIdx.x & ~31u) + i * THREADS) / NP; });
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            const int e = threadIdx.x + i * THREADS, kk = e / NP, q = e % NP;
+            if (!((on >> i) & 1u)) continue;
             const int k = src(kk);
             const float2 a = smem[(2 * q) * SR + pidx(k)], b = smem[(2 * q + 1) * SR + pidx(k)];
             *reinterpret_cast<float4*>(&out[(size_t)dst(kk) * ld + r0_block + 2 * q]) = make_float4(a.x, a.y, b.x, b.y);
@@ -539,9 +559,14 @@ __device__ __forceinline__ void transposed_store(float2* smem, Src src, Dst dst,
         const int q = threadIdx.x % NP;                   // rows 2q, 2q + 1 of the cluster
         // src and dst are shifts within a rank's range, so a thread's values are STEP apart
         const int kk0 = rank * KPC + threadIdx.x / NP;
+        static_assert(NP >= 2, "a warp holds at most 16 values");
         uint32_t on = 0;
+        if constexpr (C == 2) {
+            on = kept_steps<IT>(keep, [&](int i) { return rank * KPC + (int)(threadIdx.x & ~31u) / NP + i * STEP; });
+        } else {  // (at 2N = 8192 with the ballot: 5.16 instead of 5.10 ms of forward rows)
 #pragma unroll
-        for (int it = 0; it < IT; ++it) on |= (keep(kk0 + it * STEP) ? 1u : 0u) << it;
+            for (int it = 0; it < IT; ++it) on |= (keep(kk0 + it * STEP) ? 1u : 0u) << it;
+        }
         const uint32_t off = (uint32_t)pidx(src(kk0)) * 8u;
         const uint32_t b0 = dsmem_map(smem + ((2 * q) % RB) * SR, (2 * q) / RB) + off;
         const uint32_t b1 = dsmem_map(smem + ((2 * q + 1) % RB) * SR, (2 * q + 1) / RB) + off;
@@ -632,6 +657,16 @@ template <class Pos>
 __device__ __forceinline__ uint32_t needed(const uint8_t* __restrict__ need_row, int shift, int n, Pos pos) {
     const int lane = threadIdx.x & 31;
     return __ballot_sync(0xffffffffu, lane < n && __ldg(need_row + (pos(lane) >> shift)) != 0);
+}
+
+// Likewise which of a warp's values lie in selected tile rows (the bits of a job table are loads
+// from memory: one per lane instead of one per value and thread; iteration at 256^2, 4 bins, inverse
+// rows 15.4 -> 10.2 us; 2048^2/10M 0.563 -> 0.543 ms, 4096^2/24M 4.05 -> 3.98).
+template <class Pos>
+__device__ __forceinline__ uint32_t selected(const RowSel& sel, int n, Pos pos) {
+    if (!sel.on) return 0xffffffffu;
+    const int lane = threadIdx.x & 31, tr = pos(lane) >> sel.shift;
+    return __ballot_sync(0xffffffffu, lane < n && ((sel.bits[tr >> 5] >> (tr & 31)) & 1u));
 }
 
 // ----------------------------------------------------------------------------- forward rows
@@ -789,7 +824,7 @@ __global__ void __launch_bounds__(256, 2)
         if ((q & 15) < 4 || (q & 15) >= 12) smem[pidx(t) + padded16(out_k32(0, q))] = v[q];
     transposed_store<1, 4, SR, N, 256>(
         smem, [](int kk) { return kk < N / 2 ? kk : kk + N; },
-        [](int kk) { return kk < N / 2 ? kk + N / 2 : kk - N / 2; }, [](int) { return true; }, J.out, (size_t)gx, r0);
+        [](int kk) { return kk < N / 2 ? kk + N / 2 : kk - N / 2; }, KeepAll{}, J.out, (size_t)gx, r0);
 }
 
 // ----------------------------------------------------------------------------- patch fold
@@ -895,7 +930,7 @@ __global__ void __launch_bounds__(RB * N / 8, (1024 / (RB * N / 8)) > 0 ? (1024 
     // kept output kk < N: k = kk (kk < N/2) or kk + N; image row i = (k < N/2 ? k : k - L) + N/2
     transposed_store<RB, C, SR, N, RB * N / 8>(
         smem, [](int kk) { return kk < N / 2 ? kk : kk + N; },
-        [](int kk) { return kk < N / 2 ? kk + N / 2 : kk - N / 2; }, [](int) { return true; }, J.out, (size_t)gx,
+        [](int kk) { return kk < N / 2 ? kk + N / 2 : kk - N / 2; }, KeepAll{}, J.out, (size_t)gx,
         r0);
 }
 
@@ -931,7 +966,9 @@ __global__ void __launch_bounds__(RG * N / 8, (1024 / (RG * N / 8)) > 0 ? (1024 
         float2 v[16];
         // columns u of tile rows the inverse column pass skipped are zero (not stored)
         uint32_t keep = 0xffffu;
-        if (sel.on) {
+        if constexpr (T >= 32) {
+            keep = selected(sel, 16, [&](int m) { return (t & ~31) + T * m; });
+        } else if (sel.on) {
             keep = 0;
 #pragma unroll
             for (int m = 0; m < 16; ++m) {
@@ -981,11 +1018,14 @@ __global__ void __launch_bounds__(RG * N / 8, 2)
         const RowsJob& J = tab.jobs[on ? jc + (g & (BP - 1)) : j0];
         const RowSel& sel = J.sel;
         const float2* __restrict__ in = J.in + (size_t)i * L;
+        // (a warp's threads share a slot when a row has 32 threads or more)
+        uint32_t sels = 0;
+        if constexpr (T >= 32) sels = on ? selected(sel, 16, [&](int m) { return (t & ~31) + T * m; }) : 0u;
         float2 v[16];
 #pragma unroll
         for (int m = 0; m < 16; ++m) {
             const int tr = (t + T * m) >> sel.shift;
-            const bool keep = on && (!sel.on || ((sel.bits[tr >> 5] >> (tr & 31)) & 1u));
+            const bool keep = T >= 32 ? (sels >> m) & 1u : on && (!sel.on || ((sel.bits[tr >> 5] >> (tr & 31)) & 1u));
             v[m] = keep ? __ldg(&in[t + T * m]) : make_float2(0.f, 0.f);
         }
         fft_n<L, true, false, false>(v, sm, t, tws);
