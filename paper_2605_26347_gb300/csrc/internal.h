@@ -303,15 +303,18 @@ struct WideJob {
     float2* patch;    // tile patches of the bin's work units, (t1 - t0) PW^2
 };
 // Job of block b of a launch over a job table: the last job whose first block is <= b
-// (first: njobs + 1 non-decreasing block offsets).
+// (first: njobs + 1 non-decreasing block offsets).  Called by whole warps: 32 candidates per
+// load, where a bisection waits for log2(njobs) loads one after the other (batch of 108 jobs of
+// 1024^2 8.38 -> 8.22 ms; four jobs as before).
 __device__ __forceinline__ int job_of(const int* first, int njobs, int b) {
-    int lo = 0, hi = njobs - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(first + mid) <= b) lo = mid;
-        else hi = mid - 1;
+    int j = 0;
+    for (int n = njobs; n > 1;) {  // the job is one of [j, j + n)
+        const int step = (n + 31) >> 5, o = (int)(threadIdx.x & 31) * step;
+        const int k = __popc(__ballot_sync(0xffffffffu, o < n && __ldg(first + j + o) <= b)) - 1;
+        j += k * step;
+        n = min(step, n - k * step);
     }
-    return lo;
+    return j;
 }
 struct WideFft;   // device job tables of the transform passes (fft.cu)
 struct WideGtg;   // device unit list of the grid step (grid.cu)

@@ -124,3 +124,24 @@ def test_needed_tiles_of_the_column_passes(n, tile):
     assert rel(to_host(plan.phi(to_dev(x))), op.phi(x.astype(np.complex64).astype(np.complex128))) < TOL
     assert rel(to_host(plan.phi_adj_phi(to_dev(x))), op.phi_adj_phi(x.astype(np.complex64).astype(np.complex128))) < TOL
     plan.close()
+
+
+@pytest.mark.parametrize("bins", [[1, 2], [16, 15], [16, 16], [16, 17], [32, 32, 1], [32, 32, 31, 4]])
+def test_staged_batch_of_many_jobs(bins):
+    """A block finds its (plan, bin) job 32 candidates at a time: job counts on both sides of 32 and
+    beyond 64, against each plan's own apply bit for bit."""
+    import synth
+    import torch
+
+    import paper_2605_26347_gb300 as pkg
+    n, fov = 64, math.radians(2.0)
+    chans = synth.wideband_channels(n_chan=len(bins), m_lo=2000, m_hi=3000, seed=43)
+    plans = [pkg.Plan(uvw, pkg.default_params(n, n, fov, fov, n_wbins=b)) for (_, uvw), b in zip(chans, bins)]
+    batch = pkg.Batch(plans, form=pkg.BATCH_STAGED)
+    assert batch.layout()["jobs"] > 0.9 * sum(bins)
+    rng = np.random.default_rng(sum(bins))
+    x = torch.stack([to_dev(rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))) for _ in bins])
+    out = batch.phi_adj_phi(x)
+    for k, p in enumerate(plans):
+        assert torch.equal(torch.view_as_real(out[k].contiguous()),
+                           torch.view_as_real(p.phi_adj_phi(x[k].contiguous())))
