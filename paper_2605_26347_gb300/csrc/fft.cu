@@ -603,7 +603,7 @@ __device__ __forceinline__ int sel_row0(const RowSel& sel, int b, int rows_per_b
 // A pass over one (plan, w-bin) is a job.  A launch covers one job (the applies of a plan,
 // bin after bin: the job's arguments by value) or a table of jobs of the same transform
 // shape (a wideband batch, every channel's every bin in one launch per pass): job j owns
-// the launch's blocks [first[j], first[j + 1]), and a block finds its job from it and
+// the launch's blocks [first[j], first[j + 1]), and a block finds its job (job_of) and
 // then runs as in a one-job launch, with its block index within the job.
 // The image pointer of a rows job counts from the launch's `img` bytes: 0 with the image's
 // address in the job, or the image's address with null jobs (a plan's tables, whose images
