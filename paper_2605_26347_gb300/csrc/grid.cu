@@ -678,9 +678,7 @@ struct WideGtg {
     int* own_counter = nullptr;
     int64_t units = 0;
     ~WideGtg() {
-        cudaFree(recs);
-        cudaFree(mjobs);
-        cudaFree(mfirst);
+        cudaFree(recs);  // and mjobs, mfirst
         cudaFree(own_counter);
     }
 };
@@ -699,6 +697,7 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStr
         std::vector<MergeJob> mj;
         std::vector<int> mf{0};
         std::vector<UnitRec> recs;
+        std::vector<size_t> seg{0};  // each job's records, heaviest first as in its plan
         size_t nrec = 0;
         for (const WideJob& j : jobs) nrec += (size_t)(j.p->bins[j.bin].t1 - j.p->bins[j.bin].t0);
         // (a unit index plus the blocks' look-ahead stays an int)
@@ -715,6 +714,7 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStr
                 q.patch += (int64_t)(uintptr_t)jobs[j].patch;
                 recs.push_back(q);
             }
+            seg.push_back(recs.size());
             MergeJob m;
             m.patch = jobs[j].patch;
             m.groups = p->d_merge + br.m0;
@@ -727,7 +727,16 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStr
             std::vector<uint64_t> key(recs.size());
             for (size_t i = 0; i < recs.size(); ++i)
                 key[i] = ((uint64_t)(0xffffffffu - (uint32_t)recs[i].nvis) << 32) | (uint32_t)i;
-            std::sort(key.begin(), key.end());
+            // the jobs' runs merged two by two
+            for (; seg.size() > 2;) {
+                std::vector<size_t> up{0};
+                for (size_t k = 2; k < seg.size(); k += 2) {
+                    std::inplace_merge(key.begin() + (long)seg[k - 2], key.begin() + (long)seg[k - 1], key.begin() + (long)seg[k]);
+                    up.push_back(seg[k]);
+                }
+                if (seg.size() % 2 == 0) up.push_back(seg.back());
+                seg.swap(up);
+            }
             std::vector<UnitRec> sorted(recs.size());
             for (size_t i = 0; i < recs.size(); ++i) sorted[i] = recs[(uint32_t)key[i]];
             recs.swap(sorted);
@@ -735,9 +744,13 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStr
         w->units = (int64_t)recs.size();
         w->njobs = (int)jobs.size();
         w->merge_blocks = mf.back();
-        RIMO_CUDA(cudaMalloc(&w->recs, std::max<size_t>(1, recs.size()) * sizeof(UnitRec)));
-        RIMO_CUDA(cudaMalloc(&w->mjobs, mj.size() * sizeof(MergeJob)));
-        RIMO_CUDA(cudaMalloc(&w->mfirst, mf.size() * sizeof(int)));
+        // one allocation: records, merge jobs, their first blocks
+        const size_t at_m = recs.size() * sizeof(UnitRec), at_f = at_m + mj.size() * sizeof(MergeJob);
+        char* mem = nullptr;
+        RIMO_CUDA(cudaMalloc(&mem, at_f + mf.size() * sizeof(int)));
+        w->recs = reinterpret_cast<UnitRec*>(mem);
+        w->mjobs = reinterpret_cast<MergeJob*>(mem + at_m);
+        w->mfirst = reinterpret_cast<int*>(mem + at_f);
         if (!counter) RIMO_CUDA(cudaMalloc(&w->own_counter, sizeof(int)));
         w->counter = counter ? counter : w->own_counter;
         if (!recs.empty())
