@@ -185,14 +185,17 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(GemmArgs g) {
         for (int c = 0; c < nt; c += 16) {
             float v[16];
             tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + c, v);
-            if (row >= g.m_store) continue;
-            float4* dst = reinterpret_cast<float4*>(g.C + (size_t)row * g.ldc + n0 + c);
+            // (the warp that holds row m_store is whole again before its next, warp-collective load)
+            if (row < g.m_store) {
+                float4* dst = reinterpret_cast<float4*>(g.C + (size_t)row * g.ldc + n0 + c);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float4 x = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                if (g.atomic) atomicAdd(dst + i, x);
-                else dst[i] = x;
+                for (int i = 0; i < 4; ++i) {
+                    const float4 x = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                    if (g.atomic) atomicAdd(dst + i, x);
+                    else dst[i] = x;
+                }
             }
+            __syncwarp();
         }
     }
     tc::fence_before_sync();

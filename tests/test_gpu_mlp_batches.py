@@ -21,3 +21,18 @@ def test_gradients_of_any_batch(net, B):  # noqa: F811
         gd = pkg.unpack_params(g)
         for k in ("W3", "b3", "W2", "b2", "W1", "b1"):
             assert rel(gd[k], ref[k]) < 2e-3, (k, rel(gd[k], ref[k]))  # bf16 flips, as in test_gpu_surrogate
+
+
+@pytest.mark.parametrize("B", [128, 1408])
+def test_weight_gradients_of_the_last_outputs(net, B):  # noqa: F811
+    """dW3 has 450 rows, the product's last 128-row tile 512: one warp of it holds rows on both
+    sides of the end.  Row by row, so that two wrong rows do not hide in the norm of 450; a row
+    is a sum over B samples in which a bf16 flip moves one term by 2^-8, 2^-8 / sqrt(B) of the
+    row each (4e-4 at B = 128), a few per row."""
+    import paper_2605_26347_gb300 as pkg
+    s, p = net
+    x, t = batch(B, B + 1)
+    _, ref = omlp.loss_and_grads(p, x.astype(np.float64), t.astype(np.float64), bf=True)
+    g = pkg.unpack_params(s.gradients(x, t)[1])["W3"]
+    for j in range(384, 450):
+        assert rel(g[j], ref["W3"][j]) < 2e-3, (j, rel(g[j], ref["W3"][j]))
