@@ -444,6 +444,16 @@ rimo_status rimo_plan_status(rimo_plan_t plan, void* stream);
 rimo_status rimo_plan_set_wait_test(rimo_plan_t plan, int32_t stall, int32_t polls);
 
 /*
+ * Failure test of the library's device allocations (no counterpart in the paper): the nth
+ * device allocation that the calling thread makes from now on reports out of memory, without
+ * a call to the driver; the later ones succeed again.  nth = 0 ends the test.  left (may be
+ * null) receives what was left of the previous count: 0 when its allocation has failed or none
+ * was set.  Host-only call, for the calling thread alone.
+ * Errors: INVALID_ARG.
+ */
+rimo_status rimo_set_alloc_test(int64_t nth, int64_t* left);
+
+/*
  * Kernel surrogate (a learned replacement for the stored de-gridding taps; no
  * counterpart in the paper, which stores G or H or recomputes G on the fly, Section 3.4).
  * A multilayer perceptron maps the normalised inputs x = (2 phi_u - 1, 2 phi_v - 1,

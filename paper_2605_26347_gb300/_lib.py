@@ -106,6 +106,7 @@ _PROTOS = {
     "rimo_psf": (C.c_int, [_P, _P, _P]),
     "rimo_plan_status": (C.c_int, [_P, _P]),
     "rimo_plan_set_wait_test": (C.c_int, [_P, C.c_int32, C.c_int32]),
+    "rimo_set_alloc_test": (C.c_int, [C.c_int64, C.POINTER(C.c_int64)]),
     "rimo_plan_get_zlayer": (C.c_int, [_P, C.c_int32, _P, _P]),
     "rimo_profile_enable": (C.c_int, [_P, C.c_int32]),
     "rimo_profile_read": (C.c_int, [_P, _P, _P, C.c_int32, C.c_int32]),

@@ -180,7 +180,7 @@ void stage_plan(rimo_plan* p, cudaStream_t s) {
     // only from memory that is plentiful: what a caller allocates next fits as it did without groups
     size_t room = 0, total = 0;
     RIMO_CUDA(cudaMemGetInfo(&room, &total));
-    if (room < (size_t)(4 * each * sc.total()) || cudaMalloc(&st->scratch, (size_t)(each * sc.total())) != cudaSuccess) {
+    if (room < (size_t)(4 * each * sc.total()) || device_malloc(&st->scratch, (size_t)(each * sc.total())) != cudaSuccess) {
         cudaGetLastError();  // no room: one bin at a time
         st->scratch = nullptr;
         p->stage = nullptr;

@@ -105,7 +105,7 @@ void stage(rimo_batch* b, cudaStream_t s) {
         }
     }
     if (b->jobs.empty()) return;
-    if (cudaMalloc(&b->scratch, (size_t)total) != cudaSuccess) {
+    if (device_malloc(&b->scratch, (size_t)total) != cudaSuccess) {
         cudaGetLastError();
         fail(RIMO_ERR_OOM, "batch scratch of " + std::to_string(total) + " bytes");
     }
@@ -378,8 +378,8 @@ int tune(const double* uvw, int64_t M, const rimo_plan_params* base, const std::
     cudaStream_t s = (cudaStream_t)stream;
     float2 *x = nullptr, *o = nullptr;
     const size_t img = (size_t)q.nx * q.ny * sizeof(float2);
-    RIMO_CUDA(cudaMalloc(&x, img));
-    RIMO_CUDA(cudaMalloc(&o, img));
+    RIMO_CUDA(device_malloc(&x, img));
+    RIMO_CUDA(device_malloc(&o, img));
     double best = 1e300;
     int pick = 0;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -467,8 +467,8 @@ int tune_batch(const double* const* uvw, const int64_t* M, const rimo_plan_param
     double best = 1e300;
     int pick = 0;
     try {
-        RIMO_CUDA(cudaMalloc(&x, img * n * sizeof(float2)));
-        RIMO_CUDA(cudaMalloc(&o, img * n * sizeof(float2)));
+        RIMO_CUDA(device_malloc(&x, img * n * sizeof(float2)));
+        RIMO_CUDA(device_malloc(&o, img * n * sizeof(float2)));
         RIMO_CUDA(cudaMemsetAsync(x, 0, img * n * sizeof(float2), s));
         const float2 one = make_float2(1.f, 0.f);
         for (int i = 0; i < n; ++i)  // a point at the centre of every image: every grid is non-trivial

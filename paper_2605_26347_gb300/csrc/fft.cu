@@ -1400,7 +1400,7 @@ WideFft* wide_fft_create(const std::vector<WideJob>& jobs, const std::vector<con
         pass(w->cols_inv, ci, fci);
         pass(w->rows_inv, ri, std::vector<int>{0, w->ngroups * (p0->ny / rb)});
         const size_t gat = append(blob, grp);
-        RIMO_CUDA(cudaMalloc(&w->tables, blob.size()));
+        RIMO_CUDA(device_malloc(&w->tables, blob.size()));
         RIMO_CUDA(cudaMemcpyAsync(w->tables, blob.data(), blob.size(), cudaMemcpyHostToDevice, s));
         for (auto& q : at) {
             q.first->jobs = w->tables + q.second.first;

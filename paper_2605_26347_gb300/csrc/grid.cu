@@ -747,11 +747,11 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStr
         // one allocation: records, merge jobs, their first blocks
         const size_t at_m = recs.size() * sizeof(UnitRec), at_f = at_m + mj.size() * sizeof(MergeJob);
         char* mem = nullptr;
-        RIMO_CUDA(cudaMalloc(&mem, at_f + mf.size() * sizeof(int)));
+        RIMO_CUDA(device_malloc(&mem, at_f + mf.size() * sizeof(int)));
         w->recs = reinterpret_cast<UnitRec*>(mem);
         w->mjobs = reinterpret_cast<MergeJob*>(mem + at_m);
         w->mfirst = reinterpret_cast<int*>(mem + at_f);
-        if (!counter) RIMO_CUDA(cudaMalloc(&w->own_counter, sizeof(int)));
+        if (!counter) RIMO_CUDA(device_malloc(&w->own_counter, sizeof(int)));
         w->counter = counter ? counter : w->own_counter;
         if (!recs.empty())
             RIMO_CUDA(cudaMemcpyAsync(w->recs, recs.data(), recs.size() * sizeof(UnitRec), cudaMemcpyHostToDevice, s));

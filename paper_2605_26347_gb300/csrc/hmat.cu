@@ -716,8 +716,8 @@ static WideH* wide_h_create(const rimo_plan* p, const std::vector<WideJob>& jobs
         }
         w->njobs = (int)a.size();
         w->blocks = f.back();
-        RIMO_CUDA(cudaMalloc(&w->jobs, a.size() * sizeof(HApplyArgs)));
-        RIMO_CUDA(cudaMalloc(&w->first, f.size() * sizeof(int)));
+        RIMO_CUDA(device_malloc(&w->jobs, a.size() * sizeof(HApplyArgs)));
+        RIMO_CUDA(device_malloc(&w->first, f.size() * sizeof(int)));
         RIMO_CUDA(cudaMemcpyAsync(w->jobs, a.data(), a.size() * sizeof(HApplyArgs), cudaMemcpyHostToDevice, s));
         RIMO_CUDA(cudaMemcpyAsync(w->first, f.data(), f.size() * sizeof(int), cudaMemcpyHostToDevice, s));
         RIMO_CUDA(cudaStreamSynchronize(s));
@@ -742,7 +742,7 @@ static void stage_holographic(rimo_plan* p, int max_need, cudaStream_t s) {
     for (const auto& g : p->stage->groups) most = std::max(most, g.jobs.size());
     const size_t each = (size_t)max_need * p->PW * p->PW;
     if (most * each * sizeof(float2) > ((size_t)512 << 20)) return;
-    if (cudaMalloc(&p->stage->hpatch, most * each * sizeof(float2)) != cudaSuccess) {
+    if (device_malloc(&p->stage->hpatch, most * each * sizeof(float2)) != cudaSuccess) {
         cudaGetLastError();
         p->stage->hpatch = nullptr;
         return;
@@ -804,9 +804,9 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
         }
     }, 1);
     AnchorIndex ai;
-    RIMO_CUDA(cudaMalloc(&ai.pos, apos.size() * sizeof(int32_t)));
-    RIMO_CUDA(cudaMalloc(&ai.h0, ah0.size() * sizeof(uint16_t)));
-    RIMO_CUDA(cudaMalloc(&ai.row, arow.size() * sizeof(int64_t)));
+    RIMO_CUDA(device_malloc(&ai.pos, apos.size() * sizeof(int32_t)));
+    RIMO_CUDA(device_malloc(&ai.h0, ah0.size() * sizeof(uint16_t)));
+    RIMO_CUDA(device_malloc(&ai.row, arow.size() * sizeof(int64_t)));
     RIMO_CUDA(cudaMemcpyAsync(ai.pos, apos.data(), apos.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s));
     RIMO_CUDA(cudaMemcpyAsync(ai.h0, ah0.data(), ah0.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, s));
     RIMO_CUDA(cudaMemcpyAsync(ai.row, arow.data(), arow.size() * sizeof(int64_t), cudaMemcpyHostToDevice, s));
@@ -828,7 +828,7 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
     int max_need = 1;
     for (int b = 0; b < P; ++b) max_need = std::max(max_need, p->bins[b].n1 - p->bins[b].n0);
     DevBuf counts;
-    RIMO_CUDA(cudaMalloc(&counts.p, (size_t)max_need * sizeof(int64_t)));
+    RIMO_CUDA(device_malloc(&counts.p, (size_t)max_need * sizeof(int64_t)));
     HArgs A;
     std::memset(&A, 0, sizeof(A));
     A.meta = p->d_meta;
@@ -891,7 +891,7 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
     int64_t nnz = 0, h_bytes = 0;
     unsigned long long diag = 0;
     DevBuf dcount, ddiag;
-    RIMO_CUDA(cudaMalloc(&ddiag.p, sizeof(unsigned long long)));
+    RIMO_CUDA(device_malloc(&ddiag.p, sizeof(unsigned long long)));
     RIMO_CUDA(cudaMemsetAsync(ddiag.p, 0, sizeof(unsigned long long), s));
     try {
         for (int b = 0; b < P; ++b) {
@@ -902,7 +902,7 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
             std::vector<int64_t> roff((size_t)nown + 1, 0);
             if (nown > 0) {
                 DevBuf dense;
-                if (cudaMalloc(&dense.p, (size_t)nown * ne * sizeof(float2)) != cudaSuccess) {
+                if (device_malloc(&dense.p, (size_t)nown * ne * sizeof(float2)) != cudaSuccess) {
                     cudaGetLastError();
                     fail(RIMO_ERR_OOM, "holographic build: dense rows of one bin");
                 }
@@ -920,7 +920,7 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
                 RIMO_CUDA(cudaGetLastError());
                 cudaFree(dcount.p);
                 dcount.p = nullptr;
-                RIMO_CUDA(cudaMalloc(&dcount.p, (size_t)nown * sizeof(int32_t)));
+                RIMO_CUDA(device_malloc(&dcount.p, (size_t)nown * sizeof(int32_t)));
                 const int64_t blocks = (nown * 32 + 255) / 256;
                 hrowcount_kernel<<<(unsigned)blocks, 256, 0, s>>>((const float2*)dense.p, nown, ne, (int32_t*)dcount.p,
                                                                   (unsigned long long*)ddiag.p);

@@ -41,6 +41,12 @@ void check_cuda(cudaError_t e, const char* what);
 void validate_params(const rimo_plan_params& q);
 void validate_uvw(const double* uvw, int64_t M, const rimo_plan_params& q);
 #define RIMO_CUDA(call) ::rimo::check_cuda((call), #call)
+// cudaMalloc; the calling thread's rimo_set_alloc_test makes one of its calls fail.
+cudaError_t device_malloc_bytes(void** ptr, size_t bytes);
+template <class T>
+cudaError_t device_malloc(T** ptr, size_t bytes) {
+    return device_malloc_bytes(reinterpret_cast<void**>(ptr), bytes);
+}
 
 // ---------------------------------------------------------------------------
 // Per-visibility metadata in sorted (bin, uv-tile) order, 16 bytes.

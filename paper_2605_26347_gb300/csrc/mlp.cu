@@ -437,12 +437,13 @@ __global__ void pack_weights_kernel(const float* __restrict__ P, bf16* __restric
 // --------------------------------------------------------------------------------------
 Mlp::~Mlp() {
     for (void* p : owned) cudaFree(p);
+    cudaFree(acts);
     if (host) cudaFreeHost(host);
 }
 
 void* Mlp::alloc(size_t bytes) {
     void* p = nullptr;
-    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+    if (device_malloc(&p, bytes) != cudaSuccess) {
         cudaGetLastError();
         fail(RIMO_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes for the surrogate failed");
     }
@@ -497,23 +498,44 @@ void Mlp::pack(cudaStream_t s) {
     pack_weights_kernel<<<(n + 255) / 256, 256, 0, s>>>(P, W2b, W2Tb, W3b, W3Tb);
 }
 
+// The activations of a batch of B: one allocation, which takes the place of the previous, smaller
+// one only when it is there, so that after a failure the buffers and cap still match.
 void Mlp::reserve(int B, cudaStream_t s) {
     if (B <= cap) return;
-    cap = B;
-    Z1 = (float*)alloc((size_t)B * MLP_H * sizeof(float));
-    Z2 = (float*)alloc((size_t)B * MLP_H * sizeof(float));
-    Y = (float*)alloc((size_t)B * MLP_OUT_PAD * sizeof(float));
-    dH = (float*)alloc((size_t)B * MLP_H * sizeof(float));
-    H1 = (bf16*)alloc((size_t)B * MLP_H * sizeof(bf16));
-    H1T = (bf16*)alloc((size_t)B * MLP_H * sizeof(bf16));
-    H2 = (bf16*)alloc((size_t)B * MLP_H * sizeof(bf16));
-    H2T = (bf16*)alloc((size_t)B * MLP_H * sizeof(bf16));
-    dY = (bf16*)alloc((size_t)B * MLP_K3 * sizeof(bf16));
-    dYT = (bf16*)alloc((size_t)B * MLP_K3 * sizeof(bf16));
-    dZ = (bf16*)alloc((size_t)B * MLP_H * sizeof(bf16));
-    dZT = (bf16*)alloc((size_t)B * MLP_H * sizeof(bf16));
+    size_t total = 0;
+    auto place = [&](size_t bytes) {  // 256-byte aligned parts
+        const size_t at = total;
+        total += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t f = (size_t)B * MLP_H * sizeof(float), h = (size_t)B * MLP_H * sizeof(bf16);
+    const size_t y = (size_t)B * MLP_OUT_PAD * sizeof(float), d = (size_t)B * MLP_K3 * sizeof(bf16);
+    const size_t z1 = place(f), z2 = place(f), oy = place(y), dh = place(f), h1 = place(h), h1t = place(h), h2 = place(h),
+                 h2t = place(h), ody = place(d), dyt = place(d), dz = place(h), dzt = place(h);
+    char* q = nullptr;
+    if (device_malloc(&q, total) != cudaSuccess) {
+        cudaGetLastError();
+        fail(RIMO_ERR_OOM, "activations of " + std::to_string(B) + " samples: " + std::to_string(total) + " bytes");
+    }
     // rows past the padded outputs only fill the last 128-row tile of dW3
-    RIMO_CUDA(cudaMemsetAsync(dYT, 0, (size_t)B * MLP_K3 * sizeof(bf16), s));
+    const cudaError_t e = cudaMemsetAsync(q + dyt, 0, d, s);
+    if (e != cudaSuccess) cudaFree(q);
+    RIMO_CUDA(e);
+    cudaFree(acts);  // (waits for the kernels that use it)
+    acts = q;
+    Z1 = (float*)(q + z1);
+    Z2 = (float*)(q + z2);
+    Y = (float*)(q + oy);
+    dH = (float*)(q + dh);
+    H1 = (bf16*)(q + h1);
+    H1T = (bf16*)(q + h1t);
+    H2 = (bf16*)(q + h2);
+    H2T = (bf16*)(q + h2t);
+    dY = (bf16*)(q + ody);
+    dYT = (bf16*)(q + dyt);
+    dZ = (bf16*)(q + dz);
+    dZT = (bf16*)(q + dzt);
+    cap = B;
 }
 
 void Mlp::forward(const float* X, int B, cudaStream_t s, bool train) {
@@ -969,7 +991,7 @@ struct DevScratch {
     std::vector<void*> v;
     void* get(size_t bytes) {
         void* ptr = nullptr;
-        if (cudaMalloc(&ptr, bytes) != cudaSuccess) {
+        if (device_malloc(&ptr, bytes) != cudaSuccess) {
             cudaGetLastError();
             fail(RIMO_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes for the training set failed");
         }

@@ -31,7 +31,8 @@ struct Mlp {
     float* host = nullptr;   // pinned copy of G, loss and status
     int t = 0;
     // activations of the last batch
-    int cap = 0;
+    int cap = 0;             // its samples
+    char* acts = nullptr;    // the allocation that holds all of them
     float *Z1 = nullptr, *Z2 = nullptr, *Y = nullptr, *dH = nullptr;
     __nv_bfloat16 *H1 = nullptr, *H1T = nullptr, *H2 = nullptr, *H2T = nullptr;
     __nv_bfloat16 *dY = nullptr, *dYT = nullptr, *dZ = nullptr, *dZT = nullptr;

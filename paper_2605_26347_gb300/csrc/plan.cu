@@ -28,10 +28,17 @@ void check_cuda(cudaError_t e, const char* what) {
     }
 }
 
+static thread_local int64_t t_alloc_test = 0;  // rimo_set_alloc_test: calls until the one that fails
+
+cudaError_t device_malloc_bytes(void** ptr, size_t bytes) {
+    if (t_alloc_test > 0 && --t_alloc_test == 0) return cudaErrorMemoryAllocation;
+    return cudaMalloc(ptr, bytes);
+}
+
 void* dev_alloc(rimo_plan* p, size_t bytes) {
     void* ptr = nullptr;
     if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMalloc(&ptr, bytes);
+    cudaError_t e = device_malloc(&ptr, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         fail(RIMO_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed: " +
@@ -675,7 +682,7 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
         // several bins' tiles only where the rest of the plan surely fits beside them
         size_t room = 0, total = 0;
         if (p->stage_each > 1) RIMO_CUDA(cudaMemGetInfo(&room, &total));
-        if (p->stage_each > 1 && (room < 2 * (size_t)mx + ((size_t)4 << 30) || cudaMalloc(&taps, (size_t)mx) != cudaSuccess)) {
+        if (p->stage_each > 1 && (room < 2 * (size_t)mx + ((size_t)4 << 30) || device_malloc(&taps, (size_t)mx) != cudaSuccess)) {
             cudaGetLastError();  // no room for several bins: one at a time
             taps = nullptr;
             stage_bins(p, false);
@@ -798,6 +805,16 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
 using namespace rimo;
 
 extern "C" {
+
+rimo_status rimo_set_alloc_test(int64_t nth, int64_t* left) {
+    if (nth < 0) {
+        set_last_error("nth < 0");
+        return RIMO_ERR_INVALID_ARG;
+    }
+    if (left) *left = t_alloc_test;
+    t_alloc_test = nth;
+    return RIMO_OK;
+}
 
 void rimo_plan_params_default(rimo_plan_params* q, int32_t nx, int32_t ny, double fov_x,
                               double fov_y) {

@@ -1,0 +1,72 @@
+"""Device allocations that fail (rimo_set_alloc_test makes them, on the host): what was there
+before stays usable, and what needs no more memory goes on without it."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from oracle import mlp as omlp
+from test_gpu_surrogate import batch, rel
+
+OOM = 2
+
+
+def fail_alloc(n):
+    """The nth device allocation from now on fails; returns what was left of the last count."""
+    import paper_2605_26347_gb300 as pkg
+    left = C.c_int64()
+    pkg._lib.check(pkg._lib.load().rimo_set_alloc_test(n, C.byref(left)))
+    return left.value
+
+
+def test_the_count_is_set_read_and_ended(rimo_lib):
+    import paper_2605_26347_gb300 as pkg
+    assert fail_alloc(3) == 0
+    assert fail_alloc(0) == 3
+    assert fail_alloc(0) == 0
+    with pytest.raises(pkg.RimoError) as e:
+        fail_alloc(-1)
+    assert e.value.status == 1
+
+
+@pytest.mark.gpu
+def test_a_batch_that_does_not_fit_leaves_the_surrogate_as_it_was():
+    import paper_2605_26347_gb300 as pkg
+    s = pkg.Surrogate(seed=0)
+    p = {k: v.astype(np.float64) for k, v in pkg.unpack_params(s.get_params()).items()}
+    s.gradients(*batch(256, 1))
+    for call in (s.gradients, lambda x, t: s.forward(x)):
+        fail_alloc(1)
+        with pytest.raises(pkg.RimoError) as e:
+            call(*batch(4096, 2))
+        assert e.value.status == OOM and fail_alloc(0) == 0
+    # larger than the buffers that are there, smaller than the batch that failed
+    for B in (1408, 256, 4096):
+        x, t = batch(B, B)
+        ref_loss, ref = omlp.loss_and_grads(p, x.astype(np.float64), t.astype(np.float64), bf=True)
+        loss, g = s.gradients(x, t)
+        assert abs(loss - ref_loss) < 1e-4 * ref_loss
+        gd = pkg.unpack_params(g)
+        for k in ("W3", "b3", "W2", "b2", "W1", "b1"):
+            assert rel(gd[k], ref[k]) < 2e-3, (B, k)  # bf16 flips, as in test_gpu_surrogate
+
+
+@pytest.mark.gpu
+def test_a_larger_batch_gives_back_the_smaller_ones_memory():
+    import torch
+
+    import paper_2605_26347_gb300 as pkg
+    s = pkg.Surrogate(seed=0)
+    x = torch.zeros((65536, 3), device="cuda")
+    y = torch.empty((65536, 450), device="cuda")
+
+    def free(B):  # MiB left on the device after a batch of B
+        pkg._lib.check(s._lib.rimo_surrogate_forward(s._h, x.data_ptr(), B, y.data_ptr(), 0))
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0] / 2**20
+
+    start = free(128)  # (kernels loaded)
+    per = 6976 / 2**20  # bytes of a sample's activations
+    half, full = start - free(32768), start - free(65536)
+    assert abs(half - 32768 * per) < 16
+    assert abs(full - 65536 * per) < 16, (half, full)
