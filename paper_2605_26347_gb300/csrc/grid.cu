@@ -696,25 +696,28 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStr
         }
         std::vector<MergeJob> mj;
         std::vector<int> mf{0};
-        std::vector<UnitRec> recs;
-        std::vector<size_t> seg{0};  // each job's records, heaviest first as in its plan
+        // a sort key per unit, heaviest first over all jobs (ties: job, then the bin's order): the
+        // jobs' units come heaviest first already, so their runs are merged two by two
+        std::vector<uint64_t> key;
+        std::vector<std::pair<const UnitRec*, int>> unit;  // the plan's record, the job
+        std::vector<size_t> seg{0};
         size_t nrec = 0;
         for (const WideJob& j : jobs) nrec += (size_t)(j.p->bins[j.bin].t1 - j.p->bins[j.bin].t0);
         // (a unit index plus the blocks' look-ahead stays an int)
         if (nrec > (size_t)0x7fffffff - 8 * 4096) fail(RIMO_ERR_UNSUPPORTED, "too many work units for one launch");
-        recs.reserve(nrec);
+        key.reserve(nrec);
+        unit.reserve(nrec);
         for (size_t j = 0; j < jobs.size(); ++j) {
             const rimo_plan* p = jobs[j].p;
             if (p->TS != p0->TS || p->gx != p0->gx || p->gy != p0->gy)
                 fail(RIMO_ERR_UNSUPPORTED, "jobs of one grid-step launch need one grid and uv-tile size");
             const auto& br = p->bins[jobs[j].bin];
             for (int u = br.t0; u < br.t1; ++u) {
-                UnitRec q = p->recs_host[(size_t)u];
-                q.X = (int64_t)(uintptr_t)jobs[j].X;
-                q.patch += (int64_t)(uintptr_t)jobs[j].patch;
-                recs.push_back(q);
+                const UnitRec& q = p->recs_host[(size_t)u];
+                key.push_back(((uint64_t)(0xffffffffu - (uint32_t)q.nvis) << 32) | (uint32_t)unit.size());
+                unit.push_back({&q, (int)j});
             }
-            seg.push_back(recs.size());
+            seg.push_back(key.size());
             MergeJob m;
             m.patch = jobs[j].patch;
             m.groups = p->d_merge + br.m0;
@@ -722,24 +725,22 @@ WideGtg* wide_gtg_create(const std::vector<WideJob>& jobs, int* counter, cudaStr
             mj.push_back(m);
             mf.push_back(mf.back() + (br.m1 - br.m0));
         }
-        // heaviest first over all jobs (ties: job, then the bin's order)
-        {
-            std::vector<uint64_t> key(recs.size());
-            for (size_t i = 0; i < recs.size(); ++i)
-                key[i] = ((uint64_t)(0xffffffffu - (uint32_t)recs[i].nvis) << 32) | (uint32_t)i;
-            // the jobs' runs merged two by two
-            for (; seg.size() > 2;) {
-                std::vector<size_t> up{0};
-                for (size_t k = 2; k < seg.size(); k += 2) {
-                    std::inplace_merge(key.begin() + (long)seg[k - 2], key.begin() + (long)seg[k - 1], key.begin() + (long)seg[k]);
-                    up.push_back(seg[k]);
-                }
-                if (seg.size() % 2 == 0) up.push_back(seg.back());
-                seg.swap(up);
+        for (; seg.size() > 2;) {
+            std::vector<size_t> up{0};
+            for (size_t k = 2; k < seg.size(); k += 2) {
+                std::inplace_merge(key.begin() + (long)seg[k - 2], key.begin() + (long)seg[k - 1], key.begin() + (long)seg[k]);
+                up.push_back(seg[k]);
             }
-            std::vector<UnitRec> sorted(recs.size());
-            for (size_t i = 0; i < recs.size(); ++i) sorted[i] = recs[(uint32_t)key[i]];
-            recs.swap(sorted);
+            if (seg.size() % 2 == 0) up.push_back(seg.back());
+            seg.swap(up);
+        }
+        std::vector<UnitRec> recs;
+        recs.reserve(nrec);
+        for (const uint64_t k : key) {
+            const auto& u = unit[(uint32_t)k];
+            recs.push_back(*u.first);
+            recs.back().X = (int64_t)(uintptr_t)jobs[(size_t)u.second].X;
+            recs.back().patch += (int64_t)(uintptr_t)jobs[(size_t)u.second].patch;
         }
         w->units = (int64_t)recs.size();
         w->njobs = (int)jobs.size();

@@ -267,39 +267,44 @@ static void build_tables(rimo_plan* p, cudaStream_t s) {
 std::vector<FoldRec> fold_records(const rimo_plan* p, const std::vector<int32_t>& slot, bool whole) {
     const int TS = p->TS, H = p->H, PW = p->PW, ntu = p->gx / TS, ntv = p->gy / TS;
     std::vector<FoldRec> out(p->need_host.size());
-    planner::parallel_for(p->P, [&](int64_t b0, int64_t b1) {
-        for (int64_t b = b0; b < b1; ++b)
-            for (int k = p->bins[b].n0; k < p->bins[b].n1; ++k) {
-                const int tile = p->need_host[(size_t)k], tu = tile / ntv, tv = tile % ntv;
-                FoldRec& r = out[(size_t)k];
-                for (int q = 0; q < 4; ++q) {
-                    // source q: the tile before along u (q & 1), along v (q & 2)
-                    const int su = q & 1 ? (tu + ntu - 1) % ntu : tu, sv = q & 2 ? (tv + ntv - 1) % ntv : tv;
-                    const int oa = q & 1 ? TS : 0, ob = q & 2 ? TS : 0;  // the tile's origin in that patch
-                    const int ca = q & 1 ? H : TS, cb = q & 2 ? H : TS;  // rows, columns a patch reaches
-                    const int32_t sl = slot[(size_t)b * ntu * ntv + (size_t)su * ntv + sv];
-                    r.off[q] = 0;
-                    r.rng[q] = 0;
-                    if (sl >= 0) {
-                        const uint32_t box =
-                            whole ? box_pack(0, PW, 0, PW) : p->tiles_host[(size_t)p->bins[b].t0 + sl].box;
-                        const int64_t off = ((int64_t)sl * PW * PW + oa * PW + ob) / 2;
-                        if (off > 0x7fffffffLL) fail(RIMO_ERR_UNSUPPORTED, "too many patches in one w-bin");
-                        const int b_hi = box_c0(box) + 2 * box_pairs(box);
-                        const int a0 = std::max((int)(box & 255u) - oa, 0), a1 = std::min((int)((box >> 8) & 255u) - oa, ca);
-                        const int c0 = std::max(box_c0(box) - ob, 0), c1 = std::min(b_hi - ob, cb);
-                        if (a1 > a0 && c1 > c0) {
-                            r.off[q] = (int32_t)off;
-                            r.rng[q] = (uint32_t)a0 | (uint32_t)a1 << 7 | (uint32_t)c0 << 14 | (uint32_t)c1 << 21;
-                        }
+    // (checked here: an exception may not leave a worker thread)
+    for (const BinRange& r : p->bins)
+        if ((int64_t)(whole ? r.n1 - r.n0 : r.t1 - r.t0) * PW * PW / 2 > 0x7fffffffLL)
+            fail(RIMO_ERR_UNSUPPORTED, "too many patches in one w-bin");
+    // the records of all bins in one range: a thread's start costs as much as some thousand records
+    // (with a thread per bin however small, a plan of 128^2 / 4k / 32 bins took 0.87 ms here)
+    planner::parallel_for((int64_t)out.size(), [&](int64_t k0, int64_t k1) {
+        int b = 0;
+        for (int64_t k = k0; k < k1; ++k) {
+            while (k >= p->bins[(size_t)b].n1) ++b;
+            const int tile = p->need_host[(size_t)k], tu = tile / ntv, tv = tile % ntv;
+            FoldRec& r = out[(size_t)k];
+            for (int q = 0; q < 4; ++q) {
+                // source q: the tile before along u (q & 1), along v (q & 2)
+                const int su = q & 1 ? (tu + ntu - 1) % ntu : tu, sv = q & 2 ? (tv + ntv - 1) % ntv : tv;
+                const int oa = q & 1 ? TS : 0, ob = q & 2 ? TS : 0;  // the tile's origin in that patch
+                const int ca = q & 1 ? H : TS, cb = q & 2 ? H : TS;  // rows, columns a patch reaches
+                const int32_t sl = slot[(size_t)b * ntu * ntv + (size_t)su * ntv + sv];
+                r.off[q] = 0;
+                r.rng[q] = 0;
+                if (sl >= 0) {
+                    const uint32_t box =
+                        whole ? box_pack(0, PW, 0, PW) : p->tiles_host[(size_t)p->bins[b].t0 + sl].box;
+                    const int b_hi = box_c0(box) + 2 * box_pairs(box);
+                    const int a0 = std::max((int)(box & 255u) - oa, 0), a1 = std::min((int)((box >> 8) & 255u) - oa, ca);
+                    const int c0 = std::max(box_c0(box) - ob, 0), c1 = std::min(b_hi - ob, cb);
+                    if (a1 > a0 && c1 > c0) {
+                        r.off[q] = (int32_t)(((int64_t)sl * PW * PW + oa * PW + ob) / 2);
+                        r.rng[q] = (uint32_t)a0 | (uint32_t)a1 << 7 | (uint32_t)c0 << 14 | (uint32_t)c1 << 21;
                     }
                 }
-                r.rng[0] |= (uint32_t)(tu & 15) << 28;
-                r.rng[1] |= (uint32_t)(tu >> 4) << 28;
-                r.rng[2] |= (uint32_t)(tv & 15) << 28;
-                r.rng[3] |= (uint32_t)(tv >> 4) << 28;
             }
-    }, 1);
+            r.rng[0] |= (uint32_t)(tu & 15) << 28;
+            r.rng[1] |= (uint32_t)(tu >> 4) << 28;
+            r.rng[2] |= (uint32_t)(tv & 15) << 28;
+            r.rng[3] |= (uint32_t)(tv >> 4) << 28;
+        }
+    }, 8192);
     return out;
 }
 
