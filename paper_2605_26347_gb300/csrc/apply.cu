@@ -4,6 +4,7 @@
 //   G_p / G_p^H  : uv-tile de-grid / grid / fused G^H G           (grid.cu)
 //   Z_p^H F^H    : inverse cols pass, inverse rows pass (+ accumulate over p)
 #include <algorithm>
+#include <memory>
 
 #include "internal.h"
 
@@ -168,25 +169,15 @@ void stage_bins(rimo_plan* p, bool share_taps) {
     }
 }
 
-void stage_plan(rimo_plan* p, cudaStream_t s) {
-    if (p->stage_each < 2) return;
+// Scratch and tables of the plan's groups (an allocation that fails throws; what is made so far goes
+// with `st`).
+static void make_groups(rimo_plan* p, PlanStage* st, cudaStream_t s) {
     std::vector<int> bins;
     for (int b = 0; b < p->P; ++b)
         if (p->bins[b].t1 > p->bins[b].t0) bins.push_back(b);
     const BinScratch sc(p);
     const int64_t each = p->stage_each;
-    auto* st = new PlanStage();
-    p->stage = st;  // freed with the plan
-    // only from memory that is plentiful: what a caller allocates next fits as it did without groups
-    size_t room = 0, total = 0;
-    RIMO_CUDA(cudaMemGetInfo(&room, &total));
-    if (room < (size_t)(4 * each * sc.total()) || device_malloc(&st->scratch, (size_t)(each * sc.total())) != cudaSuccess) {
-        cudaGetLastError();  // no room: one bin at a time
-        st->scratch = nullptr;
-        p->stage = nullptr;
-        delete st;
-        return;
-    }
+    RIMO_CUDA(device_malloc(&st->scratch, (size_t)(each * sc.total())));
     st->scratch_bytes = each * sc.total();
     char* base = static_cast<char*>(st->scratch);
     int runs = 0;
@@ -211,7 +202,23 @@ void stage_plan(rimo_plan* p, cudaStream_t s) {
             h.runs.push_back(r);
         }
     }
+}
+
+void stage_plan(rimo_plan* p, cudaStream_t s) {
+    if (p->stage_each < 2) return;
+    // only from memory that is plentiful: what a caller allocates next fits as it did without groups
+    size_t room = 0, total = 0;
+    RIMO_CUDA(cudaMemGetInfo(&room, &total));
+    if (room < (size_t)(4 * p->stage_each * BinScratch(p).total())) return;
+    auto st = std::make_unique<PlanStage>();
+    try {
+        make_groups(p, st.get(), s);
+    } catch (const Error& e) {
+        if (e.status == RIMO_ERR_CUDA) throw;
+        return;  // no room for the scratch or the tables: one bin at a time, which needs neither
+    }
     p->info.scratch_bytes += st->scratch_bytes;
+    p->stage = st.release();  // freed with the plan
 }
 
 // `holo`: Phi^dagger Phi through H

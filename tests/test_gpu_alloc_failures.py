@@ -1,11 +1,13 @@
 """Device allocations that fail (rimo_set_alloc_test makes them, on the host): what was there
 before stays usable, and what needs no more memory goes on without it."""
 import ctypes as C
+import math
 
 import numpy as np
 import pytest
 
 from oracle import mlp as omlp
+from parity_util import to_dev, to_host
 from test_gpu_surrogate import batch, rel
 
 OOM = 2
@@ -70,3 +72,62 @@ def test_a_larger_batch_gives_back_the_smaller_ones_memory():
     half, full = start - free(32768), start - free(65536)
     assert abs(half - 32768 * per) < 16
     assert abs(full - 65536 * per) < 16, (half, full)
+
+
+def applies(plan, x, y):
+    """Phi x, Phi^dagger y and Phi^dagger Phi x, and the launches of forward row passes of the last:
+    one per group of bins, or per bin."""
+    out = [to_host(plan.phi(x)), to_host(plan.phi_adj(y))]
+    plan.profile_read()
+    plan.profile(True)
+    out.append(to_host(plan.phi_adj_phi(x)))
+    plan.profile(False)
+    launches = plan.profile_read()["fwd_rows"][1]
+    plan.status()
+    return out, launches
+
+
+def small_plan(bins=3, n=64, m=500, **kw):
+    import synth
+
+    import paper_2605_26347_gb300 as pkg
+    fov = math.radians(2.0)
+    return pkg.Plan(synth.make_uvw(m, 60, 1.28e9, 11), pkg.default_params(n, n, fov, fov, n_wbins=bins, **kw))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kw, optional", [
+    ({}, 3),                                # the groups' scratch, transform tables, unit list
+    (dict(mode=4, wkernel_table=64), 4),    # and the taps of several bins at a time
+])
+def test_plan_creation_goes_on_without_groups(kw, optional):
+    """Whichever allocation of plan creation fails: either creation reports it, or the plan takes
+    one bin at a time, with the results of the bins in a group bit for bit (generated tiles: to the
+    scale of the fixed-point sums, 2^-36 of their bound)."""
+    bins = 3
+    rng = np.random.default_rng(3)
+    x = to_dev(rng.standard_normal((64, 64)) + 1j * rng.standard_normal((64, 64)))
+    y = to_dev(rng.standard_normal(500) + 1j * rng.standard_normal(500))
+    plan = small_plan(bins, **kw)
+    ref, launches = applies(plan, x, y)
+    assert launches == 1  # one group
+    plan.close()
+    survived = 0
+    for nth in range(1, 200):
+        fail_alloc(nth)
+        try:
+            plan = small_plan(bins, **kw)
+        except Exception as e:
+            assert getattr(e, "status", None) == OOM and fail_alloc(0) == 0
+            continue
+        if fail_alloc(0) != 0:  # more than creation makes
+            plan.close()
+            break
+        survived += 1
+        got, launches = applies(plan, x, y)
+        for a, b in zip(got, ref):
+            assert rel(a, b) < 1e-7 if kw else np.array_equal(a, b)
+        if not kw:
+            assert launches == bins
+        plan.close()
+    assert nth > 10 and survived == optional
