@@ -126,15 +126,24 @@ constexpr int STAGE_BLOCKS = 1216;                       // four waves of two bl
 constexpr int64_t STAGE_BYTES = (int64_t)512 << 20;
 constexpr int64_t STAGE_TAPS = (int64_t)1 << 30;
 
+void PlanStage::drop_holographic() {
+    for (Group& g : groups) {
+        if (g.hfft) wide_fft_destroy(g.hfft);
+        if (g.h) wide_h_destroy(g.h);
+        g.hfft = nullptr;
+        g.h = nullptr;
+    }
+    cudaFree(hpatch);
+    hpatch = nullptr;
+}
+
 PlanStage::~PlanStage() {
+    drop_holographic();
     for (Group& g : groups) {
         if (g.fft) wide_fft_destroy(g.fft);
         for (Run& r : g.runs) wide_gtg_destroy(r.gtg);
-        if (g.hfft) wide_fft_destroy(g.hfft);
-        if (g.h) wide_h_destroy(g.h);
     }
     cudaFree(scratch);
-    cudaFree(hpatch);
 }
 
 static int64_t al256(int64_t x) { return (x + 255) & ~(int64_t)255; }

@@ -734,26 +734,32 @@ void wide_happly(const WideH* w, cudaStream_t s) {
     happly_launch(w->p, none, w->jobs, w->first, w->njobs, w->blocks, w->compressed, s);
 }
 
-// Once H is built, the plan's groups of bins apply it too (patches of their own; without room
-// for them, one bin at a time).
+// Once H is built, the plan's groups of bins apply it too, with patches of their own; where
+// those or the tables do not fit, or memory is not plentiful (as in stage_plan), one bin at a time.
 static void stage_holographic(rimo_plan* p, int max_need, cudaStream_t s) {
-    if (!p->stage) return;
+    PlanStage* st = p->stage;
+    if (!st) return;
     size_t most = 0;
-    for (const auto& g : p->stage->groups) most = std::max(most, g.jobs.size());
-    const size_t each = (size_t)max_need * p->PW * p->PW;
-    if (most * each * sizeof(float2) > ((size_t)512 << 20)) return;
-    if (device_malloc(&p->stage->hpatch, most * each * sizeof(float2)) != cudaSuccess) {
-        cudaGetLastError();
-        p->stage->hpatch = nullptr;
+    for (const auto& g : st->groups) most = std::max(most, g.jobs.size());
+    const size_t each = (size_t)max_need * p->PW * p->PW, bytes = most * each * sizeof(float2);
+    if (bytes > ((size_t)512 << 20)) return;
+    size_t room = 0, total = 0;
+    RIMO_CUDA(cudaMemGetInfo(&room, &total));
+    if (room < 4 * bytes) return;
+    try {
+        RIMO_CUDA(device_malloc(&st->hpatch, bytes));
+        for (auto& g : st->groups) {
+            std::vector<WideJob> jobs = g.jobs;
+            for (size_t k = 0; k < jobs.size(); ++k) jobs[k].patch = static_cast<float2*>(st->hpatch) + k * each;
+            g.hfft = wide_fft_create(jobs, {nullptr}, {nullptr}, s, true);
+            g.h = wide_h_create(p, jobs, s);
+        }
+    } catch (const Error& e) {
+        st->drop_holographic();
+        if (e.status == RIMO_ERR_CUDA) throw;
         return;
     }
-    for (auto& g : p->stage->groups) {
-        std::vector<WideJob> jobs = g.jobs;
-        for (size_t k = 0; k < jobs.size(); ++k) jobs[k].patch = static_cast<float2*>(p->stage->hpatch) + k * each;
-        g.hfft = wide_fft_create(jobs, {nullptr}, {nullptr}, s, true);
-        g.h = wide_h_create(p, jobs, s);
-    }
-    p->info.scratch_bytes += (int64_t)(most * each * sizeof(float2));
+    p->info.scratch_bytes += (int64_t)bytes;
 }
 
 // Builds H for every bin; see the file comment.  Synchronises s.
@@ -979,8 +985,8 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
     p->info.h_nnz = 2 * (nnz - (int64_t)diag) + (int64_t)diag;
     p->h_ne = ne;
     p->info.h_bytes = h_bytes + (int64_t)patch_bytes;
-    stage_holographic(p, max_need, s);
     p->h_built = true;
+    stage_holographic(p, max_need, s);
 }
 
 }  // namespace rimo

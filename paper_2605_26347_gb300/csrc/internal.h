@@ -365,6 +365,7 @@ struct PlanStage {
     void* scratch = nullptr;
     void* hpatch = nullptr;       // the groups' holographic patches
     int64_t scratch_bytes = 0;
+    void drop_holographic();      // hpatch, hfft and h of every group
     ~PlanStage();
 };
 // Bins of a group (1: no groups) and the runs of bins that share the tap scratch, from the

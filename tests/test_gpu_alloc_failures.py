@@ -131,3 +131,51 @@ def test_plan_creation_goes_on_without_groups(kw, optional):
             assert launches == bins
         plan.close()
     assert nth > 10 and survived == optional
+
+
+@pytest.mark.gpu
+def test_the_holographic_build_goes_on_without_groups():
+    """Whichever allocation of the build of H fails: either it reports it and a second build
+    succeeds, or H is there and applied one bin at a time, bit for bit as in groups."""
+    bins = 3
+    rng = np.random.default_rng(4)
+    x = to_dev(rng.standard_normal((64, 64)) + 1j * rng.standard_normal((64, 64)))
+
+    def normal(plan):
+        plan.profile_read()
+        plan.profile(True)
+        out = to_host(plan.phi_adj_phi(x))
+        plan.profile(False)
+        return out, plan.profile_read()["h_apply"][1]
+
+    plan = small_plan(bins)
+    plan.build_holographic()
+    ref, launches = normal(plan)
+    assert launches == 1  # one group
+    plan.close()
+    survived = 0
+    for nth in range(1, 200):
+        plan = small_plan(bins)
+        fail_alloc(nth)
+        try:
+            plan.build_holographic()
+        except Exception as e:
+            assert getattr(e, "status", None) == OOM and fail_alloc(0) == 0
+            left = 0
+            plan.build_holographic()
+            got, launches = normal(plan)
+            assert launches == 1
+        else:
+            left = fail_alloc(0)
+            got, launches = normal(plan)
+            if left == 0:
+                survived += 1
+                assert launches == bins
+        assert np.array_equal(got, ref)
+        h_bytes = plan.info()["h_bytes"]
+        plan.build_holographic()  # built already: nothing to do
+        assert plan.info()["h_bytes"] == h_bytes > 0
+        plan.close()
+        if left > 0:  # more than the build makes
+            break
+    assert survived == 4  # the groups' patches, transform tables, and the apply's jobs and their first blocks
