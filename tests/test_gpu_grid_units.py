@@ -145,3 +145,43 @@ def test_staged_batch_of_many_jobs(bins):
     for k, p in enumerate(plans):
         assert torch.equal(torch.view_as_real(out[k].contiguous()),
                            torch.view_as_real(p.phi_adj_phi(x[k].contiguous())))
+
+
+@pytest.mark.parametrize("kb, op", [(3, "phi_adj"), (3, "phi_adj_phi"), (7, "phi_adj_phi")])
+def test_scaling_by_powers_of_two_is_exact_up_to_the_largest_numbers(kb, op):
+    """The fixed-point scale of a unit is a power of two that follows its bound, so inputs times 2^k
+    give outputs times 2^k bit for bit, also where the bound is within a doubling or two of the
+    largest FP32 number."""
+    import torch
+
+    import paper_2605_26347_gb300 as pkg
+    n, m, fov = 64, 4 if kb == 3 else 1, math.radians(2.0)  # (wider tiles of several visibilities sum up to overflow)
+    rng = np.random.default_rng(kb)
+    uvw = np.zeros((m, 3))
+    uvw[:, :2] = (10.0 + 3.0 * rng.random((m, 2))) / (2.0 * fov)
+    plan = pkg.Plan(uvw, pkg.default_params(n, n, fov, fov, n_wbins=1, kb_support=kb, max_wsupport=1))
+    size = [np.abs(t.real) + np.abs(t.imag) for t in plan.tiles(np.arange(m))[3]]
+    tmax, t1 = max(s.max() for s in size), max(s.sum() for s in size)
+    if op == "phi_adj":
+        v = (rng.standard_normal(m) + 1j * rng.standard_normal(m)) * np.array([1.0, 1e-2, 1e-4, 1e-6])
+        bound = 2 * tmax * (np.abs(v.real) + np.abs(v.imag)).max()
+    else:
+        # a point source beside faint ones: |X| over the grid is that of the point source at the
+        # image centre to a few per cent, |Re X| + |Im X| between it and sqrt(2) times it
+        v = np.zeros((n, n), np.complex128)
+        v[30:33, 20:28] = 1e-4 * rng.standard_normal((3, 8))
+        v[n // 2, n // 2] = 1.0
+        bound = 4 * tmax * t1 * float(to_host(plan.zlayer(0))[n // 2, n // 2].real) * math.sqrt(2.0)
+    v = torch.view_as_real(to_dev(v * 1.6 / bound))
+    apply = getattr(plan, op)
+
+    def scaled(k):
+        out = torch.view_as_real(apply(torch.view_as_complex(v * 2.0**k)))
+        plan.status()
+        assert torch.isfinite(out).all()
+        return out.double() * 2.0**-k
+
+    ref = scaled(0)
+    for k in (-60, 20, 125, 126):  # the bound 1.1 to 1.6 times 2^k, 1.1 of it with the phases of X
+        assert torch.equal(scaled(k), ref), k
+    plan.close()
