@@ -2,30 +2,50 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
+#include <string.h>
 
 namespace rimo {
 
+__host__ __device__ __forceinline__ int cis_bits(float v) {
+#ifdef __CUDA_ARCH__
+    return __float_as_int(v);
+#else
+    int i;
+    memcpy(&i, &v, sizeof(i));
+    return i;
+#endif
+}
+__host__ __device__ __forceinline__ float cis_float(int i) {
+#ifdef __CUDA_ARCH__
+    return __int_as_float(i);
+#else
+    float v;
+    memcpy(&v, &i, sizeof(v));
+    return v;
+#endif
+}
+
 // (cos, sin) of 2 pi r for |r| <= 1/2 (a little more does no harm): the nearest quarter turn q is
 // split off by a rounding shift (1.5 x 2^23 gives 4 r + it unit spacing), and the remainder
-// |f| <= 1/8 goes through the Taylor series of sin and cos in x = 2 pi f, |x| <= pi / 4, to x^9
-// and x^10 (first omitted terms 2e-9 and 1e-10; against 64 bits over a turn: at most 8.7e-8,
-// 1.9e-8 rms, where rounding alone is 1.5e-8).  About 25 instructions, none on the special
-// function unit, where sincospif took about 45 with four there (row
-// passes 2 to 6 % faster: forward rows of 4096^2 / 32 bins 5.33 -> 5.21 ms)
-__device__ __forceinline__ float2 cis_turn(float r) {
-    const float t = __fadd_rn(4.f * r, 12582912.f);
-    const int q = __float_as_int(t);
-    const float f = fmaf(__fsub_rn(t, 12582912.f), -0.25f, r);
+// |f| <= 1/8 goes through polynomials in g = f^2, sin(2 pi f) = f (6.28125 + p(g)) (6.28125 is exact in
+// FP32, so that the product with the leading term is rounded once) and cos(2 pi f) = 1 + g (...).  Their
+// coefficients are minimax fits (linear programme over [0, 1/64]; relative error 3.6e-9 of the sine,
+// 4e-10 of the cosine), each rounded to FP32 before the next ones are fitted.  Against 64 bits, over
+// a turn: at most 5.2e-8, 0.86 ulp, 1.50e-8 rms; sincospif 5.3e-8, 0.97 ulp, 1.51e-8 (the Taylor
+// series with 2 pi in one FP32 number, two terms more: 8.8e-8, 1.7 ulp, 1.9e-8).  About 24
+// instructions, none on the special function unit, where sincospif took about 45 with four there
+// (row passes 2 to 6 % faster: forward rows of 4096^2 / 32 bins 5.33 -> 5.21 ms).
+__host__ __device__ __forceinline__ float2 cis_turn(float r) {
+    const float t = 4.f * r + 12582912.f;  // (4 r is exact: the same with or without a fused multiply-add)
+    const int q = cis_bits(t);
+    const float f = fmaf(t - 12582912.f, -0.25f, r);
     const float g = f * f;
-    // sin: f (2 pi - (2 pi)^3 / 3! g + ...), cos: 1 - (2 pi)^2 / 2! g + ...
-    const float s = f * fmaf(g, fmaf(g, fmaf(g, fmaf(g, 42.0586939448f, -76.7058597531f), 81.6052492761f), -41.3417022404f),
-                             6.2831853072f);
-    const float c = fmaf(g, fmaf(g, fmaf(g, fmaf(g, fmaf(g, -26.4262567834f, 60.2446413719f), -85.4568172066f), 64.9393940227f),
-                                 -19.7392088022f),
-                         1.f);
+    const float p = fmaf(g, fmaf(g, fmaf(g, -75.3683167f, 81.5918808f), -41.3416595f), 1.9352868e-3f);
+    const float s = fmaf(f, 6.28125f, f * p);
+    const float c = fmaf(g, fmaf(g, fmaf(g, fmaf(g, 58.5611687f, -85.4231186f), 64.9391403f), -19.7392082f), 1.f);
     const float cq = (q & 1) ? s : c, sq = (q & 1) ? c : s;  // up to sign
-    return make_float2(__int_as_float(__float_as_int(cq) ^ (((q + 1) & 2) << 30)),
-                       __int_as_float(__float_as_int(sq) ^ ((q & 2) << 30)));
+    return make_float2(cis_float(cis_bits(cq) ^ (((q + 1) & 2) << 30)), cis_float(cis_bits(sq) ^ ((q & 2) << 30)));
 }
 
 }  // namespace rimo
