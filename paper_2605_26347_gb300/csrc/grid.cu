@@ -132,11 +132,11 @@ __device__ __forceinline__ void fx_scale(float maxterm, int n, float& s1, float&
     s1 = 1.f;
     inv = 1.f;
     if (!(maxterm > 0.f)) return;  // all contributions vanish (or the input was flagged)
-    const float lim = fminf(2097152.f, 1073741824.f / (float)(n > 1 ? n : 1));
-    // the exponent of lim / maxterm: the difference of theirs, one less where lim has the smaller
-    // significand (an approximate division gives 0 for divisors above 2^126)
-    const uint32_t a = __float_as_uint(lim), b = __float_as_uint(maxterm);
-    int ex = (int)(a >> 23) - (int)(b >> 23) - ((a & 0x7fffffu) < (b & 0x7fffffu) ? 1 : 0);
+    // = 2^30 / N, N = max(n, 512): with maxterm = m 2^e, 1 <= m < 2, the exponent 30 - e - ceil(log2(m N)),
+    // for any normal maxterm (an approximate division gives 0 for divisors above 2^126)
+    const uint32_t b = __float_as_uint(maxterm);
+    const uint32_t q = __float_as_uint(__uint_as_float((b & 0x7fffffu) | 0x3f800000u) * (float)max(n, 512));
+    int ex = 30 - ((int)(b >> 23) - 127) - ((int)((q + 0x7fffffu) >> 23) - 127);
     ex = ex < -120 ? -120 : (ex > 120 ? 120 : ex);
     s1 = __uint_as_float((uint32_t)(ex + 127) << 23);
     inv = __uint_as_float((uint32_t)(127 - ex) << 23);
