@@ -87,7 +87,9 @@ static void inv(rimo_plan* p, int b, float2* out, bool first, int real_only, cud
     prof_end(p, 1, s);
 }
 
-// Plans without stored G: the tiles of bins [b0, b1] into the tap scratch.
+// Plans without stored G: the tiles of bins [b0, b1] into the tap scratch.  Their largest tap raises
+// the plan's bound before the grid step of any of them, so a bin's fixed-point scale may be coarser
+// than by itself by the ratio of its largest tap to the run's (2^-36 of the bound instead of 2^-37).
 static void generate(rimo_plan* p, int b0, int b1, cudaStream_t s) {
     const int64_t v0 = p->bins[b0].vb, n = p->bins[b1].ve - v0;
     if (p->mode == RIMO_MODE_SURROGATE) {
@@ -111,11 +113,15 @@ static void gtg(rimo_plan* p, int b, int mode, const float2* y_in, float2* y_out
 // ---- the bins of a plan in groups
 // A pass over one bin of a small image does not fill the GPU: its grid is nx ny / 4096 blocks,
 // 304 of which are resident at once, and 4 bins of 256^2 took 27 launches of 4 to 10 us.  Plans
-// of several bins whose passes have fewer than STAGE_BLOCKS blocks therefore run as many bins
-// at a time, every pass one launch over a table of (bin) jobs with a grid, half transforms
-// and patches of their own (the kernels and the order of every sum are those of one bin at a
-// time, so the results are the same bit for bit).  The scratch of a group is at most
-// STAGE_BYTES; from 2048^2 on that is less than two bins, whose passes fill the GPU anyway.
+// of several bins, two of which have at most STAGE_BLOCKS blocks in a pass, therefore run as many
+// bins at a time as have about that many, every pass one launch over a table of (bin) jobs with a
+// grid, half transforms and patches of their own.  The kernels and the order of every sum are those
+// of one bin at a time, so with stored G and with H the results are the same bit for bit; generated
+// tiles share the bound of their run of bins (see generate), so that the fixed-point scale, hence
+// the last bits, may depend on whether memory allowed a run.  The scratch of a group is at most
+// STAGE_BYTES.  The line lies between 2048 x 1024 (512 blocks a bin; 20k visibilities, 6 bins,
+// groups of three 0.656 ms, one by one 0.706; 5M, 8 bins 2.99 and 3.06) and 2048^2 (1024 blocks; 2k
+// visibilities, 4 bins, two by two 0.677 and 0.677 ms for 512 MiB).
 // Plans that generate their tiles do so for as many bins of a group as fit STAGE_TAPS (at
 // 1024^2/1M/16 bins, generation and grid step of four bins instead of one at a time: tabulated
 // kernels 0.82 -> 0.56 and 0.96 -> 0.87 ms per apply, the network 1.03 -> 0.80 ms).
@@ -160,8 +166,9 @@ void stage_bins(rimo_plan* p, bool share_taps) {
     int nb = 0;
     for (int b = 0; b < p->P; ++b) nb += p->bins[b].t1 > p->bins[b].t0;
     const int per_bin = std::max(1, p->nx * p->ny / 4096);
-    const int64_t most = std::min<int64_t>({(int64_t)nb, (STAGE_BLOCKS + per_bin - 1) / per_bin,
-                                            STAGE_BYTES / BinScratch(p).total()});
+    const int64_t most =
+        2 * per_bin > STAGE_BLOCKS ? 1 : std::min<int64_t>({(int64_t)nb, (STAGE_BLOCKS + per_bin - 1) / per_bin,
+                                                            STAGE_BYTES / BinScratch(p).total()});
     // groups of nearly equal size
     const int64_t ng = most < 2 ? nb : (nb + most - 1) / most;
     p->stage_each = ng > 0 ? (int)((nb + ng - 1) / ng) : 1;

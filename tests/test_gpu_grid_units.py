@@ -40,16 +40,41 @@ def test_units_of_every_size_and_tile_side(m, kb, cap, tile, spread):
     plan.close()
 
 
+def row_passes(plan, call):
+    """Launches of the forward row pass in a call: one per group of bins, or per bin."""
+    plan.profile_read()
+    plan.profile(True)
+    call()
+    plan.profile(False)
+    return plan.profile_read()["fwd_rows"][1]
+
+
+def test_no_groups_where_a_bins_passes_fill_the_gpu():
+    """At 2048^2 two bins side by side are no faster than one after the other: no scratch for them."""
+    import synth
+
+    import paper_2605_26347_gb300 as pkg
+    n, bins, fov = 2048, 4, math.radians(2.0)
+    plan = pkg.Plan(synth.make_uvw(500, 60, 1.28e9, 11), pkg.default_params(n, n, fov, fov, n_wbins=bins))
+    x = to_dev(np.ones((n, n)))
+    assert row_passes(plan, lambda: plan.phi_adj_phi(x)) == bins
+    # one bin's scratch: 2 n^2 half transforms, 4 n^2 grid, n^2 delta image, patches
+    assert plan.info()["scratch_bytes"] < 8 * 8 * n * n
+    plan.close()
+
+
 @pytest.mark.parametrize("nx, ny, m, bins, kw", [
     (64, 64, 500, 2, {}), (64, 64, 40, 9, {}), (256, 64, 3000, 5, {}), (64, 256, 3000, 5, dict(tile_size=64)),
     (512, 512, 20000, 23, {}), (1024, 1024, 30000, 7, {}), (4096, 64, 3000, 3, {}), (64, 4096, 3000, 3, {}),
     (128, 128, 4000, 4, dict(mode=4, wkernel_table=64)), (128, 128, 4000, 4, dict(kb_support=11)),
+    (2048, 1024, 3000, 3, {}),
 ])
 def test_bins_in_groups_equal_one_bin_at_a_time(nx, ny, m, bins, kw):
     """Plans of small images run their bins in groups; a call that selects every bin by a mask
     takes them one at a time: the same sums in the same order, bit for bit with stored G.  With
     tiles generated per group the fixed-point scale comes from the group's tap bound, which may
-    be a power of two above a bin's: 2^-46 of the bound, far below an FP32 rounding."""
+    be a power of two above a bin's: 2^-36 of the bound instead of 2^-37 per contribution, far below
+    an FP32 rounding."""
     import synth
     import torch
 
@@ -60,6 +85,8 @@ def test_bins_in_groups_equal_one_bin_at_a_time(nx, ny, m, bins, kw):
     plan = pkg.Plan(uvw, pkg.default_params(nx, ny, fov_x, fov_y, n_wbins=bins, **kw))
     rng = np.random.default_rng(5)
     x = torch.from_numpy((rng.standard_normal((ny, nx)) + 1j * rng.standard_normal((ny, nx))).astype(np.complex64)).cuda()
+    assert row_passes(plan, lambda: plan.phi_adj_phi(x)) < row_passes(
+        plan, lambda: plan.phi_adj_phi_bins(x, np.ones(bins, np.uint8)))  # the plan has groups
     for real in (False, True):
         a = plan.phi_adj_phi(x, real_part_only=real)
         b = plan.phi_adj_phi_bins(x, np.ones(bins, np.uint8), real_part_only=real)
