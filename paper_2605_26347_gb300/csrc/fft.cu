@@ -30,8 +30,6 @@
 #include <cstring>
 #include <cstdio>
 
-#include <map>
-#include <mutex>
 #include <type_traits>
 
 #include "internal.h"
@@ -1110,21 +1108,6 @@ static void launch_clustered(void (*kernel)(KArgs...), int grid, int block, size
     at[1].val.clusterSchedulingPolicyPreference = cudaClusterSchedulingPolicyLoadBalancing;
     cfg.numAttrs = 2;
     RIMO_CUDA(cudaLaunchKernelEx(&cfg, kernel, args...));
-}
-
-// Raises a kernel's dynamic shared-memory limit once per (device, kernel, size).
-template <class K>
-static void set_smem(K kernel, size_t bytes) {
-    static std::mutex mu;
-    static std::map<std::pair<int, const void*>, size_t> done;
-    int dev = 0;
-    RIMO_CUDA(cudaGetDevice(&dev));
-    std::lock_guard<std::mutex> lock(mu);
-    size_t& have = done[{dev, reinterpret_cast<const void*>(kernel)}];
-    if (have < bytes) {
-        RIMO_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-        have = bytes;
-    }
 }
 
 #define RIMO_DISPATCH_N(N_, CALL)                                                      \

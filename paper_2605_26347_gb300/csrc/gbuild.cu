@@ -534,7 +534,7 @@ void launch_kwtab(const rimo_plan* p, cudaStream_t s) {
     const size_t sm = gbuild_smem(p->L, p->hmax);
     void (*kern)(BuildArgs) = p->L == 16 ? kwtab_kernel<16> : p->L == 32 ? kwtab_kernel<32>
                             : p->L == 64 ? kwtab_kernel<64> : kwtab_kernel<128>;
-    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    set_smem(kern, sm);
     const int blocks = (p->kw_n + 3 + BUILD_WARPS - 1) / BUILD_WARPS;
     kern<<<blocks, BUILD_WARPS * 32, sm, s>>>(A);
     RIMO_CUDA(cudaGetLastError());
@@ -548,7 +548,7 @@ void launch_gbuild_range(const rimo_plan* p, int64_t v0, int64_t n, cudaStream_t
     const size_t sm = gbuild_smem(p->L, p->hmax);
     void (*kern)(BuildArgs) = p->L == 16 ? gbuild_kernel<16> : p->L == 32 ? gbuild_kernel<32>
                             : p->L == 64 ? gbuild_kernel<64> : gbuild_kernel<128>;
-    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    set_smem(kern, sm);
     int dev = 0, nsm = 0;
     RIMO_CUDA(cudaGetDevice(&dev));
     RIMO_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));

@@ -654,7 +654,7 @@ static void gtg_run(const rimo_plan* p, int bin, const float2* y_in, float2* y_o
     A.y_out = y_out;
     const GtgShape g = gtg_shape(p, p->PW, p->max_S, MODE, A);
     void (*kern)(GtgArgs) = gtg_kernel_for<MODE>(p->PW);
-    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+    set_smem(kern, g.smem);
     kern<<<std::min(nu, p->n_sm * g.blocks_per_sm), g.warps * 32, g.smem, s>>>(A);
     if (MODE != 0 && br.m1 > br.m0) {
         MergeJob mj;
@@ -784,7 +784,7 @@ int wide_gtg(const WideGtg* w, int mode, const float2* y_in, float2* y_out, cuda
     A.y_out = y_out;
     const int pw = w->one_pw ? w->PW : 0;
     void (*kern)(GtgArgs) = mode == 0 ? gtg_kernel_for<0>(pw) : mode == 1 ? gtg_kernel_for<1>(pw) : gtg_kernel_for<2>(pw);
-    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+    set_smem(kern, g.smem);
     if (w->own_counter) RIMO_CUDA(cudaMemsetAsync(w->counter, 0, sizeof(int), s));
     kern<<<(int)std::min<int64_t>(w->units, (int64_t)w->p0->n_sm * g.blocks_per_sm), g.warps * 32, g.smem, s>>>(A);
     if (mode == 0 || w->merge_blocks == 0) return 1;

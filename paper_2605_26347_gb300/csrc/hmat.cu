@@ -681,7 +681,7 @@ static void happly_launch(const rimo_plan* p, const HApplyArgs& one, const HAppl
     if (blocks <= 0) return;
     auto kern = happly_for(p->max_S);
     const size_t sm = happly_smem(p->PW, p->max_S, compressed);
-    RIMO_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    set_smem(kern, sm);
     kern<<<blocks, HA_WARPS * 32, sm, s>>>(one, jobs, first, njobs);
 }
 
@@ -876,7 +876,7 @@ static void build_holographic(rimo_plan* p, cudaStream_t s) {
     p->d_hpatch = (float2*)dev_alloc(p, patch_bytes);
     const size_t sm = hbuild_smem(ne, p->max_S, D);
     if (sm > 227 * 1024) fail(RIMO_ERR_UNSUPPORTED, "holographic build: owner rows exceed shared memory");
-    RIMO_CUDA(cudaFuncSetAttribute(hbuild_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    set_smem(hbuild_kernel, sm);
     const int per_tile = (TS / HB_OWN) * (TS / HB_OWN);
     // bin by bin: dense rows into a temporary, then only their non-zero entries kept
     std::vector<void*> made;  // the compressed arrays, released again if the budget refuses

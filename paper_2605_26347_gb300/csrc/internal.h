@@ -47,6 +47,14 @@ template <class T>
 cudaError_t device_malloc(T** ptr, size_t bytes) {
     return device_malloc_bytes(reinterpret_cast<void**>(ptr), bytes);
 }
+// Raises a kernel's dynamic shared-memory limit on the current device to `bytes` where it is lower.
+// The limit belongs to the process: lowered to one plan's need, it would refuse the launch of a
+// larger plan that another thread is about to make.
+void raise_smem(const void* kernel, size_t bytes);
+template <class K>
+void set_smem(K kernel, size_t bytes) {
+    raise_smem(reinterpret_cast<const void*>(kernel), bytes);
+}
 
 // ---------------------------------------------------------------------------
 // Per-visibility metadata in sorted (bin, uv-tile) order, 16 bytes.

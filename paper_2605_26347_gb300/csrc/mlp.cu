@@ -14,7 +14,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <random>
@@ -211,13 +210,7 @@ __global__ void __launch_bounds__(128) gemm_tc_kernel(GemmArgs g) {
 static void gemm(const bf16* A, int lda, const bf16* B, int ldb, float* C, int ldc, int M, int N, int K, int nt,
                  int splits, bool atomic, int* status, cudaStream_t s, int m_store = 1 << 30) {
     constexpr int most = 2 * (128 + GEMM_MAX_NT) * GEMM_KC * 2;
-    static std::atomic<uint64_t> ready{0};  // devices whose limit is raised
-    int dev = 0;
-    RIMO_CUDA(cudaGetDevice(&dev));
-    if (dev >= 64 || !((ready.load() >> dev) & 1u)) {
-        RIMO_CUDA(cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-        if (dev < 64) ready.fetch_or(1ull << dev);
-    }
+    set_smem(gemm_tc_kernel, most);
     GemmArgs g;
     g.A = A;
     g.B = B;
@@ -945,7 +938,7 @@ int surrogate_generate(rimo_plan* p, int64_t v0, int64_t n, cudaStream_t s) {
     A.fx = p->d_fx;
     A.status = p->d_status;
     A.wt = p->d_wt;
-    RIMO_CUDA(cudaFuncSetAttribute(sur_gen_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GEN_SMEM));
+    set_smem(sur_gen_kernel, GEN_SMEM);
     const int64_t ntile = (n + 127) / 128;
     const int grid = (int)std::min<int64_t>(ntile, (int64_t)p->n_sm);
     sur_gen_kernel<<<grid, GEN_THREADS, GEN_SMEM, s>>>(A);

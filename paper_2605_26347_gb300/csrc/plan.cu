@@ -5,6 +5,8 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <numeric>
 #include <string>
 
@@ -33,6 +35,19 @@ static thread_local int64_t t_alloc_test = 0;  // rimo_set_alloc_test: calls unt
 cudaError_t device_malloc_bytes(void** ptr, size_t bytes) {
     if (t_alloc_test > 0 && --t_alloc_test == 0) return cudaErrorMemoryAllocation;
     return cudaMalloc(ptr, bytes);
+}
+
+void raise_smem(const void* kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> done;
+    int dev = 0;
+    RIMO_CUDA(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    size_t& have = done[{dev, kernel}];
+    if (have < bytes) {
+        RIMO_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        have = bytes;
+    }
 }
 
 void* dev_alloc(rimo_plan* p, size_t bytes) {

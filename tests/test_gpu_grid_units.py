@@ -212,3 +212,43 @@ def test_scaling_by_powers_of_two_is_exact_up_to_the_largest_numbers(kb, op):
     for k in (-60, 20, 125, 126):  # the bound 1.1 to 1.6 times 2^k, 1.1 of it with the phases of X
         assert torch.equal(scaled(k), ref), k
     plan.close()
+
+
+def test_plans_of_other_shapes_in_other_threads():
+    """The grid step's kernel for run-time strides serves plans of 13 x 13 and of 19 x 19 tiles, whose
+    blocks need different shared memory: launches from two threads do not disturb each other."""
+    import threading
+
+    import torch
+
+    import paper_2605_26347_gb300 as pkg
+    n, fov, m = 64, math.radians(2.0), 300
+    rng = np.random.default_rng(2)
+    uvw = (rng.random((m, 3)) - 0.5) * np.array([2 * n / (2 * fov), 2 * n / (2 * fov), 3000.0])
+    x = to_dev(rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n)))
+    work = []
+    for kb in (5, 11):
+        plan = pkg.Plan(uvw, pkg.default_params(n, n, fov, fov, n_wbins=1, kb_support=kb))
+        work.append((plan, torch.cuda.Stream(), plan.phi_adj_phi(x), torch.empty_like(x)))
+    torch.cuda.synchronize()
+    failed = []
+
+    def run(plan, stream, ref, out):
+        try:
+            for _ in range(400):
+                plan.phi_adj_phi(x, out=out, stream=stream)
+            stream.synchronize()
+            if not torch.equal(torch.view_as_real(out), torch.view_as_real(ref)):
+                failed.append("result")
+        except Exception as e:
+            failed.append(e)
+
+    threads = [threading.Thread(target=run, args=w) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed
+    for plan, *_ in work:
+        plan.status()
+        plan.close()
