@@ -1,10 +1,10 @@
 """Failure detection on the device without a fault (GPU).
 
 Every wait of the grid step is bounded.  rimo_plan_set_wait_test makes one of them run
-out: the consumer warps withhold their release of tap-ring slots (a flag that nothing
-sets) and the producer's waits on them give up after a few polls.  The launch must end by
-itself, the plan's status must report RIMO_ERR_TIMEOUT (and clear), and the next apply
-at the normal limit must be clean and equal, bit for bit, to the apply before the test.
+out: every warp fills the slots of its tap ring once and never again (a copy that nothing
+starts), and its waits for taps give up after a few polls.  The launch must end by itself,
+the plan's status must report RIMO_ERR_TIMEOUT (and clear), and the next apply at the normal
+limit must be clean and equal, bit for bit, to the apply before the test.
 """
 import math
 import time
@@ -22,9 +22,9 @@ TIMEOUT = 5
 
 @pytest.mark.parametrize("n, m, fov_deg", [
     # 128^2, 20k visibilities, one w-bin: a few dozen uv-tiles of ~300 visibilities, so every
-    # block of the grid step streams more tap chunks than its ring holds (two X buffers)
+    # warp of the grid step has more visibilities than its ring has slots
     (128, 20000, 2.0),
-    # 512^2, 60k visibilities: units of a few chunks (three X buffers, two units ahead)
+    # 512^2, 60k visibilities: units of a few visibilities per warp, blocks that take several units
     (512, 60000, 2.0),
 ])
 def test_bounded_wait_runs_out_then_the_plan_recovers(n, m, fov_deg):
@@ -41,7 +41,7 @@ def test_bounded_wait_runs_out_then_the_plan_recovers(n, m, fov_deg):
     t = time.time()
     plan.phi_adj_phi(x)
     torch.cuda.synchronize()
-    assert time.time() - t < 2.0          # each block gives up after <= 16 polls of <= 100 us
+    assert time.time() - t < 2.0          # each warp gives up after <= 16 polls of <= 100 us
     with pytest.raises(pkg.RimoError) as e:
         plan.status()
     assert e.value.status == TIMEOUT

@@ -1,5 +1,6 @@
-"""Gradients of the surrogate at batch sizes around its tiles (GPU): one 128-row tile, odd
-numbers of them (odd splits of the weight-gradient products), a full training batch."""
+"""The surrogate at the batch sizes it takes, multiples of 128 (GPU): gradients and forward pass of
+one 128-row tile, odd numbers of them (odd splits of the weight-gradient products), a full
+training batch; smaller batches in the buffers of larger ones."""
 import numpy as np
 import pytest
 
@@ -36,3 +37,17 @@ def test_weight_gradients_of_the_last_outputs(net, B):  # noqa: F811
     g = pkg.unpack_params(s.gradients(x, t)[1])["W3"]
     for j in range(384, 450):
         assert rel(g[j], ref["W3"][j]) < 2e-3, (j, rel(g[j], ref["W3"][j]))
+
+
+@pytest.mark.parametrize("sizes", [(128, 384, 1408), (4096, 128, 1408)])
+def test_forward_of_any_batch(sizes):
+    """The forward pass alone (no transposed activations), in growing buffers and in those of a larger
+    batch and of its gradients; bf16 flips as in test_gpu_surrogate."""
+    import paper_2605_26347_gb300 as pkg
+    s = pkg.Surrogate(seed=0)
+    p = {k: v.astype(np.float64) for k, v in pkg.unpack_params(s.get_params()).items()}
+    for B in sizes:
+        x, t = batch(B, B + 2)
+        y = s.forward(x).cpu().numpy().astype(np.float64)
+        assert rel(y, omlp.forward(p, x.astype(np.float64), bf=True)["y"]) < 1e-3, B
+        s.gradients(x, t)
