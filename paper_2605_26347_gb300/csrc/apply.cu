@@ -50,10 +50,7 @@ static void prof_collect(rimo_plan* p) {
     p->prof_pending.clear();
 }
 
-static int gtg_launches(const rimo_plan* p, int b, int mode) {
-    (void)mode;
-    return p->bins[b].t1 > p->bins[b].t0 ? 1 : 0;
-}
+static int gtg_launches(const rimo_plan* p, int b) { return p->bins[b].t1 > p->bins[b].t0 ? 1 : 0; }
 
 static void check_plan(rimo_plan* p) {
     if (!p) fail(RIMO_ERR_INVALID_ARG, "null plan");
@@ -107,7 +104,7 @@ static void gtg(rimo_plan* p, int b, int mode, const float2* y_in, float2* y_out
     prof_begin(p, ST_GTG, s);
     launch_gtg(p, b, mode, y_in, y_out, s);
     const bool merge = mode != 0 && p->bins[b].m1 > p->bins[b].m0;
-    prof_end(p, gtg_launches(p, b, mode) + (merge ? 1 : 0), s);
+    prof_end(p, gtg_launches(p, b) + (merge ? 1 : 0), s);
 }
 
 // ---- the bins of a plan in groups

@@ -4,7 +4,7 @@
 // Section 2 and Section 3.5: the wideband model applies the monochromatic one per
 // channel).  Its Phi^dagger Phi is recorded once into a CUDA graph and replayed by one
 // cudaGraphLaunch per call for as long as the buffers stay the same, in one of two forms:
-//  * staged (plans with stored G and one image, uv-tile, patch and tap-ring shape): every
+//  * staged (plans with stored G, square images of one size and one uv-tile size): every
 //    (channel, w-bin) is a job with its own scratch, and each pass runs as ONE launch over
 //    all jobs - forward rows, forward cols, the grid step as one persistent launch that
 //    takes the work units of every job heaviest first from one queue (channels and bins of
@@ -276,7 +276,7 @@ rimo_status rimo_batch_create_form(const rimo_plan_t* plans, int32_t n_plans, in
     }
     const bool eligible = stage_eligible(b->plans);
     if (form == RIMO_BATCH_STAGED && !eligible)
-        fail(RIMO_ERR_UNSUPPORTED, "staged batches need stored-G plans of one image, tile, patch and ring shape");
+        fail(RIMO_ERR_UNSUPPORTED, "staged batches need stored-G plans of one square image size and one uv-tile size");
     b->staged = form != RIMO_BATCH_BRANCHES && eligible;
     RIMO_CUDA(cudaStreamCreateWithFlags(&b->root, cudaStreamNonBlocking));
     if (b->staged) stage(b, b->root);

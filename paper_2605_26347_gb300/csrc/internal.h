@@ -12,7 +12,7 @@
 namespace rimo {
 // rows of the time interleave of a uv-tile's visibilities (uv_order 0): that many visibilities
 // in a row come from far-apart instants
-constexpr int GTG_CHUNK = 20;
+constexpr int UV_INTERLEAVE = 20;
 
 // ---------------------------------------------------------------------------
 // Error handling: every public entry point catches rimo::Error and returns its status.
@@ -318,8 +318,9 @@ struct WideJob {
 };
 // Job of block b of a launch over a job table: the last job whose first block is <= b
 // (first: njobs + 1 non-decreasing block offsets).  Called by whole warps: 32 candidates per
-// load, where a bisection waits for log2(njobs) loads one after the other (batch of 108 jobs of
-// 1024^2 8.38 -> 8.22 ms; four jobs as before).
+// load, where a bisection waits for log2(njobs) loads one after the other before the block's first
+// row can be asked for (with 108 jobs seven against two; what that gives of a batch of 8.4 ms is no
+// more than the batch varies between runs).
 __device__ __forceinline__ int job_of(const int* first, int njobs, int b) {
     int j = 0;
     for (int n = njobs; n > 1;) {  // the job is one of [j, j + n)

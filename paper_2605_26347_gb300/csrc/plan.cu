@@ -459,17 +459,17 @@ static void create_plan(const double* uvw, int64_t M, const rimo_plan_params& q,
             x.r = std::sqrt(cu * cu + cv * cv);
             // Interleave the tile's visibilities (arrival order within a tile is time, so
             // neighbours are the same few baselines a fraction of a cell apart): viewed
-            // as GTG_CHUNK rows of nc, the new order reads the list column by column, so
+            // as UV_INTERLEAVE rows of nc, the new order reads the list column by column, so
             // that consecutive visibilities, de-gridded and gridded at the same time by as
             // many warps, come from far-apart instants and rarely update the same grid cells.
             // (uv_order 0; 1 keeps the time order; 2 orders the tile's visibilities by a
             // SplitMix64 hash of their index)
             if (q.uv_order == 0) {
-                const int64_t n = x.ve - x.vb, nc = (n + GTG_CHUNK - 1) / GTG_CHUNK;
+                const int64_t n = x.ve - x.vb, nc = (n + UV_INTERLEAVE - 1) / UV_INTERLEAVE;
                 tmp.assign(order.begin() + x.vb, order.begin() + x.ve);
                 int64_t o = x.vb;
                 for (int64_t c = 0; c < nc; ++c)
-                    for (int64_t r = 0; r < GTG_CHUNK; ++r)
+                    for (int64_t r = 0; r < UV_INTERLEAVE; ++r)
                         if (r * nc + c < n) order[o++] = tmp[r * nc + c];
             } else if (q.uv_order == 2) {
                 std::stable_sort(order.begin() + x.vb, order.begin() + x.ve, [](int32_t a, int32_t b) {
