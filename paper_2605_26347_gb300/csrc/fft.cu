@@ -19,8 +19,8 @@
 // 6.90 ms, while the row passes, which also evaluate Z_p per point, were slower so: 5.32 -> 5.55
 // and 4.30 -> 4.61 ms).  What bounds the passes at 4096^2 (32 bins, 24M visibilities, per apply):
 // forward cols 2.91 ms, issue and the FMA pipe (63 and 62 %) and latency; fold + inverse cols 5.25
-// ms, memory latency and the clusters' barriers; forward rows 5.10 ms, barriers (block and cluster), the exchange and the
-// 32-byte pieces of the transposed store (69 % of the load/store pipe); inverse rows 3.98 ms,
+// ms, memory latency and the clusters' barriers; forward rows 5.12 ms, barriers (block and cluster), the exchange and the
+// 32-byte pieces of the transposed store (69 % of the load/store pipe); inverse rows 3.95 ms,
 // memory latency at 4.3 TB/s with two 512-thread rows per SM (with the 8192 points as two halves of
 // 4096, two exchanges instead of three, they took the same 5.18 and 4.09 ms).  The
 // zero padding and the crop are exploited where they cost nothing: forward passes never
